@@ -426,7 +426,7 @@ enum {
   HKBE_PHASE_BOOT = 8,    /* bootstrap square                                  */
   HKBE_PHASE_CTRL = 9,    /* convergence bookkeeping                           */
   HKBE_PHASE_COMPRESS = 10, /* HODLR leaf copy + TSVD block updates (update_blocks) */
-  HKBE_PHASE_CHUNKINV = 11, /* inverses of frozen 32-point sweep chunks           */
+  HKBE_PHASE_CHUNKINV = 11, /* inverses of the 32-point sweep chunks and the head */
   HKBE_NPHASE = 12
 };
 

@@ -51,6 +51,14 @@ struct hkbe_s {
   double2 *rowbuf_r = nullptr, *rowbuf_l = nullptr;
   int* status_dev = nullptr;
   double2* diagbuf = nullptr;  // [n_inst][no2] density matrices of one time
+  // points whose rows the chunk inverses hold (retarded [0, rowsR), lesser [1, rowsL))
+  int rowsR = 0, rowsL = 1;
+  // the rows of a growing chunk's inverse are rebuilt from the first step after a
+  // restart (their FP64 copies are not part of snapshots and files)
+  void restart_rows() {
+    rowsR = 32 * d.nfrozR;
+    rowsL = std::max(1, 32 * d.nfrozL);
+  }
   // device arrays that make up the propagation state, zeroed by hkbe_rewind so
   // that a rewound run starts from exactly the state that followed bootstrap
   std::vector<std::pair<void*, size_t>> state_arrays;
@@ -436,6 +444,16 @@ int hkbe_create(const hkbe_params* p, const int32_t* nt_per_inst, void* stream, 
     return rc;
   }
   h->scratch.insert(h->scratch.end(), {d.cinv_ws, h->diagbuf});
+  {  // inverses of the retarded heads: rebuilt at every step, in neither snapshots nor files
+    const size_t b = (size_t)d.n_inst * 4 * d.k * d.k * d.no * d.no * sizeof(double2);
+    const cudaError_t e = cudaMalloc((void**)&d.hinv, b);
+    if (e != cudaSuccess) {
+      g_create_error = std::string("cudaMalloc: ") + cudaGetErrorString(e);
+      hkbe_destroy(h);
+      return HKBE_ERR_NOMEM;
+    }
+    h->bytes += b;
+  }
   cudaError_t e = cudaStreamSynchronize(h->s);
   if (e != cudaSuccess) {
     g_create_error = std::string("cudaStreamSynchronize: ") + cudaGetErrorString(e);
@@ -452,6 +470,7 @@ int hkbe_destroy(hkbe_t* h) {
   drain(h);
   for (cudaEvent_t e : h->event_pool) cudaEventDestroy(e);
   for (void* p : h->allocs) cudaFree(p);
+  if (h->d.hinv) cudaFree(h->d.hinv);
   for (void* p : h->snap_dev)
     if (p) cudaFree(p);
   delete h;
@@ -616,6 +635,7 @@ int hkbe_set_hamiltonian(hkbe_t* h, const double* eps) {
   HK_CUDA(h, cudaMemcpyAsync(d.eps_ext, eps, cnt * sizeof(double), cudaMemcpyHostToDevice, h->s));
   HK_CUDA(h, cudaStreamSynchronize(h->s));
   h->have_eps = true;
+  if (h->cur >= 0) h->restart_rows();   // eps(t) of the growing chunks may have changed
   return HKBE_OK;
 }
 
@@ -974,19 +994,15 @@ int hkbe_step(hkbe_t* h, int n_steps, int32_t* iters, double* err) {
   bool any_failed = false;
   for (int st = 0; st < n_steps; ++st) {
     const int T = h->cur + 1;
-    // inverses of the chunks that became frozen (their rows are final and far enough from T)
+    // inverses of the sweeps' chunks: append the points that became final, and the head of step T
     if (h->scheme == HKBE_SCHEME_PAPER) {
-      const int tR = std::max(0, (T - 2 * d.k) / 32), tL = std::max(0, T / 32);
-      if (tR > d.nfrozR) {
-        HK_CUDA(h, run_phase(h, HKBE_PHASE_CHUNKINV, tR - d.nfrozR,
-                             [&]() { return hk::launch_chunk_inv(d, 0, d.nfrozR, tR, h->s); }));
-        d.nfrozR = tR;
-      }
-      if (tL > d.nfrozL) {
-        HK_CUDA(h, run_phase(h, HKBE_PHASE_CHUNKINV, tL - d.nfrozL,
-                             [&]() { return hk::launch_chunk_inv(d, 1, d.nfrozL, tL, h->s); }));
-        d.nfrozL = tL;
-      }
+      const int rR = std::max(0, T - 2 * d.k), rL = T;
+      HK_CUDA(h, run_phase(h, HKBE_PHASE_CHUNKINV, 1,
+                           [&]() { return hk::launch_inv_rows(d, T, h->rowsR, rR, h->rowsL, rL, h->s); }));
+      h->rowsR = rR;
+      h->rowsL = rL;
+      d.nfrozR = rR / 32;
+      d.nfrozL = rL / 32;
     }
     HK_CUDA(h, run_phase(h, HKBE_PHASE_EXTRAP, 1, [&]() { return hk::launch_extrapolate(d, T, h->s); }));
     std::vector<int> act0(N);
@@ -1280,6 +1296,7 @@ int hkbe_snapshot_restore(hkbe_t* h) {
   h->d.cdir = h->snap_cdir;
   h->d.nfrozR = h->snap_nfrozR;
   h->d.nfrozL = h->snap_nfrozL;
+  h->restart_rows();
   return HKBE_OK;
 }
 
@@ -1319,6 +1336,7 @@ int hkbe_rewind(hkbe_t* h) {
   HK_CUDA(h, put_tv(h->snap_stv, d.STV));
   HK_CUDA(h, hk::launch_diag_seed(d, h->s));
   d.nfrozR = d.nfrozL = 0;
+  h->restart_rows();
   if (h->hodlr) {
     d.cdir = 0;
     for (int X = 0; X < 4; ++X)
@@ -1533,6 +1551,7 @@ int hkbe_load(const char* path, void* stream, hkbe_t** out) {
   d.cdir = sc.cdir;
   d.nfrozR = sc.nfrozR;
   d.nfrozL = sc.nfrozL;
+  h->restart_rows();
   *out = h;
   return HKBE_OK;
 }

@@ -5,19 +5,27 @@
 //
 // Within one chunk the unknowns couple through the near-diagonal part of the
 // discretised equation: the BDF stencil, eps, and Sigma^R entries inside the
-// chunk with their Gregory weights.  Once every coefficient of that local
-// system is final and its weights no longer depend on T, the system is frozen
-// and its inverse is computed once (k_chunk_inv) and reused at every later
-// iteration and step:
-//   retarded chunk [a, a+32): frozen when a + 32 + 2k <= T (all points see the
-//     standard Gregory weights at their end of the integral, and no row of the
-//     chunk is within k of T);
-//   lesser chunk [a, a+32): frozen when a + 32 <= T (its rows are final; the
-//     lesser weights depend on the row and column only).  Chunk 0 holds rows
-//     1..31 including the start block.
+// chunk with their Gregory weights.  Row T of Sigma^R, the only one that the
+// corrector iterations of step T change, multiplies known values there
+// (retarded: y(T) = -i) or belongs to one unknown (lesser: x(T)), so the
+// coefficients between the other unknowns are final before the step's first
+// iteration.  k_inv_rows brings the inverses of these triangular systems up
+// to date once per step and instance, one appended row at a time:
+//   retarded chunk [a, a+32): points t' < T - 2k, whose integrals end in the
+//     standard Gregory weights; the 2k points above them (the head: the start
+//     block and the points of the k < n < 2k+1 rule) form a system of their
+//     own, inverted anew for every T;
+//   lesser chunk [a, a+32): rows t < T; chunk 0 holds rows 1..31 and begins
+//     with the start block.  Row T (horizontal density matrix) is one point
+//     solve at the end.
 // A chunk's solve is then F times the inverse (retarded, row vector) or the
 // inverse times F (lesser), where F holds everything outside the chunk (the
-// far field).  Only the chunks near T are solved point by point in one warp.
+// far field), also for the chunk that is still growing, so no point waits
+// for its neighbour.  Solving the growing chunks point by point in one warp
+// (a chain of up to 64 FP64 point solves per sweep, and an LU of the start
+// block) took 75 of the 89 thousand cycles of a retarded sweep at N_o = 1,
+// T <= 64, and 820 of 1900 thousand at N_o = 4, T = 290; the two sweeps of
+// those runs went from 89 to 35 us and from 1650 to 1040 us.
 #include "bulk_copy.cuh"
 #include "hodlr_util.cuh"
 
@@ -27,18 +35,14 @@ namespace {
 
 constexpr int CK = 32;   // chunk length
 using Y = double2;       // element type of the row / column being solved
-template <int NO> constexpr bool kStage = NO <= 2;   // hot-chunk coefficients staged in shared memory
+template <int NO> constexpr bool kStage = NO <= 2;   // chunk inverses staged in shared memory
 template <int NO> constexpr size_t kStageBytes = kStage<NO> ? sizeof(zd) * CK * CK * NO * NO : 0;
-// Bytes of a frozen chunk inverse that are staged in shared memory (the
-// dynamic buffer of the hot-chunk coefficients, free while a frozen chunk is
-// solved) by a bulk copy issued before the chunk's far field, so the copy
-// overlaps that phase: the whole inverse (FP64, or the hi and lo matrices of
-// the complex64 form, 16 bytes per entry either way); 0 (read from global
-// memory) for N_o > 2.
+// Bytes of a chunk inverse that are staged in shared memory by a bulk copy
+// issued before the chunk's far field, so the copy overlaps that phase: the
+// whole inverse (FP64, or the hi and lo matrices of the complex64 form, 16
+// bytes per entry either way); 0 (read from global memory) for N_o > 2.
 template <int NO, typename S>
 constexpr uint32_t kInvStage = kStage<NO> ? (uint32_t)(CK * NO * CK * NO * sizeof(double2)) : 0u;
-static_assert(kInvStage<2, double2> <= kStageBytes<2> && kInvStage<1, double2> <= kStageBytes<1>,
-              "a staged inverse must fit the hot-chunk buffer");
 constexpr int kCopyWaitPolls = 1 << 20;   // bound of the wait for a staged inverse
 
 // Sum over the 8 lanes of an aligned lane group of their history
@@ -67,7 +71,7 @@ struct Row64<NO, double2> {
   __device__ static Y* get(const Dev&, int, int, int, double2* p) { return p; }
 };
 
-// Inverse of frozen chunk cc of sweep `which`, (32 N_o)^2 entries.  FP64
+// Inverse of chunk cc of sweep `which`, (32 N_o)^2 entries (rows of points not yet built: unused).  FP64
 // storage form: complex128.  Complex64 form: the same 16 bytes per entry
 // hold a complex64 pair hi + lo (hi = the inverse rounded to complex64, lo =
 // the rounding of hi), [hi matrix][lo matrix].  The chunk's right-hand side
@@ -206,8 +210,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
   const int k = d.k, c = d.cdir, L = d.L;
   const double h = d.h;
   const DevW& W = d.w;
-  __shared__ zd sA[20 * 20];
-  __shared__ zd sB[20];
+  __shared__ zd sB[10 * NO];     // right-hand side of the head
   __shared__ zd FB[64][NO];
   __shared__ zd pbuf[8][128];
   __shared__ zd Fs[CK][NO];
@@ -216,9 +219,9 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
   __shared__ zf Ff[CK][NO];      // complex64 form: the far field (Fs - Fb) rounded to complex64
   __shared__ cff FbF[CK][NO];    // complex64 form: Fb in float-float
   __shared__ double serr;
-  extern __shared__ __align__(16) zd ctile[];  // [CK][CK][NO2] hot-chunk coefficients (N_o <= 2);
+  extern __shared__ __align__(16) zd ctile[];  // for each chunk its staged inverse (N_o <= 2);
                                  // at leaf entry (staged != 0) the block projections
-                                 // [maxl][NO2][rmax]; for a frozen chunk its staged inverse
+                                 // [maxl][NO2][rmax]
   __shared__ __align__(8) uint64_t cbar;   // completion of the inverse's bulk copy
   __shared__ int s_stage;                  // 0 once a wait for a copy has timed out
   uint32_t cphase = 0;
@@ -238,47 +241,48 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
   auto yp = [&](int tp) { return rowy + (long long)tp * NO2 + irow * NO; };
   auto sp = [&](int tp) { return rowp + (long long)tp * NO2 + irow * NO; };
   double myerr = 0.0;
-  // ---- start block t' = T-k .. T-1 (s = 1..k), and y(T) = -i ----
-  const int ns = k * NO;
-  if (warp == 0) {
-    for (int e = lane; e < ns * ns; e += 32) {
-      const int row = e / ns, col = e % ns;
-      const int s = row / NO + 1, j = row % NO, l = col / NO + 1, m = col % NO;
-      zd v = srx_any<NO, S>(d, n, T - l, T - s, m, j) * (-h * W.I0[s][l]);
-      if (m == j) v += zd(0, W.D[s][l] / h);
-      if (l == s) v -= ld(epsp<NO>(d, n, T - s) + m * NO + j);
-      sA[row * ns + col] = v;
-    }
-    for (int row = lane; row < ns; row += 32) {
-      const int s = row / NO + 1, j = row % NO;
-      zd cc = srx_any<NO, S>(d, n, T, T - s, irow, j) * (-h * W.I0[s][0]);
-      if (irow == j) cc += zd(0, W.D[s][0] / h);
-      sB[row] = zd(0, 1) * cc;
-    }
-    __syncwarp();
-    warp_lu_solve(ns, sA, sB, 1, nullptr);
-    for (int row = lane; row < ns; row += 32) {
-      const int s = row / NO + 1, j = row % NO;
-      myerr = fmax(myerr, (sB[row] - ld(sp(T - s) + j)).abs2());
-      st(yp(T - s) + j, sB[row]);
-      if constexpr (Row64<NO, S>::separate) st(sp(T - s) + j, sB[row]);
-    }
-    if (lane == 0) {
-      for (int j = 0; j < NO; ++j) {
-        zd v = (j == irow) ? zd(0, -1) : zd();
-        myerr = fmax(myerr, (ld(sp(T) + j) - v).abs2());
-        st(yp(T) + j, v);
-        if constexpr (Row64<NO, S>::separate) st(sp(T) + j, v);
+  // ---- the head: points T-s, s = 1..hs, and y(T) = -i.  Its right-hand side
+  // is row T of Sigma^R (and the derivative's y(T) term) alone; 8 threads per
+  // element of the product with the head's inverse ----
+  const int hs = min(2 * k, T), nh = hs * NO;
+  for (int e = tid; e < nh; e += blockDim.x) {
+    const int s = e / NO + 1, j = e % NO;
+    zd cc = ld(el<NO, S>(d.SR, d, n, T, T - s) + irow * NO + j) * (-h * (s <= k ? W.I0[s][0] : rule_w(W, s, 0)));
+    if (s <= k && irow == j) cc += zd(0, W.D[s][0] / h);
+    sB[e] = zd(0, 1) * cc;
+  }
+  __syncthreads();
+  {
+    const double2* Hi = d.hinv + (long long)n * (4 * k * k * NO2);
+    for (int o8 = tid; o8 < nh * 8; o8 += blockDim.x) {
+      const int o = o8 >> 3, sl = o8 & 7, s = o / NO + 1, j = o % NO;
+      const int nb = max(s, min(k, hs)) * NO;   // the inverse is lower triangular below the start block
+      zd y = zd();
+      for (int b = sl; b < nb; b += 8) y = cfma(ld(Hi + (long long)o * nh + b), sB[b], y);
+      const unsigned grp = 0xffu << (lane & 24);
+#pragma unroll
+      for (int off = 1; off < 8; off <<= 1)
+        y += zd(__shfl_xor_sync(grp, y.re, off), __shfl_xor_sync(grp, y.im, off));
+      if (sl == 0) {
+        myerr = fmax(myerr, (y - ld(sp(T - s) + j)).abs2());
+        st(yp(T - s) + j, y);
+        if constexpr (Row64<NO, S>::separate) st(sp(T - s) + j, y);
       }
     }
   }
+  if (tid < NO) {
+    const zd v = (tid == irow) ? zd(0, -1) : zd();
+    myerr = fmax(myerr, (ld(sp(T) + tid) - v).abs2());
+    st(yp(T) + tid, v);
+    if constexpr (Row64<NO, S>::separate) st(sp(T) + tid, v);
+  }
   __syncthreads();
-  const int top = T - k - 1;
-  for (int cc = top / CK; cc >= 0; --cc) {
+  const int top = T - 2 * k - 1;   // the highest point of the chunks (none while T <= 2k)
+  for (int cc = top >= 0 ? top / CK : -1; cc >= 0; --cc) {
     const int a = cc * CK, b = min(a + CK, top + 1), cn = b - a;
     const bool comp = (c > 0 && b <= c);
     const int jl = comp ? a / L : 0, A = jl * L, E = comp ? (jl + 1) * L : 0;
-    if (comp && b == E) {
+    if (comp && (b == E || b == top + 1)) {   // (the top chunk may end inside its leaf)
       // Entering leaf jl from above.  (1) projections pi_B = sum_s y(s) U_B(s,:) S_B
       // of the blocks whose columns end at E, rows summed in 4 slices.
       for (int lv = 0; lv < d.maxl; ++lv) {
@@ -328,8 +332,8 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
       }
       __syncthreads();
       // projections of every block over this leaf's columns, staged in shared
-      // memory for the far-field loop below (the buffer of the hot-chunk
-      // coefficients, which the chunk solves fill only after it)
+      // memory for the far-field loop below (the buffer of the chunk
+      // inverses, whose copies are issued only after it)
       cx<R>* Ps = reinterpret_cast<cx<R>*>(ctile);
       if (staged) {
         const int per = NO2 * d.rmax;
@@ -417,8 +421,8 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
       }
       __syncthreads();
     }
-    // the frozen inverse of this chunk into shared memory, overlapping the far field
-    const bool stage_now = kInvStage<NO, S> && cc < d.nfrozR && s_stage;
+    // the inverse of this chunk into shared memory, overlapping the far field
+    const bool stage_now = kInvStage<NO, S> && s_stage;
     if (stage_now && tid == 0) bulk_g2s(ctile, Cinv<NO>(d, n, cc, 0), kInvStage<NO, S>, &cbar);
     // ---- far field of the chunk: rows s >= b not covered above; 8 threads per column ----
     {
@@ -489,8 +493,8 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
         for (int j = 0; j < NO; ++j) Old[col][j] = ld(sp(tp) + j);
     }
     __syncthreads();
-    if (cc < d.nfrozR) {
-      // frozen chunk: y = F C^-1 (row vector times the precomputed inverse),
+    {
+      // y = F C^-1 (row vector times the chunk's inverse, lower triangular),
       // 8 threads per output element
       const double2* Mi = Cinv<NO>(d, n, cc, 0);
       bool smem_inv = false;
@@ -513,12 +517,12 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
           const float2* Mh = reinterpret_cast<const float2*>(Mg);
           const float2* Ml = Mh + LD * LD;
           zf s32 = zf(0);
-          for (int si = sl; si < CK; si += 8)
+          for (int si = (ti & ~7) + sl; si < cn; si += 8)
 #pragma unroll
             for (int m = 0; m < NO; ++m)
               s32 = cfma(Ff[si][m], ldr<float>(Mh + (long long)(si * NO + m) * LD + ti * NO + j), s32);
           cff sf = cff_of(s32);
-          for (int si = CK - k + sl; si < CK; si += 8)
+          for (int si = max(cn - k, 0) + sl; si < cn; si += 8)
 #pragma unroll
             for (int m = 0; m < NO; ++m) {
               const long long e = (long long)(si * NO + m) * LD + ti * NO + j;
@@ -529,97 +533,18 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
           for (int off = 1; off < 8; off <<= 1) sf = cff_add(sf, cff_shfl_xor(sf, off));
           if (sl == 0) sacc = cff_val(sf);
         } else {
-          for (int si = sl; si < CK; si += 8)
+          for (int si = (ti & ~7) + sl; si < cn; si += 8)
 #pragma unroll
             for (int m = 0; m < NO; ++m) sacc = cfma(Fs[si][m], ld(Mg + (long long)(si * NO + m) * LD + ti * NO + j), sacc);
 #pragma unroll
           for (int off = 1; off < 8; off <<= 1)
             sacc += zd(__shfl_xor_sync(FULL, sacc.re, off), __shfl_xor_sync(FULL, sacc.im, off));
         }
-        if (sl == 0) {
+        if (sl == 0 && ti < cn) {
           myerr = fmax(myerr, (sacc - Old[ti][j]).abs2());
           st(yp(a + ti) + j, sacc);
           if constexpr (Row64<NO, S>::separate) st(sp(a + ti) + j, sacc);
         }
-      }
-    } else {
-      // chunk near T: right-looking triangular solve in one warp.  Lane L owns
-      // t'' = a + L; after point s is solved every lane with t'' < s removes
-      // y(s) C(s, t'') from its right-hand side.  The coefficients C(s, t'')
-      // are first staged in shared memory by the whole block (N_o <= 2), so
-      // the 32 dependent steps of the solve wait on no global load.
-      auto coef = [&](int i, int L0, zd* cf) {
-        const int spt = a + i, tq = a + L0;
-        const double wl = -h * rule_w(W, T - tq, T - spt);
-        const S* sr = comp ? Lf<NO, S>(d, 2, n, jl, spt, tq) : el<NO, S>(d.SR, d, n, spt, tq);
-        const int dd = spt - tq;
-#pragma unroll
-        for (int q = 0; q < NO2; ++q) {
-          cf[q] = ld(sr + q) * wl;
-          if (dd <= k && (q / NO) == (q % NO)) cf[q] += zd(0, W.a[dd] / h);
-        }
-      };
-      if constexpr (kStage<NO>) {
-        for (int e = tid; e < CK * CK; e += blockDim.x) {
-          const int i = e / CK, L0 = e % CK;
-          if (L0 < i && i < cn) coef(i, L0, ctile + (long long)e * NO2);
-        }
-        __syncthreads();
-      }
-      if (warp == 0) {
-      const int L0 = lane, tq = a + L0;
-      M<NO> Dinv;
-      zd f[NO];
-      if (L0 < cn) {
-        const double ws = h * rule_w(W, T - tq, T - tq);
-        const S* sd = comp ? Lf<NO, S>(d, 2, n, jl, tq, tq) : el<NO, S>(d.SR, d, n, tq, tq);
-        const double2* ep = epsp<NO>(d, n, tq);
-        M<NO> Mm;
-#pragma unroll
-        for (int x = 0; x < NO; ++x)
-#pragma unroll
-          for (int y2 = 0; y2 < NO; ++y2)
-            Mm.a[x][y2] = (x == y2 ? zd(0, W.a[0] / h) : zd()) - ld(ep + x * NO + y2) - ld(sd + x * NO + y2) * ws;
-        Dinv = solve_left<NO>(Mm, M<NO>::eye(zd(1.0)));
-#pragma unroll
-        for (int j = 0; j < NO; ++j) f[j] = Fs[L0][j];
-      }
-      for (int i = cn - 1; i >= 0; --i) {
-        const int spt = a + i;
-        // coefficient C(spt, tq) for this lane (only lanes with tq < spt use it)
-        zd cf[NO2];
-        if (L0 < i) {
-          if constexpr (kStage<NO>) {
-#pragma unroll
-            for (int q = 0; q < NO2; ++q) cf[q] = ctile[(long long)(i * CK + L0) * NO2 + q];
-          } else {
-            coef(i, L0, cf);
-          }
-        }
-        zd y[NO];
-        if (L0 == i) {
-#pragma unroll
-          for (int j = 0; j < NO; ++j) {
-            y[j] = zd();
-#pragma unroll
-            for (int m = 0; m < NO; ++m) y[j] = cfma(f[m], Dinv.a[m][j], y[j]);
-          }
-#pragma unroll
-          for (int j = 0; j < NO; ++j) {
-            myerr = fmax(myerr, (y[j] - ld(sp(spt) + j)).abs2());
-            st(yp(spt) + j, y[j]);
-            if constexpr (Row64<NO, S>::separate) st(sp(spt) + j, y[j]);
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < NO; ++j) y[j] = zd(__shfl_sync(FULL, y[j].re, i), __shfl_sync(FULL, y[j].im, i));
-        if (L0 < i) {
-#pragma unroll
-          for (int m = 0; m < NO; ++m)
-#pragma unroll
-            for (int j = 0; j < NO; ++j) f[j] -= y[m] * cf[m * NO + j];
-        }
-      }
       }
     }
     __syncthreads();
@@ -646,8 +571,6 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
   const int k = d.k, c = d.cdir, L = d.L;
   const double h = d.h;
   const DevW& W = d.w;
-  __shared__ zd sA[20 * 20];
-  __shared__ zd sB[20];
   __shared__ zd FB[64][NO];
   __shared__ zd pbuf[8][128];
   __shared__ zd Fs[CK][NO];
@@ -656,9 +579,9 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
   __shared__ zf Ff[CK][NO];      // complex64 form: the far field (Fs - Fb) rounded to complex64
   __shared__ cff FbF[CK][NO];    // complex64 form: Fb in float-float
   __shared__ double serr;
-  extern __shared__ __align__(16) zd ctile[];  // [CK][CK][NO2] hot-chunk coefficients (N_o <= 2);
+  extern __shared__ __align__(16) zd ctile[];  // for each chunk its staged inverse (N_o <= 2);
                                  // at leaf entry (staged != 0) the block projections
-                                 // [maxl][NO2][rmax]; for a frozen chunk its staged inverse
+                                 // [maxl][NO2][rmax]
   __shared__ __align__(8) uint64_t cbar;   // completion of the inverse's bulk copy
   __shared__ int s_stage;                  // 0 once a wait for a copy has timed out
   uint32_t cphase = 0;
@@ -741,8 +664,8 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
       }
       __syncthreads();
       // projections of every block left of this leaf's rows, staged in shared
-      // memory for the loop below (the buffer of the hot-chunk coefficients,
-      // which the chunk solves fill only after it)
+      // memory for the loop below (the buffer of the chunk inverses, whose
+      // copies are issued only after it)
       cx<R>* Ps = reinterpret_cast<cx<R>*>(ctile);
       if (staged) {
         const int per = NO2 * d.rmax;
@@ -805,9 +728,9 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
       }
       __syncthreads();
     }
-    const bool frozen = (cc < d.nfrozL) && (b - a == ((cc == 0) ? CK - 1 : CK));
-    // the frozen inverse of this chunk into shared memory, overlapping the far field
-    const bool stage_now = kInvStage<NO, S> && frozen && s_stage;
+    const int fn = min(b, T) - a;   // rows solved with the chunk's inverse; row T, if it is here, follows them
+    // the inverse of this chunk into shared memory, overlapping the far field
+    const bool stage_now = kInvStage<NO, S> && fn > 0 && s_stage;
     if (stage_now && tid == 0) bulk_g2s(ctile, Cinv<NO>(d, n, cc, 1), kInvStage<NO, S>, &cbar);
     // ---- far field F(t) = q(t) - sum_{l < a} C(t,l) x(l); 8 threads per row ----
     {
@@ -904,7 +827,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
         for (int m = 0; m < NO; ++m) Old[row][m] = ld(sp(t) + m * NO + jc);
     }
     __syncthreads();
-    if (frozen) {
+    if (fn > 0) {
       const double2* Mi = Cinv<NO>(d, n, cc, 1);
       bool smem_inv = false;
       if (stage_now) {
@@ -926,14 +849,14 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
           const float2* Mh = reinterpret_cast<const float2*>(Mg);
           const float2* Ml = Mh + LD * LD;
           cff sf = cff_of(zf(0));
-          if (ti < cn) {
+          if (ti < fn) {
             zf s32 = zf(0);
-            for (int li = sl; li < cn; li += 8)
+            for (int li = sl; li < max(ti + 1, min(k, fn)); li += 8)
 #pragma unroll
               for (int y = 0; y < NO; ++y)
                 s32 = cfma(ldr<float>(Mh + (long long)(ti * NO + m) * LD + li * NO + y), Ff[li][y], s32);
             sf = cff_of(s32);
-            for (int li = sl; li < k && li < cn; li += 8)
+            for (int li = sl; li < k && li < fn; li += 8)
 #pragma unroll
               for (int y = 0; y < NO; ++y) {
                 const long long e = (long long)(ti * NO + m) * LD + li * NO + y;
@@ -945,8 +868,8 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
           for (int off = 1; off < 8; off <<= 1) sf = cff_add(sf, cff_shfl_xor(sf, off));
           if (sl == 0) sacc = cff_val(sf);
         } else {
-          if (ti < cn)
-            for (int li = sl; li < cn; li += 8)
+          if (ti < fn)
+            for (int li = sl; li < max(ti + 1, min(k, fn)); li += 8)
 #pragma unroll
               for (int y = 0; y < NO; ++y)
                 sacc = cfma(ld(Mg + (long long)(ti * NO + m) * LD + li * NO + y), Fs[li][y], sacc);
@@ -954,129 +877,55 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
           for (int off = 1; off < 8; off <<= 1)
             sacc += zd(__shfl_xor_sync(FULL, sacc.re, off), __shfl_xor_sync(FULL, sacc.im, off));
         }
-        if (sl == 0 && ti < cn) {
+        if (sl == 0 && ti < fn) {
           myerr = fmax(myerr, (sacc - Old[ti][m]).abs2());
           st(xp(a + ti) + m * NO + jc, sacc);
           if constexpr (Row64<NO, S>::separate) st(sp(a + ti) + m * NO + jc, sacc);
         }
       }
-    } else {
-      // chunk near T: right-looking triangular solve in one warp; lane L owns
-      // row t'' = a + L.  Chunk 0 first solves its start block t = 1..k.  The
-      // coefficients C(t'', tp) are staged in shared memory first (N_o <= 2).
-      auto coef = [&](int L0, int i, zd* cf) {
-        const int tq = a + L0, tp = a + i;
-        const double wl = -h * rule_w(W, tq, tp);
-        const S* sr = comp ? Lf<NO, S>(d, 2, n, jl, tq, tp) : el<NO, S>(d.SR, d, n, tq, tp);
-        const int dd = tq - tp;
-#pragma unroll
-        for (int q = 0; q < NO2; ++q) {
-          cf[q] = ld(sr + q) * wl;
-          if (dd <= k && (q / NO) == (q % NO)) cf[q] += zd(0, W.a[dd] / h);
-        }
-      };
-      if constexpr (kStage<NO>) {
-        const int i0s = (cc == 0) ? k : 0;
-        for (int e = tid; e < CK * CK; e += blockDim.x) {
-          const int L0 = e / CK, i = e % CK;
-          if (i >= i0s && i < L0 && L0 < cn) coef(L0, i, ctile + (long long)e * NO2);
-        }
-        __syncthreads();
-      }
+    }
+    if (fn < cn) {
+      // row T (horizontal density matrix): x(T) from the rows of its chunk and
+      // the current Sigma^R(T, .), one lane of warp 0 per row
+      __syncthreads();
       if (warp == 0) {
-      const int L0 = lane, tq = a + L0;
-      int i0 = 0;
-      zd f[NO];
-      if (L0 < cn)
+        zd f[NO];
 #pragma unroll
-        for (int m = 0; m < NO; ++m) f[m] = Fs[L0][m];
-      if (cc == 0) {
-        const int nsb = k * NO;
-        for (int e = lane; e < nsb * nsb; e += 32) {
-          const int row = e / nsb, col = e % nsb;
-          const int t = row / NO + 1, m = row % NO, l = col / NO + 1, y = col % NO;
-          zd v = srx_any<NO, S>(d, n, t, l, m, y) * (-h * W.I0[t][l]);
-          if (m == y) v += zd(0, W.D[t][l] / h);
-          if (l == t) v -= ld(epsp<NO>(d, n, t) + m * NO + y);
-          sA[row * nsb + col] = v;
-        }
-        for (int row = lane; row < nsb; row += 32) sB[row] = Fs[row / NO][row % NO];
-        __syncwarp();
-        warp_lu_solve(nsb, sA, sB, 1, nullptr);
-        for (int row = lane; row < nsb; row += 32) {
-          const int t = row / NO + 1, m = row % NO;
-          if (t <= last) {
-            myerr = fmax(myerr, (sB[row] - ld(sp(t) + m * NO + jc)).abs2());
-            st(xp(t) + m * NO + jc, sB[row]);
-            if constexpr (Row64<NO, S>::separate) st(sp(t) + m * NO + jc, sB[row]);
+        for (int m = 0; m < NO; ++m) f[m] = zd();
+        if (lane < fn) {
+          const int l = a + lane, dd = T - l;
+          const double wl = h * rule_w(W, T, l);
+          const S* sr = el<NO, S>(d.SR, d, n, T, l);
+#pragma unroll
+          for (int y = 0; y < NO; ++y) {
+            const zd x = ld(xp(l) + y * NO + jc), xw = x * wl;
+#pragma unroll
+            for (int m = 0; m < NO; ++m) f[m] = cfma(ld(sr + m * NO + y), xw, f[m]);
+            if (dd <= k) f[y] += zd(W.ah[dd] * x.im, -W.ah[dd] * x.re);   // (-i a_d / h) x(l)
           }
         }
-        __syncwarp();
-        if (L0 < cn && tq > k) {  // rows below the start block remove its contribution
-          for (int l = 1; l <= k; ++l) {
-            const double wl = -h * rule_w(W, tq, l);
-            const S* sr = comp ? Lf<NO, S>(d, 2, n, jl, tq, l) : el<NO, S>(d.SR, d, n, tq, l);
-            const int dd = tq - l;
+        warp_sum<NO>(f);
+        if (lane == 0) {
+          const double wt = h * rule_w(W, T, T);
+          const S* sd = el<NO, S>(d.SR, d, n, T, T);
+          const double2* ep = epsp<NO>(d, n, T);
+          M<NO> Mm;
+          zd x[NO];
 #pragma unroll
-            for (int m = 0; m < NO; ++m)
+          for (int x2 = 0; x2 < NO; ++x2) {
+            f[x2] += Fs[fn][x2];
 #pragma unroll
-              for (int y = 0; y < NO; ++y) {
-                zd cfv = ld(sr + m * NO + y) * wl;
-                if (dd <= k && m == y) cfv += zd(0, W.a[dd] / h);
-                f[m] -= cfv * sB[(l - 1) * NO + y];
-              }
+            for (int y = 0; y < NO; ++y)
+              Mm.a[x2][y] = (x2 == y ? zd(0, W.a[0] / h) : zd()) - ld(ep + x2 * NO + y) - ld(sd + x2 * NO + y) * wt;
           }
-        }
-        i0 = k;  // rows a..k (a = 1) are done
-      }
-      M<NO> Dinv;
-      if (L0 < cn && L0 >= i0) {
-        const double wt = h * rule_w(W, tq, tq);
-        const S* sd = comp ? Lf<NO, S>(d, 2, n, jl, tq, tq) : el<NO, S>(d.SR, d, n, tq, tq);
-        const double2* ep = epsp<NO>(d, n, tq);
-        M<NO> Mm;
-#pragma unroll
-        for (int x2 = 0; x2 < NO; ++x2)
-#pragma unroll
-          for (int y = 0; y < NO; ++y)
-            Mm.a[x2][y] = (x2 == y ? zd(0, W.a[0] / h) : zd()) - ld(ep + x2 * NO + y) - ld(sd + x2 * NO + y) * wt;
-        Dinv = solve_left<NO>(Mm, M<NO>::eye(zd(1.0)));
-      }
-      for (int i = i0; i < cn; ++i) {
-        const int tp = a + i;
-        zd cf[NO2];
-        if (L0 > i && L0 < cn) {
-          if constexpr (kStage<NO>) {
-#pragma unroll
-            for (int q = 0; q < NO2; ++q) cf[q] = ctile[(long long)(L0 * CK + i) * NO2 + q];
-          } else {
-            coef(L0, i, cf);
-          }
-        }
-        zd x[NO];
-        if (L0 == i) {
+          solve_col<NO>(Mm, f, x);
 #pragma unroll
           for (int m = 0; m < NO; ++m) {
-            x[m] = zd();
-#pragma unroll
-            for (int y = 0; y < NO; ++y) x[m] = cfma(Dinv.a[m][y], f[y], x[m]);
-          }
-#pragma unroll
-          for (int m = 0; m < NO; ++m) {
-            myerr = fmax(myerr, (x[m] - ld(sp(tp) + m * NO + jc)).abs2());
-            st(xp(tp) + m * NO + jc, x[m]);
-            if constexpr (Row64<NO, S>::separate) st(sp(tp) + m * NO + jc, x[m]);
+            myerr = fmax(myerr, (x[m] - Old[fn][m]).abs2());
+            st(xp(T) + m * NO + jc, x[m]);
+            if constexpr (Row64<NO, S>::separate) st(sp(T) + m * NO + jc, x[m]);
           }
         }
-#pragma unroll
-        for (int m = 0; m < NO; ++m) x[m] = zd(__shfl_sync(FULL, x[m].re, i), __shfl_sync(FULL, x[m].im, i));
-        if (L0 > i && L0 < cn) {
-#pragma unroll
-          for (int m = 0; m < NO; ++m)
-#pragma unroll
-            for (int y = 0; y < NO; ++y) f[m] -= cf[m * NO + y] * x[y];
-        }
-      }
       }
     }
     __syncthreads();
@@ -1091,115 +940,194 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
 }
 
 // ---------------------------------------------------------------------------
-// Inverse of a frozen chunk's local system, by Gauss-Jordan with partial
-// pivoting (FP64), one CTA per instance.  Retarded (which 0): unknowns
-// y(t'), t' in [a, a+32), matrix C[(s,m),(t',j)] = (i/h) a_{s-t'} [0 <= s-t' <= k]
-// delta_mj - delta_{s t'} eps(t')_mj - h w(s-t') Sigma^R(s,t')_mj with the
-// standard Gregory end weight w(d) = omega_d (d <= k) else 1.  Lesser (which 1):
-// unknowns x(t), rows t of the chunk; rows t <= k are the start equations with
-// D and I_{0,t,.}, other rows the BDF/Gregory equation with the weights w^(t)_l.
+// Inverses of the sweeps' triangular systems, brought up to date once per time
+// step (before its first iteration), one CTA per (instance, system):
+//   system 0, retarded chunks: points s in [r0, r1).  C[(s,m),(t',j)] =
+//     (i/h) a_{s-t'} [0 <= s-t' <= k] delta_mj - delta_{s t'} eps(t')_mj
+//     - h w(s-t') Sigma^R(s,t')_mj, w(d) = omega_d (d <= k) else 1;
+//   system 1, lesser chunks: rows t in [l0, l1) of E[(t,m),(l,y)] = (i/h)
+//     a_{t-l} delta - delta_{tl} eps(t) - h w^(t)_l Sigma^R(t,l); rows t <= k
+//     are the start equations with D and I_{0,t,.}, inverted together;
+//   system 2, the retarded head of step T: unknowns y(T-s), s = 1..min(2k,T),
+//     H[(s,j),(l,m)] = C[l,s]_mj of Eq. KBER: the start block s <= k with D and
+//     I_{0,s,.}, then rows with w^(s)_l, s <= 2k.
+// Each matrix is block lower triangular (below its start block), so a new row
+// s of an inverse M follows from the rows before it,
+//   M(s, c) = -A(s,s)^-1 sum_{c <= u < s} A(s, u) M(u, c),  M(s,s) = A(s,s)^-1,
+// and a completed chunk is never touched again.  All FP64; the complex64 form
+// keeps the growing chunk's rows in FP64 (cinv_ws) and writes their hi + lo
+// pair into the chunk's slot.
+// One launch per step, bound by the chain of the head's small inverse: 36 us at
+// N_o = 1, 88 us at N_o = 2, 270 us at N_o = 4 (16 instances).  A Gauss-Jordan
+// of the whole chunk every 32 steps took 0.2 ms (N_o = 1) to 7 ms (N_o = 4) and
+// left the growing chunks without an inverse.
 // ---------------------------------------------------------------------------
+// In-place Gauss-Jordan inverse with partial pivoting of the n x n matrix A
+// (leading dimension ld, shared memory, n <= 20); every thread calls it.
+__device__ void gj_inverse(int n, zd* A, int ld) {
+  __shared__ zd col[20];
+  __shared__ int prow[20];
+  const int tid = threadIdx.x;
+  for (int c = 0; c < n; ++c) {
+    if (tid < 32) {
+      double v = (tid >= c && tid < n) ? A[tid * ld + c].abs2() : -1.0;
+      int p = tid;
+#pragma unroll
+      for (int off = 16; off; off >>= 1) {
+        const double v2 = __shfl_xor_sync(FULL, v, off);
+        const int p2 = __shfl_xor_sync(FULL, p, off);
+        if (v2 > v || (v2 == v && p2 < p)) { v = v2; p = p2; }
+      }
+      if (p != c && tid < n) { const zd t = A[c * ld + tid]; A[c * ld + tid] = A[p * ld + tid]; A[p * ld + tid] = t; }
+      if (tid == 0) prow[c] = p;
+      __syncwarp();
+      if (tid < n) col[tid] = tid == c ? cdiv(zd(1.0), A[c * ld + c]) : A[tid * ld + c];
+      __syncwarp();
+      if (tid < n) A[c * ld + tid] = tid == c ? col[c] : A[c * ld + tid] * col[c];   // the scaled pivot row
+    }
+    __syncthreads();
+    for (int e = tid; e < n * n; e += blockDim.x) {
+      const int r = e / n, j = e % n;
+      if (r == c) continue;
+      const zd f = col[r];
+      A[r * ld + j] = j == c ? -(f * col[c]) : A[r * ld + j] - f * A[c * ld + j];
+    }
+    __syncthreads();
+  }
+  if (tid < n)   // undo the row exchanges on the columns, last first
+    for (int c = n - 1; c >= 0; --c)
+      if (prow[c] != c) { const zd t = A[tid * ld + c]; A[tid * ld + c] = A[tid * ld + prow[c]]; A[tid * ld + prow[c]] = t; }
+  __syncthreads();
+}
+
+// Row s of an inverse: Mi(s, .) from the coefficients crow[u][m][p] = A(s,u)_mp,
+// u = 0..s (diagonal block last), and the rows u < s of Mi (leading dimension
+// ld_m, columns u N_o + p; the first sb rows are a full start block).  out(m,
+// col, value) stores.  Every thread calls it.
+template <int NO, typename P, typename OUT>
+__device__ void append_row(int s, int sb, const zd* crow, const P* Mi, int ld_m, zd* part, zd* dinv, OUT out) {
+  constexpr int NO2 = NO * NO, SL = NO == 1 ? 8 : NO == 2 ? 2 : 1;   // slices of the sum over u
+  const int tid = threadIdx.x, nc = s * NO, tps = blockDim.x / SL, slice = tid / tps;
+  if (tid == 0) {
+    M<NO> D;
+#pragma unroll
+    for (int q = 0; q < NO2; ++q) D.a[q / NO][q % NO] = crow[s * NO2 + q];
+    const M<NO> I = solve_left<NO>(D, M<NO>::eye(zd(1.0)));
+#pragma unroll
+    for (int q = 0; q < NO2; ++q) dinv[q] = I.a[q / NO][q % NO];
+  }
+  for (int e = tid % tps; e < NO * nc; e += tps) {
+    const int m = e / nc, col = e % nc;
+    zd acc = zd();
+    for (int u = (col < sb * NO ? 0 : col / NO) + slice; u < s; u += SL)
+#pragma unroll
+      for (int p = 0; p < NO; ++p) acc = cfma(crow[u * NO2 + m * NO + p], ldr<double>(Mi + (long long)(u * NO + p) * ld_m + col), acc);
+    part[slice * (NO * nc) + e] = acc;
+  }
+  __syncthreads();
+  for (int e = tid; e < NO * (nc + NO); e += blockDim.x) {
+    const int m = e / (nc + NO), col = e % (nc + NO);
+    zd v = zd();
+    if (col >= nc) {
+      v = dinv[m * NO + col - nc];
+    } else {
+#pragma unroll
+      for (int q = 0; q < NO; ++q) {
+        zd w = zd();
+#pragma unroll
+        for (int sl = 0; sl < SL; ++sl) w += part[sl * (NO * nc) + q * nc + col];
+        v -= dinv[m * NO + q] * w;
+      }
+    }
+    out(m, col, v);
+  }
+  __syncthreads();
+}
+
 template <int NO, typename S>
-__global__ void __launch_bounds__(256) k_chunk_inv(Dev d, int which, int cc, double2* ws) {
-  const int n = blockIdx.x;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+__global__ void __launch_bounds__(256) k_inv_rows(Dev d, int T, int r0, int r1, int l0, int l1) {
+  constexpr int NO2 = NO * NO, LD = CK * NO, NH = 10 * NO;
+  const int n = blockIdx.y, sys = blockIdx.x, tid = threadIdx.x;
+  if (T > d.last[n]) return;   // the instance has ended
   const int k = d.k;
   const double h = d.h;
   const DevW& W = d.w;
-  const int a = (which == 1 && cc == 0) ? 1 : cc * CK;
-  const int cnt = (which == 1 && cc == 0) ? CK - 1 : CK;
-  if (cc * CK + CK + (which == 0 ? 2 * k : 0) > d.last[n]) return;   // frozen only after the instance ends
-  const int nn = cnt * NO;
-  constexpr int LD = CK * NO;
-  double2* Bout = Cinv<NO>(d, n, cc, which);
-  double2* Am = ws + (long long)n * 2 * LD * LD;   // FP64 work matrix
-  double2* B = Am + (long long)LD * LD;            // FP64 inverse under construction
-  __shared__ zd fcol[CK * 4];
-  __shared__ int s_piv;
-  __shared__ zd s_inv;
-  for (int e = tid; e < nn * nn; e += blockDim.x) {
-    const int r = e / nn, col = e % nn;
-    const int ri = r / NO, m = r % NO, ci = col / NO, j = col % NO;
-    zd v = zd();
-    if (which == 0) {
-      const int s = a + ri, tp = a + ci, dd = s - tp;
-      if (dd >= 0) {
-        const double wf = (dd <= k) ? W.omega[dd] : 1.0;
-        v = sr_any<NO, S>(d, n, s, tp, m, j) * (-h * wf);
-        if (dd <= k && m == j) v += zd(0, W.a[dd] / h);
-        if (dd == 0) v -= ld(epsp<NO>(d, n, tp) + m * NO + j);
-      }
-    } else {
-      const int t = a + ri, l = a + ci;
-      if (t <= k) {
-        if (l <= k) {
-          v = srx_any<NO, S>(d, n, t, l, m, j) * (-h * W.I0[t][l]);
-          if (m == j) v += zd(0, W.D[t][l] / h);
-          if (l == t) v -= ld(epsp<NO>(d, n, t) + m * NO + j);
-        }
-      } else if (l <= t) {
-        v = sr_any<NO, S>(d, n, t, l, m, j) * (-h * rule_w(W, t, l));
-        if (t - l <= k && m == j) v += zd(0, W.a[t - l] / h);
-        if (l == t) v -= ld(epsp<NO>(d, n, t) + m * NO + j);
-      }
+  __shared__ zd part[NO <= 2 ? 256 : CK * NO2];
+  __shared__ zd crow[CK * NO2];
+  __shared__ zd dinv[NO2];
+  __shared__ zd Hm[NH * NH];       // the head, or the lesser start block
+  if (sys == 2) {
+    const int hs = min(2 * k, T), kb = min(k, hs), nh = hs * NO, nb = kb * NO;
+    auto coef = [&](int s, int l, int j, int m) {   // H[(s,j),(l,m)]
+      const double wl = s <= k ? W.I0[s][l] : rule_w(W, s, l);
+      zd v = srx_any<NO, S>(d, n, T - l, T - s, m, j) * (-h * wl);
+      if (m == j) v += zd(0, s <= k ? W.D[s][l] / h : s - l <= k ? W.ah[s - l] : 0.0);
+      if (l == s) v -= ld(epsp<NO>(d, n, T - s) + m * NO + j);
+      return v;
+    };
+    for (int e = tid; e < nh * nh; e += blockDim.x) {
+      const int row = e / nh, col = e % nh;
+      Hm[e] = (row < nb && col < nb) ? coef(row / NO + 1, col / NO + 1, row % NO, col % NO) : zd();
     }
-    st(Am + (long long)r * LD + col, v);
-    st(B + (long long)r * LD + col, (r == col) ? zd(1.0) : zd());
+    __syncthreads();
+    gj_inverse(nb, Hm, nh);
+    for (int s = kb; s < hs; ++s) {
+      for (int e = tid; e < (s + 1) * NO2; e += blockDim.x)
+        crow[e] = coef(s + 1, e / NO2 + 1, (e % NO2) / NO, e % NO);
+      __syncthreads();
+      append_row<NO>(s, kb, crow, Hm, nh, part, dinv, [&](int m, int col, const zd& v) { Hm[(s * NO + m) * nh + col] = v; });
+    }
+    double2* Hi = d.hinv + (long long)n * (4 * k * k * NO2);
+    for (int e = tid; e < nh * nh; e += blockDim.x) st(Hi + e, Hm[e]);
+    return;
   }
-  __syncthreads();
-  for (int piv = 0; piv < nn; ++piv) {
-    if (warp == 0) {
-      double best = -1.0;
-      int arg = piv;
-      for (int r = piv + lane; r < nn; r += 32) {
-        const double v = ld(Am + (long long)r * LD + piv).abs2();
-        if (v > best) { best = v; arg = r; }
+  // chunk rows (systems 0 and 1)
+  constexpr bool f64 = sizeof(S) == sizeof(double2);
+  double2* wsm = d.cinv_ws + ((long long)n * 2 + sys) * (LD * LD);
+  const int q0 = sys == 0 ? r0 : l0, q1 = sys == 0 ? r1 : l1;
+  for (int s = q0; s < q1; ++s) {
+    const int cc = s / CK, a = (sys == 1 && cc == 0) ? 1 : cc * CK;
+    double2* slot = Cinv<NO>(d, n, cc, sys);
+    double2* Mi = f64 ? slot : wsm;
+    auto put = [&](int row, int col, const zd& v) {
+      st(Mi + (long long)row * LD + col, v);
+      if constexpr (!f64) {   // complex64 form: hi and lo matrices (see Cinv)
+        float2* Oh = reinterpret_cast<float2*>(slot);
+        const float2 hi = make_float2((float)v.re, (float)v.im);
+        Oh[(long long)row * LD + col] = hi;
+        Oh[(long long)LD * LD + (long long)row * LD + col] =
+            make_float2((float)(v.re - (double)hi.x), (float)(v.im - (double)hi.y));
       }
-#pragma unroll
-      for (int off = 16; off; off >>= 1) {
-        const double b2 = __shfl_xor_sync(0xffffffffu, best, off);
-        const int a2 = __shfl_xor_sync(0xffffffffu, arg, off);
-        if (b2 > best || (b2 == best && a2 < arg)) { best = b2; arg = a2; }
+    };
+    if (sys == 1 && s == 1) {   // the lesser start block, rows 1..k together
+      const int nb = k * NO;
+      for (int e = tid; e < nb * nb; e += blockDim.x) {
+        const int row = e / nb, col = e % nb;
+        const int t = row / NO + 1, m = row % NO, l = col / NO + 1, y = col % NO;
+        zd v = srx_any<NO, S>(d, n, t, l, m, y) * (-h * W.I0[t][l]);
+        if (m == y) v += zd(0, W.D[t][l] / h);
+        if (l == t) v -= ld(epsp<NO>(d, n, t) + m * NO + y);
+        Hm[e] = v;
       }
-      if (lane == 0) s_piv = arg;
+      __syncthreads();
+      gj_inverse(nb, Hm, nb);
+      for (int e = tid; e < nb * nb; e += blockDim.x) put(e / nb, e % nb, Hm[e]);
+      __syncthreads();
+      s = k;
+      continue;
+    }
+    const int ri = s - a;
+    for (int e = tid; e < (ri + 1) * NO2; e += blockDim.x) {
+      const int u = a + e / NO2, m = (e % NO2) / NO, p = e % NO, dd = s - u;
+      const double wl = sys == 1 ? rule_w(W, s, u) : dd <= k ? W.omega[dd] : 1.0;
+      zd v = sr_any<NO, S>(d, n, s, u, m, p) * (-h * wl);
+      if (dd <= k && m == p) v += zd(0, W.ah[dd]);
+      if (dd == 0) v -= ld(epsp<NO>(d, n, s) + m * NO + p);
+      crow[e] = v;
     }
     __syncthreads();
-    const int p = s_piv;
-    if (p != piv) {
-      for (int j = tid; j < nn; j += blockDim.x) {
-        double2 t1 = Am[(long long)piv * LD + j]; Am[(long long)piv * LD + j] = Am[(long long)p * LD + j]; Am[(long long)p * LD + j] = t1;
-        double2 t2 = B[(long long)piv * LD + j]; B[(long long)piv * LD + j] = B[(long long)p * LD + j]; B[(long long)p * LD + j] = t2;
-      }
-    }
-    __syncthreads();
-    if (tid == 0) s_inv = cdiv(zd(1.0), ld(Am + (long long)piv * LD + piv));
-    __syncthreads();
-    for (int j = tid; j < nn; j += blockDim.x) {
-      st(Am + (long long)piv * LD + j, ld(Am + (long long)piv * LD + j) * s_inv);
-      st(B + (long long)piv * LD + j, ld(B + (long long)piv * LD + j) * s_inv);
-    }
-    for (int r = tid; r < nn; r += blockDim.x) fcol[r] = ld(Am + (long long)r * LD + piv);
-    __syncthreads();
-    for (int e = tid; e < nn * nn; e += blockDim.x) {
-      const int r = e / nn, j = e % nn;
-      if (r == piv) continue;
-      const zd f = fcol[r];
-      st(Am + (long long)r * LD + j, ld(Am + (long long)r * LD + j) - f * ld(Am + (long long)piv * LD + j));
-      st(B + (long long)r * LD + j, ld(B + (long long)r * LD + j) - f * ld(B + (long long)piv * LD + j));
-    }
-    __syncthreads();
-  }
-  for (int e = tid; e < nn * nn; e += blockDim.x) {
-    const int r = e / nn, col = e % nn;
-    const zd v = ld(B + (long long)r * LD + col);
-    if constexpr (sizeof(S) == sizeof(float2)) {   // complex64 form: hi and lo matrices (see Cinv)
-      float2* Oh = reinterpret_cast<float2*>(Bout);
-      const float2 hi = make_float2((float)v.re, (float)v.im);
-      Oh[(long long)r * LD + col] = hi;
-      Oh[(long long)LD * LD + (long long)r * LD + col] = make_float2((float)(v.re - (double)hi.x), (float)(v.im - (double)hi.y));
-    } else {
-      st(Bout + (long long)r * LD + col, v);
-    }
+    const int sb = sys == 1 && cc == 0 ? k : 0;   // rows of the start block in this chunk: full columns
+    append_row<NO>(ri, sb, crow, Mi, LD, part, dinv, [&](int m, int col, const zd& v) { put(ri * NO + m, col, v); });
   }
 }
 
@@ -1227,7 +1155,7 @@ static cudaError_t allow_smem(K kern, size_t bytes) {
   if (a.sharedSizeBytes + bytes > 227 * 1024) return cudaErrorInvalidValue;
   return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
-// Dynamic shared memory of a sweep: the hot-chunk coefficients (N_o <= 2)
+// Dynamic shared memory of a sweep: the staged chunk inverse (N_o <= 2)
 // and, in the compressed form, the staged block projections, which share one
 // buffer; staging is used when it fits in 64 KiB.
 template <int NO, typename S>
@@ -1263,13 +1191,9 @@ cudaError_t launch_les_h(const Dev& d, int T, cudaStream_t s) {
   HK_DISPATCH(d.no, return (sweep_les<NO, S>(d, T, s)));
   return cudaSuccess;
 }
-cudaError_t launch_chunk_inv(const Dev& d, int which, int c0, int c1, cudaStream_t s) {
-  for (int cc = c0; cc < c1; ++cc) {
-    HK_DISPATCH(d.no, (k_chunk_inv<NO, S><<<d.n_inst, 256, 0, s>>>(d, which, cc, d.cinv_ws)));
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+cudaError_t launch_inv_rows(const Dev& d, int T, int r0, int r1, int l0, int l1, cudaStream_t s) {
+  HK_DISPATCH(d.no, (k_inv_rows<NO, S><<<dim3(3, d.n_inst), 256, 0, s>>>(d, T, r0, r1, l0, l1)));
+  return cudaGetLastError();
 }
 
 }  // namespace hk

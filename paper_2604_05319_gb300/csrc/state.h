@@ -50,11 +50,13 @@ struct Dev {
   int tsvd_group;         // runs tsvd_group instances at a time on one shared workspace
   const long long* ws_lvoff;
   int* status;         // [0] rank overflow count, [1] Jacobi non-convergence count
-  // frozen 32-point chunk inverses of the two sweeps (FP64): [n][nchunk][2][(32 no)^2]
+  // 32-point chunk inverses of the two sweeps: [n][nchunk][2][(32 no)^2]; entries above
+  // the diagonal stay zero from the allocation
   double2* cinv;
-  double2* cinv_ws;    // [n][(32 no)^2] Gauss-Jordan workspace
+  double2* cinv_ws;    // [n][2][(32 no)^2] complex64 form: FP64 rows of the growing chunks
+  double2* hinv;       // [n][(2k no)^2] inverse of the retarded head of the current step
   int nchunk;          // ceil(nt / 32)
-  int nfrozR, nfrozL;  // chunks [0, nfroz) of each sweep have a valid inverse
+  int nfrozR, nfrozL;  // chunks [0, nfroz) of each sweep have a complete inverse
   long long ntri;  // nt*(nt+1)/2
   double h, beta;
   DevW w;
@@ -109,7 +111,7 @@ cudaError_t launch_density_at(const Dev& d, int t, double2* out, cudaStream_t s)
 cudaError_t launch_sigma_lattice(const Dev& d, int T, cudaStream_t s);   // model 4, all k at once
 cudaError_t launch_lattice_obs(const Dev& d, int t, double* out, cudaStream_t s);
 cudaError_t launch_row_out(const Dev& d, int n, int T, double2* out_r, double2* out_l, cudaStream_t s);
-// inverses of the frozen chunks [c0, c1) of sweep `which` (0 retarded, 1 lesser)
-cudaError_t launch_chunk_inv(const Dev& d, int which, int c0, int c1, cudaStream_t s);
+// inverse rows of retarded points [r0, r1) and lesser points [l0, l1), and the retarded head of step T
+cudaError_t launch_inv_rows(const Dev& d, int T, int r0, int r1, int l0, int l1, cudaStream_t s);
 
 }  // namespace hk
