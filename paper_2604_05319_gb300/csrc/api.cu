@@ -330,6 +330,10 @@ int hkbe_create(const hkbe_params* p, const int32_t* nt_per_inst, void* stream, 
   for (int i = 0; i < 6; ++i) {
     d.w.ah[i] = w.a[i] / p->h;
     d.w.omegaf[i] = (float)w.omega[i];
+    auto pair = [](double x) { const float hi = (float)x; return make_float2(hi, (float)(x - (double)hi)); };
+    d.w.hf = pair(p->h);
+    d.w.ahf[i] = pair(d.w.ah[i]);
+    d.w.wm1f[i] = pair(w.omega[i] - 1.0);
     for (int j = 0; j < 6; ++j) d.w.I0f[i][j] = (float)w.I0[i][j];
   }
   h->hodlr = p->svd_tol > 0;

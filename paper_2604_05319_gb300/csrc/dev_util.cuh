@@ -102,6 +102,33 @@ __device__ __forceinline__ R rule_wr(const DevW& w, int n, int l) {
   }
 }
 
+// Element of the lesser source q(t): FP64, or in the complex64 form a
+// float-float pair of the same 16 bytes, so that the lesser sweep takes it
+// without FP64 conversions.
+template <typename S>
+__device__ __forceinline__ auto ldv(const double2* p) {
+  if constexpr (sizeof(S) == sizeof(double2)) {
+    return ld(p);
+  } else {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    return cff{{v.x, v.y}, {v.z, v.w}};
+  }
+}
+template <typename S>
+__device__ __forceinline__ zd ldv64(const double2* p) {
+  if constexpr (sizeof(S) == sizeof(double2)) return ld(p);
+  else return cff_val(ldv<S>(p));
+}
+template <typename S>
+__device__ __forceinline__ void stv(double2* p, const zd& v) {
+  if constexpr (sizeof(S) == sizeof(double2)) {
+    st(p, v);
+  } else {
+    const cff f = cff_of(v);
+    *reinterpret_cast<float4*>(p) = make_float4(f.re.hi, f.re.lo, f.im.hi, f.im.lo);
+  }
+}
+
 constexpr int FOLD = 8;  // terms summed in R before they enter the compensated accumulator
 
 __device__ __forceinline__ zd wshfl(zd v, int off) {

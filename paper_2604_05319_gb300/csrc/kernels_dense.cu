@@ -442,7 +442,7 @@ __global__ void k_src(Dev d, int T) {
   if (lane == 0) {
     double2* p = d.qsrc + ((long long)n * d.nt + t) * NO2;
 #pragma unroll
-    for (int q = 0; q < NO2; ++q) st(p + q, acc[q]);
+    for (int q = 0; q < NO2; ++q) stv<S>(p + q, acc[q]);
   }
 }
 
@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(256) k_les(Dev d, int T) {
     }
     for (int row = lane; row < ns; row += 32) {
       const int t = row / NO + 1, m = row % NO;
-      zd b = ld(qs + t * NO2 + m * NO + jc);
+      zd b = ldv64<S>(qs + t * NO2 + m * NO + jc);
       for (int y = 0; y < NO; ++y) {
         zd c = srx<NO, S>(d, n, t, 0, m, y) * (-h * W.I0[t][0]);
         if (m == y) c += zd(0, W.D[t][0] / h);
@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(256) k_les(Dev d, int T) {
         if (lane == 0) {
           zd rhs[NO], x[NO];
 #pragma unroll
-          for (int m = 0; m < NO; ++m) rhs[m] = part[m] + farsh[tl][m] + ld(qs + (long long)t * NO2 + m * NO + jc);
+          for (int m = 0; m < NO; ++m) rhs[m] = part[m] + farsh[tl][m] + ldv64<S>(qs + (long long)t * NO2 + m * NO + jc);
           const double wt = h * rule_w(W, t, t);
           const S* sd = el<NO, S>(d.SR, d, n, t, t);
           const double2* ep = epsp<NO>(d, n, t);
@@ -625,7 +625,7 @@ __global__ void k_rho(Dev d, int T) {
   if (threadIdx.x != 0) return;
   zd r0[NO2];
   for (int q = 0; q < NO2; ++q) {
-    r0[q] = ld(d.qsrc + ((long long)n * d.nt + T) * NO2 + q);
+    r0[q] = ldv64<S>(d.qsrc + ((long long)n * d.nt + T) * NO2 + q);
     for (int w2 = 0; w2 < (int)(blockDim.x >> 5); ++w2) r0[q] += part[w2][q];
   }
   const double xi = d.xi;

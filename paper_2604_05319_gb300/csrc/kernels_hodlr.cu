@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(128) k_src_c(Dev d, int T) {
   }
   double2* qp = d.qsrc + ((long long)n * d.nt + t) * NO2;
 #pragma unroll
-  for (int q = 0; q < NO2; ++q) st(qp + q, acc[q]);
+  for (int q = 0; q < NO2; ++q) stv<S>(qp + q, acc[q]);
 }
 
 // q(t) for the uncompressed rows t in [c, T]: one warp per t (lanes along the row).
@@ -412,7 +412,7 @@ __global__ void k_src_h(Dev d, int T) {
   if (lane == 0) {
     double2* p = d.qsrc + ((long long)n * d.nt + t) * NO2;
 #pragma unroll
-    for (int q = 0; q < NO2; ++q) st(p + q, acc[q]);
+    for (int q = 0; q < NO2; ++q) stv<S>(p + q, acc[q]);
   }
 }
 

@@ -26,6 +26,8 @@
 // block) took 75 of the 89 thousand cycles of a retarded sweep at N_o = 1,
 // T <= 64, and 820 of 1900 thousand at N_o = 4, T = 290; the two sweeps of
 // those runs went from 89 to 35 us and from 1650 to 1040 us.
+#include <algorithm>
+
 #include "bulk_copy.cuh"
 #include "hodlr_util.cuh"
 
@@ -36,22 +38,72 @@ namespace {
 constexpr int CK = 32;   // chunk length
 using Y = double2;       // element type of the row / column being solved
 template <int NO> constexpr bool kStage = NO <= 2;   // chunk inverses staged in shared memory
-template <int NO> constexpr size_t kStageBytes = kStage<NO> ? sizeof(zd) * CK * CK * NO * NO : 0;
 // Bytes of a chunk inverse that are staged in shared memory by a bulk copy
-// issued before the chunk's far field, so the copy overlaps that phase: the
-// whole inverse (FP64, or the hi and lo matrices of the complex64 form, 16
-// bytes per entry either way); 0 (read from global memory) for N_o > 2.
-template <int NO, typename S>
+// issued before the chunk's far field, so the copy overlaps it: the whole
+// inverse (FP64, or the hi and lo matrices of the complex64 form, 16 bytes
+// per entry either way); 0 (read from global memory) for N_o > 2.
+template <int NO>
 constexpr uint32_t kInvStage = kStage<NO> ? (uint32_t)(CK * NO * CK * NO * sizeof(double2)) : 0u;
+// Orbital pairs that one pass of proj_block takes, and the bytes of its
+// cross-warp partial sums (which share the buffer of the staged inverse).
+template <int NO> constexpr int kPG = NO == 1 ? 1 : NO == 3 ? 3 : 4;
+template <int NO>
+constexpr size_t kBufBytes = std::max((size_t)kInvStage<NO>, (size_t)8 * kPG<NO> * 64 * 16);
+// Leaf rows (of four per thread) that a chunk's far field keeps in flight.
+template <int NO, typename S> constexpr int kLB = NO == 1 ? 4 : NO == 2 ? (sizeof(S) == 8 ? 4 : 2) : 1;
 constexpr int kCopyWaitPolls = 1 << 20;   // bound of the wait for a staged inverse
+constexpr int kRingRows = 80;             // >= leaf + k + 1 uncompressed rows
 
 // Sum over the 8 lanes of an aligned lane group of their history
 // accumulators (every lane receives it).  Complex64 form: the compensated
 // FP32 sums are combined in float-float, so the reduction runs on the FP32
-// pipes; FP64 form: plain FP64.  val_of converts to FP64 (once, by the lane
-// that uses the sum).
+// pipes; FP64 form: plain FP64.
 template <typename R>
 __device__ __forceinline__ auto reduce8(const KAcc<R>& k) { return kacc_lanes(k, 1, 8); }
+
+// A solved value: FP64, or float-float in the complex64 form (about 48 bits
+// on the FP32 pipes; an FP64 instruction holds a warp's pipe for 64 cycles,
+// and a chunk's epilogue in FP64 took most of the chunk's time).
+template <typename S> struct Val { using t = zd; };
+template <> struct Val<float2> { using t = cff; };
+__device__ __forceinline__ void vset(zd& v, const zd& x) { v = x; }
+__device__ __forceinline__ void vset(cff& v, const zd& x) { v = cff_of(x); }
+__device__ __forceinline__ zd v64(const zd& v) { return v; }
+__device__ __forceinline__ zd v64(const cff& v) { return cff_val(v); }
+__device__ __forceinline__ zd vadd(const zd& a, const zd& b) { return a + b; }
+__device__ __forceinline__ cff vadd(const cff& a, const cff& b) { return cff_add(a, b); }
+__device__ __forceinline__ zd vbulk(const zd& v) { return v; }                      // in the bulk arithmetic
+__device__ __forceinline__ zf vbulk(const cff& v) { return zf(v.re.hi, v.im.hi); }
+__device__ __forceinline__ zd vreal(const zd& a, double s, float2) { return a * s; }
+__device__ __forceinline__ cff vreal(const cff& a, double, float2 s) {
+  return {ff_mul(a.re, {s.x, s.y}), ff_mul(a.im, {s.x, s.y})};
+}
+// acc + (-i a_j / h) y
+__device__ __forceinline__ zd vbdf(const zd& acc, const zd& y, const DevW& W, int j) {
+  return zd(fma(W.ah[j], y.im, acc.re), fma(-W.ah[j], y.re, acc.im));
+}
+__device__ __forceinline__ cff vbdf(const cff& acc, const cff& y, const DevW& W, int j) {
+  const ffl a{W.ahf[j].x, W.ahf[j].y};
+  return {ff_add(acc.re, ff_mul(a, y.im)), ff_add(acc.im, ff_neg(ff_mul(a, y.re)))};
+}
+__device__ __forceinline__ zd vshfl_xor(const zd& a, int off) { return wshfl(a, off); }
+__device__ __forceinline__ cff vshfl_xor(const cff& a, int off) { return cff_shfl_xor(a, off); }
+// |new - old|^2, old a stored element
+__device__ __forceinline__ double vdist(const zd& a, const zd& o) { return (a - o).abs2(); }
+__device__ __forceinline__ float vdist(const cff& a, const zf& o) {
+  const float x = (a.re.hi - o.re) + a.re.lo, y = (a.im.hi - o.im) + a.im.lo;
+  return x * x + y * y;
+}
+__device__ __forceinline__ void vstore(double2* p, const zd& v) { st(p, v); }
+__device__ __forceinline__ void vstore(float2* p, const cff& v) { *p = make_float2(v.re.hi, v.im.hi); }
+template <typename T, int N>
+__device__ __forceinline__ T pick(const T (&v)[N], int i) {   // v[i] without indexed registers
+  T r = v[0];
+#pragma unroll
+  for (int j = 1; j < N; ++j)
+    if (i == j) r = v[j];
+  return r;
+}
 
 // Where a sweep keeps the row it solves: in place (FP64 storage), or in FP64
 // next to the complex64 storage: the row's slot of the FP64 ring copies of the
@@ -71,7 +123,8 @@ struct Row64<NO, double2> {
   __device__ static Y* get(const Dev&, int, int, int, double2* p) { return p; }
 };
 
-// Inverse of chunk cc of sweep `which`, (32 N_o)^2 entries (rows of points not yet built: unused).  FP64
+// Inverse of chunk cc of sweep `which`, (32 N_o)^2 entries (rows of points not
+// yet built: unused).  FP64
 // storage form: complex128.  Complex64 form: the same 16 bytes per entry
 // hold a complex64 pair hi + lo (hi = the inverse rounded to complex64, lo =
 // the rounding of hi), [hi matrix][lo matrix].  The chunk's right-hand side
@@ -87,152 +140,247 @@ __device__ __forceinline__ double2* Cinv(const Dev& d, int n, int cc, int which)
   return d.cinv + (((long long)n * d.nchunk + cc) * 2 + which) * nn;
 }
 
-// Projections of one block of Sigma^R for all N_o^2 orbital pairs in one pass
-// (complex64 form, N_o <= 2, rank <= 64): out_p[q] = S_p[q] sum_{l in [l0, l1)}
-// v_p(l) F_p(l, q) for q < rank_p, with F = U (ROWS: the retarded sweep, v_p =
-// y_m, m = p / N_o) or F = conj(V) (the lesser sweep, v_p = w_l x_nn, nn =
-// p % N_o); vf(l, i) returns the vector's component i at l.  A warp covers
-// 32 / lpr rows per step, lpr = 8, 16 or 32 lanes per row (the smallest that
-// holds the largest rank), so small ranks keep every lane loading; warps split
-// the rows, and the pairs share the vector loads.  Partial sums (compensated
-// FP32) are combined across a warp's rows in float-float and across warps in
-// red ([8][N_o^2][64], shared memory).  Every thread calls it.
-template <int NO, typename S, bool ROWS, typename VF>
-__device__ __forceinline__ void proj_block(const Dev& d, int n, int blk, int lv, int slot, int l0, int l1, VF vf,
-                                           zd* red) {
-  constexpr int NO2 = NO * NO;
-  using R = typename Bulk<S>::R;
-  static_assert(sizeof(R) == sizeof(float), "the one-pass projections serve the complex64 form");
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int rk[NO2];
-  const S* F[NO2];
-  int rkmax = 0;
-#pragma unroll
-  for (int p = 0; p < NO2; ++p) {
-    rk[p] = *Rk<NO>(d, 2, n, blk, p);
-    F[p] = ROWS ? Up<NO, S>(d, 2, n, blk, p) : Vp<NO, S>(d, 2, n, blk, p);
-    rkmax = max(rkmax, rk[p]);
+// Dynamic shared memory of a sweep: the buffer of the staged inverse, the
+// projections Ps[slot][rmax] of the blocks that cover the current leaf (slot =
+// (target m or j, level, other index), target-major), the same packed without
+// the gaps between ranks (Pk, and the factor entry Off each belongs to), and
+// per slot its factor base, rank, first packed entry and block, for this leaf
+// and the next (ranks and blocks).
+template <int NO, typename R>
+struct SweepMem {
+  cx<R>*Ps, *Pk;
+  long long* base;
+  unsigned* off;
+  int *start, *rk, *blk;
+  int nslot;
+  __host__ __device__ static size_t bytes(int maxl, int rmax) {
+    const size_t ns = (size_t)maxl * NO * NO;
+    return ns * rmax * (2 * sizeof(cx<R>) + 4) + ns * 8 + (ns + 1) * 4 + 2 * (ns + maxl) * 4 + 16;
   }
+  __device__ SweepMem(char* p, int maxl, int rmax) {
+    nslot = maxl * NO * NO;
+    Ps = reinterpret_cast<cx<R>*>(p);
+    Pk = Ps + (size_t)nslot * rmax;
+    base = reinterpret_cast<long long*>(Pk + (size_t)nslot * rmax);
+    off = reinterpret_cast<unsigned*>(base + nslot);
+    start = reinterpret_cast<int*>(off + (size_t)nslot * rmax);
+    rk = start + nslot + 1;
+    blk = rk + 2 * nslot;
+  }
+};
+
+// Projections of one block of Sigma^R for all N_o^2 orbital pairs: P_p[q] =
+// S_p[q] sum_{l in [l0, l1)} v_p(l) F_p(l, q) for q < rank_p, with F = U
+// (ROWS: the retarded sweep, v_p = y_m, m = p / N_o) or F = conj(V) (the
+// lesser sweep, v_p = w_l x_nn, nn = p % N_o); vf(l, i) returns the vector's
+// component i at l.  A warp covers 32 / lpr rows per step, lpr = 8, 16 or 32
+// lanes per row (the smallest that holds the largest rank), so small ranks
+// keep every lane loading; warps split the rows, and the pairs of a group
+// share the vector loads.  Partial sums (compensated FP32, or FP64) are
+// combined across a warp's rows by shuffles and across warps in red
+// ([8][group][64], shared memory).  out(p, q, value).  Every thread calls it.
+template <int NO, typename S, bool ROWS, typename VF, typename RK, typename OUT>
+__device__ __forceinline__ void proj_block(const Dev& d, int n, int blk, int l0, int l1, VF vf, RK rank_of, void* buf,
+                                           OUT out) {
+  constexpr int NO2 = NO * NO, PG = kPG<NO>;
+  using R = typename Bulk<S>::R;
+  using V = typename Val<S>::t;
+  V* red = static_cast<V*>(buf);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int base = ROWS ? d.b_r0[blk] : d.b_c0[blk];
-  const int lpr = rkmax <= 8 ? 8 : rkmax <= 16 ? 16 : 32;   // lanes per row
-  const int rps = 32 / lpr, sub = lane / lpr, q0 = lane % lpr;
-  const int stride = 8 * rps;                               // rows per CTA step
-  KAcc<R> part[NO2][2];
-  for (int sb = l0 + warp * rps + sub; sb < l1; sb += stride * FOLD) {
-    cx<R> pp[NO2][2];
+#pragma unroll 1
+  for (int p0 = 0; p0 < NO2; p0 += PG) {
+    int rk[PG], rkmax = 0;
+    const S* F[PG];
 #pragma unroll
-    for (int p = 0; p < NO2; ++p) pp[p][0] = pp[p][1] = cx<R>(0);
+    for (int g = 0; g < PG; ++g) {
+      rk[g] = rank_of(p0 + g);
+      F[g] = ROWS ? Up<NO, S>(d, 2, n, blk, p0 + g) : Vp<NO, S>(d, 2, n, blk, p0 + g);
+      rkmax = max(rkmax, rk[g]);
+    }
+    for (int qb = 0; qb < rkmax; qb += 64) {   // 64 entries of the rank at a time
+      const int rem = min(rkmax - qb, 64), lpr = rem <= 8 ? 8 : rem <= 16 ? 16 : 32;   // lanes per row
+      const int rps = 32 / lpr, sub = lane / lpr, q0 = qb + lane % lpr;
+      const int stride = 8 * rps;   // rows per CTA step
+      double sv = 0.0;              // the singular value this thread multiplies at the end
+      if (tid < PG * 64) {
+        const int g = tid >> 6, q = qb + (tid & 63);
+        if (q < d.rmax) sv = Sp<NO>(d, 2, n, blk, p0 + g)[q];
+      }
+      KAcc<R> part[PG][2];
+      for (int sb = l0 + warp * rps + sub; sb < l1; sb += stride * FOLD) {
+        cx<R> pp[PG][2];
 #pragma unroll
-    for (int jj = 0; jj < FOLD; ++jj) {
-      const int l = sb + stride * jj;
-      if (l < l1) {
-        cx<R> v[NO];
+        for (int g = 0; g < PG; ++g) pp[g][0] = pp[g][1] = cx<R>(0);
 #pragma unroll
-        for (int i = 0; i < NO; ++i) v[i] = vf(l, i);
+        for (int jj = 0; jj < FOLD; ++jj) {
+          const int l = sb + stride * jj;
+          if (l < l1) {
+            cx<R> v[NO];
 #pragma unroll
-        for (int p = 0; p < NO2; ++p) {
-          const S* fr = F[p] + (long long)(l - base) * d.rmax;
-          const cx<R> vp = v[ROWS ? p / NO : p % NO];
+            for (int i = 0; i < NO; ++i) v[i] = vf(l, i);
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int q = q0 + lpr * u;
-            if (q < rk[p]) {
-              const cx<R> f = ROWS ? ldr<R>(fr + q) : ldr<R>(fr + q).conj();
-              pp[p][u] = cfma(vp, f, pp[p][u]);
+            for (int g = 0; g < PG; ++g) {
+              const S* fr = F[g] + (long long)(l - base) * d.rmax;
+              const cx<R> vp = pick(v, ROWS ? (p0 + g) / NO : (p0 + g) % NO);
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                const int q = q0 + lpr * u;
+                if (q < rk[g]) {
+                  const cx<R> f = ROWS ? ldr<R>(fr + q) : ldr<R>(fr + q).conj();
+                  pp[g][u] = cfma(vp, f, pp[g][u]);
+                }
+              }
             }
           }
         }
+#pragma unroll
+        for (int g = 0; g < PG; ++g) {
+          part[g][0].add(pp[g][0]);
+          part[g][1].add(pp[g][1]);
+        }
       }
-    }
 #pragma unroll
-    for (int p = 0; p < NO2; ++p) {
-      part[p][0].add(pp[p][0]);
-      part[p][1].add(pp[p][1]);
+      for (int g = 0; g < PG; ++g)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int q = q0 + lpr * u - qb;
+          if (lpr * u < rem) {
+            const V r = kacc_lanes(part[g][u], lpr, 32);
+            if (sub == 0 && q < 64) red[(warp * PG + g) * 64 + q] = r;
+          }
+        }
+      __syncthreads();
+      if (tid < PG * 64) {
+        const int g = tid >> 6, q = tid & 63;
+        if (q < min(pick(rk, g) - qb, 64)) {   // (entries past rem are not written by the warps)
+          V a[8];
+#pragma unroll
+          for (int w2 = 0; w2 < 8; ++w2) a[w2] = red[(w2 * PG + g) * 64 + q];
+#pragma unroll
+          for (int s2 = 4; s2; s2 >>= 1)
+#pragma unroll
+            for (int w2 = 0; w2 < s2; ++w2) a[w2] = vadd(a[w2], a[w2 + s2]);
+          out(p0 + g, qb + q, a[0], sv);
+        }
+      }
+      __syncthreads();
     }
   }
-#pragma unroll
-  for (int p = 0; p < NO2; ++p)
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const cff r = kacc_lanes(part[p][u], lpr, 32);
-      const int q = q0 + lpr * u;
-      if (sub == 0 && q < 64) red[(warp * NO2 + p) * 64 + q] = cff_val(r);
-    }
-  __syncthreads();
-  for (int e = tid; e < NO2 * d.rmax; e += blockDim.x) {
-    const int p = e / d.rmax, q = e % d.rmax;
-    int rkp = 0;
-#pragma unroll
-    for (int pp2 = 0; pp2 < NO2; ++pp2)
-      if (pp2 == p) rkp = rk[pp2];
-    zd acc = zd();
-    if (q < rkp)   // entries q >= the pair's rank are not written by every warp
-      for (int w2 = 0; w2 < 8; ++w2) acc += red[(w2 * NO2 + p) * 64 + q];
-    st(Pj<NO>(d, n, slot, lv, p) + q, q < rkp ? acc * Sp<NO>(d, 2, n, blk, p)[q] : zd());
-  }
-  __syncthreads();
+}
+__device__ __forceinline__ zd scale_sv(const zd& a, double s) { return a * s; }
+__device__ __forceinline__ zf scale_sv(const cff& a, double s) {
+  const ffl f = ff_of(s);
+  return zf(ff_mul(a.re, f).hi, ff_mul(a.im, f).hi);
 }
 
-// Sum over q < rk of P[q] * F[q] (or P[q] * conj(F[q])): the far field of one
-// compressed block at one row or column, P its projection vector staged in
-// shared memory, F the block's factor row in global memory.  Four threads
-// share an output (q = sl, sl + 4, ...) and each keeps eight loads of F in
-// flight, so the row streams instead of waiting on one load per term.
-template <typename R, typename S, bool CONJ>
-__device__ __forceinline__ cx<R> lr_dot4(const cx<R>* P, const S* F, int rk, int sl) {
-  cx<R> acc = cx<R>(0);
-  for (int q0 = sl; q0 < rk; q0 += 32) {
-    cx<R> f[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int q = q0 + 4 * u;
-      f[u] = q < rk ? ldr<R>(F + q) : cx<R>(0);
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) acc = cfma(P[q0 + 4 * u < rk ? q0 + 4 * u : 0], CONJ ? f[u].conj() : f[u], acc);
+// The blocks and ranks of Sigma^R that cover leaf jl (of tab = colblk or
+// rowblk; retarded: only blocks with built rows), slot by slot, into rk, blk.
+template <int NO, typename R>
+__device__ __forceinline__ void leaf_table(const Dev& d, int n, int jl, bool cols, int* rk, int* blk, int t0) {
+  constexpr int NO2 = NO * NO;
+  const int* tab = cols ? d.colblk : d.rowblk;
+  for (int e = t0; e < d.maxl * NO2; e += blockDim.x) {
+    // slot order: target-major (retarded: target j = p % N_o; lesser: m = p / N_o)
+    const int tg = e / (d.maxl * NO), lv = (e / NO) % d.maxl, oth = e % NO, p = cols ? oth * NO + tg : tg * NO + oth;
+    int b = tab[jl * d.maxl + lv];
+    if (b >= 0 && cols && d.b_r0[b] >= d.cdir) b = -1;
+    rk[e] = b >= 0 ? *Rk<NO>(d, 2, n, b, p) : 0;
+    if (tg == 0 && oth == 0) blk[lv] = b;
   }
-  return acc;
+}
+// Pack the projections of the current leaf: entry e of target tg belongs to
+// e in [start[tg maxl NO], start[(tg + 1) maxl NO]).  Every thread calls it.
+template <int NO, typename R>
+__device__ __forceinline__ void leaf_pack(const Dev& d, int A, bool cols, const SweepMem<NO, R>& sm, const int* rk,
+                                          const int* blk) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (warp == 0) {   // first packed entry of each slot
+    int carry = 0;
+    for (int s0 = 0; s0 < sm.nslot; s0 += 32) {
+      const int r = s0 + lane < sm.nslot ? rk[s0 + lane] : 0;
+      int x = r;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, x, o);
+        if (lane >= o) x += y;
+      }
+      if (s0 + lane < sm.nslot) sm.start[s0 + lane] = carry + x - r;
+      carry += __shfl_sync(FULL, x, 31);
+    }
+    if (lane == 0) sm.start[sm.nslot] = carry;
+  }
+  __syncthreads();
+  for (int s = warp; s < sm.nslot; s += 8) {
+    const int r = rk[s];
+    if (!r) continue;
+    const int tg = s / (d.maxl * NO), lv = (s / NO) % d.maxl, oth = s % NO, p = cols ? oth * NO + tg : tg * NO + oth;
+    const int b = blk[lv], r0 = d.b_r0[b], c0 = d.b_c0[b];
+    const long long base = cols ? (d.b_voff[b] + (long long)p * (d.b_c1[b] - c0) + (A - c0)) * d.rmax
+                                : (d.b_uoff[b] + (long long)p * (d.b_r1[b] - r0) + (A - r0)) * d.rmax;
+    for (int q = lane; q < r; q += 32) {
+      sm.Pk[sm.start[s] + q] = sm.Ps[(size_t)s * d.rmax + q];
+      sm.off[sm.start[s] + q] = (unsigned)(base + q);
+    }
+  }
+  __syncthreads();
 }
 
 }  // namespace
 
 // ---------------------------------------------------------------------------
 // Retarded row, Eq. KBER: unknown y(t') = G^R(T, t') (row irow), solved for
-// t' = T-1 .. 0; the start block t' >= T-k is solved together.
+// t' = T-1 .. 0; the 2k points of the head are solved together.
+//
+// One CTA per (instance, orbital row) walks the chunks; its time is the
+// dependency chain of their phases, not bandwidth.  What keeps a phase short:
+// the last 64 solved points stay in shared memory (the far field of the lower
+// half of a leaf, the BDF terms and the band read them there), the complex64
+// form computes on the FP32 pipes throughout (FP64 copies of the row are
+// written a phase later, off the chain), the ranks of the next leaf are read
+// while this one is worked on, and the factors of all blocks over a leaf are
+// read as one packed list with eight loads in flight per thread (one block and
+// pair after the other, each waited for its rank and then for its row).
+// Both sweeps of an iteration, before and after these: 1.05 -> 0.53 ms (N_o = 2,
+// complex64, 128 instances, T = 600), 1.34 -> 0.69 ms (one instance, T = 1089),
+// 0.75 -> 0.43 ms (N_o = 2, FP64, 16 instances, T = 300).
 // ---------------------------------------------------------------------------
 template <int NO, typename S>
 __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, int staged) {
   constexpr int NO2 = NO * NO;
+  constexpr bool MX = Row64<NO, S>::separate;
   using R = typename Bulk<S>::R;
+  using V = typename Val<S>::t;
   const int n = blockIdx.y, irow = blockIdx.x;
   if (!d.active[n]) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   const int k = d.k, c = d.cdir, L = d.L;
   const double h = d.h;
   const DevW& W = d.w;
-  __shared__ zd sB[10 * NO];     // right-hand side of the head
-  __shared__ zd FB[64][NO];
-  __shared__ zd pbuf[8][128];
-  __shared__ zd Fs[CK][NO];
-  __shared__ zd Fb[CK][NO];      // the BDF part of Fs (rows at the chunk edge; zero elsewhere)
-  __shared__ zd Old[CK][NO];     // the chunk's previous iterate (convergence measure)
-  __shared__ zf Ff[CK][NO];      // complex64 form: the far field (Fs - Fb) rounded to complex64
-  __shared__ cff FbF[CK][NO];    // complex64 form: Fb in float-float
+  __shared__ zd sB[10 * NO];      // right-hand side of the head
+  __shared__ V FB[64][NO];        // far field of the leaf's columns from the rows beyond the leaf
+  __shared__ V Yl[64][NO];        // the last 64 solved points, y(t') in slot t' mod 64
+  __shared__ cx<R> yr[kRingRows][NO];   // y on the uncompressed rows, times the weights at the end T
+  __shared__ cx<R> Ff[CK][NO];    // the chunk's far field (FP64 form: with its BDF part)
+  __shared__ V Fb[CK][NO];        // the BDF terms reaching beyond the chunk (complex64 form)
+  __shared__ cx<R> Old[CK][NO];   // the chunk's previous iterate (convergence measure)
   __shared__ double serr;
-  extern __shared__ __align__(16) zd ctile[];  // for each chunk its staged inverse (N_o <= 2);
-                                 // at leaf entry (staged != 0) the block projections
-                                 // [maxl][NO2][rmax]
+  extern __shared__ __align__(16) char dyn[];
+  zd* ctile = reinterpret_cast<zd*>(dyn);
+  SweepMem<NO, R> sm(dyn + kBufBytes<NO>, d.maxl, d.rmax);
   __shared__ __align__(8) uint64_t cbar;   // completion of the inverse's bulk copy
   __shared__ int s_stage;                  // 0 once a wait for a copy has timed out
   uint32_t cphase = 0;
+  const int top = T - 2 * k - 1;   // the highest point of the chunks (none while T <= 2k)
+  int buf = 0;                     // table buffer of the current leaf
   if (tid == 0) {
     serr = 0.0;
     s_stage = 1;
-    if (kInvStage<NO, S>) mbar_init(&cbar);
+    if (kInvStage<NO>) mbar_init(&cbar);
   }
   // The row being solved lives in FP64 during the sweep (in the complex64
   // storage form a separate buffer), so the point-to-point recursion of the
-  // sweep (BDF terms, point solves) does not accumulate storage rounding.
+  // sweep (BDF terms, chunk solves) does not accumulate storage rounding.
   // yp: the FP64 row; sp: its storage, written at the same time (rounded in
   // the complex64 form), which the FP32 bulk sums read; it holds the previous
   // iterate until an element is overwritten (the convergence measure).
@@ -240,7 +388,8 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
   Y* rowy = Row64<NO, S>::get(d, n, 0, T, rowp);
   auto yp = [&](int tp) { return rowy + (long long)tp * NO2 + irow * NO; };
   auto sp = [&](int tp) { return rowp + (long long)tp * NO2 + irow * NO; };
-  double myerr = 0.0;
+  decltype(vdist(V(), cx<R>())) myerr = 0;
+  if (staged && top >= 0 && c > 0) leaf_table<NO, R>(d, n, (min(c, top + 1) - 1) / L, true, sm.rk, sm.blk, tid);
   // ---- the head: points T-s, s = 1..hs, and y(T) = -i.  Its right-hand side
   // is row T of Sigma^R (and the derivative's y(T) term) alone; 8 threads per
   // element of the product with the head's inverse ----
@@ -264,104 +413,214 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
       for (int off = 1; off < 8; off <<= 1)
         y += zd(__shfl_xor_sync(grp, y.re, off), __shfl_xor_sync(grp, y.im, off));
       if (sl == 0) {
-        myerr = fmax(myerr, (y - ld(sp(T - s) + j)).abs2());
+        V v;
+        vset(v, y);
+        myerr = fmax(myerr, vdist(v, ldr<R>(sp(T - s) + j)));
+        Yl[(T - s) & 63][j] = v;
         st(yp(T - s) + j, y);
-        if constexpr (Row64<NO, S>::separate) st(sp(T - s) + j, y);
+        if constexpr (MX) vstore(sp(T - s) + j, v);
       }
     }
   }
   if (tid < NO) {
-    const zd v = (tid == irow) ? zd(0, -1) : zd();
-    myerr = fmax(myerr, (ld(sp(T) + tid) - v).abs2());
-    st(yp(T) + tid, v);
-    if constexpr (Row64<NO, S>::separate) st(sp(T) + tid, v);
+    V v;
+    vset(v, (tid == irow) ? zd(0, -1) : zd());
+    myerr = fmax(myerr, vdist(v, ldr<R>(sp(T) + tid)));
+    st(yp(T) + tid, v64(v));
+    if constexpr (MX) vstore(sp(T) + tid, v);
   }
   __syncthreads();
-  const int top = T - 2 * k - 1;   // the highest point of the chunks (none while T <= 2k)
+  // FP64 copies of the points [wa, wa + wn) (complex64 form), by the last threads first
+  auto write64 = [&](int wa, int wn) {
+    if constexpr (MX)
+      for (int e = blockDim.x - 1 - tid; e < wn * NO; e += blockDim.x)
+        st(yp(wa + e / NO) + e % NO, cff_val(Yl[(wa + e / NO) & 63][e % NO]));
+  };
+  bool first_comp = true;
+  int wa = 0, wn = 0;
   for (int cc = top >= 0 ? top / CK : -1; cc >= 0; --cc) {
     const int a = cc * CK, b = min(a + CK, top + 1), cn = b - a;
     const bool comp = (c > 0 && b <= c);
     const int jl = comp ? a / L : 0, A = jl * L, E = comp ? (jl + 1) * L : 0;
     if (comp && (b == E || b == top + 1)) {   // (the top chunk may end inside its leaf)
-      // Entering leaf jl from above.  (1) projections pi_B = sum_s y(s) U_B(s,:) S_B
-      // of the blocks whose columns end at E, rows summed in 4 slices.
+      // Entering leaf jl from above.
+      const int* rk = sm.rk + buf * sm.nslot;
+      const int* blks = sm.blk + buf * d.maxl;
+      const int nr = T + 1 - c;
+      if (first_comp) {   // the uncompressed rows with their weights at the end T
+        first_comp = false;
+        for (int e = tid; e < nr * NO; e += blockDim.x) {
+          const int s2 = c + e / NO;
+          const cx<R> v = ldr<R>(sp(s2) + e % NO);
+          yr[e / NO][e % NO] = T - s2 <= k ? v * rule_wr<R>(W, T + 2 * k + 1, T - s2) : v;
+        }
+      }
+      // (1) projections pi_B = sum_s y(s) U_B(s,:) S_B of the blocks whose columns end at E
       for (int lv = 0; lv < d.maxl; ++lv) {
-        const int blk = d.colblk[jl * d.maxl + lv];
-        if (blk < 0 || d.b_c1[blk] != E) continue;
+        const int blk = staged ? blks[lv] : d.colblk[jl * d.maxl + lv];
+        if (blk < 0 || d.b_c1[blk] != E || d.b_r0[blk] >= c) continue;
         const int r0 = d.b_r0[blk], rl = min(d.b_r1[blk], c);
-        if constexpr (kStage<NO> && Row64<NO, S>::separate) {   // complex64 form: all pairs in one
-          if (d.rmax <= 64) {                                     // pass (ctile is free here)
-            proj_block<NO, S, true>(d, n, blk, lv, irow, r0, rl,
-                                    [&](int s2, int m) { return ldr<R>(sp(s2) + m); }, ctile);
-            continue;
+        auto slot = [&](int p) { return ((p % NO) * d.maxl + lv) * NO + p / NO; };
+        proj_block<NO, S, true>(
+            d, n, blk, r0, rl, [&](int s2, int m) { return ldr<R>(sp(s2) + m); },
+            [&](int p) { return staged ? rk[slot(p)] : *Rk<NO>(d, 2, n, blk, p); }, dyn,
+            [&](int p, int q, const V& v, double sv) {
+              if (staged) sm.Ps[(size_t)slot(p) * d.rmax + q] = scale_sv(v, sv);
+              else reinterpret_cast<cx<R>*>(Pj<NO>(d, n, irow, lv, p))[q] = scale_sv(v, sv);
+            });
+      }
+      __syncthreads();
+      if (staged) leaf_pack<NO, R>(d, A, true, sm, rk, blks);
+      // (2) for every column of the leaf: uncompressed rows s in [c, T], the
+      // blocks below the leaf (weight 1) and the near-diagonal corrections;
+      // 256 / L threads per column.
+      if (staged && jl > 0)
+        leaf_table<NO, R>(d, n, jl - 1, true, sm.rk + (buf ^ 1) * sm.nslot, sm.blk + (buf ^ 1) * d.maxl, blockDim.x - 1 - tid);
+      {
+        const int lpc = blockDim.x / L, col = tid / lpc, sl = tid % lpc, tp = A + col;
+        KAcc<R> ka[NO];   // FP32 history sums, compensated (FP64 in the FP64 form)
+        constexpr int RB = NO == 1 ? 8 : NO == 2 ? (MX ? 4 : 2) : 1;   // rows in flight
+        const S* Sr = static_cast<const S*>(d.SR) + ((long long)n * d.ring * d.nt + tp) * NO2;
+        const int s0 = c % d.ring;
+        for (int i0 = sl; i0 < nr; i0 += lpc * RB) {
+          cx<R> sv[RB][NO2];
+#pragma unroll
+          for (int u = 0; u < RB; ++u) {
+            const int i = i0 + lpc * u;
+            int slot = s0 + i;
+            if (slot >= d.ring) slot -= d.ring;
+            const S* s = Sr + (long long)slot * d.nt * NO2;
+#pragma unroll
+            for (int q = 0; q < NO2; ++q) sv[u][q] = i < nr ? ldr<R>(s + q) : cx<R>(0);
+          }
+          cx<R> pa[NO];
+#pragma unroll
+          for (int j = 0; j < NO; ++j) pa[j] = cx<R>(0);
+#pragma unroll
+          for (int u = 0; u < RB; ++u) {
+            const int i = min(i0 + lpc * u, nr - 1), dd = c + i - tp;
+            const R wd = dd <= k && dd >= 0 ? rule_wr<R>(W, 2 * k + 1 + dd, dd) : (R)1;
+#pragma unroll
+            for (int m = 0; m < NO; ++m) {
+              const cx<R> ym = yr[i][m] * wd;
+#pragma unroll
+              for (int j = 0; j < NO; ++j) pa[j] = cfma(ym, sv[u][m * NO + j], pa[j]);
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < NO; ++j) ka[j].add(pa[j]);
+        }
+        if (staged) {
+          const S* Vb = static_cast<const S*>(d.hod[2].V) + (long long)n * d.vtot * d.rmax + (long long)col * d.rmax;
+#pragma unroll
+          for (int j = 0; j < NO; ++j) {
+            const int e1 = sm.start[(j + 1) * d.maxl * NO];
+            for (int e0 = sm.start[j * d.maxl * NO] + sl; e0 < e1; e0 += lpc * FOLD) {
+              cx<R> f[FOLD], pb = cx<R>(0);
+#pragma unroll
+              for (int u = 0; u < FOLD; ++u) {
+                const int e = e0 + lpc * u;
+                f[u] = e < e1 ? ldr<R>(Vb + sm.off[e]) : cx<R>(0);
+              }
+#pragma unroll
+              for (int u = 0; u < FOLD; ++u) pb = cfma(sm.Pk[min(e0 + lpc * u, e1 - 1)], f[u].conj(), pb);
+              ka[j].add(pb);
+            }
+          }
+        } else {
+          for (int lv = 0; lv < d.maxl; ++lv) {
+            const int blk = d.colblk[jl * d.maxl + lv];
+            if (blk < 0 || d.b_r0[blk] >= c) continue;
+#pragma unroll
+            for (int p = 0; p < NO2; ++p) {
+              const int rkp = *Rk<NO>(d, 2, n, blk, p);
+              const S* Vr = Vp<NO, S>(d, 2, n, blk, p) + (long long)(tp - d.b_c0[blk]) * d.rmax;
+              const cx<R>* P = reinterpret_cast<const cx<R>*>(Pj<NO>(d, n, irow, lv, p));
+              cx<R> pb = cx<R>(0);
+              for (int q = sl; q < rkp; q += lpc) pb = cfma(P[q], ldr<R>(Vr + q).conj(), pb);
+              ka[p % NO].add(pb);
+            }
           }
         }
-        for (int p = 0; p < NO2; ++p) {
-          const int m = p / NO;
-          const int rk = *Rk<NO>(d, 2, n, blk, p);
-          const S* U = Up<NO, S>(d, 2, n, blk, p);
-          KAcc<R> part[4];
-          for (int s0 = r0 + warp; s0 < rl; s0 += 8 * FOLD) {  // warps over rows, lanes over rank
-            cx<R> pp[4] = {cx<R>(0), cx<R>(0), cx<R>(0), cx<R>(0)};
+        V acc[NO];
 #pragma unroll
-            for (int jj = 0; jj < FOLD; ++jj) {
-              const int s2 = s0 + 8 * jj;
-              if (s2 < rl) {
-                const cx<R> yv = ldr<R>(sp(s2) + m);
-                const S* ur = U + (long long)(s2 - r0) * d.rmax;
+        for (int j = 0; j < NO; ++j) vset(acc[j], zd());
+        if (E < c && __any_sync(FULL, tp + k >= E))
+          for (int s2 = E + sl; s2 <= tp + k && s2 < c; s2 += lpc) {   // (w - 1) of the band's entries
+            const S* bd = Bd<NO, S>(d, n, s2, s2 - tp);
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  const int q = lane + 32 * u;
-                  if (q < rk) pp[u] = cfma(yv, ldr<R>(ur + q), pp[u]);
+            for (int m = 0; m < NO; ++m) {
+              const V ym = vreal(Yl[s2 & 63][m], W.omega[s2 - tp] - 1.0, W.wm1f[s2 - tp]);
+#pragma unroll
+              for (int j = 0; j < NO; ++j) {
+                if constexpr (MX) acc[j] = cff_add(acc[j], cff_mul(ym, cff_of(ldr<R>(bd + m * NO + j))));
+                else acc[j] = cfma(ym, ld(bd + m * NO + j), acc[j]);
+              }
+            }
+          }
+#pragma unroll
+        for (int j = 0; j < NO; ++j) {
+          V r = kacc_lanes(ka[j], 1, lpc);
+          if (E < c && __any_sync(FULL, tp + k >= E)) {
+            for (int off = 1; off < lpc; off <<= 1) acc[j] = vadd(acc[j], vshfl_xor(acc[j], off));
+            r = vadd(r, acc[j]);
+          }
+          if (sl == 0) FB[col][j] = r;
+        }
+      }
+      buf ^= 1;
+      __syncthreads();
+    }
+    // the inverse of this chunk into shared memory, overlapping the far field
+    const bool stage_now = kInvStage<NO> && s_stage;
+    if (stage_now && tid == 0) bulk_g2s(ctile, Cinv<NO>(d, n, cc, 0), kInvStage<NO>, &cbar);
+    // ---- far field of the chunk: rows s >= b not covered above; 8 threads per column ----
+    {
+      const int col = tid >> 3, sl = tid & 7;
+      const int tp = a + col;
+      KAcc<R> ka[NO];   // FP32 history sums, compensated (FP64 in the FP64 form)
+      cx<R> old = cx<R>(0);
+      if (sl < NO && col < cn) old = ldr<R>(sp(tp) + sl);
+      if (col < cn) {
+        if (comp) {   // the rest of the leaf (at most 32 points, solved last)
+          const S* lf = static_cast<const S*>(d.hod[2].leaf) +
+                        ((long long)n * d.leaftot + (long long)jl * ((long long)L * (L + 1) / 2) + (tp - A)) * NO2;
+          cx<R> pa[NO];
+#pragma unroll
+          for (int j = 0; j < NO; ++j) pa[j] = cx<R>(0);
+#pragma unroll
+          for (int u0 = 0; u0 < 4; u0 += kLB<NO, S>) {
+            cx<R> sv[kLB<NO, S>][NO2];
+#pragma unroll
+            for (int u = 0; u < kLB<NO, S>; ++u) {
+              const int s2 = b + sl + 8 * (u0 + u);
+#pragma unroll
+              for (int q = 0; q < NO2; ++q) sv[u][q] = s2 < E ? ldr<R>(lf + tri(s2 - A) * NO2 + q) : cx<R>(0);
+            }
+#pragma unroll
+            for (int u = 0; u < kLB<NO, S>; ++u) {
+              const int s2 = b + sl + 8 * (u0 + u);
+              if (s2 < E) {
+                const R ws = rule_wr<R>(W, T - tp, T - s2);
+#pragma unroll
+                for (int m = 0; m < NO; ++m) {
+                  const cx<R> ym = vbulk(Yl[s2 & 63][m]) * ws;
+#pragma unroll
+                  for (int j = 0; j < NO; ++j) pa[j] = cfma(ym, sv[u][m * NO + j], pa[j]);
                 }
               }
             }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) part[u].add(pp[u]);
           }
 #pragma unroll
-          for (int u = 0; u < 4; ++u) pbuf[warp][lane + 32 * u] = part[u].get();
-          __syncthreads();
-          if (tid < d.rmax) {
-            zd acc = zd();
-            for (int w2 = 0; w2 < 8; ++w2) acc += pbuf[w2][tid];
-            st(Pj<NO>(d, n, irow, lv, p) + tid, tid < rk ? acc * Sp<NO>(d, 2, n, blk, p)[tid] : zd());
-          }
-          __syncthreads();
-        }
-      }
-      __syncthreads();
-      // projections of every block over this leaf's columns, staged in shared
-      // memory for the far-field loop below (the buffer of the chunk
-      // inverses, whose copies are issued only after it)
-      cx<R>* Ps = reinterpret_cast<cx<R>*>(ctile);
-      if (staged) {
-        const int per = NO2 * d.rmax;
-        for (int e = tid; e < d.maxl * per; e += blockDim.x) {
-          const int lv = e / per, p = (e / d.rmax) % NO2, q = e % d.rmax;
-          const int blk = d.colblk[jl * d.maxl + lv];
-          Ps[e] = (blk >= 0 && d.b_r0[blk] < c) ? ldr<R>(Pj<NO>(d, n, irow, lv, p) + q) : cx<R>(0);
-        }
-        __syncthreads();
-      }
-      // (2) for every column of the leaf: uncompressed rows s in [c, T], the
-      // blocks below the leaf (weight 1) and the near-diagonal corrections;
-      // 4 threads per column.
-      {
-        const int col = tid >> 2, sl = tid & 3;
-        zd acc[NO];
-#pragma unroll
-        for (int j = 0; j < NO; ++j) acc[j] = zd();
-        KAcc<R> ka[NO];   // FP32 history sums, compensated (FP64 in the FP64 form)
-        const int tp = A + col;
-        if (col < L) {
-          for (int s0 = c + sl; s0 <= T; s0 += 4 * FOLD) {
+          for (int j = 0; j < NO; ++j) ka[j].add(pa[j]);
+        } else {
+          for (int s0 = b + sl; s0 <= T; s0 += 8 * FOLD) {
             cx<R> pa[NO];
 #pragma unroll
             for (int j = 0; j < NO; ++j) pa[j] = cx<R>(0);
 #pragma unroll
             for (int jj = 0; jj < FOLD; ++jj) {
-              const int s2 = s0 + 4 * jj;
+              const int s2 = s0 + 8 * jj;
               if (s2 <= T) {
                 const R ws = rule_wr<R>(W, T - tp, T - s2);
                 const S* yl = sp(s2);
@@ -377,121 +636,28 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
 #pragma unroll
             for (int j = 0; j < NO; ++j) ka[j].add(pa[j]);
           }
-          for (int lv = 0; lv < d.maxl; ++lv) {
-            const int blk = d.colblk[jl * d.maxl + lv];
-            if (blk < 0 || d.b_r0[blk] >= c) continue;
-            const int c0 = d.b_c0[blk];
-#pragma unroll
-            for (int p = 0; p < NO2; ++p) {
-              const int j = p % NO;
-              const int rk = *Rk<NO>(d, 2, n, blk, p);
-              const S* V = Vp<NO, S>(d, 2, n, blk, p) + (long long)(tp - c0) * d.rmax;
-              cx<R> pb = cx<R>(0);
-              if (staged) {
-                pb = lr_dot4<R, S, true>(Ps + (lv * NO2 + p) * d.rmax, V, rk, sl);
-              } else {
-                const double2* P = Pj<NO>(d, n, irow, lv, p);
-                for (int q = sl; q < rk; q += 4) pb = cfma(ldr<R>(P + q), ldr<R>(V + q).conj(), pb);
-              }
-              ka[j].add(pb);
-            }
-          }
-          for (int s2 = E + sl; s2 <= tp + k && s2 < c; s2 += 4) {
-            const double ws = rule_w(W, T - tp, T - s2) - 1.0;
-            const S* bd = Bd<NO, S>(d, n, s2, s2 - tp);
-            const Y* yl = yp(s2);
-#pragma unroll
-            for (int m = 0; m < NO; ++m) {
-              const zd ym = ld(yl + m) * ws;
-#pragma unroll
-              for (int j = 0; j < NO; ++j) acc[j] = cfma(ym, ld(bd + m * NO + j), acc[j]);
-            }
-          }
         }
-#pragma unroll
-        for (int j = 0; j < NO; ++j) acc[j] += ka[j].get();
-#pragma unroll
-        for (int j = 0; j < NO; ++j) {
-          acc[j] += zd(__shfl_xor_sync(FULL, acc[j].re, 1), __shfl_xor_sync(FULL, acc[j].im, 1));
-          acc[j] += zd(__shfl_xor_sync(FULL, acc[j].re, 2), __shfl_xor_sync(FULL, acc[j].im, 2));
-        }
-        if (sl == 0 && col < L)
-#pragma unroll
-          for (int j = 0; j < NO; ++j) FB[col][j] = acc[j];
       }
-      __syncthreads();
+      V r[NO];
+#pragma unroll
+      for (int j = 0; j < NO; ++j) r[j] = reduce8(ka[j]);
+      if (sl < NO && col < cn) {   // lane sl of the group finishes component sl
+        V F = pick(r, sl), fb;
+        if (comp) F = vadd(F, FB[tp - A][sl]);
+        F = vreal(F, h, W.hf);
+        vset(fb, zd());
+        if (col >= cn - k)   // BDF terms reaching above the chunk: (-i a_j / h) y(s2)
+          for (int jj = b - tp; jj <= k; ++jj) fb = vbdf(fb, Yl[(tp + jj) & 63][sl], W, jj);
+        if constexpr (MX) {
+          Ff[col][sl] = vbulk(F);
+          Fb[col][sl] = fb;
+        } else {
+          Ff[col][sl] = F + fb;
+        }
+        Old[col][sl] = old;
+      }
     }
-    // the inverse of this chunk into shared memory, overlapping the far field
-    const bool stage_now = kInvStage<NO, S> && s_stage;
-    if (stage_now && tid == 0) bulk_g2s(ctile, Cinv<NO>(d, n, cc, 0), kInvStage<NO, S>, &cbar);
-    // ---- far field of the chunk: rows s >= b not covered above; 8 threads per column ----
-    {
-      const int col = tid >> 3, sl = tid & 7;
-      const int tp = a + col;
-      zd acc[NO];
-#pragma unroll
-      for (int j = 0; j < NO; ++j) acc[j] = zd();
-        KAcc<R> ka[NO];   // FP32 history sums, compensated (FP64 in the FP64 form)
-      if (col < cn) {
-        const int s_end = comp ? E : T + 1;   // compressed: the rest of the leaf; else every later row
-        for (int s0 = b + sl; s0 < s_end; s0 += 8 * FOLD) {
-          cx<R> pa[NO];
-#pragma unroll
-          for (int j = 0; j < NO; ++j) pa[j] = cx<R>(0);
-#pragma unroll
-          for (int jj = 0; jj < FOLD; ++jj) {
-            const int s2 = s0 + 8 * jj;
-            if (s2 < s_end) {
-              const R ws = rule_wr<R>(W, T - tp, T - s2);
-              const S* yl = sp(s2);
-              const S* sr = comp ? Lf<NO, S>(d, 2, n, jl, s2, tp) : el<NO, S>(d.SR, d, n, s2, tp);
-#pragma unroll
-              for (int m = 0; m < NO; ++m) {
-                const cx<R> ym = ldr<R>(yl + m) * ws;
-#pragma unroll
-                for (int j = 0; j < NO; ++j) pa[j] = cfma(ym, ldr<R>(sr + m * NO + j), pa[j]);
-              }
-            }
-          }
-#pragma unroll
-          for (int j = 0; j < NO; ++j) ka[j].add(pa[j]);
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < NO; ++j) {
-        const auto r = reduce8(ka[j]);
-        if (sl == 0) acc[j] = val_of(r);
-      }
-      if (sl == 0 && col < cn) {
-        zd F[NO];
-        zd Fbd[NO];
-#pragma unroll
-        for (int j = 0; j < NO; ++j) {
-          F[j] = (acc[j] + (comp ? FB[tp - A][j] : zd())) * h;
-          Fbd[j] = zd();
-        }
-        for (int jj = 1; jj <= k; ++jj) {  // BDF terms reaching above the chunk: (-i a_j / h) y(s2)
-          const int s2 = tp + jj;
-          if (s2 < b) continue;
-          const double cj = W.ah[jj];
-#pragma unroll
-          for (int m = 0; m < NO; ++m) {
-            const zd y = ld(yp(s2) + m);
-            Fbd[m] = zd(fma(cj, y.im, Fbd[m].re), fma(-cj, y.re, Fbd[m].im));
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < NO; ++j) {
-          Fs[col][j] = F[j] + Fbd[j];
-          Fb[col][j] = Fbd[j];
-          Ff[col][j] = zf((float)F[j].re, (float)F[j].im);
-          FbF[col][j] = cff_of(Fbd[j]);
-        }
-      }
-      if (sl == 1 && col < cn)
-#pragma unroll
-        for (int j = 0; j < NO; ++j) Old[col][j] = ld(sp(tp) + j);
-    }
+    write64(wa, wn);
     __syncthreads();
     {
       // y = F C^-1 (row vector times the chunk's inverse, lower triangular),
@@ -510,8 +676,8 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
       constexpr int LD = CK * NO;
       for (int o8 = tid; o8 < CK * NO * 8; o8 += blockDim.x) {
         const int o = o8 >> 3, sl = o8 & 7, ti = o / NO, j = o % NO;
-        zd sacc = zd();
-        if constexpr (Row64<NO, S>::separate) {
+        V out;
+        if constexpr (MX) {
           // complex64 form: far field x hi in FP32, the k edge rows x (hi + lo)
           // in float-float, reduced over the 8 lanes in float-float
           const float2* Mh = reinterpret_cast<const float2*>(Mg);
@@ -521,74 +687,77 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
 #pragma unroll
             for (int m = 0; m < NO; ++m)
               s32 = cfma(Ff[si][m], ldr<float>(Mh + (long long)(si * NO + m) * LD + ti * NO + j), s32);
-          cff sf = cff_of(s32);
+          out = cff_of(s32);
           for (int si = max(cn - k, 0) + sl; si < cn; si += 8)
 #pragma unroll
             for (int m = 0; m < NO; ++m) {
               const long long e = (long long)(si * NO + m) * LD + ti * NO + j;
               const float2 hv = Mh[e], lv = Ml[e];
-              sf = cff_add(sf, cff_mul(FbF[si][m], cff{{hv.x, lv.x}, {hv.y, lv.y}}));
+              out = cff_add(out, cff_mul(Fb[si][m], cff{{hv.x, lv.x}, {hv.y, lv.y}}));
             }
-#pragma unroll
-          for (int off = 1; off < 8; off <<= 1) sf = cff_add(sf, cff_shfl_xor(sf, off));
-          if (sl == 0) sacc = cff_val(sf);
         } else {
+          out = zd();
           for (int si = (ti & ~7) + sl; si < cn; si += 8)
 #pragma unroll
-            for (int m = 0; m < NO; ++m) sacc = cfma(Fs[si][m], ld(Mg + (long long)(si * NO + m) * LD + ti * NO + j), sacc);
-#pragma unroll
-          for (int off = 1; off < 8; off <<= 1)
-            sacc += zd(__shfl_xor_sync(FULL, sacc.re, off), __shfl_xor_sync(FULL, sacc.im, off));
+            for (int m = 0; m < NO; ++m) out = cfma(Ff[si][m], ld(Mg + (long long)(si * NO + m) * LD + ti * NO + j), out);
         }
+#pragma unroll
+        for (int off = 1; off < 8; off <<= 1) out = vadd(out, vshfl_xor(out, off));
         if (sl == 0 && ti < cn) {
-          myerr = fmax(myerr, (sacc - Old[ti][j]).abs2());
-          st(yp(a + ti) + j, sacc);
-          if constexpr (Row64<NO, S>::separate) st(sp(a + ti) + j, sacc);
+          myerr = fmax(myerr, vdist(out, Old[ti][j]));
+          Yl[(a + ti) & 63][j] = out;
+          vstore(sp(a + ti) + j, out);
         }
       }
+      wa = a;
+      wn = cn;
     }
     __syncthreads();
   }
-  myerr = sqrt(warp_max(myerr));
-  if (lane == 0 && myerr > 0) atomic_max_nonneg(&serr, myerr);
+  write64(wa, wn);
+  const double e1 = sqrt(warp_max((double)myerr));
+  if (lane == 0 && e1 > 0) atomic_max_nonneg(&serr, e1);
   __syncthreads();
   if (tid == 0) atomic_max_nonneg(d.err + n, serr);
   // after a timed-out wait, a copy may still be in flight into this CTA's
   // shared memory: wait for it (bounded) before the CTA exits
-  if (kInvStage<NO, S> && tid == 0 && !s_stage) mbar_wait(&cbar, cphase ^ 1u, kCopyWaitPolls);
+  if (kInvStage<NO> && tid == 0 && !s_stage) mbar_wait(&cbar, cphase ^ 1u, kCopyWaitPolls);
 }
 
 // ---------------------------------------------------------------------------
-// Lesser column, Eq. KBEL: unknown x(t) = G^<(t, T) (column jc), t = 0..T.
+// Lesser column, Eq. KBEL: unknown x(t) = G^<(t, T) (column jc), t = 0..T; the
+// same phases as the retarded sweep, upwards.
 // ---------------------------------------------------------------------------
 template <int NO, typename S>
 __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, int staged) {
   constexpr int NO2 = NO * NO;
+  constexpr bool MX = Row64<NO, S>::separate;
   using R = typename Bulk<S>::R;
+  using V = typename Val<S>::t;
   const int n = blockIdx.y, jc = blockIdx.x;
   if (!d.active[n]) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int k = d.k, c = d.cdir, L = d.L;
   const double h = d.h;
   const DevW& W = d.w;
-  __shared__ zd FB[64][NO];
-  __shared__ zd pbuf[8][128];
-  __shared__ zd Fs[CK][NO];
-  __shared__ zd Fb[CK][NO];      // the BDF part of Fs (rows at the chunk edge; zero elsewhere)
-  __shared__ zd Old[CK][NO];     // the chunk's previous iterate (convergence measure)
-  __shared__ zf Ff[CK][NO];      // complex64 form: the far field (Fs - Fb) rounded to complex64
-  __shared__ cff FbF[CK][NO];    // complex64 form: Fb in float-float
+  __shared__ V FB[64][NO];        // far field of the leaf's rows from the columns before the leaf
+  __shared__ V Xl[64][NO];        // the last 64 solved points, x(t) in slot t mod 64
+  __shared__ V FT[NO];            // right-hand side of row T
+  __shared__ cx<R> Ff[CK][NO];    // the chunk's far field (FP64 form: with its BDF part)
+  __shared__ V Fb[CK][NO];        // the BDF terms reaching beyond the chunk (complex64 form)
+  __shared__ cx<R> Old[CK][NO];   // the chunk's previous iterate (convergence measure)
   __shared__ double serr;
-  extern __shared__ __align__(16) zd ctile[];  // for each chunk its staged inverse (N_o <= 2);
-                                 // at leaf entry (staged != 0) the block projections
-                                 // [maxl][NO2][rmax]
+  extern __shared__ __align__(16) char dyn[];
+  zd* ctile = reinterpret_cast<zd*>(dyn);
+  SweepMem<NO, R> sm(dyn + kBufBytes<NO>, d.maxl, d.rmax);
   __shared__ __align__(8) uint64_t cbar;   // completion of the inverse's bulk copy
   __shared__ int s_stage;                  // 0 once a wait for a copy has timed out
   uint32_t cphase = 0;
+  int buf = 0;
   if (tid == 0) {
     serr = 0.0;
     s_stage = 1;
-    if (kInvStage<NO, S>) mbar_init(&cbar);
+    if (kInvStage<NO>) mbar_init(&cbar);
   }
   // FP64 column during the sweep (see k_ret2); xp: as solved, sp: storage
   S* colp = el<NO, S>(d.GL, d, n, T, 0);
@@ -596,176 +765,173 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
   auto xp = [&](int t) { return coly + (long long)t * NO2; };  // element [m*NO + jc]
   auto sp = [&](int t) { return colp + (long long)t * NO2; };
   const double2* qs = d.qsrc + (long long)n * d.nt * NO2;
-  double myerr = 0.0;
+  decltype(vdist(V(), cx<R>())) myerr = 0;
   const int last = (d.rho_mode == 1) ? T - 1 : T;
-  if (warp == 0 && lane < NO) {  // x(0) = -[G^tv(T, 0+)]^dagger
-    const int m = lane;
-    zd v = ld(d.x0 + (long long)n * NO2 + m * NO + jc);
-    myerr = fmax(myerr, (v - ld(sp(0) + m * NO + jc)).abs2());
-    st(xp(0) + m * NO + jc, v);
-    if constexpr (Row64<NO, S>::separate) st(sp(0) + m * NO + jc, v);
+  if (staged && c > 0) leaf_table<NO, R>(d, n, 0, false, sm.rk, sm.blk, tid);
+  if (tid < NO) {  // x(0) = -[G^tv(T, 0+)]^dagger
+    const int m = tid;
+    const zd x = ld(d.x0 + (long long)n * NO2 + m * NO + jc);
+    V v;
+    vset(v, x);
+    myerr = fmax(myerr, vdist(v, ldr<R>(sp(0) + m * NO + jc)));
+    Xl[0][m] = v;
+    st(xp(0) + m * NO + jc, x);
+    if constexpr (MX) vstore(sp(0) + m * NO + jc, v);
   }
   __syncthreads();
+  auto write64 = [&](int wa, int wn) {
+    if constexpr (MX)
+      for (int e = blockDim.x - 1 - tid; e < wn * NO; e += blockDim.x)
+        st(xp(wa + e / NO) + (e % NO) * NO + jc, cff_val(Xl[(wa + e / NO) & 63][e % NO]));
+  };
+  int wa = 0, wn = 0;
   for (int cc = 0; cc * CK <= last; ++cc) {
     const int a = (cc == 0) ? 1 : cc * CK, b = min((cc + 1) * CK, last + 1), cn = b - a;
     if (cn <= 0) break;
     const bool comp = (c > 0 && b <= c);
     const int jl = comp ? a / L : 0, A = jl * L;
     if (comp && cc * CK == A) {
+      const int* rk = sm.rk + buf * sm.nslot;
+      const int* blks = sm.blk + buf * d.maxl;
       // Entering leaf jl.  (1) rho_B = S_B sum_l w_l conj(V_B(l,:)) x(l) for the
       // blocks whose rows start at A (w_l = omega_l for l <= k, else 1).
       for (int lv = 0; lv < d.maxl && jl > 0; ++lv) {
-        const int blk = d.rowblk[jl * d.maxl + lv];
+        const int blk = staged ? blks[lv] : d.rowblk[jl * d.maxl + lv];
         if (blk < 0 || d.b_r0[blk] != A) continue;
-        const int c0 = d.b_c0[blk], c1 = d.b_c1[blk];
-        if constexpr (kStage<NO> && Row64<NO, S>::separate) {   // complex64 form: all pairs in one
-          if (d.rmax <= 64) {                                     // pass (ctile is free here)
-            proj_block<NO, S, false>(d, n, blk, lv, jc, c0, c1, [&](int l, int nn) {
-              const R wl = (l <= k) ? (R)W.omega[l] : (R)1;
-              return ldr<R>(sp(l) + nn * NO + jc) * wl;
-            }, ctile);
-            continue;
-          }
-        }
-        for (int p = 0; p < NO2; ++p) {
-          const int nn = p % NO;
-          const int rk = *Rk<NO>(d, 2, n, blk, p);
-          const S* V = Vp<NO, S>(d, 2, n, blk, p);
-          KAcc<R> part[4];
-          for (int l0 = c0 + warp; l0 < c1; l0 += 8 * FOLD) {  // warps over columns, lanes over rank
-            cx<R> pp[4] = {cx<R>(0), cx<R>(0), cx<R>(0), cx<R>(0)};
-#pragma unroll
-            for (int jj = 0; jj < FOLD; ++jj) {
-              const int l = l0 + 8 * jj;
-              if (l < c1) {
-                const R wl = (l <= k) ? (R)W.omega[l] : (R)1;
-                const cx<R> xv = ldr<R>(sp(l) + nn * NO + jc) * wl;
-                const S* vr = V + (long long)(l - c0) * d.rmax;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  const int q = lane + 32 * u;
-                  if (q < rk) pp[u] = cfma(ldr<R>(vr + q).conj(), xv, pp[u]);
-                }
-              }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) part[u].add(pp[u]);
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) pbuf[warp][lane + 32 * u] = part[u].get();
-          __syncthreads();
-          if (tid < d.rmax) {
-            zd acc = zd();
-            for (int w2 = 0; w2 < 8; ++w2) acc += pbuf[w2][tid];
-            st(Pj<NO>(d, n, jc, lv, p) + tid, tid < rk ? acc * Sp<NO>(d, 2, n, blk, p)[tid] : zd());
-          }
-          __syncthreads();
-        }
+        auto slot = [&](int p) { return ((p / NO) * d.maxl + lv) * NO + p % NO; };
+        proj_block<NO, S, false>(
+            d, n, blk, d.b_c0[blk], d.b_c1[blk],
+            [&](int l, int nn) {
+              const cx<R> x = ldr<R>(sp(l) + nn * NO + jc);
+              return l <= k ? x * (R)W.omega[l] : x;
+            },
+            [&](int p) { return staged ? rk[slot(p)] : *Rk<NO>(d, 2, n, blk, p); }, dyn,
+            [&](int p, int q, const V& v, double sv) {
+              if (staged) sm.Ps[(size_t)slot(p) * d.rmax + q] = scale_sv(v, sv);
+              else reinterpret_cast<cx<R>*>(Pj<NO>(d, n, jc, lv, p))[q] = scale_sv(v, sv);
+            });
       }
       __syncthreads();
-      // projections of every block left of this leaf's rows, staged in shared
-      // memory for the loop below (the buffer of the chunk inverses, whose
-      // copies are issued only after it)
-      cx<R>* Ps = reinterpret_cast<cx<R>*>(ctile);
-      if (staged) {
-        const int per = NO2 * d.rmax;
-        for (int e = tid; e < d.maxl * per; e += blockDim.x) {
-          const int lv = e / per, p = (e / d.rmax) % NO2, q = e % d.rmax;
-          const int blk = d.rowblk[jl * d.maxl + lv];
-          Ps[e] = blk >= 0 ? ldr<R>(Pj<NO>(d, n, jc, lv, p) + q) : cx<R>(0);
-        }
-        __syncthreads();
-      }
+      if (staged) leaf_pack<NO, R>(d, A, false, sm, rk, blks);
       // (2) every row of the leaf: blocks left of it and near-diagonal corrections
+      if (staged && (jl + 1) * L < c)
+        leaf_table<NO, R>(d, n, jl + 1, false, sm.rk + (buf ^ 1) * sm.nslot, sm.blk + (buf ^ 1) * d.maxl, blockDim.x - 1 - tid);
       {
-        const int row = tid >> 2, sl = tid & 3;
+        const int lpc = blockDim.x / L, row = tid / lpc, sl = tid % lpc;
         const int t = A + row;
-        zd acc[NO];
-#pragma unroll
-        for (int m = 0; m < NO; ++m) acc[m] = zd();
         KAcc<R> ka[NO];   // FP32 history sums, compensated (FP64 in the FP64 form)
-        if (row < L) {
-          for (int lv = 0; lv < d.maxl; ++lv) {
-            const int blk = d.rowblk[jl * d.maxl + lv];
-            if (blk < 0) continue;
-            const int r0 = d.b_r0[blk];
+        if (staged) {
+          const S* Ub = static_cast<const S*>(d.hod[2].U) + (long long)n * d.utot * d.rmax + (long long)row * d.rmax;
 #pragma unroll
-            for (int p = 0; p < NO2; ++p) {
-              const int m = p / NO;
-              const int rk = *Rk<NO>(d, 2, n, blk, p);
-              const S* U = Up<NO, S>(d, 2, n, blk, p) + (long long)(t - r0) * d.rmax;
-              cx<R> pb = cx<R>(0);
-              if (staged) {
-                pb = lr_dot4<R, S, false>(Ps + (lv * NO2 + p) * d.rmax, U, rk, sl);
-              } else {
-                const double2* P = Pj<NO>(d, n, jc, lv, p);
-                for (int q = sl; q < rk; q += 4) pb = cfma(ldr<R>(U + q), ldr<R>(P + q), pb);
+          for (int m = 0; m < NO; ++m) {
+            const int e1 = sm.start[(m + 1) * d.maxl * NO];
+            for (int e0 = sm.start[m * d.maxl * NO] + sl; e0 < e1; e0 += lpc * FOLD) {
+              cx<R> f[FOLD], pb = cx<R>(0);
+#pragma unroll
+              for (int u = 0; u < FOLD; ++u) {
+                const int e = e0 + lpc * u;
+                f[u] = e < e1 ? ldr<R>(Ub + sm.off[e]) : cx<R>(0);
               }
+#pragma unroll
+              for (int u = 0; u < FOLD; ++u) pb = cfma(sm.Pk[min(e0 + lpc * u, e1 - 1)], f[u], pb);
               ka[m].add(pb);
             }
           }
-          for (int l = max(t - k, 0) + sl; l < A; l += 4) {
-            const double wl = rule_w(W, t, l) - 1.0;
-            const S* bd = Bd<NO, S>(d, n, t, t - l);
+        } else {
+          for (int lv = 0; lv < d.maxl; ++lv) {
+            const int blk = d.rowblk[jl * d.maxl + lv];
+            if (blk < 0) continue;
 #pragma unroll
-            for (int y = 0; y < NO; ++y) {
-              const zd xy = ld(xp(l) + y * NO + jc) * wl;
-#pragma unroll
-              for (int m = 0; m < NO; ++m) acc[m] = cfma(ld(bd + m * NO + y), xy, acc[m]);
+            for (int p = 0; p < NO2; ++p) {
+              const int rkp = *Rk<NO>(d, 2, n, blk, p);
+              const S* Ur = Up<NO, S>(d, 2, n, blk, p) + (long long)(t - d.b_r0[blk]) * d.rmax;
+              const cx<R>* P = reinterpret_cast<const cx<R>*>(Pj<NO>(d, n, jc, lv, p));
+              cx<R> pb = cx<R>(0);
+              for (int q = sl; q < rkp; q += lpc) pb = cfma(ldr<R>(Ur + q), P[q], pb);
+              ka[p / NO].add(pb);
             }
           }
         }
+        V acc[NO];
 #pragma unroll
-        for (int m = 0; m < NO; ++m) acc[m] += ka[m].get();
+        for (int m = 0; m < NO; ++m) vset(acc[m], zd());
+        const bool band = jl > 0 && __any_sync(FULL, t - k < A);
+        if (band)
+          for (int l = max(t - k, 0) + sl; l < A; l += lpc) {
+            const S* bd = Bd<NO, S>(d, n, t, t - l);
+#pragma unroll
+            for (int y = 0; y < NO; ++y) {
+              const V xy = vreal(Xl[l & 63][y], W.omega[t - l] - 1.0, W.wm1f[t - l]);
+#pragma unroll
+              for (int m = 0; m < NO; ++m) {
+                if constexpr (MX) acc[m] = cff_add(acc[m], cff_mul(cff_of(ldr<R>(bd + m * NO + y)), xy));
+                else acc[m] = cfma(ld(bd + m * NO + y), xy, acc[m]);
+              }
+            }
+          }
 #pragma unroll
         for (int m = 0; m < NO; ++m) {
-          acc[m] += zd(__shfl_xor_sync(FULL, acc[m].re, 1), __shfl_xor_sync(FULL, acc[m].im, 1));
-          acc[m] += zd(__shfl_xor_sync(FULL, acc[m].re, 2), __shfl_xor_sync(FULL, acc[m].im, 2));
+          V r = kacc_lanes(ka[m], 1, lpc);
+          if (band) {
+            for (int off = 1; off < lpc; off <<= 1) acc[m] = vadd(acc[m], vshfl_xor(acc[m], off));
+            r = vadd(r, acc[m]);
+          }
+          if (sl == 0) FB[row][m] = r;
         }
-        if (sl == 0 && row < L)
-#pragma unroll
-          for (int m = 0; m < NO; ++m) FB[row][m] = acc[m];
       }
+      buf ^= 1;
       __syncthreads();
     }
     const int fn = min(b, T) - a;   // rows solved with the chunk's inverse; row T, if it is here, follows them
     // the inverse of this chunk into shared memory, overlapping the far field
-    const bool stage_now = kInvStage<NO, S> && fn > 0 && s_stage;
-    if (stage_now && tid == 0) bulk_g2s(ctile, Cinv<NO>(d, n, cc, 1), kInvStage<NO, S>, &cbar);
+    const bool stage_now = kInvStage<NO> && fn > 0 && s_stage;
+    if (stage_now && tid == 0) bulk_g2s(ctile, Cinv<NO>(d, n, cc, 1), kInvStage<NO>, &cbar);
     // ---- far field F(t) = q(t) - sum_{l < a} C(t,l) x(l); 8 threads per row ----
     {
       const int row = tid >> 3, sl = tid & 7;
       const int t = a + row;
-      zd acc[NO], fbo[NO];   // fbo: this lane's BDF part (only the owner lane's is nonzero)
+      KAcc<R> ka[NO];   // FP32 history sums, compensated (FP64 in the FP64 form)
+      cx<R> old = cx<R>(0);
+      V q;
+      if (sl < NO && row < cn) {
+        old = ldr<R>(sp(t) + sl * NO + jc);
+        q = ldv<S>(qs + (long long)t * NO2 + sl * NO + jc);
+      }
+      if (row < cn && t > k) {
+        if (comp) {   // the leaf's rows before the chunk (at most 32 points, solved last)
+          const S* lf = static_cast<const S*>(d.hod[2].leaf) +
+                        ((long long)n * d.leaftot + (long long)jl * ((long long)L * (L + 1) / 2) + tri(t - A)) * NO2;
+          cx<R> pa[NO];
 #pragma unroll
-      for (int m = 0; m < NO; ++m) acc[m] = fbo[m] = zd();
-        KAcc<R> ka[NO];   // FP32 history sums, compensated (FP64 in the FP64 form)
-      if (row < cn) {
-        if (t <= k) {
-          if (sl == 0) {  // start rows: only l = 0 lies left of chunk 0 (a derivative term: kept in Fb)
-            zd fb[NO];
+          for (int m = 0; m < NO; ++m) pa[m] = cx<R>(0);
 #pragma unroll
-            for (int m = 0; m < NO; ++m) fb[m] = zd();
-            for (int y = 0; y < NO; ++y) {
-              const zd xv = ld(xp(0) + y * NO + jc);
+          for (int u0 = 0; u0 < 4; u0 += kLB<NO, S>) {
+            cx<R> sv[kLB<NO, S>][NO2];
 #pragma unroll
-              for (int m = 0; m < NO; ++m) {
-                zd cf = srx_any<NO, S>(d, n, t, 0, m, y) * (-h * W.I0[t][0]);
-                if (m == y) cf += zd(0, W.D[t][0] / h);
-                fb[m] -= cf * xv;
+            for (int u = 0; u < kLB<NO, S>; ++u) {
+              const int l = A + sl + 8 * (u0 + u);
+#pragma unroll
+              for (int e = 0; e < NO2; ++e) sv[u][e] = l < a ? ldr<R>(lf + (l - A) * NO2 + e) : cx<R>(0);
+            }
+#pragma unroll
+            for (int u = 0; u < kLB<NO, S>; ++u) {
+              const int l = A + sl + 8 * (u0 + u);
+              if (l < a) {
+                const R wl = rule_wr<R>(W, t, l);
+#pragma unroll
+                for (int y = 0; y < NO; ++y) {
+                  const cx<R> xy = vbulk(Xl[l & 63][y]) * wl;
+#pragma unroll
+                  for (int m = 0; m < NO; ++m) pa[m] = cfma(sv[u][m * NO + y], xy, pa[m]);
+                }
               }
             }
-#pragma unroll
-            for (int m = 0; m < NO; ++m) {
-              fbo[m] = fb[m];
-              Fb[row][m] = fb[m];
-            }
           }
+#pragma unroll
+          for (int m = 0; m < NO; ++m) ka[m].add(pa[m]);
         } else {
-          const int l0 = comp ? A : 0;
-          const S* srow = comp ? nullptr : el<NO, S>(d.SR, d, n, t, 0);
-          const R hr = (R)h;
-          for (int lb = l0 + sl; lb < a; lb += 8 * FOLD) {
+          const S* srow = el<NO, S>(d.SR, d, n, t, 0);
+          for (int lb = sl; lb < a; lb += 8 * FOLD) {
             cx<R> pa[NO];
 #pragma unroll
             for (int m = 0; m < NO; ++m) pa[m] = cx<R>(0);
@@ -773,8 +939,8 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
             for (int jj = 0; jj < FOLD; ++jj) {
               const int l = lb + 8 * jj;
               if (l < a) {
-                const R wl = hr * rule_wr<R>(W, t, l);
-                const S* sr = comp ? Lf<NO, S>(d, 2, n, jl, t, l) : srow + (long long)l * NO2;
+                const R wl = rule_wr<R>(W, t, l);
+                const S* sr = srow + (long long)l * NO2;
 #pragma unroll
                 for (int y = 0; y < NO; ++y) {
                   const cx<R> xy = ldr<R>(sp(l) + y * NO + jc) * wl;
@@ -786,46 +952,38 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
 #pragma unroll
             for (int m = 0; m < NO; ++m) ka[m].add(pa[m]);
           }
-          if (sl == 1) {  // BDF terms reaching left of the chunk, kept apart in Fb
-            zd fb[NO];
+        }
+      }
+      V r[NO];
 #pragma unroll
-            for (int m = 0; m < NO; ++m) fb[m] = zd();
-            for (int jj = 1; jj <= k; ++jj) {   // (-i a_j / h) x(t - j)
-              if (t - jj >= a) continue;
-              const double cj = W.ah[jj];
-#pragma unroll
-              for (int m = 0; m < NO; ++m) {
-                const zd x = ld(xp(t - jj) + m * NO + jc);
-                fb[m] = zd(fma(cj, x.im, fb[m].re), fma(-cj, x.re, fb[m].im));
-              }
-            }
-#pragma unroll
-            for (int m = 0; m < NO; ++m) {
-              fbo[m] = fb[m];
-              Fb[row][m] = fb[m];
-            }
+      for (int m = 0; m < NO; ++m) r[m] = reduce8(ka[m]);
+      if (sl < NO && row < cn) {   // lane sl of the group finishes component sl
+        V F = pick(r, sl), fb;
+        if (comp && t > k) F = vadd(F, FB[t - A][sl]);
+        F = vadd(vreal(F, h, W.hf), q);
+        vset(fb, zd());
+        if (t <= k) {   // start rows: only l = 0 lies left of chunk 0 (a derivative term: kept in Fb)
+          zd f0 = zd();
+          for (int y = 0; y < NO; ++y) {
+            zd cf = srx_any<NO, S>(d, n, t, 0, sl, y) * (-h * W.I0[t][0]);
+            if (sl == y) cf += zd(0, W.D[t][0] / h);
+            f0 -= cf * ld(d.x0 + (long long)n * NO2 + y * NO + jc);
           }
+          vset(fb, f0);
+        } else if (row < k) {   // BDF terms reaching left of the chunk: (-i a_j / h) x(t - j)
+          for (int jj = t - a + 1; jj <= k; ++jj) fb = vbdf(fb, Xl[(t - jj) & 63][sl], W, jj);
         }
-      }
-      // the BDF part from its owner lane (sl 0 for the start rows, else sl 1)
-      const int owner = (lane & ~7) | (t <= k ? 0 : 1);
-#pragma unroll
-      for (int m = 0; m < NO; ++m) {
-        const auto r = reduce8(ka[m]);
-        const zd fbm(__shfl_sync(FULL, fbo[m].re, owner), __shfl_sync(FULL, fbo[m].im, owner));
-        if (sl == 0 && row < cn) {
-          const zd far = val_of(r) + (comp && t > k ? FB[t - A][m] * h : zd()) +
-                         ld(qs + (long long)t * NO2 + m * NO + jc);
-          Fs[row][m] = far + fbm;
-          Ff[row][m] = zf((float)far.re, (float)far.im);
-          FbF[row][m] = cff_of(fbm);
+        if (t == T) FT[sl] = vadd(F, fb);
+        if constexpr (MX) {
+          Ff[row][sl] = vbulk(F);
+          Fb[row][sl] = fb;
+        } else {
+          Ff[row][sl] = F + fb;
         }
+        Old[row][sl] = old;
       }
-      (void)acc;
-      if (sl == 1 && row < cn)
-#pragma unroll
-        for (int m = 0; m < NO; ++m) Old[row][m] = ld(sp(t) + m * NO + jc);
     }
+    write64(wa, wn);
     __syncthreads();
     if (fn > 0) {
       const double2* Mi = Cinv<NO>(d, n, cc, 1);
@@ -842,48 +1000,43 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
       constexpr int LD = CK * NO;
       for (int o8 = tid; o8 < CK * NO * 8; o8 += blockDim.x) {
         const int o = o8 >> 3, sl = o8 & 7, ti = o / NO, m = o % NO;
-        zd sacc = zd();
-        if constexpr (Row64<NO, S>::separate) {
+        const int le = ti < fn ? max(ti + 1, min(k, fn)) : 0;   // lower triangular below the start block
+        V out;
+        if constexpr (MX) {
           // complex64 form: far field x hi in FP32, the k edge rows x (hi + lo) in
           // float-float, reduced over the 8 lanes in float-float
           const float2* Mh = reinterpret_cast<const float2*>(Mg);
           const float2* Ml = Mh + LD * LD;
-          cff sf = cff_of(zf(0));
-          if (ti < fn) {
-            zf s32 = zf(0);
-            for (int li = sl; li < max(ti + 1, min(k, fn)); li += 8)
+          zf s32 = zf(0);
+          for (int li = sl; li < le; li += 8)
 #pragma unroll
-              for (int y = 0; y < NO; ++y)
-                s32 = cfma(ldr<float>(Mh + (long long)(ti * NO + m) * LD + li * NO + y), Ff[li][y], s32);
-            sf = cff_of(s32);
-            for (int li = sl; li < k && li < fn; li += 8)
+            for (int y = 0; y < NO; ++y)
+              s32 = cfma(ldr<float>(Mh + (long long)(ti * NO + m) * LD + li * NO + y), Ff[li][y], s32);
+          out = cff_of(s32);
+          for (int li = sl; li < k && li < le; li += 8)
 #pragma unroll
-              for (int y = 0; y < NO; ++y) {
-                const long long e = (long long)(ti * NO + m) * LD + li * NO + y;
-                const float2 hv = Mh[e], lv = Ml[e];
-                sf = cff_add(sf, cff_mul(cff{{hv.x, lv.x}, {hv.y, lv.y}}, FbF[li][y]));
-              }
-          }
-#pragma unroll
-          for (int off = 1; off < 8; off <<= 1) sf = cff_add(sf, cff_shfl_xor(sf, off));
-          if (sl == 0) sacc = cff_val(sf);
+            for (int y = 0; y < NO; ++y) {
+              const long long e = (long long)(ti * NO + m) * LD + li * NO + y;
+              const float2 hv = Mh[e], lv = Ml[e];
+              out = cff_add(out, cff_mul(cff{{hv.x, lv.x}, {hv.y, lv.y}}, Fb[li][y]));
+            }
         } else {
-          if (ti < fn)
-            for (int li = sl; li < max(ti + 1, min(k, fn)); li += 8)
+          out = zd();
+          for (int li = sl; li < le; li += 8)
 #pragma unroll
-              for (int y = 0; y < NO; ++y)
-                sacc = cfma(ld(Mg + (long long)(ti * NO + m) * LD + li * NO + y), Fs[li][y], sacc);
-#pragma unroll
-          for (int off = 1; off < 8; off <<= 1)
-            sacc += zd(__shfl_xor_sync(FULL, sacc.re, off), __shfl_xor_sync(FULL, sacc.im, off));
+            for (int y = 0; y < NO; ++y) out = cfma(ld(Mg + (long long)(ti * NO + m) * LD + li * NO + y), Ff[li][y], out);
         }
+#pragma unroll
+        for (int off = 1; off < 8; off <<= 1) out = vadd(out, vshfl_xor(out, off));
         if (sl == 0 && ti < fn) {
-          myerr = fmax(myerr, (sacc - Old[ti][m]).abs2());
-          st(xp(a + ti) + m * NO + jc, sacc);
-          if constexpr (Row64<NO, S>::separate) st(sp(a + ti) + m * NO + jc, sacc);
+          myerr = fmax(myerr, vdist(out, Old[ti][m]));
+          Xl[(a + ti) & 63][m] = out;
+          vstore(sp(a + ti) + m * NO + jc, out);
         }
       }
     }
+    wa = a;
+    wn = fn;
     if (fn < cn) {
       // row T (horizontal density matrix): x(T) from the rows of its chunk and
       // the current Sigma^R(T, .), one lane of warp 0 per row
@@ -898,7 +1051,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
           const S* sr = el<NO, S>(d.SR, d, n, T, l);
 #pragma unroll
           for (int y = 0; y < NO; ++y) {
-            const zd x = ld(xp(l) + y * NO + jc), xw = x * wl;
+            const zd x = v64(Xl[l & 63][y]), xw = x * wl;
 #pragma unroll
             for (int m = 0; m < NO; ++m) f[m] = cfma(ld(sr + m * NO + y), xw, f[m]);
             if (dd <= k) f[y] += zd(W.ah[dd] * x.im, -W.ah[dd] * x.re);   // (-i a_d / h) x(l)
@@ -913,7 +1066,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
           zd x[NO];
 #pragma unroll
           for (int x2 = 0; x2 < NO; ++x2) {
-            f[x2] += Fs[fn][x2];
+            f[x2] += v64(FT[x2]);
 #pragma unroll
             for (int y = 0; y < NO; ++y)
               Mm.a[x2][y] = (x2 == y ? zd(0, W.a[0] / h) : zd()) - ld(ep + x2 * NO + y) - ld(sd + x2 * NO + y) * wt;
@@ -921,22 +1074,25 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
           solve_col<NO>(Mm, f, x);
 #pragma unroll
           for (int m = 0; m < NO; ++m) {
-            myerr = fmax(myerr, (x[m] - Old[fn][m]).abs2());
+            V v;
+            vset(v, x[m]);
+            myerr = fmax(myerr, vdist(v, Old[fn][m]));
             st(xp(T) + m * NO + jc, x[m]);
-            if constexpr (Row64<NO, S>::separate) st(sp(T) + m * NO + jc, x[m]);
+            if constexpr (MX) vstore(sp(T) + m * NO + jc, v);
           }
         }
       }
     }
     __syncthreads();
   }
-  myerr = sqrt(warp_max(myerr));
-  if (lane == 0 && myerr > 0) atomic_max_nonneg(&serr, myerr);
+  write64(wa, wn);
+  const double e1 = sqrt(warp_max((double)myerr));
+  if (lane == 0 && e1 > 0) atomic_max_nonneg(&serr, e1);
   __syncthreads();
   if (tid == 0) atomic_max_nonneg(d.err + n, serr);
   // after a timed-out wait, a copy may still be in flight into this CTA's
   // shared memory: wait for it (bounded) before the CTA exits
-  if (kInvStage<NO, S> && tid == 0 && !s_stage) mbar_wait(&cbar, cphase ^ 1u, kCopyWaitPolls);
+  if (kInvStage<NO> && tid == 0 && !s_stage) mbar_wait(&cbar, cphase ^ 1u, kCopyWaitPolls);
 }
 
 // ---------------------------------------------------------------------------
@@ -1155,15 +1311,16 @@ static cudaError_t allow_smem(K kern, size_t bytes) {
   if (a.sharedSizeBytes + bytes > 227 * 1024) return cudaErrorInvalidValue;
   return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
-// Dynamic shared memory of a sweep: the staged chunk inverse (N_o <= 2)
-// and, in the compressed form, the staged block projections, which share one
-// buffer; staging is used when it fits in 64 KiB.
+// Dynamic shared memory of a sweep: the buffer of the staged inverse and, in
+// the compressed form, the projections of the blocks over a leaf, unless ranks
+// and levels make them larger than 200 KB in all (then they stay in global
+// memory).
 template <int NO, typename S>
 static size_t sweep_smem(const Dev& d, int* staged) {
-  using R = typename Bulk<S>::R;
-  const size_t ps = d.ring ? (size_t)d.maxl * NO * NO * d.rmax * sizeof(cx<R>) : 0;
-  *staged = (d.ring && ps <= 65536) ? 1 : 0;
-  return std::max(kStageBytes<NO>, *staged ? ps : (size_t)0);
+  const size_t b = kBufBytes<NO> + (d.ring ? SweepMem<NO, typename Bulk<S>::R>::bytes(d.maxl, d.rmax) : 0);
+  const bool off32 = std::max(d.utot, d.vtot) * d.rmax < (1ll << 32);
+  *staged = (d.ring && b <= 200 * 1024 && off32) ? 1 : 0;
+  return *staged ? b : kBufBytes<NO>;
 }
 template <int NO, typename S>
 static cudaError_t sweep_ret(const Dev& d, int T, cudaStream_t s) {
@@ -1171,6 +1328,7 @@ static cudaError_t sweep_ret(const Dev& d, int T, cudaStream_t s) {
   const size_t bytes = sweep_smem<NO, S>(d, &staged);
   cudaError_t e = allow_smem(k_ret2<NO, S>, bytes);
   if (e != cudaSuccess) return e;
+  if (d.ring && T + 1 - d.cdir > kRingRows && d.cdir > 0) return cudaErrorInvalidValue;
   k_ret2<NO, S><<<dim3(d.no, d.n_inst), 256, bytes, s>>>(d, T, staged);
   return cudaGetLastError();
 }

@@ -12,6 +12,7 @@ struct DevW {
   double a[6], omega[6], D[6][6], I0[6][6];
   float omegaf[6], I0f[6][6];   // float copies for the bulk sums of the complex64 form
   double ah[6];                  // a_j / h (the BDF coefficients of the time derivative)
+  float2 hf, ahf[6], wm1f[6];    // h, a_j / h and omega_i - 1 as float-float pairs (complex64 form)
 };
 
 constexpr int MP = 64;  // doubles of model parameters per instance
@@ -70,7 +71,7 @@ struct Dev {
   double2 *wconv;              // [n][r(a)][r(i)][no2]
   double *tau, *e0, *ebeta, *rev, *q;  // [r], [r], [r], [r*r], [r*r]
   double *mpar;                // [n][MP]
-  double2 *qsrc;               // [n][nt][no2]   lesser source q(t)
+  double2 *qsrc;               // [n][nt][no2]   lesser source q(t) (complex64 form: float-float pairs)
   double2 *vvec;               // [n][r][no2]    v_a = sum_b Q_ab G^vt(tau_b, T)
   double2 *x0;                 // [n][no2]       -[G^tv(T,0)]^dagger
   double2 *scratch;            // [n][scratch_per_inst]  start-block right-hand sides
