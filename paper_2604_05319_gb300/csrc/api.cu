@@ -51,6 +51,8 @@ struct hkbe_s {
   double2 *rowbuf_r = nullptr, *rowbuf_l = nullptr;
   int* status_dev = nullptr;
   double2* diagbuf = nullptr;  // [n_inst][no2] density matrices of one time
+  std::vector<int> src_r0;   // first block row of each source-projection job (ascending)
+  std::vector<void*> work;   // device buffers that are in neither snapshots nor files
   // points whose rows the chunk inverses hold (retarded [0, rowsR), lesser [1, rowsL))
   int rowsR = 0, rowsL = 1;
   // the rows of a growing chunk's inverse are rebuilt from the first step after a
@@ -156,6 +158,51 @@ int dalloc_el(hkbe_t* h, void** p, size_t count) {
   int rc = h->d.prec ? dalloc(h, reinterpret_cast<float2**>(p), count) : dalloc(h, reinterpret_cast<double2**>(p), count);
   if (rc == HKBE_OK) h->state_arrays.push_back({*p, std::max<size_t>(count, 1) * (h->d.prec ? sizeof(float2) : sizeof(double2))});
   return rc;
+}
+
+// working buffer of a handle, zeroed; in neither its snapshots nor its files
+template <typename T>
+int walloc(hkbe_t* h, T** p, size_t count) {
+  count = std::max<size_t>(count, 1);
+  cudaError_t e = cudaMalloc((void**)p, count * sizeof(T));
+  if (e != cudaSuccess) return fail(h, HKBE_ERR_NOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  h->work.push_back(*p);
+  h->bytes += count * sizeof(T);
+  e = cudaMemsetAsync(*p, 0, count * sizeof(T), h->s);
+  return e == cudaSuccess ? HKBE_OK : fail(h, HKBE_ERR_CUDA, cudaGetErrorString(e));
+}
+
+// Jobs of the source projections (block, side, chunk of kSrcChunk rows, first
+// partial-sum slot of a side longer than one chunk), sorted by the block's
+// first row so that the jobs of the built blocks come first.
+int src_jobs(hkbe_t* h) {
+  hk::Dev& d = h->d;
+  std::vector<int> order(d.nblk);
+  for (int b = 0; b < d.nblk; ++b) order[b] = b;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return h->g_r0[a] < h->g_r0[b]; });
+  std::vector<int4> tab;
+  h->src_r0.clear();
+  int parts = 0;
+  for (int b : order)
+    for (int side = 0; side < 2; ++side) {
+      const int len = side == 0 ? h->g_r1[b] - h->g_r0[b] : h->g_c1[b] - h->g_c0[b];
+      const int nch = (len + hk::kSrcChunk - 1) / hk::kSrcChunk;
+      for (int c = 0; c < nch; ++c) {
+        tab.push_back(make_int4(b, side, c, parts));
+        h->src_r0.push_back(h->g_r0[b]);
+      }
+      if (nch > 1) parts += nch;
+    }
+  d.s_parts = parts;
+  int rc;
+  int4* t = nullptr;
+  if ((rc = walloc(h, &t, tab.size())) || (rc = walloc(h, &d.s_cnt, (size_t)d.n_inst * d.nblk * 2)) ||
+      (rc = walloc(h, &d.spart, (size_t)d.n_inst * parts * d.no * d.no * d.no * d.rmax)))
+    return rc;
+  d.s_tab = t;
+  cudaError_t e = cudaMemcpyAsync(t, tab.data(), tab.size() * sizeof(int4), cudaMemcpyHostToDevice, h->s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->s);
+  return e == cudaSuccess ? HKBE_OK : fail(h, HKBE_ERR_CUDA, cudaGetErrorString(e));
 }
 
 // mixed components: complex128 in both precision forms
@@ -449,14 +496,12 @@ int hkbe_create(const hkbe_params* p, const int32_t* nt_per_inst, void* stream, 
   }
   h->scratch.insert(h->scratch.end(), {d.cinv_ws, h->diagbuf});
   {  // inverses of the retarded heads: rebuilt at every step, in neither snapshots nor files
-    const size_t b = (size_t)d.n_inst * 4 * d.k * d.k * d.no * d.no * sizeof(double2);
-    const cudaError_t e = cudaMalloc((void**)&d.hinv, b);
-    if (e != cudaSuccess) {
-      g_create_error = std::string("cudaMalloc: ") + cudaGetErrorString(e);
+    const size_t n2 = (size_t)d.no * d.no;
+    if ((rc = walloc(h, &d.hinv, (size_t)d.n_inst * 4 * d.k * d.k * n2)) || (h->hodlr && (rc = src_jobs(h)))) {
+      g_create_error = h->err;
       hkbe_destroy(h);
-      return HKBE_ERR_NOMEM;
+      return rc;
     }
-    h->bytes += b;
   }
   cudaError_t e = cudaStreamSynchronize(h->s);
   if (e != cudaSuccess) {
@@ -474,7 +519,7 @@ int hkbe_destroy(hkbe_t* h) {
   drain(h);
   for (cudaEvent_t e : h->event_pool) cudaEventDestroy(e);
   for (void* p : h->allocs) cudaFree(p);
-  if (h->d.hinv) cudaFree(h->d.hinv);
+  for (void* p : h->work) cudaFree(p);
   for (void* p : h->snap_dev)
     if (p) cudaFree(p);
   delete h;
@@ -1009,6 +1054,7 @@ int hkbe_step(hkbe_t* h, int n_steps, int32_t* iters, double* err) {
       d.nfrozL = rL / 32;
     }
     HK_CUDA(h, run_phase(h, HKBE_PHASE_EXTRAP, 1, [&]() { return hk::launch_extrapolate(d, T, h->s); }));
+    const int njob = (int)(std::lower_bound(h->src_r0.begin(), h->src_r0.end(), d.cdir) - h->src_r0.begin());
     std::vector<int> act0(N);
     for (int n = 0; n < N; ++n) act0[n] = T <= h->last[n] ? 1 : 0;
     bool failed = false;
@@ -1024,8 +1070,8 @@ int hkbe_step(hkbe_t* h, int n_steps, int32_t* iters, double* err) {
                    if ((e = run_phase(h, HKBE_PHASE_MIXED, 1, [&]() { return hk::launch_mixed(d, T, h->s); })))
                      return e;
                    if ((e = run_phase(h, HKBE_PHASE_VT, 1, [&]() { return hk::launch_vt(d, T, h->s); }))) return e;
-                   if ((e = run_phase(h, HKBE_PHASE_SRC, (h->hodlr && d.cdir > 0) ? 3 : 1, [&]() {
-                          return h->hodlr ? hk::launch_src_h(d, T, h->s) : hk::launch_src(d, T, h->s);
+                   if ((e = run_phase(h, HKBE_PHASE_SRC, (h->hodlr && d.cdir > 0) ? 2 : 1, [&]() {
+                          return h->hodlr ? hk::launch_src_h(d, T, njob, h->s) : hk::launch_src(d, T, h->s);
                         })))
                      return e;
                    if ((e = run_phase(h, HKBE_PHASE_LES, 1, [&]() {

@@ -120,6 +120,19 @@ __device__ __forceinline__ float f32_of(double x) {
   const unsigned mag = ((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
   return __uint_as_float(sign | (mag + ((lo >> 28) & 1u)));
 }
+// The same as an unevaluated pair: hi the top 24 bits of x (truncated), lo the
+// 29 bits after them (rounded to 24): x to about 2^-47 of it, without an FP64
+// instruction.  Magnitudes below 2^-74 keep hi only, below the FP32 range 0.
+__device__ __forceinline__ ffl ff_of_bits(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu) - 1023 + 127;
+  const unsigned sign = hi & 0x80000000u;
+  if (e <= 0) return {__uint_as_float(sign), 0.f};
+  if (e >= 255) return {__uint_as_float(sign | 0x7f800000u), 0.f};
+  const float h = __uint_as_float(sign | ((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+  const float l = e > 52 ? (float)(lo & 0x1fffffffu) * __uint_as_float(sign | ((unsigned)(e - 52) << 23)) : 0.f;
+  return {h, l};
+}
 __device__ __forceinline__ zf ld_f32(const double2* p) {
   const double2 v = *p;
   return zf(f32_of(v.x), f32_of(v.y));

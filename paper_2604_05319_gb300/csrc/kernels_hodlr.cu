@@ -26,6 +26,8 @@
 namespace hk {
 
 
+constexpr int kSrcRing = 80;   // >= leaf + k + 1 uncompressed rows
+
 // ---------------------------------------------------------------------------
 // Lesser source with compressed Sigma^< (two-sided HODLR matvec).
 // Stored S[r][c] = Sigma^<(c, r), c <= r.  q(t) = h sum_l w_l Sigma^<(t,l) g_l,
@@ -33,386 +35,416 @@ namespace hk {
 // -S[t][l]^dagger (row t).
 // Projections per (block, pair (x,z), y):
 //   P1 = S o sum_{rows l} w_l g_l[z][y] U(l,:),  q(t in cols) += P1 . conj(V(t,:))
-//   P2 = S o sum_{cols l} w_l g_l[z][y] V(l,:),  q(t in rows) -= conj(U(t,:)) . P2
+//   P2 = - S o sum_{cols l} w_l g_l[z][y] V(l,:),  q(t in rows) += conj(U(t,:)) . P2
 // ---------------------------------------------------------------------------
-// Slot of P1 (which = 0) or P2 (which = 1), rmax complex values in the bulk
-// arithmetic R of the form (FP32 in the complex64 form: the products with the
-// factor rows need no conversion), inside a complex128-sized slot.
+// P1 (which = 0) or P2 (which = 1) of (block, pair), entry q, all y < N_o, in
+// the bulk arithmetic R of the form, inside complex128-sized slots.
 template <int NO, typename R>
-__device__ __forceinline__ cx<R>* Psrc(const Dev& d, int n, int b, int p, int y, int which) {
+__device__ __forceinline__ cx<R>* Psrc(const Dev& d, int n, int b, int p, int which) {
   return reinterpret_cast<cx<R>*>(d.proj + (long long)d.n_inst * NO * d.maxl * NO * NO * d.rmax +
-                                  (((((long long)n * d.nblk + b) * (NO * NO) + p) * NO + y) * 2 + which) * d.rmax);
+                                  ((((long long)n * d.nblk + b) * (NO * NO) + p) * 2 + which) * d.rmax * NO);
 }
 
-// sum_{q < rk} P[q] conj(F[q]) for one thread: P (bulk type, shared by the
-// CTA, cached) and F (a factor row in global memory) with eight loads of F in
-// flight rather than one load per term.
-template <typename R, typename S>
-__device__ __forceinline__ cx<R> lr_dot_conj(const cx<R>* P, const S* F, int rk) {
-  cx<R> acc = cx<R>(0);
-  for (int q0 = 0; q0 < rk; q0 += 8) {
-    cx<R> f[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) f[u] = q0 + u < rk ? ldr<R>(F + q0 + u) : cx<R>(0);
-#pragma unroll
-    for (int u = 0; u < 8; ++u) acc = cfma(P[q0 + u < rk ? q0 + u : 0], f[u].conj(), acc);
-  }
-  return acc;
-}
-
+// The projections: one CTA per instance, block side and 256 of its rows (or
+// columns), so that a block of a thousand rows is not one warp's loop over
+// all of them.  A warp takes one pair (N_o = 1, 2: 8 or 2 warps share a pair's
+// rows), all y, lanes packed by the pair's rank (8, 16 or 32 per factor row,
+// 64 entries of the rank per pass).  Sides longer than 256 leave one partial
+// sum per CTA in spart; the CTA that finds itself the last of its side (a
+// counter that it sets back) adds them in their order, so the sum does not
+// depend on which one that is.
+// s_tab: (block, side, first row / 256, first slot of the side's partial sums).
 template <int NO, typename S>
 __global__ void __launch_bounds__(256) k_src_proj(Dev d, int T) {
   constexpr int NO2 = NO * NO;
   using R = typename Bulk<S>::R;
-  const int b = blockIdx.x, n = blockIdx.y;
-  if (!d.active[n]) return;
+  using V = typename Val<S>::t;
+  const int4 job = d.s_tab[blockIdx.x];
+  const int b = job.x, which = job.y, ch = job.z, n = blockIdx.y;
   const int c = d.cdir;
-  if (d.b_r0[b] >= c) return;
-  const int r0 = d.b_r0[b], rl = min(d.b_r1[b], c), c0 = d.b_c0[b], c1 = d.b_c1[b];
+  if (!d.active[n] || d.b_r0[b] >= c) return;
+  const int lo = which == 0 ? d.b_r0[b] : d.b_c0[b], hi = which == 0 ? min(d.b_r1[b], c) : d.b_c1[b];
+  const int l0 = lo + ch * kSrcChunk, l1 = min(l0 + kSrcChunk, hi), nch = (hi - lo + kSrcChunk - 1) / kSrcChunk;
+  if (l0 >= hi) return;
   const DevW& W = d.w;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // YB values of y per pass over a factor row (N_o <= 2: all of them), so each
-  // factor row is read once per pair and side.
-  constexpr int YB = NO <= 2 ? NO : 1;
-  // A job is one (side, pair, y-block); it runs on a group of wpj warps (one
-  // warp per job when there are at least 8 jobs), the group splitting the
-  // job's rows.  Within a warp, lpr = 8, 16 or 32 lanes cover the rank of a
-  // factor row (with up to 4 entries per lane: ranks up to 128), so a small
-  // rank keeps every lane loading (32 / lpr rows per step).  P1 serves pair p = (x, z) (uses g[z]); P2 serves pair p = (z, x)
-  // (uses g[z]); g_l[z][y] = conj(G^R(T,l)[y][z]).
-  constexpr int NJOB = NO2 * 2 * (NO / YB);
-  constexpr int WPJ = NJOB >= 8 ? 1 : 8 / NJOB;
-  constexpr int NGRP = 8 / WPJ;
-  __shared__ zd pbuf[WPJ > 1 ? 8 : 1][YB * 128];  // a group's per-warp partial sums
+  constexpr int WPJ = NO == 1 ? 8 : NO == 2 ? 2 : 1, NGRP = 8 / WPJ;   // warps per pair
+  __shared__ V red[WPJ > 1 ? 8 : 1][NO * 64];
+  __shared__ int s_last;
   const int grp = warp / WPJ, wig = warp % WPJ;
-  for (int job0 = 0; job0 < NJOB; job0 += NGRP) {
-    const int job = job0 + grp;
-    const bool act = job < NJOB;
-    const int which = job & 1, rest = job >> 1;
-    const int yb = (rest % (NO / YB)) * YB, p = act ? rest / (NO / YB) : 0;
+  V* part = reinterpret_cast<V*>(d.spart) + ((long long)n * d.s_parts + job.w) * (NO2 * NO) * d.rmax;   // [chunk][p][q][y]
+  auto finish = [&](int p, int q, int y, const V& v) {   // the whole side's sum
+    const double s = Sp<NO>(d, 3, n, b, p)[q];
+    const zd r = v64(v) * (which == 0 ? s : -s);
+    Psrc<NO, R>(d, n, b, p, which)[q * NO + y] = cx<R>((R)r.re, (R)r.im);
+  };
+  for (int p0 = 0; p0 < NO2; p0 += NGRP) {
+    const int p = p0 + grp;
+    const bool act = p < NO2;
     const int z = which == 0 ? p % NO : p / NO;
     const int rk = act ? *Rk<NO>(d, 3, n, b, p) : 0;
-    const S* F = which == 0 ? Up<NO, S>(d, 3, n, b, p) : Vp<NO, S>(d, 3, n, b, p);
-    const int lo = which == 0 ? r0 : c0, hi = act ? (which == 0 ? rl : c1) : lo;
-    const int lpr = rk <= 8 ? 8 : rk <= 16 ? 16 : 32;
-    const int rps = 32 / lpr, sub = lane / lpr, q0 = lane % lpr;
-    const int stride = WPJ * rps;
-    KAcc<R> part[YB][4];   // compensated FP32 sums in the complex64 form
-    for (int l0 = lo + wig * rps + sub; l0 < hi; l0 += stride * FOLD) {
-      cx<R> pp[YB][4];
+    const S* F = which == 0 ? Up<NO, S>(d, 3, n, b, act ? p : 0) : Vp<NO, S>(d, 3, n, b, act ? p : 0);
+    int rkall = rk;   // of the pairs taken together (the groups meet at barriers)
+    if (WPJ > 1) {
+      for (int g = 0; g < NGRP; ++g) rkall = max(rkall, *Rk<NO>(d, 3, n, b, p0 + g));
+    }
+    for (int qb = 0; qb < rkall; qb += 64) {
+      const int rem = max(0, min(rk - qb, 64)), lpr = rem <= 8 ? 8 : rem <= 16 ? 16 : 32;
+      const int rps = 32 / lpr, sub = lane / lpr, q0 = qb + lane % lpr;
+      const int stride = WPJ * rps;
+      KAcc<R> acc[NO][2];
+      if (rem > 0)
+        for (int lb = l0 + wig * rps + sub; lb < l1; lb += stride * FOLD) {
+          cx<R> pp[NO][2];
 #pragma unroll
-      for (int yy = 0; yy < YB; ++yy)
+          for (int y = 0; y < NO; ++y) pp[y][0] = pp[y][1] = cx<R>(0);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) pp[yy][u] = cx<R>(0);
+          for (int jj = 0; jj < FOLD; ++jj) {
+            const int l = lb + stride * jj;
+            if (l < l1) {
+              const R wl = rule_wr<R>(W, T, l);
+              const S* gp = el<NO, S>(d.GR, d, n, T, l);
+              cx<R> g[NO];   // w_l g_l[z][y] = w_l conj(G^R(T,l)[y][z])
 #pragma unroll
-      for (int jj = 0; jj < FOLD; ++jj) {
-        const int l = l0 + stride * jj;
-        if (l < hi) {
-          const R wl = rule_wr<R>(W, T, l);
-          const S* gp = el<NO, S>(d.GR, d, n, T, l);
-          cx<R> g[YB];
+              for (int y = 0; y < NO; ++y) g[y] = ldr<R>(gp + y * NO + z).conj() * wl;
+              const S* fr = F + (long long)(l - lo) * d.rmax;
 #pragma unroll
-          for (int yy = 0; yy < YB; ++yy) g[yy] = ldr<R>(gp + (yb + yy) * NO + z).conj() * wl;
-          const S* fr = F + (long long)(l - lo) * d.rmax;
+              for (int u = 0; u < 2; ++u) {
+                const int q = q0 + lpr * u;
+                if (q < rk) {
+                  const cx<R> f = ldr<R>(fr + q);
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int q = q0 + lpr * u;
-            if (q < rk) {
-              const cx<R> f = ldr<R>(fr + q);
+                  for (int y = 0; y < NO; ++y) pp[y][u] = cfma(g[y], f, pp[y][u]);
+                }
+              }
+            }
+          }
 #pragma unroll
-              for (int yy = 0; yy < YB; ++yy) pp[yy][u] = cfma(g[yy], f, pp[yy][u]);
+          for (int y = 0; y < NO; ++y) {
+            acc[y][0].add(pp[y][0]);
+            acc[y][1].add(pp[y][1]);
+          }
+        }
+#pragma unroll
+      for (int y = 0; y < NO; ++y)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int q = q0 + lpr * u;
+          if (lpr * u < rem) {   // (warp-uniform)
+            const V r = kacc_lanes(acc[y][u], lpr, 32);
+            if (sub == 0 && q < rk && q < qb + 64) {
+              if (WPJ > 1) red[warp][y * 64 + q - qb] = r;
+              else if (nch == 1) finish(p, q, y, r);
+              else part[((long long)(ch * NO2 + p) * d.rmax + q) * NO + y] = r;
             }
           }
         }
-      }
+      if (WPJ > 1) {
+        __syncthreads();
+        if (act)
+          for (int e = wig * 32 + lane; e < NO * rem; e += WPJ * 32) {
+            const int y = e / rem, qq = e % rem;
+            V r = red[grp * WPJ][y * 64 + qq];
 #pragma unroll
-      for (int yy = 0; yy < YB; ++yy)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) part[yy][u].add(pp[yy][u]);
-    }
-    // the warp's rows combined (every lane calls the shuffles)
-#pragma unroll
-    for (int yy = 0; yy < YB; ++yy)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const auto r = kacc_lanes(part[yy][u], lpr, 32);
-        const int q = q0 + lpr * u;   // < 128
-        if (sub == 0 && q < rk) {
-          if (WPJ == 1) {
-            const zd v = val_of(r) * Sp<NO>(d, 3, n, b, p)[q];
-            Psrc<NO, R>(d, n, b, p, yb + yy, which)[q] = cx<R>((R)v.re, (R)v.im);
-          } else {
-            pbuf[warp][yy * 128 + q] = val_of(r);
+            for (int w2 = 1; w2 < WPJ; ++w2) r = vadd(r, red[grp * WPJ + w2][y * 64 + qq]);
+            if (nch == 1) finish(p, qb + qq, y, r);
+            else part[((long long)(ch * NO2 + p) * d.rmax + qb + qq) * NO + y] = r;
           }
-        }
+        __syncthreads();
       }
-    if (WPJ > 1) {   // the group's warps combined: at most one job per group here (NJOB <= 8)
-      __syncthreads();
-      if (act && wig == 0)
-        for (int e = lane; e < YB * rk; e += 32) {
-          const int yy = e / rk, q = e % rk;
-          zd acc = zd();
-          for (int w2 = 0; w2 < WPJ; ++w2) acc += pbuf[grp * WPJ + w2][yy * 128 + q];
-          const zd v = acc * Sp<NO>(d, 3, n, b, p)[q];
-          Psrc<NO, R>(d, n, b, p, yb + yy, which)[q] = cx<R>((R)v.re, (R)v.im);
-        }
-      __syncthreads();
+    }
+  }
+  if (nch == 1) return;
+  __threadfence();
+  __syncthreads();
+  int* cnt = d.s_cnt + ((long long)n * d.nblk + b) * 2 + which;
+  if (tid == 0) {
+    s_last = atomicAdd(cnt, 1) == nch - 1;
+    if (s_last) *cnt = 0;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  for (int p = 0; p < NO2; ++p) {
+    const int rk = *Rk<NO>(d, 3, n, b, p);
+    for (int e = tid; e < rk * NO; e += blockDim.x) {
+      V r;
+      vset(r, zd());
+      for (int i = 0; i < nch; ++i) r = vadd(r, part[(long long)(i * NO2 + p) * d.rmax * NO + e]);
+      finish(p, e / NO, e % NO, r);
     }
   }
 }
 
-// q(t) for the compressed columns t < c, one thread per t (adjacent threads
-// read adjacent elements of every row).  The weighted G^A(l, T) of the
-// uncompressed rows l in [c, T] (at most a leaf plus k+1 rows) is staged in
-// shared memory once per block.
-constexpr int kSrcRing = 80;   // >= leaf + k + 1 uncompressed rows
+// Sum of products of FP64 data.  Complex64 form: both factors as float-float
+// pairs, every product's rounding error kept by a fused multiply-add and every
+// sum's by TwoSum, both collected in a second float (the compensated dot
+// product of Ogita, Rump and Oishi): about 48 bits on the FP32 pipes, 12
+// instructions per real product where an FP64 one holds the pipe for 64 cycles.
+struct Dot2 {
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(const ffl& a, const ffl& b) {
+    const float p = a.hi * b.hi;
+    const float e = fmaf(a.hi, b.hi, -p);
+    const ffl t = ff_two_sum(s, p);
+    s = t.hi;
+    c = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, c + (t.lo + e)));
+  }
+};
+template <typename S> struct DotC;
+template <> struct DotC<double2> {
+  zd a{};
+  __device__ __forceinline__ DotC() : a(0.0) {}
+  __device__ __forceinline__ void add(const zd& x, const zd& y) { a = cfma(x, y, a); }
+  __device__ __forceinline__ zd get() const { return a; }
+};
+template <> struct DotC<float2> {
+  Dot2 re, im;
+  __device__ __forceinline__ void add(const cff& x, const cff& y) {
+    re.add(x.re, y.re);
+    re.add(ff_neg(x.im), y.im);
+    im.add(x.re, y.im);
+    im.add(x.im, y.re);
+  }
+  __device__ __forceinline__ cff get() const { return {ff_two_sum(re.s, re.c), ff_two_sum(im.s, im.c)}; }
+};
+template <typename S>
+__device__ __forceinline__ auto ld_split(const double2* p) {   // complex128 data as a Val<S>
+  if constexpr (sizeof(S) == sizeof(double2)) {
+    return ld(p);
+  } else {
+    const double2 v = *p;
+    return cff{ff_of_bits(v.x), ff_of_bits(v.y)};
+  }
+}
+__device__ __forceinline__ zd vmul_mi(const zd& a) { return zd(a.im, -a.re); }   // -i a
+__device__ __forceinline__ cff vmul_mi(const cff& a) { return {a.im, ff_neg(a.re)}; }
+
+// q(t).  CTAs x < c / 32: 32 compressed columns t < c; lanes along t (adjacent
+// elements of every uncompressed row), the terms of the sum split over the 8
+// warps: uncompressed rows l in [c, T] (at most a leaf plus k + 1, staged
+// weighted G^A), the leaf, the packed entries of all blocks over the leaf
+// (both sides) with kEB loads in flight, and the mixed part - i sum_a
+// Sigma^tv(t, tau_a) v_a.  The other CTAs: 8 uncompressed rows t >= c, one warp
+// each, lanes along the row.  One thread per t over all terms (the earlier form)
+// was a chain of some thousand loads and FP64 products, on T / 128 CTAs; projections
+// and source together took 554 us at N_o = 2, complex64, 128 instances, T = 600
+// (now 360), 400 us in FP64 at 16 instances, T = 300 (123), 970 us at N_o = 4,
+// complex64, 16 instances, T = 290 (152).
+constexpr int kEB = 4;
 template <int NO, typename S>
-__global__ void __launch_bounds__(128) k_src_c(Dev d, int T) {
+__global__ void __launch_bounds__(256) k_src_q(Dev d, int T, int uselist) {
   constexpr int NO2 = NO * NO;
   using R = typename Bulk<S>::R;
+  using V = typename Val<S>::t;
   const int n = blockIdx.y;
   if (!d.active[n]) return;
-  const int c = d.cdir, L = d.L;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int c = d.cdir, L = d.L, ntile = c / 32;
   const DevW& W = d.w;
-  __shared__ cx<R> gs[kSrcRing][NO2];  // gs[l - c][z][y] = w_l conj(G^R(T, l)[y][z])
-  const int nr = T + 1 - c;
-  for (int e = threadIdx.x; e < nr * NO2; e += blockDim.x) {
-    const int li = e / NO2, q = e % NO2, z = q / NO, y = q % NO, l = c + li;
-    gs[li][q] = ldr<R>(el<NO, S>(d.GR, d, n, T, l) + y * NO + z).conj() * rule_wr<R>(W, T, l);
-  }
-  __syncthreads();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= c) return;
-  const int jt = t / L, A = jt * L, E = min(A + L, c);
-  zd acc[NO2];
-#pragma unroll
-  for (int q = 0; q < NO2; ++q) acc[q] = zd();
+  extern __shared__ __align__(16) char dyn[];
+  V* vs = reinterpret_cast<V*>(dyn);              // [r][NO2] v_a
+  V* red = vs + d.r * NO2;                        // [8][NO2][32] partial sums of the warps
+  for (int e = tid; e < d.r * NO2; e += blockDim.x) vset(vs[e], ld(d.vvec + (long long)n * d.r * NO2 + e));
   KAcc<R> ka[NO2];   // the history sums: compensated FP32 in the complex64 form
+  DotC<S> mx[NO2];   // the mixed part
   cx<R> pa[NO2];
-  auto zero = [&]() {
-#pragma unroll
-    for (int q = 0; q < NO2; ++q) pa[q] = cx<R>(0);
-  };
   auto fold = [&]() {
 #pragma unroll
-    for (int q = 0; q < NO2; ++q) ka[q].add(pa[q]);
-    zero();
+    for (int q = 0; q < NO2; ++q) {
+      ka[q].add(pa[q]);
+      pa[q] = cx<R>(0);
+    }
   };
-  // pa[x][y] += sum_z Sx[x][z] g[z][y], Sx = S or S^dagger
-  auto mac_g = [&](const S* sp, bool dagS, const cx<R>* g) {
+#pragma unroll
+  for (int q = 0; q < NO2; ++q) pa[q] = cx<R>(0);
+  auto gw = [&](int l, int z, int y) {   // w_l g_l[z][y]
+    return ldr<R>(el<NO, S>(d.GR, d, n, T, l) + y * NO + z).conj() * rule_wr<R>(W, T, l);
+  };
+  // pa[x][y] += sum_z Sx[x][z] g[z][y], Sx = S or -S^dagger
+  auto mac = [&](const cx<R>* s, bool low, const cx<R>* g) {
 #pragma unroll
     for (int x = 0; x < NO; ++x)
 #pragma unroll
       for (int z = 0; z < NO; ++z) {
-        const cx<R> sxz = dagS ? ldr<R>(sp + z * NO + x).conj() : ldr<R>(sp + x * NO + z);
+        const cx<R> sxz = low ? -s[z * NO + x].conj() : s[x * NO + z];
 #pragma unroll
         for (int y = 0; y < NO; ++y) pa[x * NO + y] = cfma(sxz, g[z * NO + y], pa[x * NO + y]);
       }
   };
-  auto gload = [&](int l, cx<R>* g) {  // g[z][y] = w_l conj(G^R(T,l)[y][z])
-    const R wl = rule_wr<R>(W, T, l);
-    const S* gp = el<NO, S>(d.GR, d, n, T, l);
+  auto mixed = [&](int t, int a0, int da) {
+    const double2* sv = tv<NO>(d.STV, d, n, t, 0);
+#pragma unroll(NO <= 2 ? 2 : 1)
+    for (int a = a0; a < d.r; a += da)
 #pragma unroll
-    for (int z = 0; z < NO; ++z)
+      for (int x = 0; x < NO; ++x)
 #pragma unroll
-      for (int y = 0; y < NO; ++y) g[z * NO + y] = ldr<R>(gp + y * NO + z).conj() * wl;
+        for (int z = 0; z < NO; ++z) {
+          const V s = ld_split<S>(sv + (long long)a * NO2 + x * NO + z);
+#pragma unroll
+          for (int y = 0; y < NO; ++y) mx[x * NO + y].add(s, vs[a * NO2 + z * NO + y]);
+        }
   };
-  zero();
-  // l >= t: Sigma^<(t, l) = S[l][t]; the uncompressed rows [c, T] (coalesced over t)
-  for (int l0 = 0; l0 < nr; l0 += FOLD) {
-#pragma unroll
-    for (int jj = 0; jj < FOLD; ++jj)
-      if (l0 + jj < nr) mac_g(el<NO, S>(d.SL, d, n, c + l0 + jj, t), false, gs[l0 + jj]);
-    fold();
-  }
-  // the same leaf, l in [t, E)
-  cx<R> g[NO2];
-  for (int l0 = t; l0 < E; l0 += FOLD) {
-#pragma unroll
-    for (int jj = 0; jj < FOLD; ++jj) {
-      const int l = l0 + jj;
-      if (l < E) {
-        gload(l, g);
-        mac_g(Lf<NO, S>(d, 3, n, jt, l, t), false, g);
-      }
-    }
-    fold();
-  }
-  // l < t in the same leaf: -S[t][l]^dagger
-  for (int l0 = A; l0 < t; l0 += FOLD) {
-#pragma unroll
-    for (int jj = 0; jj < FOLD; ++jj) {
-      const int l = l0 + jj;
-      if (l < t) {
-        gload(l, g);
-#pragma unroll
-        for (int q = 0; q < NO2; ++q) g[q] = -g[q];
-        mac_g(Lf<NO, S>(d, 3, n, jt, t, l), true, g);
-      }
-    }
-    fold();
-  }
-  // blocks with t in their columns (P1 . conj V) and in their rows (-conj U . P2)
-  for (int lv = 0; lv < d.maxl; ++lv) {
-    const int b = d.colblk[jt * d.maxl + lv];
-    if (b < 0 || d.b_r0[b] >= c) continue;
-    const int c0 = d.b_c0[b];
-#pragma unroll
-    for (int p = 0; p < NO2; ++p) {
-      const int x = p / NO;
-      const int rk = *Rk<NO>(d, 3, n, b, p);
-      const S* V = Vp<NO, S>(d, 3, n, b, p) + (long long)(t - c0) * d.rmax;
-#pragma unroll
-      for (int y = 0; y < NO; ++y) {
-        ka[x * NO + y].add(lr_dot_conj<R, S>(Psrc<NO, R>(d, n, b, p, y, 0), V, rk));
-      }
-    }
-  }
-  for (int lv = 0; lv < d.maxl; ++lv) {
-    const int b = d.rowblk[jt * d.maxl + lv];
-    if (b < 0) continue;
-    const int r0 = d.b_r0[b];
-#pragma unroll
-    for (int p = 0; p < NO2; ++p) {  // p = (z, x)
-      const int x = p % NO;
-      const int rk = *Rk<NO>(d, 3, n, b, p);
-      const S* U = Up<NO, S>(d, 3, n, b, p) + (long long)(t - r0) * d.rmax;
-#pragma unroll
-      for (int y = 0; y < NO; ++y) {
-        ka[x * NO + y].add(-lr_dot_conj<R, S>(Psrc<NO, R>(d, n, b, p, y, 1), U, rk));
-      }
-    }
-  }
-#pragma unroll
-#pragma unroll
-  for (int q = 0; q < NO2; ++q) acc[q] += ka[q].get();
-  for (int q = 0; q < NO2; ++q) acc[q] = acc[q] * d.h;
-  for (int a = 0; a < d.r; ++a) {  // -i sum_a Sigma^tv(t, tau_a) v_a
-    const double2* sv = tv<NO>(d.STV, d, n, t, a);
-    const double2* vv = d.vvec + ((long long)n * d.r + a) * NO2;
-#pragma unroll
-    for (int x = 0; x < NO; ++x)
-#pragma unroll
-      for (int z = 0; z < NO; ++z) {
-        const zd sxz = ld(sv + x * NO + z) * zd(0, -1);
-#pragma unroll
-        for (int y = 0; y < NO; ++y) acc[x * NO + y] = cfma(sxz, ld(vv + z * NO + y), acc[x * NO + y]);
-      }
-  }
-  double2* qp = d.qsrc + ((long long)n * d.nt + t) * NO2;
-#pragma unroll
-  for (int q = 0; q < NO2; ++q) stv<S>(qp + q, acc[q]);
-}
-
-// q(t) for the uncompressed rows t in [c, T]: one warp per t (lanes along the row).
-template <int NO, typename S>
-__global__ void k_src_h(Dev d, int T) {
-  constexpr int NO2 = NO * NO;
-  using R = typename Bulk<S>::R;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int nrow = T + 1 - d.cdir;
-  const int n = gw / nrow, t = d.cdir + gw % nrow;
-  if (n >= d.n_inst || !d.active[n]) return;
-  const int c = d.cdir, L = d.L;
-  const double h = d.h;
-  const DevW& W = d.w;
-  zd acc[NO2];
-#pragma unroll
-  for (int q = 0; q < NO2; ++q) acc[q] = zd();
-  KAcc<R> ka[NO2];   // the history sums: compensated FP32 in the complex64 form
-  const int jt = t / L, A = jt * L, E = min(A + L, d.nt);
-  // pa[x][y] += wl sum_z Sx[x][z] conj(G^R(T,l)[y][z]), Sx = S or S^dagger (in R)
-  auto sg = [&](cx<R>* pa, const S* sp, bool dagS, const S* gp, R wl) {
-#pragma unroll
-    for (int x = 0; x < NO; ++x)
-#pragma unroll
-      for (int z = 0; z < NO; ++z) {
-        const cx<R> sxz = (dagS ? ldr<R>(sp + z * NO + x).conj() : ldr<R>(sp + x * NO + z)) * wl;
-#pragma unroll
-        for (int y = 0; y < NO; ++y) pa[x * NO + y] = cfma(sxz, ldr<R>(gp + y * NO + z).conj(), pa[x * NO + y]);
-      }
-  };
-  auto fold = [&](cx<R>* pa) {
-#pragma unroll
-    for (int q = 0; q < NO2; ++q) { ka[q].add(pa[q]); pa[q] = cx<R>(0); }
-  };
-  cx<R> pa[NO2];
-#pragma unroll
-  for (int q = 0; q < NO2; ++q) pa[q] = cx<R>(0);
-  // part 1, l >= t: S[l][t]
-  for (int l = max(t, c) + lane; l <= T; l += 32)  // uncompressed rows (at most a leaf and k+8)
-    sg(pa, el<NO, S>(d.SL, d, n, l, t), false, el<NO, S>(d.GR, d, n, T, l), rule_wr<R>(W, T, l));
-  if (t < c) {
-    for (int l = t + lane; l < min(E, c); l += 32)  // same leaf
-      sg(pa, Lf<NO, S>(d, 3, n, jt, l, t), false, el<NO, S>(d.GR, d, n, T, l), rule_wr<R>(W, T, l));
-  }
-  fold(pa);
-  for (int lv = 0; lv < d.maxl; ++lv) {  // blocks with t in their columns
-    const int b = d.colblk[jt * d.maxl + lv];
-    if (b < 0 || d.b_r0[b] >= c) continue;
-    const int c0 = d.b_c0[b];
-#pragma unroll
-    for (int p = 0; p < NO2; ++p) {
-      const int x = p / NO;
-      const int rk = *Rk<NO>(d, 3, n, b, p);
-      const S* V = Vp<NO, S>(d, 3, n, b, p) + (long long)(t - c0) * d.rmax;
-#pragma unroll
-      for (int y = 0; y < NO; ++y) {
-        const cx<R>* P = Psrc<NO, R>(d, n, b, p, y, 0);
-        cx<R> sb = cx<R>(0);
-        for (int q = lane; q < rk; q += 32) sb = cfma(P[q], ldr<R>(V + q).conj(), sb);
-        ka[x * NO + y].add(sb);
-      }
-    }
-  }
-  // part 2, l < t: -S[t][l]^dagger
-  if (t >= c) {
-    for (int l0 = lane; l0 < t; l0 += 32 * FOLD) {  // the whole (uncompressed) row t
+  if ((int)blockIdx.x >= ntile) {   // uncompressed rows, one warp each, lanes along the row
+    __syncthreads();
+    const int t = c + ((int)blockIdx.x - ntile) * 8 + warp;
+    if (t > T) return;
+    cx<R> g[NO2], s[NO2];
+    for (int l0 = lane; l0 <= T; l0 += 32 * FOLD) {
 #pragma unroll
       for (int jj = 0; jj < FOLD; ++jj) {
         const int l = l0 + 32 * jj;
-        if (l < t) sg(pa, el<NO, S>(d.SL, d, n, t, l), true, el<NO, S>(d.GR, d, n, T, l), -rule_wr<R>(W, T, l));
-      }
-      fold(pa);
-    }
-  } else {
-    for (int l = A + lane; l < t; l += 32)
-      sg(pa, Lf<NO, S>(d, 3, n, jt, t, l), true, el<NO, S>(d.GR, d, n, T, l), -rule_wr<R>(W, T, l));
-    fold(pa);
-    for (int lv = 0; lv < d.maxl; ++lv) {  // blocks with t in their rows
-      const int b = d.rowblk[jt * d.maxl + lv];
-      if (b < 0) continue;
-      const int r0 = d.b_r0[b];
+        if (l <= T) {
+          const S* sp = l >= t ? el<NO, S>(d.SL, d, n, l, t) : el<NO, S>(d.SL, d, n, t, l);
 #pragma unroll
-      for (int p = 0; p < NO2; ++p) {  // p = (z, x): conj(U^{zx}(t,:)) . P2^{(zx), y} -> q_xy
-        const int x = p % NO;
-        const int rk = *Rk<NO>(d, 3, n, b, p);
-        const S* U = Up<NO, S>(d, 3, n, b, p) + (long long)(t - r0) * d.rmax;
-#pragma unroll
-        for (int y = 0; y < NO; ++y) {
-          const cx<R>* P = Psrc<NO, R>(d, n, b, p, y, 1);
-          cx<R> sb = cx<R>(0);
-          for (int q = lane; q < rk; q += 32) sb = cfma(ldr<R>(U + q).conj(), P[q], sb);
-          ka[x * NO + y].add(-sb);
+          for (int q = 0; q < NO2; ++q) {
+            s[q] = ldr<R>(sp + q);
+            g[q] = gw(l, q / NO, q % NO);
+          }
+          mac(s, l < t, g);
         }
       }
+      fold();
+    }
+    V hist[NO2];
+#pragma unroll
+    for (int q = 0; q < NO2; ++q) hist[q] = vreal(kacc_lanes(ka[q], 1, 32), d.h, W.hf);
+    mixed(t, lane, 32);
+#pragma unroll
+    for (int q = 0; q < NO2; ++q) {
+      V v = vmul_mi(mx[q].get());
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) v = vadd(v, vshfl_xor(v, off));
+      if (lane == 0) stV(d.qsrc + ((long long)n * d.nt + t) * NO2 + q, vadd(hist[q], v));
+    }
+    return;
+  }
+  // 32 compressed columns
+  const int t = blockIdx.x * 32 + lane, jt = blockIdx.x * 32 / L, A = jt * L;
+  cx<R>* gr = reinterpret_cast<cx<R>*>(red + 8 * NO2 * 32);   // [kSrcRing][NO2] w_l g_l of the uncompressed rows
+  cx<R>* gl = gr + kSrcRing * NO2;                            // [L][NO2] of the leaf
+  int* rk = reinterpret_cast<int*>(gl + 64 * NO2);            // per slot (target x, side, level, other index): rank,
+  const int nslot = 2 * d.maxl * NO2;
+  int* start = rk + nslot;                                    // first packed entry,
+  int* blk = start + nslot + 1;                               // block,
+  long long* base = reinterpret_cast<long long*>(((unsigned long long)(blk + nslot) + 7) & ~7ull);   // factor row of t0
+  unsigned short* list = reinterpret_cast<unsigned short*>(base + nslot);   // entries: slot * 128 + q
+  const int nr = T + 1 - c;
+  for (int e = tid; e < nr * NO2; e += blockDim.x) gr[e] = gw(c + e / NO2, (e % NO2) / NO, e % NO);
+  for (int e = tid; e < L * NO2; e += blockDim.x) gl[e] = gw(A + e / NO2, (e % NO2) / NO, e % NO);
+  for (int s = tid; s < nslot; s += blockDim.x) {
+    const int x = s / (2 * d.maxl * NO), which = (s / (d.maxl * NO)) & 1, lv = (s / NO) % d.maxl, z = s % NO;
+    const int p = which == 0 ? x * NO + z : z * NO + x;
+    int b = (which == 0 ? d.colblk : d.rowblk)[jt * d.maxl + lv];
+    if (b >= 0 && d.b_r0[b] >= c) b = -1;
+    blk[s] = b;
+    rk[s] = b >= 0 ? *Rk<NO>(d, 3, n, b, p) : 0;
+    if (b >= 0) {
+      const int r0 = d.b_r0[b], c0 = d.b_c0[b];
+      base[s] = which == 0 ? ((long long)n * d.vtot + d.b_voff[b] + (long long)p * (d.b_c1[b] - c0) + (blockIdx.x * 32 - c0)) * d.rmax
+                           : ((long long)n * d.utot + d.b_uoff[b] + (long long)p * (d.b_r1[b] - r0) + (blockIdx.x * 32 - r0)) * d.rmax;
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    int carry = 0;
+    for (int s0 = 0; s0 < nslot; s0 += 32) {
+      const int r = s0 + lane < nslot ? rk[s0 + lane] : 0;
+      int x = r;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, x, o);
+        if (lane >= o) x += y;
+      }
+      if (s0 + lane < nslot) start[s0 + lane] = carry + x - r;
+      carry += __shfl_sync(FULL, x, 31);
+    }
+    if (lane == 0) start[nslot] = carry;
+  }
+  __syncthreads();
+  if (uselist) {
+    for (int s = warp; s < nslot; s += 8)
+      for (int q = lane; q < rk[s]; q += 32) list[start[s] + q] = (unsigned short)(s * 128 + q);
+    __syncthreads();
+  }
+  cx<R> s[NO2];
+  for (int l0 = warp; l0 < nr; l0 += 8 * FOLD) {   // the uncompressed rows
+#pragma unroll
+    for (int jj = 0; jj < FOLD; ++jj) {
+      const int l = l0 + 8 * jj;
+      if (l < nr) {
+        const S* sp = el<NO, S>(d.SL, d, n, c + l, t);
+#pragma unroll
+        for (int q = 0; q < NO2; ++q) s[q] = ldr<R>(sp + q);
+        mac(s, false, gr + l * NO2);
+      }
+    }
+    fold();
+  }
+  for (int l0 = warp; l0 < L; l0 += 8 * FOLD) {   // the leaf, both triangles
+#pragma unroll
+    for (int jj = 0; jj < FOLD; ++jj) {
+      const int l = A + l0 + 8 * jj;
+      if (l < A + L) {
+        const S* sp = Lf<NO, S>(d, 3, n, jt, max(l, t), min(l, t));
+#pragma unroll
+        for (int q = 0; q < NO2; ++q) s[q] = ldr<R>(sp + q);
+        mac(s, l < t, gl + (l - A) * NO2);
+      }
+    }
+    fold();
+  }
+  const int tstr = lane * d.rmax;
+#pragma unroll
+  for (int x = 0; x < NO; ++x) {   // the blocks
+    auto entries = [&](auto at, int e0, int e1, int stride) {   // kEB entries from e0, at(e) = slot * 128 + q
+      cx<R> f[kEB], P[kEB][NO];
+#pragma unroll
+      for (int u = 0; u < kEB; ++u) {
+        const int e = e0 + stride * u, le = at(min(e, e1 - 1)), sl = le >> 7, q = le & 127;
+        const int which = (sl / (d.maxl * NO)) & 1, z = sl % NO, p = which == 0 ? x * NO + z : z * NO + x;
+        const S* F = static_cast<const S*>(which == 0 ? d.hod[3].V : d.hod[3].U) + base[sl] + tstr;
+        const cx<R>* pp = Psrc<NO, R>(d, n, blk[sl], p, which) + q * NO;
+        f[u] = e < e1 ? ldr<R>(F + q).conj() : cx<R>(0);
+#pragma unroll
+        for (int y = 0; y < NO; ++y) P[u][y] = pp[y];
+      }
+#pragma unroll
+      for (int y = 0; y < NO; ++y) {
+        cx<R> sum = cx<R>(0);
+#pragma unroll
+        for (int u = 0; u < kEB; ++u) sum = cfma(P[u][y], f[u], sum);
+        ka[x * NO + y].add(sum);
+      }
+    };
+    if (uselist) {
+      const int e1 = start[(x + 1) * 2 * d.maxl * NO];
+      for (int e0 = start[x * 2 * d.maxl * NO] + warp; e0 < e1; e0 += 8 * kEB)
+        entries([&](int e) { return (int)list[e]; }, e0, e1, 8);
+    } else {
+      for (int sl = x * 2 * d.maxl * NO; sl < (x + 1) * 2 * d.maxl * NO; ++sl)
+        for (int q0 = warp; q0 < rk[sl]; q0 += 8 * kEB) entries([&](int q) { return sl * 128 + q; }, q0, rk[sl], 8);
     }
   }
 #pragma unroll
-  for (int q = 0; q < NO2; ++q) acc[q] += ka[q].get();
+  for (int q = 0; q < NO2; ++q) red[(warp * NO2 + q) * 32 + lane] = vreal(kacc_lanes(ka[q], 32, 32), d.h, W.hf);
+  mixed(t, warp, 8);
 #pragma unroll
-  for (int q = 0; q < NO2; ++q) acc[q] = acc[q] * h;
-  for (int a = lane; a < d.r; a += 32) {
-    M<NO> Sm = load<NO>(tv<NO>(d.STV, d, n, t, a));
-    M<NO> V = load<NO>(d.vvec + ((long long)n * d.r + a) * NO2);
-    mac<NO>(*reinterpret_cast<M<NO>*>(acc), Sm, V, zd(0, -1));
+  for (int q = 0; q < NO2; ++q) {
+    V& v = red[(warp * NO2 + q) * 32 + lane];
+    v = vadd(v, vmul_mi(mx[q].get()));
   }
-  warp_sum<NO2>(acc);
-  if (lane == 0) {
-    double2* p = d.qsrc + ((long long)n * d.nt + t) * NO2;
+  __syncthreads();
+  for (int e = tid; e < 32 * NO2; e += blockDim.x) {
+    const int tt = e / NO2, q = e % NO2;
+    V a[8];
 #pragma unroll
-    for (int q = 0; q < NO2; ++q) stv<S>(p + q, acc[q]);
+    for (int w2 = 0; w2 < 8; ++w2) a[w2] = red[(w2 * NO2 + q) * 32 + tt];
+#pragma unroll
+    for (int s2 = 4; s2; s2 >>= 1)
+#pragma unroll
+      for (int w2 = 0; w2 < s2; ++w2) a[w2] = vadd(a[w2], a[w2 + s2]);
+    stV(d.qsrc + ((long long)n * d.nt + blockIdx.x * 32) * NO2 + e, a[0]);
   }
 }
 
@@ -912,19 +944,27 @@ __global__ void __launch_bounds__(kLatMaxK) k_lattice_obs(Dev d, int t, double* 
     default: return cudaErrorInvalidValue;                                      \
   }
 
-cudaError_t launch_src_h(const Dev& d, int T, cudaStream_t s) {
-  if (d.cdir > 0) {
-    dim3 g(d.nblk, d.n_inst);
-    HK_DISPATCH(d.no, (k_src_proj<NO, S><<<g, 256, 0, s>>>(d, T)));
-  }
-  if (d.cdir > 0) {
-    if (T + 1 - d.cdir > kSrcRing) return cudaErrorInvalidValue;
-    dim3 g((d.cdir + 127) / 128, d.n_inst);
-    HK_DISPATCH(d.no, (k_src_c<NO, S><<<g, 128, 0, s>>>(d, T)));
-  }
-  const long long warps = (long long)d.n_inst * (T + 1 - d.cdir);
-  HK_DISPATCH(d.no, (k_src_h<NO, S><<<(unsigned)((warps * 32 + 127) / 128), 128, 0, s>>>(d, T)));
+// Dynamic shared memory of k_src_q; the list of packed entries is left out
+// where ranks, levels and orbitals would make it too large.
+template <int NO, typename S>
+static cudaError_t src_q(const Dev& d, int T, cudaStream_t s) {
+  const size_t n2 = NO * NO, es = sizeof(S), ns = 2 * (size_t)d.maxl * n2;
+  size_t bytes = ((size_t)d.r * n2 + 8 * n2 * 32) * 16 + (kSrcRing + 64) * n2 * es + (3 * ns + 1) * 4 + 8 + ns * 8;
+  const size_t list = ns * d.rmax * 2;
+  const int uselist = ns * 128 <= 65536 && bytes + list <= 200 * 1024;
+  if (uselist) bytes += list;
+  if (bytes > 227 * 1024) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(k_src_q<NO, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  const int nrow = T + 1 - d.cdir;
+  k_src_q<NO, S><<<dim3(d.cdir / 32 + (nrow + 7) / 8, d.n_inst), 256, bytes, s>>>(d, T, uselist);
   return cudaGetLastError();
+}
+cudaError_t launch_src_h(const Dev& d, int T, int njob, cudaStream_t s) {
+  if (d.cdir > 0 && T + 1 - d.cdir > kSrcRing) return cudaErrorInvalidValue;
+  if (njob > 0) HK_DISPATCH(d.no, (k_src_proj<NO, S><<<dim3(njob, d.n_inst), 256, 0, s>>>(d, T)));
+  HK_DISPATCH(d.no, return (src_q<NO, S>(d, T, s)));
+  return cudaSuccess;
 }
 cudaError_t launch_compress(const Dev& d, int A, int nb, cudaStream_t s) {
   {

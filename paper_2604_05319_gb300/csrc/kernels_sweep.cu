@@ -61,33 +61,6 @@ constexpr int kRingRows = 80;             // >= leaf + k + 1 uncompressed rows
 template <typename R>
 __device__ __forceinline__ auto reduce8(const KAcc<R>& k) { return kacc_lanes(k, 1, 8); }
 
-// A solved value: FP64, or float-float in the complex64 form (about 48 bits
-// on the FP32 pipes; an FP64 instruction holds a warp's pipe for 64 cycles,
-// and a chunk's epilogue in FP64 took most of the chunk's time).
-template <typename S> struct Val { using t = zd; };
-template <> struct Val<float2> { using t = cff; };
-__device__ __forceinline__ void vset(zd& v, const zd& x) { v = x; }
-__device__ __forceinline__ void vset(cff& v, const zd& x) { v = cff_of(x); }
-__device__ __forceinline__ zd v64(const zd& v) { return v; }
-__device__ __forceinline__ zd v64(const cff& v) { return cff_val(v); }
-__device__ __forceinline__ zd vadd(const zd& a, const zd& b) { return a + b; }
-__device__ __forceinline__ cff vadd(const cff& a, const cff& b) { return cff_add(a, b); }
-__device__ __forceinline__ zd vbulk(const zd& v) { return v; }                      // in the bulk arithmetic
-__device__ __forceinline__ zf vbulk(const cff& v) { return zf(v.re.hi, v.im.hi); }
-__device__ __forceinline__ zd vreal(const zd& a, double s, float2) { return a * s; }
-__device__ __forceinline__ cff vreal(const cff& a, double, float2 s) {
-  return {ff_mul(a.re, {s.x, s.y}), ff_mul(a.im, {s.x, s.y})};
-}
-// acc + (-i a_j / h) y
-__device__ __forceinline__ zd vbdf(const zd& acc, const zd& y, const DevW& W, int j) {
-  return zd(fma(W.ah[j], y.im, acc.re), fma(-W.ah[j], y.re, acc.im));
-}
-__device__ __forceinline__ cff vbdf(const cff& acc, const cff& y, const DevW& W, int j) {
-  const ffl a{W.ahf[j].x, W.ahf[j].y};
-  return {ff_add(acc.re, ff_mul(a, y.im)), ff_add(acc.im, ff_neg(ff_mul(a, y.re)))};
-}
-__device__ __forceinline__ zd vshfl_xor(const zd& a, int off) { return wshfl(a, off); }
-__device__ __forceinline__ cff vshfl_xor(const cff& a, int off) { return cff_shfl_xor(a, off); }
 // |new - old|^2, old a stored element
 __device__ __forceinline__ double vdist(const zd& a, const zd& o) { return (a - o).abs2(); }
 __device__ __forceinline__ float vdist(const cff& a, const zf& o) {
@@ -96,15 +69,6 @@ __device__ __forceinline__ float vdist(const cff& a, const zf& o) {
 }
 __device__ __forceinline__ void vstore(double2* p, const zd& v) { st(p, v); }
 __device__ __forceinline__ void vstore(float2* p, const cff& v) { *p = make_float2(v.re.hi, v.im.hi); }
-template <typename T, int N>
-__device__ __forceinline__ T pick(const T (&v)[N], int i) {   // v[i] without indexed registers
-  T r = v[0];
-#pragma unroll
-  for (int j = 1; j < N; ++j)
-    if (i == j) r = v[j];
-  return r;
-}
-
 // Where a sweep keeps the row it solves: in place (FP64 storage), or in FP64
 // next to the complex64 storage: the row's slot of the FP64 ring copies of the
 // compressed form (which the TSVD later compresses), else the buffer

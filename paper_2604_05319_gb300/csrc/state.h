@@ -45,6 +45,12 @@ struct Dev {
   long long utot, vtot, leaftot;
   Hod hod[4];          // 0 G^R, 1 G^<, 2 Sigma^R, 3 Sigma^<
   void* band;          // [n][nt][k][no2] Sigma^R(t, t-d), d = 1..k
+  // jobs of the source projections, sorted by the block's first row; partial sums
+  // of the long block sides and the counters of their finished CTAs
+  const int4* s_tab;
+  double2* spart;
+  long long s_parts;
+  int* s_cnt;
   double2* proj;       // sweep projections [n][no][maxl][no2][rmax] (+ source: see kernels)
   double2* tsvd_ws;    // TSVD workspace: [tsvd_group][4][no2] slots of tsvd_ws_per entries,
   long long tsvd_ws_per;  // level lv of a slot at offset ws_lvoff[lv]; the compression
@@ -92,6 +98,8 @@ struct Dev {
   const int *last;             // [n] last time step of each instance (N_t of the instance - 1)
 };
 
+constexpr int kSrcChunk = 256;   // rows of a block side that one CTA of the source projections takes
+
 // ---- launchers (all on `s`) ----
 cudaError_t launch_extrapolate(const Dev& d, int T, cudaStream_t s);
 cudaError_t launch_sigma(const Dev& d, int T, cudaStream_t s);
@@ -106,7 +114,7 @@ cudaError_t launch_set_active(const Dev& d, double tol, int iter, int min_iter, 
 // compressed (HODLR) form
 cudaError_t launch_ret_h(const Dev& d, int T, cudaStream_t s);
 cudaError_t launch_les_h(const Dev& d, int T, cudaStream_t s);
-cudaError_t launch_src_h(const Dev& d, int T, cudaStream_t s);
+cudaError_t launch_src_h(const Dev& d, int T, int njob, cudaStream_t s);   // njob: jobs with built rows
 cudaError_t launch_compress(const Dev& d, int A, int nb, cudaStream_t s);
 cudaError_t launch_density_at(const Dev& d, int t, double2* out, cudaStream_t s);  // rho(t), every instance
 cudaError_t launch_sigma_lattice(const Dev& d, int T, cudaStream_t s);   // model 4, all k at once
