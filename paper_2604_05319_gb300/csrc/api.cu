@@ -546,8 +546,16 @@ int hkbe_set_dlr(hkbe_t* h, int r, const double* tau, const double* omega) {
       (rc = dalloc_tv(h, &d.STV, (size_t)d.n_inst * d.nt * r * n2)) ||
       (rc = dalloc(h, &d.gm, (size_t)d.n_inst * r * n2)) ||
       (rc = dalloc(h, &d.wconv, (size_t)d.n_inst * r * r * n2)) ||
-      (rc = dalloc(h, &d.vvec, (size_t)d.n_inst * r * n2)))
+      (rc = dalloc(h, &d.vvec, (size_t)d.n_inst * r * n2)) || (rc = walloc(h, &d.qrev, (size_t)r * r)))
     return rc;
+  std::vector<double> qrev((size_t)r * r);
+  for (int a = 0; a < r; ++a)
+    for (int c = 0; c < r; ++c) {
+      long double v = 0;
+      for (int b = 0; b < r; ++b) v += (long double)h->dm.q[a * r + b] * h->dm.rev[b * r + c];
+      qrev[a * r + c] = (double)v;
+    }
+  HK_CUDA(h, cudaMemcpyAsync(d.qrev, qrev.data(), qrev.size() * sizeof(double), cudaMemcpyHostToDevice, h->s));
   HK_CUDA(h, cudaMemcpyAsync(d.tau, tau, r * sizeof(double), cudaMemcpyHostToDevice, h->s));
   HK_CUDA(h, cudaMemcpyAsync(d.e0, h->dm.e0.data(), r * sizeof(double), cudaMemcpyHostToDevice, h->s));
   HK_CUDA(h, cudaMemcpyAsync(d.ebeta, h->dm.ebeta.data(), r * sizeof(double), cudaMemcpyHostToDevice, h->s));

@@ -211,6 +211,44 @@ __device__ __forceinline__ void lu_apply(int n, const zd* A, const int* piv, zd*
   }
 }
 
+// In-place Gauss-Jordan inverse with partial pivoting of the n x n matrix A
+// (leading dimension ld, shared memory, n <= 20); every thread calls it.
+static __device__ __noinline__ void gj_inverse(int n, zd* A, int ld) {
+  __shared__ zd col[20];
+  __shared__ int prow[20];
+  const int tid = threadIdx.x;
+  for (int c = 0; c < n; ++c) {
+    if (tid < 32) {
+      double v = (tid >= c && tid < n) ? A[tid * ld + c].abs2() : -1.0;
+      int p = tid;
+#pragma unroll
+      for (int off = 16; off; off >>= 1) {
+        const double v2 = __shfl_xor_sync(FULL, v, off);
+        const int p2 = __shfl_xor_sync(FULL, p, off);
+        if (v2 > v || (v2 == v && p2 < p)) { v = v2; p = p2; }
+      }
+      if (p != c && tid < n) { const zd t = A[c * ld + tid]; A[c * ld + tid] = A[p * ld + tid]; A[p * ld + tid] = t; }
+      if (tid == 0) prow[c] = p;
+      __syncwarp();
+      if (tid < n) col[tid] = tid == c ? cdiv(zd(1.0), A[c * ld + c]) : A[tid * ld + c];
+      __syncwarp();
+      if (tid < n) A[c * ld + tid] = tid == c ? col[c] : A[c * ld + tid] * col[c];   // the scaled pivot row
+    }
+    __syncthreads();
+    for (int e = tid; e < n * n; e += blockDim.x) {
+      const int r = e / n, j = e % n;
+      if (r == c) continue;
+      const zd f = col[r];
+      A[r * ld + j] = j == c ? -(f * col[c]) : A[r * ld + j] - f * A[c * ld + j];
+    }
+    __syncthreads();
+  }
+  if (tid < n)   // undo the row exchanges on the columns, last first
+    for (int c = n - 1; c >= 0; --c)
+      if (prow[c] != c) { const zd t = A[tid * ld + c]; A[tid * ld + c] = A[tid * ld + prow[c]]; A[tid * ld + prow[c]] = t; }
+  __syncthreads();
+}
+
 // small vector solves: y M = r (row vector) and M x = r (column vector)
 template <int NO>
 __device__ void solve_row(const M<NO>& Mm, const zd* r, zd* y) {

@@ -8,8 +8,8 @@
 // Per self-consistency iteration at step T the launches are
 //   k_sigma  Sigma^R(T, .), Sigma^<(., T), Sigma^tv(T, .) from the current G
 //   (the retarded row, Eq. KBER, is solved by k_ret2 in kernels_sweep.cu)
-//   k_mixed  G^tv(T, tau_i) (Eq. KBET), one warp per (instance, node)
-//   k_vt     v_a = sum_b Q_ab G^vt(tau_b, T) and x_0 = -[G^tv(T, 0)]^dagger
+//   k_mixed  G^tv(T, tau_i) (Eq. KBET), one CTA per (instance, group of nodes)
+//   k_vt_qr  v_a = sum_b Q_ab G^vt(tau_b, T) and x_0 = -[G^tv(T, 0)]^dagger
 //   k_src    lesser source q(t), t = 0..T, one warp per (instance, t)
 //   k_les    lesser column x_t = G^<(t, T) (Eq. KBEL), one CTA per
 //            (instance, orbital column): start block t <= k solved together,
@@ -269,104 +269,179 @@ constexpr int CH = 32;     // chunk of the sequential sweeps
 constexpr int NWARP = 8;   // warps per sweep CTA
 
 // ---------------------------------------------------------------------------
-// Mixed component at step T, Eq. KBET (one warp per (instance, node)).
+// Mixed component at step T, Eq. KBET.  One CTA per instance and group of NI
+// nodes: a lane owns element (i, z, y) of the group's rows of G^tv (adjacent
+// elements, 16-byte loads) and all N_o products with column z of Sigma^R; the
+// warps, and the lanes left over by a small group, split the history l and the
+// convolution sum a.  Groups fill a warp (32 elements) where that gives a CTA to
+// every SM (256 lattice points: 38 us an iteration, 76 us with small groups);
+// with fewer, groups of 64 bytes or one node spread the FP64 products over more
+// SMs (3 instances, FP64, N_o = 1, T = 256: 19 us with groups of 32, 16 with 4).  (One
+// warp per node over all l read 16 bytes of every row and node apart, and its
+// lane 0 solved an N_o x N_o system per node: 158 us for 128 instances at
+// N_o = 2, T = 600; 110 us for 16 at N_o = 4, T = 290.)
 // ---------------------------------------------------------------------------
-template <int NO, typename S>
-__global__ void k_mixed(Dev d, int T) {
-  constexpr int NO2 = NO * NO;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int n = gw / d.r, i = gw % d.r;
-  if (n >= d.n_inst || !d.active[n]) return;
-  const int k = d.k;
+template <int NO> constexpr int kNodes = 32 / (NO * NO);                      // nodes per CTA
+template <int NO> constexpr int kNodesFew = NO == 1 ? 4 : NO == 2 ? 2 : 1;    // with few instances
+template <int NO, typename S, int NI>
+__global__ void __launch_bounds__(256) k_mixed(Dev d, int T) {
+  constexpr int NO2 = NO * NO, E = NI * NO2, LS = 32 / E, NS = 8 * LS;   // elements, slices per warp and CTA
+  constexpr bool kLanes = LS > 1 && E * LS == 32;   // a warp's slices are combined by shuffles
+  constexpr int NR = kLanes ? 8 : NS;               // partial sums per element
+  constexpr bool MX = sizeof(S) == sizeof(float2);
+  using R = typename Bulk<S>::R;
+  const int n = blockIdx.y, i0 = blockIdx.x * NI;
+  if (!d.active[n]) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int k = d.k, ni = min(NI, d.r - i0);
   const double h = d.h;
   const DevW& W = d.w;
-  zd acc[NO2];
+  __shared__ zd red[NR][NO][E];
+  __shared__ zd Mi[NO2];       // inverse of the point's matrix
+  __shared__ double serr[8];
+  if (tid < NO2) {
+    const int x = tid / NO, y = tid % NO;
+    Mi[tid] = (x == y ? zd(0, W.a[0] / h) : zd()) - ld(epsp<NO>(d, n, T) + tid) -
+              ld(el<NO, S>(d.SR, d, n, T, T) + tid) * (h * rule_w(W, T, T));
+  }
+  const int el_ = lane % E, slice = warp * LS + lane / E;
+  const bool act = lane < LS * E && el_ < ni * NO2;
+  const int z = (el_ % NO2) / NO;
+  const double2* G = tv<NO>(d.GTV, d, n, 0, i0) + (act ? el_ : 0);
+  const long long gs = (long long)d.r * NO2;   // from row l to row l + 1
+  const S* Sr = el<NO, S>(d.SR, d, n, T, 0) + z;
+  constexpr int UB = 8;        // rows in flight
+  KAcc<R> ka[NO];              // h sum_l w_l Sigma^R(T,l) G^tv(l, tau_i): FP32 products, compensated, in the complex64 form
+  for (int l0 = slice; l0 < T; l0 += NS * UB) {
+    double2 g[UB];
 #pragma unroll
-  for (int q = 0; q < NO2; ++q) acc[q] = zd();
-  if constexpr (sizeof(S) == sizeof(float2)) {
-    // complex64 form: h sum_l w_l Sigma^R(T,l) G^tv(l, tau_i) with FP32 products
-    // (G^tv truncated to FP32 on the integer pipes) in compensated FP32 sums
-    KAcc<float> ka[NO2];
-    const float hf = (float)h;
-    for (int l0 = lane; l0 < T; l0 += 32 * 4) {
-      zf pa[NO2];
+    for (int u = 0; u < UB; ++u) {
+      const int l = l0 + NS * u;
+      g[u] = l < T ? G[l * gs] : make_double2(0, 0);
+    }
 #pragma unroll
-      for (int q = 0; q < NO2; ++q) pa[q] = zf(0.f);
+    for (int u0 = 0; u0 < UB; u0 += 4) {
+      cx<R> pa[NO];
 #pragma unroll
-      for (int jj = 0; jj < 4; ++jj) {
-        const int l = l0 + 32 * jj;
+      for (int x = 0; x < NO; ++x) pa[x] = cx<R>(0);
+#pragma unroll
+      for (int u = u0; u < u0 + 4; ++u) {
+        const int l = l0 + NS * u;
         if (l < T) {
-          const float wl = hf * rule_wr<float>(W, T, l);
-          const S* sp = el<NO, S>(d.SR, d, n, T, l);
-          const double2* gp = tv<NO>(d.GTV, d, n, l, i);
-          zf g[NO2];
+          const R wl = (R)h * rule_wr<R>(W, T, l);
+          cx<R> gv;
+          if constexpr (MX) gv = zf(f32_of(g[u].x), f32_of(g[u].y));
+          else gv = zd(g[u].x, g[u].y);
 #pragma unroll
-          for (int q = 0; q < NO2; ++q) g[q] = ld_f32(gp + q);
-#pragma unroll
-          for (int x = 0; x < NO; ++x)
-#pragma unroll
-            for (int z = 0; z < NO; ++z) {
-              const zf sx = ldr<float>(sp + x * NO + z) * wl;
-#pragma unroll
-              for (int y = 0; y < NO; ++y) pa[x * NO + y] = cfma(sx, g[z * NO + y], pa[x * NO + y]);
-            }
+          for (int x = 0; x < NO; ++x) pa[x] = cfma(ldr<R>(Sr + (long long)l * NO2 + x * NO) * wl, gv, pa[x]);
         }
       }
 #pragma unroll
-      for (int q = 0; q < NO2; ++q) ka[q].add(pa[q]);
+      for (int x = 0; x < NO; ++x) ka[x].add(pa[x]);
     }
+  }
+  zd acc[NO];
 #pragma unroll
-    for (int q = 0; q < NO2; ++q) acc[q] = ka[q].get();
+  for (int x = 0; x < NO; ++x) acc[x] = ka[x].get();
+  const double2* C = d.wconv + ((long long)n * d.r * d.r + i0) * NO2 + (act ? el_ : 0);
+  const double2* St = tv<NO>(d.STV, d, n, T, 0) + z;
+#pragma unroll 4
+  for (int a = slice; a < d.r; a += NS) {   // sum_a Sigma^tv(T, tau_a) W[a][i]
+    const zd c = ld(C + (long long)a * gs);
+#pragma unroll
+    for (int x = 0; x < NO; ++x) acc[x] = cfma(ld(St + (long long)a * NO2 + x * NO), c, acc[x]);
+  }
+#pragma unroll
+  for (int x = 0; x < NO; ++x) {
+    if constexpr (kLanes) {
+#pragma unroll
+      for (int off = 16; off >= E; off >>= 1) acc[x] += wshfl(acc[x], off);
+      if (lane < E) red[warp][x][el_] = acc[x];
+    } else {
+      if (lane < LS * E) red[slice][x][el_] = acc[x];
+    }
+  }
+  __syncthreads();
+  if constexpr (NO == 1) {
+    if (tid == 0) Mi[0] = cdiv(zd(1.0), Mi[0]);
+    __syncthreads();
   } else {
-    for (int l = lane; l < T; l += 32) {  // h sum_l w_l Sigma^R(T,l) G^tv(l, tau_i)
-      const double wl = h * rule_w(W, T, l);
-      M<NO> Sm = load<NO>(el<NO, S>(d.SR, d, n, T, l));
-      M<NO> G = load<NO>(tv<NO>(d.GTV, d, n, l, i));
+    gj_inverse(NO, Mi, NO);
+  }
+  zd rhs = zd();
+  double e = 0.0;
+  const int i = tid / NO2, x = (tid % NO2) / NO, y = tid % NO;
+  if (tid < ni * NO2) {
+    for (int w2 = 0; w2 < NR; ++w2)
 #pragma unroll
-      for (int x = 0; x < NO; ++x)
-#pragma unroll
-        for (int z = 0; z < NO; ++z) {
-          zd sx = Sm.a[x][z] * wl;
-#pragma unroll
-          for (int y = 0; y < NO; ++y) acc[x * NO + y] = cfma(sx, G.a[z][y], acc[x * NO + y]);
-        }
+      for (int zz = 0; zz < NO; ++zz) rhs += red[w2][x][i * NO2 + zz * NO + y];
+    const double2* gp = tv<NO>(d.GTV, d, n, T, i0) + tid;
+    for (int j = 1; j <= k; ++j) {
+      const zd g = ld(gp - j * gs);
+      rhs += zd(W.ah[j] * g.im, -W.ah[j] * g.re);
     }
   }
-  for (int a = lane; a < d.r; a += 32) {  // sum_a Sigma^tv(T, tau_a) W[a][i]
-    M<NO> Sm = load<NO>(tv<NO>(d.STV, d, n, T, a));
-    M<NO> C = load<NO>(d.wconv + (((long long)n * d.r + a) * d.r + i) * NO2);
-    mac<NO>(*reinterpret_cast<M<NO>*>(acc), Sm, C, zd(1.0));
+  __syncthreads();
+  zd* rs = &red[0][0][0];
+  if (tid < ni * NO2) rs[tid] = rhs;
+  __syncthreads();
+  if (tid < ni * NO2) {
+    zd v = zd();
+#pragma unroll
+    for (int m = 0; m < NO; ++m) v = cfma(Mi[x * NO + m], rs[i * NO2 + m * NO + y], v);
+    double2* p = tv<NO>(d.GTV, d, n, T, i0) + tid;
+    e = sqrt((v - ld(p)).abs2());
+    st(p, v);
   }
-  if (lane >= 1 && lane <= k) {
-    M<NO> G = load<NO>(tv<NO>(d.GTV, d, n, T - lane, i));
-    const zd c(0, -W.a[lane] / h);
-#pragma unroll
-    for (int q = 0; q < NO2; ++q) acc[q] += c * G.a[q / NO][q % NO];
-  }
-  warp_sum<NO2>(acc);
-  if (lane == 0) {
-    const double wt = h * rule_w(W, T, T);
-    M<NO> Mm, R;
-    const S* sd = el<NO, S>(d.SR, d, n, T, T);
-    const double2* ep = epsp<NO>(d, n, T);
-#pragma unroll
-    for (int x = 0; x < NO; ++x)
-#pragma unroll
-      for (int y = 0; y < NO; ++y) {
-        Mm.a[x][y] = (x == y ? zd(0, W.a[0] / h) : zd()) - ld(ep + x * NO + y) - ld(sd + x * NO + y) * wt;
-        R.a[x][y] = acc[x * NO + y];
-      }
-    M<NO> X = solve_left<NO>(Mm, R);
-    double2* p = tv<NO>(d.GTV, d, n, T, i);
-    M<NO> old = load<NO>(p);
-    store<NO>(p, X);
-    atomic_max_nonneg(d.err + n, maxabs_diff<NO>(X, old));
+  e = warp_max(e);
+  if (lane == 0) serr[warp] = e;
+  __syncthreads();
+  if (tid == 0) {
+    for (int w2 = 1; w2 < 8; ++w2) e = fmax(e, serr[w2]);
+    atomic_max_nonneg(d.err + n, e);
   }
 }
 
 // v_a = sum_b Q_ab G^vt(tau_b, T), G^vt(tau_b, T) = -xi [G^tv(T, beta - tau_b)]^dagger,
-// x_0 = -[G^tv(T, 0+)]^dagger.  One CTA per instance, thread per node.
+// x_0 = -[G^tv(T, 0+)]^dagger, with the product Q Rev formed once at set-up:
+// v_a = -xi sum_c (Q Rev)_ac [G^tv(T, tau_c)]^dagger.  16 rows a (row r: the
+// boundary value) per CTA, 16 lanes over c.  FP64-bound; the two products one
+// after the other, a row per thread, took 15 us (N_o = 1) to 126 us (N_o = 4).
+template <int NO, typename S>
+__global__ void __launch_bounds__(256) k_vt_qr(Dev d, int T) {
+  constexpr int NO2 = NO * NO;
+  const int n = blockIdx.y;
+  if (!d.active[n]) return;
+  const int r = d.r, a = blockIdx.x * 16 + (threadIdx.x >> 4), sl = threadIdx.x & 15;
+  if (a > r) return;   // (whole 16-lane groups)
+  const double* row = a < r ? d.qrev + (long long)a * r : d.e0;
+  zd acc[NO2];
+#pragma unroll
+  for (int q = 0; q < NO2; ++q) acc[q] = zd();
+  for (int c = sl; c < r; c += 16) {
+    const double rv = row[c];
+    const double2* g = tv<NO>(d.GTV, d, n, T, c);
+#pragma unroll
+    for (int q = 0; q < NO2; ++q) {
+      const zd v = ld(g + q);
+      acc[q] = zd(fma(v.re, rv, acc[q].re), fma(v.im, rv, acc[q].im));
+    }
+  }
+  const unsigned grp = 0xffffu << (threadIdx.x & 16);
+#pragma unroll
+  for (int off = 8; off; off >>= 1)
+#pragma unroll
+    for (int q = 0; q < NO2; ++q)
+      acc[q] += zd(__shfl_xor_sync(grp, acc[q].re, off), __shfl_xor_sync(grp, acc[q].im, off));
+  if (sl) return;
+  double2* p = a < r ? d.vvec + ((long long)n * r + a) * NO2 : d.x0 + (long long)n * NO2;
+  const double s = a < r ? -(double)d.xi : -1.0;
+#pragma unroll
+  for (int q = 0; q < NO2; ++q) st(p + q, acc[(q % NO) * NO + q / NO].conj() * s);
+}
+
+// The same from Q and Rev themselves, for the allocation-free entry point (it has
+// no buffer for their product).  One CTA per instance, thread per node.
 template <int NO, typename S>
 __global__ void k_vt(Dev d, int T) {
   constexpr int NO2 = NO * NO;
@@ -600,94 +675,80 @@ __global__ void __launch_bounds__(256) k_les(Dev d, int T) {
 // Diagonal density matrix (Sec. 3.3): (a_0/h) rho + i (A rho - rho A^dag) =
 //   -(1/h) sum_{j>=1} a_j rho(T-j) + xi (r0 + r0^dag),
 // A = eps(T) + h w_T Sigma^R(T,T), r0 = h sum_{l<T} w_l Sigma^R(T,l) x_l + q(T).
+// One CTA per instance; the N_o^2 x N_o^2 system is inverted by the whole CTA
+// (one thread's elimination took 0.6 of the 0.67 ms at N_o = 4).
 // ---------------------------------------------------------------------------
 template <int NO, typename S>
-__global__ void k_rho(Dev d, int T) {
+__global__ void __launch_bounds__(256) k_rho(Dev d, int T) {
   constexpr int NO2 = NO * NO;
   const int n = blockIdx.x;
   if (!d.active[n]) return;
   const double h = d.h;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ zd part[8][NO2];
+  __shared__ zd A[NO2], r0[NO2], b[NO2], Lm[NO2 * NO2];
   zd acc[NO2];
 #pragma unroll
   for (int q = 0; q < NO2; ++q) acc[q] = zd();
-  for (int l = threadIdx.x; l < T; l += blockDim.x) {
+  for (int l = tid; l < T; l += blockDim.x) {
     const double wl = h * rule_w(d.w, T, l);
     M<NO> Sm = load<NO>(el<NO, S>(d.SR, d, n, T, l));
     M<NO> X = load<NO>(el<NO, S>(d.GL, d, n, T, l));
     mac<NO>(*reinterpret_cast<M<NO>*>(acc), Sm, X, zd(wl));
   }
+  if (tid < NO2)
+    A[tid] = ld(epsp<NO>(d, n, T) + tid) + ld(el<NO, S>(d.SR, d, n, T, T) + tid) * (h * rule_w(d.w, T, T));
   warp_sum<NO2>(acc);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane == 0)
     for (int q = 0; q < NO2; ++q) part[warp][q] = acc[q];
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  zd r0[NO2];
-  for (int q = 0; q < NO2; ++q) {
-    r0[q] = ldv64<S>(d.qsrc + ((long long)n * d.nt + T) * NO2 + q);
-    for (int w2 = 0; w2 < (int)(blockDim.x >> 5); ++w2) r0[q] += part[w2][q];
+  if (tid < NO2) {
+    zd v = ldv64<S>(d.qsrc + ((long long)n * d.nt + T) * NO2 + tid);
+    for (int w2 = 0; w2 < 8; ++w2) v += part[w2][tid];
+    r0[tid] = v;
   }
+  // L vec(rho) = vec(rhs), vec row-major: (a0/h) E + i (A E - E A^dag) with E = e_u e_v^T
+  for (int e = tid; e < NO2 * NO2; e += blockDim.x) {
+    const int x = (e / NO2) / NO, y = (e / NO2) % NO, u = (e % NO2) / NO, v = e % NO;
+    zd val = (x == u && y == v) ? zd(d.w.ah[0]) : zd();
+    if (y == v) val += zd(0, 1) * A[x * NO + u];
+    if (x == u) val -= zd(0, 1) * A[y * NO + v].conj();
+    Lm[e] = val;
+  }
+  __syncthreads();
   const double xi = d.xi;
-  const double wt = h * rule_w(d.w, T, T);
-  M<NO> A, rhs;
-  const S* sd = el<NO, S>(d.SR, d, n, T, T);
-  const double2* ep = epsp<NO>(d, n, T);
-  for (int x = 0; x < NO; ++x)
-    for (int y = 0; y < NO; ++y) {
-      A.a[x][y] = ld(ep + x * NO + y) + ld(sd + x * NO + y) * wt;
-      rhs.a[x][y] = (r0[x * NO + y] + r0[y * NO + x].conj()) * xi;
-    }
   constexpr bool f64 = sizeof(S) == sizeof(double2);  // else: FP64 diagonal history in diag64
-  for (int j = 1; j <= d.k; ++j) {
-    const M<NO> gd = f64 ? load<NO>(el<NO, S>(d.GL, d, n, T - j, T - j))
-                         : load<NO>(d.diag64 + ((long long)n * d.nt + T - j) * NO2);
-    M<NO> rho = scale<NO>(gd, zd(0, xi));
-    rhs = rhs - scale<NO>(rho, zd(d.w.a[j] / h));
-  }
-  // L vec(rho) = vec(rhs), vec row-major, L[(x,y),(u,v)]
-  zd L[NO2 * NO2], b[NO2];
-  for (int p = 0; p < NO2; ++p) {
-    const int u = p / NO, v = p % NO;
-    for (int q = 0; q < NO2; ++q) {
-      const int x = q / NO, y = q % NO;
-      // (a0/h) E + i (A E - E A^dag) with E = e_u e_v^T
-      zd val = (x == u && y == v) ? zd(d.w.a[0] / h) : zd();
-      if (y == v) val += zd(0, 1) * A.a[x][u];
-      if (x == u) val -= zd(0, 1) * A.a[y][v].conj();
-      L[q * NO2 + p] = val;
+  if (tid < NO2) {
+    zd rhs = (r0[tid] + r0[(tid % NO) * NO + tid / NO].conj()) * xi;
+    for (int j = 1; j <= d.k; ++j) {   // rho(T - j) = xi i G^<(T-j, T-j)
+      const zd g = f64 ? ld(el<NO, S>(d.GL, d, n, T - j, T - j) + tid)
+                       : ld(d.diag64 + ((long long)n * d.nt + T - j) * NO2 + tid);
+      rhs += zd(g.im, -g.re) * (xi * d.w.ah[j]);
     }
-    b[p] = rhs.a[u][v];
+    b[tid] = rhs;
   }
-  for (int c = 0; c < NO2; ++c) {  // Gaussian elimination with pivoting
-    int pv = c;
-    for (int r = c + 1; r < NO2; ++r)
-      if (L[r * NO2 + c].abs2() > L[pv * NO2 + c].abs2()) pv = r;
-    if (pv != c) {
-      for (int j = 0; j < NO2; ++j) { zd t = L[c * NO2 + j]; L[c * NO2 + j] = L[pv * NO2 + j]; L[pv * NO2 + j] = t; }
-      zd t = b[c]; b[c] = b[pv]; b[pv] = t;
-    }
-    for (int r = c + 1; r < NO2; ++r) {
-      zd f = cdiv(L[r * NO2 + c], L[c * NO2 + c]);
-      for (int j = c; j < NO2; ++j) L[r * NO2 + j] -= f * L[c * NO2 + j];
-      b[r] -= f * b[c];
-    }
+  if constexpr (NO == 1) {
+    if (tid == 0) Lm[0] = cdiv(zd(1.0), Lm[0]);
+    __syncthreads();
+  } else {
+    __syncthreads();
+    gj_inverse(NO2, Lm, NO2);
   }
-  for (int c = NO2 - 1; c >= 0; --c) {
-    zd s = b[c];
-    for (int j = c + 1; j < NO2; ++j) s -= L[c * NO2 + j] * b[j];
-    b[c] = cdiv(s, L[c * NO2 + c]);
-  }
-  S* p = el<NO, S>(d.GL, d, n, T, T);
   double e = 0.0;
-  for (int q = 0; q < NO2; ++q) {
-    zd x = b[q] * zd(0, -xi);  // G^<(T,T) = -i xi rho
-    e = fmax(e, sqrt((x - ld(p + q)).abs2()));
-    st(p + q, x);
-    if (d.ring64[1]) st(el64<NO>(d, 1, n, T, T) + q, x);
-    if (!f64) st(d.diag64 + ((long long)n * d.nt + T) * NO2 + q, x);
+  if (tid < NO2) {
+    zd x = zd();
+    for (int j = 0; j < NO2; ++j) x = cfma(Lm[tid * NO2 + j], b[j], x);
+    x = x * zd(0, -xi);  // G^<(T,T) = -i xi rho
+    S* p = el<NO, S>(d.GL, d, n, T, T);
+    e = sqrt((x - ld(p + tid)).abs2());
+    st(p + tid, x);
+    if (d.ring64[1]) st(el64<NO>(d, 1, n, T, T) + tid, x);
+    if (!f64) st(d.diag64 + ((long long)n * d.nt + T) * NO2 + tid, x);
   }
-  atomic_max_nonneg(d.err + n, e);
+  if (warp == 0) {
+    e = warp_max(e);
+    if (lane == 0) atomic_max_nonneg(d.err + n, e);
+  }
 }
 
 template <int NO, typename S>
@@ -937,16 +998,16 @@ __global__ void k_set_active(Dev d, double tol, int iter, int min_iter, int* any
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-#define HK_DISPATCH(NOV, CALL)                                                  \
+#define HK_DISPATCH(NOV, ...)                                                   \
   switch ((NOV) * 2 + d.prec) {                                                 \
-    case 2: { constexpr int NO = 1; using S = double2; CALL; break; }           \
-    case 3: { constexpr int NO = 1; using S = float2; CALL; break; }            \
-    case 4: { constexpr int NO = 2; using S = double2; CALL; break; }           \
-    case 5: { constexpr int NO = 2; using S = float2; CALL; break; }            \
-    case 6: { constexpr int NO = 3; using S = double2; CALL; break; }           \
-    case 7: { constexpr int NO = 3; using S = float2; CALL; break; }            \
-    case 8: { constexpr int NO = 4; using S = double2; CALL; break; }           \
-    case 9: { constexpr int NO = 4; using S = float2; CALL; break; }            \
+    case 2: { constexpr int NO = 1; using S = double2; __VA_ARGS__; break; }           \
+    case 3: { constexpr int NO = 1; using S = float2; __VA_ARGS__; break; }            \
+    case 4: { constexpr int NO = 2; using S = double2; __VA_ARGS__; break; }           \
+    case 5: { constexpr int NO = 2; using S = float2; __VA_ARGS__; break; }            \
+    case 6: { constexpr int NO = 3; using S = double2; __VA_ARGS__; break; }           \
+    case 7: { constexpr int NO = 3; using S = float2; __VA_ARGS__; break; }            \
+    case 8: { constexpr int NO = 4; using S = double2; __VA_ARGS__; break; }           \
+    case 9: { constexpr int NO = 4; using S = float2; __VA_ARGS__; break; }            \
     default: return cudaErrorInvalidValue;                                      \
   }
 
@@ -962,12 +1023,18 @@ cudaError_t launch_sigma(const Dev& d, int T, cudaStream_t s) {
   return cudaGetLastError();
 }
 cudaError_t launch_mixed(const Dev& d, int T, cudaStream_t s) {
-  const long long warps = (long long)d.n_inst * d.r;
-  HK_DISPATCH(d.no, (k_mixed<NO, S><<<(unsigned)((warps * 32 + 127) / 128), 128, 0, s>>>(d, T)));
+  HK_DISPATCH(d.no, {
+    constexpr int N1 = kNodes<NO>, N2 = kNodesFew<NO>;
+    if ((d.r + N1 - 1) / N1 * d.n_inst >= 152)
+      k_mixed<NO, S, N1><<<dim3((d.r + N1 - 1) / N1, d.n_inst), 256, 0, s>>>(d, T);
+    else
+      k_mixed<NO, S, N2><<<dim3((d.r + N2 - 1) / N2, d.n_inst), 256, 0, s>>>(d, T);
+  })
   return cudaGetLastError();
 }
 cudaError_t launch_vt(const Dev& d, int T, cudaStream_t s) {
-  HK_DISPATCH(d.no, (k_vt<NO, S><<<d.n_inst, 128, d.r * NO * NO * sizeof(zd), s>>>(d, T)));
+  if (d.qrev) HK_DISPATCH(d.no, (k_vt_qr<NO, S><<<dim3((d.r + 16) / 16, d.n_inst), 256, 0, s>>>(d, T)))
+  else HK_DISPATCH(d.no, (k_vt<NO, S><<<d.n_inst, 128, d.r * NO * NO * sizeof(zd), s>>>(d, T)))
   return cudaGetLastError();
 }
 cudaError_t launch_src(const Dev& d, int T, cudaStream_t s) {

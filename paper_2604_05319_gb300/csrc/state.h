@@ -76,6 +76,7 @@ struct Dev {
   double2 *gm;                 // [n][r][no2]
   double2 *wconv;              // [n][r(a)][r(i)][no2]
   double *tau, *e0, *ebeta, *rev, *q;  // [r], [r], [r], [r*r], [r*r]
+  double *qrev;                // [r*r] Q Rev (null: the allocation-free entry point)
   double *mpar;                // [n][MP]
   double2 *qsrc;               // [n][nt][no2]   lesser source q(t) (complex64 form: float-float pairs)
   double2 *vvec;               // [n][r][no2]    v_a = sum_b Q_ab G^vt(tau_b, T)
