@@ -837,67 +837,102 @@ __global__ void k_density_at(Dev d, int t, double2* out) {
 // k = 2 pi (m_x, m_y)/L (instance m_x L + m_y), or, with the reflection
 // k_y -> -k_y of a drive along x (Sec. 4.2, the L(L/2+1) k-set), one
 // instance per m_y <= L/2 (instance m_x (L/2+1) + m_y; k-point (m_x, L - m_y)
-// reads instance (m_x, m_y)).  One CTA per time t of the current row (and
-// per DLR node for the mixed row); thread q owns grid point q = m_x L + m_y
-// and real-space point r = (q / L, q % L):
-//   X_r = (1/N_k) sum_k e^{+i k.r} X_k,  Y_{-r} = (1/N_k) sum_k e^{-i k.r} Y_k,
+// reads instance (m_x, m_y)):
+//   X_r = (1/N_k) sum_k e^{+i k.r} X_k,
 //   Sigma^>_r = U(T)U(t) G^>_r(T,t)^2 G^<_{-r}(t,T),
 //   Sigma^<_r = U(T)U(t) G^<_r(T,t)^2 G^>_{-r}(t,T),
-//   Sigma_k = sum_r e^{-i k.r} Sigma_r,  Sigma^R = Sigma^> - Sigma^<;
-// mixed: Sigma^tv_r = U(T)U(0_|) G^tv_r(T,tau)^2 G^vt_{-r}(tau,T).
-// The 2D transforms are done as two passes of L-point sums (rows, columns).
+//   Sigma_k = sum_r e^{-i k.r} Sigma_r,  Sigma^R = Sigma^> - Sigma^<,
+// where Y_{-r} = (1/N_k) sum_k e^{-i k.r} Y_k of Y_k = -[X_k]^* is -[X_r]^*, so
+// G^<_{-r}(t,T) and G^>_{-r}(t,T) come from the transforms of G^<(T,t) and
+// G^>(T,t).  Mixed: Sigma^tv_r = U(T)U(0_|) G^tv_r(T,tau)^2 G^vt_{-r}(tau,T).
+// One CTA per kLatT times of the current row (or DLR nodes of the mixed row):
+// two grids each, FP64-bound.
 // ---------------------------------------------------------------------------
 template <typename S>
-__global__ void __launch_bounds__(kLatMaxK) k_sigma_lattice(Dev d, int T) {
-  __shared__ zd X1[kLatMaxK], X2[kLatMaxK], Y1[kLatMaxK], Y2[kLatMaxK], tmp[kLatMaxK], tw[16];
-  const int L = (int)d.mpar[0], ys = (int)d.mpar[1], N = L * L, q = threadIdx.x;
-  const int nq = lat_inst(q, L, ys);
+__global__ void __launch_bounds__(128) k_sigma_lattice(Dev d, int T) {
+  extern __shared__ __align__(16) zd grid[];   // [2][kLatT] grids of L rows of L + 1
+  __shared__ zd tw[16];
+  const int L = (int)d.mpar[0], ys = (int)d.mpar[1], N = L * L, gsz = L * (L + 1);
+  const int ntb = (T + kLatT) / kLatT, tid = threadIdx.x;
   lat_twiddles(tw, L);
   const double* U = d.drU;   // U(t) of instance 0 (the same for every k)
   const double invN = 1.0 / N;
-  const int b = blockIdx.x;
-  __syncthreads();
-  if (b <= T) {
-    const int t = b;
-    if (q < N) {
-      const zd gr = ldx<1, S>(d, 0, nq, T, t, 0);
-      const zd glc = ldx<1, S>(d, 1, nq, T, t, 0);        // G^<(t, T)
-      const zd glr = -glc.conj();                         // G^<(T, t)
-      const zd ggr = gr + glr;                            // G^>(T, t)
-      X1[q] = ggr; X2[q] = glr; Y1[q] = glc; Y2[q] = -ggr.conj();
+  zd *X1 = grid, *X2 = grid + kLatT * gsz;
+  auto at = [&](int e, int* q) {   // element e: time (fastest) and grid point
+    *q = e / kLatT;
+    return (e % kLatT) * gsz + (*q / L) * (L + 1) + *q % L;
+  };
+  if ((int)blockIdx.x < ntb) {
+    const int t0 = blockIdx.x * kLatT;
+    for (int e = tid; e < kLatT * N; e += blockDim.x) {
+      int q;
+      const int o = at(e, &q), t = t0 + e % kLatT, nq = lat_inst(q, L, ys);
+      zd gg = zd(), gl = zd();
+      if (t <= T) {
+        gl = -ldx<1, S>(d, 1, nq, T, t, 0).conj();   // G^<(T, t)
+        gg = ldx<1, S>(d, 0, nq, T, t, 0) + gl;      // G^>(T, t)
+      }
+      X1[o] = gg;
+      X2[o] = gl;
     }
     __syncthreads();
-    lat_dft2(X1, tmp, tw, L, +1, invN);
-    lat_dft2(X2, tmp, tw, L, +1, invN);
-    lat_dft2(Y1, tmp, tw, L, -1, invN);
-    lat_dft2(Y2, tmp, tw, L, -1, invN);
-    const double uu = U[T + 1] * U[t + 1];
-    if (q < N) {
-      X1[q] = X1[q] * X1[q] * Y1[q] * uu;    // Sigma^>_r
-      X2[q] = X2[q] * X2[q] * Y2[q] * uu;    // Sigma^<_r
+    lat_fft2(grid, 2 * kLatT, tw, L, +1);
+    for (int e = tid; e < kLatT * N; e += blockDim.x) {
+      int q;
+      const int o = at(e, &q), t = t0 + e % kLatT;
+      const double uu = t <= T ? U[T + 1] * U[t + 1] : 0.0;
+      const zd g = X1[o] * invN, l = X2[o] * invN;
+      X1[o] = g * g * -l.conj() * uu;    // Sigma^>_r
+      X2[o] = l * l * -g.conj() * uu;    // Sigma^<_r
     }
     __syncthreads();
-    lat_dft2(X1, tmp, tw, L, -1, 1.0);
-    lat_dft2(X2, tmp, tw, L, -1, 1.0);
-    if (q < N && lat_owner(q, L, ys)) {
-      stx<1, S>(d, 2, nq, T, t, 0, X1[q] - X2[q]);
-      stx<1, S>(d, 3, nq, T, t, 0, -X2[q].conj());
+    lat_fft2(grid, 2 * kLatT, tw, L, -1);
+    for (int e = tid; e < kLatT * N; e += blockDim.x) {
+      int q;
+      const int o = at(e, &q), t = t0 + e % kLatT;
+      if (t > T || !lat_owner(q, L, ys)) continue;
+      const int nq = lat_inst(q, L, ys);
+      stx<1, S>(d, 2, nq, T, t, 0, X1[o] - X2[o]);
+      stx<1, S>(d, 3, nq, T, t, 0, -X2[o].conj());
     }
   } else {
-    const int i = b - (T + 1), r = d.r;
-    if (q < N) {
-      X1[q] = ld(tv<1>(d.GTV, d, nq, T, i));
-      zd gb = zd();                                        // G^tv(T, beta - tau_i)
-      for (int c = 0; c < r; ++c) gb += ld(tv<1>(d.GTV, d, nq, T, c)) * d.rev[i * r + c];
-      Y1[q] = gb.conj() * (-(double)d.xi);                 // G^vt(tau_i, T)
+    const int i0 = (blockIdx.x - ntb) * kLatT, r = d.r, ni = min(kLatT, r - i0);
+    for (int q = tid; q < N; q += blockDim.x) {
+      const int nq = lat_inst(q, L, ys), o = (q / L) * (L + 1) + q % L;
+      const double2* G = tv<1>(d.GTV, d, nq, T, 0);
+      zd gb[kLatT];                                          // G^tv(T, beta - tau_i)
+#pragma unroll
+      for (int i = 0; i < kLatT; ++i) gb[i] = zd();
+      for (int c = 0; c < r; ++c) {
+        const zd g = ld(G + c);
+#pragma unroll
+        for (int i = 0; i < kLatT; ++i) {
+          const double rv = i < ni ? d.rev[(i0 + i) * r + c] : 0.0;
+          gb[i] = zd(fma(g.re, rv, gb[i].re), fma(g.im, rv, gb[i].im));
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < kLatT; ++i) {
+        X1[i * gsz + o] = i < ni ? ld(G + i0 + i) : zd();
+        X2[i * gsz + o] = gb[i];
+      }
     }
     __syncthreads();
-    lat_dft2(X1, tmp, tw, L, +1, invN);
-    lat_dft2(Y1, tmp, tw, L, -1, invN);
-    if (q < N) X1[q] = X1[q] * X1[q] * Y1[q] * (U[T + 1] * U[0]);
+    lat_fft2(grid, 2 * kLatT, tw, L, +1);
+    const double uu = U[T + 1] * U[0] * -(double)d.xi;       // G^vt_{-r}(tau_i, T) = -xi [G^tv_r(T, beta - tau_i)]^*
+    for (int e = tid; e < kLatT * N; e += blockDim.x) {
+      int q;
+      const int o = at(e, &q);
+      const zd x = X1[o] * invN, y = X2[o] * invN;
+      X1[o] = x * x * y.conj() * uu;
+    }
     __syncthreads();
-    lat_dft2(X1, tmp, tw, L, -1, 1.0);
-    if (q < N && lat_owner(q, L, ys)) st(tv<1>(d.STV, d, nq, T, i), X1[q]);
+    lat_fft2(grid, kLatT, tw, L, -1);
+    for (int e = tid; e < kLatT * N; e += blockDim.x) {
+      int q;
+      const int o = at(e, &q), i = i0 + e % kLatT;
+      if (i < r && lat_owner(q, L, ys)) st(tv<1>(d.STV, d, lat_inst(q, L, ys), T, i), X1[o]);
+    }
   }
 }
 
@@ -983,8 +1018,10 @@ cudaError_t launch_density_at(const Dev& d, int t, double2* out, cudaStream_t s)
 }
 cudaError_t launch_sigma_lattice(const Dev& d, int T, cudaStream_t s) {
   if (d.no != 1 || d.n_inst > kLatMaxK) return cudaErrorInvalidValue;
-  if (d.prec) k_sigma_lattice<float2><<<T + 1 + d.r, kLatMaxK, 0, s>>>(d, T);
-  else k_sigma_lattice<double2><<<T + 1 + d.r, kLatMaxK, 0, s>>>(d, T);
+  const int nb = (T + kLatT) / kLatT + (d.r + kLatT - 1) / kLatT;
+  const size_t smem = lat_smem(16);   // 35 KB
+  if (d.prec) k_sigma_lattice<float2><<<nb, 128, smem, s>>>(d, T);
+  else k_sigma_lattice<double2><<<nb, 128, smem, s>>>(d, T);
   return cudaGetLastError();
 }
 cudaError_t launch_lattice_obs(const Dev& d, int t, double* out, cudaStream_t s) {

@@ -64,30 +64,46 @@ __global__ void __launch_bounds__(128) k_mats_sigma(MatsDev m) {
   }
 }
 
-// ---- Sigma^M(tau_i) of LATTICE2B, one CTA per DLR node ------------------
-// thread q owns grid point q = m_x L + m_y (instance lat_inst(q)) and the
-// real-space point (q / L, q % L):
+// ---- Sigma^M(tau_i) of LATTICE2B, one CTA per kLatNode DLR nodes ----------
 //   G_r(tau) = (1/N) sum_k e^{ikr} G_k(tau),  G_{-r}(-tau) = (1/N) sum_k e^{-ikr} G_k(-tau),
 //   Sigma_r = -U^2 G_r^2 G_{-r}(-tau),  Sigma_k = sum_r e^{-ikr} Sigma_r.
-__global__ void __launch_bounds__(kLatMaxK) k_mats_sigma_lattice(MatsDev m) {
-  __shared__ zd X[kLatMaxK], Y[kLatMaxK], tmp[kLatMaxK], tw[16];
-  const int L = m.L, N = L * L, q = threadIdx.x, i = blockIdx.x, r = m.r;
-  const int nq = lat_inst(q, L, m.ys);
+constexpr int kLatNode = 2;
+__global__ void __launch_bounds__(256) k_mats_sigma_lattice(MatsDev m) {
+  extern __shared__ __align__(16) zd grid[];   // [2][kLatNode] grids of L rows of L + 1
+  __shared__ zd tw[16];
+  const int L = m.L, N = L * L, gsz = L * (L + 1), i0 = blockIdx.x * kLatNode, r = m.r, ni = min(kLatNode, r - i0);
   lat_twiddles(tw, L);
-  if (q < N) {
-    const double2* G = m.G + (size_t)nq * r;
-    X[q] = ld(G + i);
-    zd s = zd();
-    for (int c = 0; c < r; ++c) s += ld(G + c) * m.rev[i * r + c];
-    Y[q] = s * (double)m.xi;
+  zd *X = grid, *Y = grid + kLatNode * gsz;
+  for (int q = threadIdx.x; q < N; q += blockDim.x) {
+    const double2* G = m.G + (size_t)lat_inst(q, L, m.ys) * r;
+    const int o = (q / L) * (L + 1) + q % L;
+    zd s[kLatNode];
+#pragma unroll
+    for (int i = 0; i < kLatNode; ++i) s[i] = zd();
+    for (int c = 0; c < r; ++c) {
+      const zd g = ld(G + c);
+#pragma unroll
+      for (int i = 0; i < kLatNode; ++i) {
+        const double rv = i < ni ? m.rev[(i0 + i) * r + c] : 0.0;
+        s[i] = zd(fma(g.re, rv, s[i].re), fma(g.im, rv, s[i].im));
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kLatNode; ++i) {
+      X[i * gsz + o] = i < ni ? ld(G + i0 + i) : zd();
+      Y[i * gsz + o] = (s[i] * (double)m.xi).conj();   // the transform with e^{-ikr} of Y is [that of Y^* with e^{ikr}]^*
+    }
   }
   __syncthreads();
-  lat_dft2(X, tmp, tw, L, +1, 1.0 / N);
-  lat_dft2(Y, tmp, tw, L, -1, 1.0 / N);
-  if (q < N) X[q] = X[q] * X[q] * Y[q] * (-m.U * m.U);
+  lat_fft2(grid, 2 * kLatNode, tw, L, +1);
+  const double sc = -m.U * m.U / ((double)N * N * N);
+  for (int e = threadIdx.x; e < kLatNode * gsz; e += blockDim.x) X[e] = X[e] * X[e] * Y[e].conj() * sc;
   __syncthreads();
-  lat_dft2(X, tmp, tw, L, -1, 1.0);
-  if (q < N && lat_owner(q, L, m.ys)) st(m.S + (size_t)nq * r + i, X[q]);
+  lat_fft2(grid, kLatNode, tw, L, -1);
+  for (int e = threadIdx.x; e < ni * N; e += blockDim.x) {
+    const int i = e % ni, q = e / ni;
+    if (lat_owner(q, L, m.ys)) st(m.S + (size_t)lat_inst(q, L, m.ys) * r + i0 + i, X[i * gsz + (q / L) * (L + 1) + q % L]);
+  }
 }
 
 // in-place inverse of an N x N complex matrix in registers (Gauss-Jordan,
@@ -223,7 +239,7 @@ cudaError_t launch_mats_sigma(const MatsDev& m, cudaStream_t s) {
   if (m.r > 128) return cudaErrorInvalidValue;
   if (m.model == kMatsLattice) {
     if (m.no != 1 || m.L * m.L > kLatMaxK) return cudaErrorInvalidValue;
-    k_mats_sigma_lattice<<<m.r, kLatMaxK, 0, s>>>(m);
+    k_mats_sigma_lattice<<<(m.r + kLatNode - 1) / kLatNode, 256, sizeof(zd) * 2 * kLatNode * m.L * (m.L + 1), s>>>(m);
   } else {
     MATS_DISPATCH((k_mats_sigma<NO><<<m.n_inst, 128, 0, s>>>(m)));
   }
