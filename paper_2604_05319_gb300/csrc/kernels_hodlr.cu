@@ -489,65 +489,164 @@ __global__ void k_comp_copy(Dev d, int A, int nb) {
   }
 }
 
-// One CTA per (component X, level slot, pair p) x instance.  Workspace per
-// CTA (complex doubles): E [nb][ncol], Q [nb][ncol], P [nb][rmax], C [nb][nb],
-// K [(rmax+nb)][(rmax+nb)] column-major, Vh [(rmax+nb)][(rmax+nb)] column-major.
-//
-// FP64 throughout, in both storage forms.  The complex64 form truncates at
-// the rounding floor of its stored rows (below), so every step must round
-// well below that floor; measured on the C4 batch, FP32 variants of the
-// projections (even with FP64 folds), of the residual rows, of the rotation
-// of V, or of the core Jacobi each put rounding directions above it and the
-// ranks grew to r_max within a few hundred steps.
+// ---------------------------------------------------------------------------
+// update_blocks, the TSVD.  One CTA per (component X, level slot, pair p) x
+// instance.  With E the new rows of the block, V the block's right factor:
+//   P = E V, E -= P V^dagger (twice in the complex64 form);
+//   Gram-Schmidt of the residual rows, E = C Q: row by row, a row whose residual
+//     is below a quarter of the threshold adds no basis direction;
+//   the core K = [[S, 0], [P, C]]: R of a column-pivoted QR, then one-sided
+//     Jacobi (round-robin pairs) on the columns of R^dagger, whose normalised
+//     columns are the right singular vectors W of K;
+//   truncation, U' = [[U, 0], [0, I]] K W / sigma, V' = [V, Q^dagger] W.
+// It is bound by the arithmetic of one SM and the latency of its phases, so:
+// tiles of E and V in shared memory; the Gram-Schmidt's second pass (against V
+// and Q) for accepted rows only, which then update every later row at once
+// (two passes over all 64 rows one after the other, five barriers each, were
+// the largest part); the pivoted QR makes the Jacobi matrix n x n and graded (4
+// to 6 sweeps instead of up to 12 on 64 + r rows), and needs no accumulation of
+// the rotations; a rotation's angle is found in FP32 and only its
+// normalisation in full precision.
+// Precision: FP64, and in the complex64 form float-float throughout (about 48
+// bits, on the FP32 pipes).  That form truncates at the rounding floor of its
+// stored rows (below), so every step must round well below that floor;
+// measured on the C4 batch, FP32 variants of the projections (even with FP64
+// folds), of the residual rows, of the rotation of V, or of the core Jacobi
+// each put rounding directions above it and the ranks grew to r_max within a
+// few hundred steps.
+// ---------------------------------------------------------------------------
 constexpr double kF32Unit = 5.9604644775390625e-8;  // 2^-24, complex64 unit roundoff
+constexpr size_t kTsvdSmem = 100 * 1024;            // dynamic shared memory: two CTAs per SM
+
+// real numbers of the same precision as Val<S>
+__device__ __forceinline__ double rmul(double a, double b) { return a * b; }
+__device__ __forceinline__ ffl rmul(const ffl& a, const ffl& b) { return ff_mul(a, b); }
+__device__ __forceinline__ zd vscl(const zd& a, double s) { return a * s; }
+__device__ __forceinline__ cff vscl(const cff& a, const ffl& s) { return {ff_mul(a.re, s), ff_mul(a.im, s)}; }
+__device__ __forceinline__ zd vmul(const zd& a, const zd& b) { return a * b; }
+__device__ __forceinline__ cff vmul(const cff& a, const cff& b) { return cff_mul(a, b); }
+__device__ __forceinline__ zd vneg(const zd& a) { return -a; }
+__device__ __forceinline__ cff vneg(const cff& a) { return {ff_neg(a.re), ff_neg(a.im)}; }
+__device__ __forceinline__ zd vconj(const zd& a) { return a.conj(); }
+__device__ __forceinline__ cff vconj(const cff& a) { return {a.re, ff_neg(a.im)}; }
+__device__ __forceinline__ zd vof(const double2& a) { return zd(a.x, a.y); }
+__device__ __forceinline__ cff vof(const float2& a) { return {{a.x, 0.f}, {a.y, 0.f}}; }
+__device__ __forceinline__ double vnorm2(const zd& a) { return a.abs2(); }
+__device__ __forceinline__ float vnorm2(const cff& a) { return a.re.hi * a.re.hi + a.im.hi * a.im.hi; }
+// 1 / sqrt(x) from an FP32 estimate by two Newton steps
+__device__ __forceinline__ double rsq(double x) {
+  const int e = ((__double2hiint(x) >> 20) & 0x7ff) - 1023;   // scale by an even power of two into the FP32 range
+  const int e2 = e & ~1;
+  const double xs = x * __hiloint2double((1023 - e2) << 20, 0);
+  double y = (double)rsqrtf((float)xs);
+  y = y * fma(-0.5 * xs * y, y, 1.5);
+  y = y * fma(-0.5 * xs * y, y, 1.5);
+  return y * __hiloint2double((1023 - e2 / 2) << 20, 0);
+}
+__device__ __forceinline__ ffl rsq(const ffl& x) {
+  const float y0 = rsqrtf(x.hi);
+  ffl y{y0, 0.f};
+  const ffl xh{-0.5f * x.hi, -0.5f * x.lo};
+#pragma unroll
+  for (int i = 0; i < 2; ++i) y = ff_mul(y, ff_add(ff_mul(ff_mul(xh, y), y), {1.5f, 0.f}));
+  return y;
+}
+__device__ __forceinline__ float r32(double x) { return (float)x; }
+__device__ __forceinline__ float r32(const ffl& x) { return x.hi; }
+__device__ __forceinline__ double r64(double x) { return x; }
+__device__ __forceinline__ double r64(const ffl& x) { return ff_val(x); }
+template <typename S> struct Re { using t = double; };
+template <> struct Re<float2> { using t = ffl; };
+__device__ __forceinline__ double rof1(float x, double2*) { return (double)x; }
+__device__ __forceinline__ ffl rof1(float x, float2*) { return {x, 0.f}; }
+__device__ __forceinline__ float vnorm32(const zd& a) { return (float)a.abs2(); }
+__device__ __forceinline__ float vnorm32(const cff& a) { return vnorm2(a); }
+__device__ __forceinline__ double rof(double x, double2*) { return x; }
+__device__ __forceinline__ ffl rof(double x, float2*) { return ff_of(x); }
+// sum of |a|^2
+template <typename S> struct Nrm2;
+template <> struct Nrm2<double2> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(const zd& a) { s = fma(a.re, a.re, fma(a.im, a.im, s)); }
+  __device__ __forceinline__ double get() const { return s; }
+};
+template <> struct Nrm2<float2> {
+  Dot2 s;
+  __device__ __forceinline__ void add(const cff& a) { s.add(a.re, a.re); s.add(a.im, a.im); }
+  __device__ __forceinline__ ffl get() const { return ff_two_sum(s.s, s.c); }
+};
+__device__ __forceinline__ double rshfl(double a, int off) { return __shfl_xor_sync(FULL, a, off); }
+__device__ __forceinline__ ffl rshfl(const ffl& a, int off) {
+  return {__shfl_xor_sync(FULL, a.hi, off), __shfl_xor_sync(FULL, a.lo, off)};
+}
+__device__ __forceinline__ double radd(double a, double b) { return a + b; }
+__device__ __forceinline__ ffl radd(const ffl& a, const ffl& b) { return ff_add(a, b); }
+// sums over the lanes reached by xor offsets from n / 2 down (all lanes call)
+template <typename T> __device__ __forceinline__ T vsum(T v, int n) {
+  for (int off = n >> 1; off; off >>= 1) v = vadd(v, vshfl_xor(v, off));
+  return v;
+}
+template <typename T> __device__ __forceinline__ T rsum(T v, int n) {
+  for (int off = n >> 1; off; off >>= 1) v = radd(v, rshfl(v, off));
+  return v;
+}
+// a - sum of products, the sum started from a
+__device__ __forceinline__ void dot_from(DotC<double2>& s, const zd& a) { s.a = a; }
+__device__ __forceinline__ void dot_from(DotC<float2>& s, const cff& a) {
+  s.re.s = a.re.hi; s.re.c = a.re.lo;
+  s.im.s = a.im.hi; s.im.c = a.im.lo;
+}
 
 template <int NO, typename S>
-__global__ void __launch_bounds__(256) k_tsvd(Dev d, int A, int nb, int n0) {
+__global__ void __launch_bounds__(256, 2) k_tsvd(Dev d, int A, int nb, int n0) {
   constexpr int NO2 = NO * NO;
+  using V = typename Val<S>::t;
+  using R = typename Re<S>::t;
   const int n = n0 + blockIdx.y;   // instances n0 .. n0 + gridDim.y - 1 share the workspace
   const int X = blockIdx.x / (d.maxl * NO2);
   const int lv = (blockIdx.x / NO2) % d.maxl;
   const int p = blockIdx.x % NO2;
-  const int j = A / d.L;
-  const int b = d.rowblk[j * d.maxl + lv];
+  const int b = d.rowblk[(A / d.L) * d.maxl + lv];
   if (b < 0 || A + nb + d.k > d.last[n]) return;   // the instance's rows end before this leaf is final
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r0 = d.b_r0[b], c0 = d.b_c0[b];
-  const int ncol = d.b_c1[b] - c0;
-  const int rmax = d.rmax;
-  const int ld_k = rmax + d.L;  // leading dimension of K and Vh
+  const int ncol = d.b_c1[b] - c0, rmax = d.rmax, L = d.L;
+  const int ld_k = rmax + L;
   double2* ws = d.tsvd_ws + (((long long)blockIdx.y * 4 + X) * NO2 + p) * d.tsvd_ws_per + d.ws_lvoff[lv];
-  double2* Em = ws;                                   // [nb][ncol]
-  double2* Qm = Em + (long long)d.L * ncol;           // [nb][ncol]
-  double2* Pm = Qm + (long long)d.L * ncol;           // [nb][rmax]
-  double2* Cm = Pm + (long long)d.L * rmax;           // [nb][nb]
-  double2* Km = Cm + (long long)d.L * d.L;            // [ld_k cols][ld_k rows]
-  double2* Vh = Km + (long long)ld_k * ld_k;          // [ld_k cols][ld_k rows]
-  __shared__ int s_rnew;
-  __shared__ double s_wpart[32];
-  __shared__ double s_sig[256];
-  __shared__ int s_ord[256];
+  V* Em = reinterpret_cast<V*>(ws);                   // [nb][ncol]
+  V* Qm = Em + (long long)L * ncol;                   // [nb][ncol]
+  V* Pm = Qm + (long long)L * ncol;                   // [nb][rmax]
+  V* Cm = Pm + (long long)L * rmax;                   // [nb][nb]
+  V* g1 = Cm + (long long)L * L;                      // [ld_k][ld_k] R^dagger, where it does not fit in shared memory
+  V* g2 = g1 + (long long)ld_k * ld_k;                // [ld_k][ld_k] the core while it is factorised, then K W / sigma
+  extern __shared__ __align__(16) char dyn[];
+  V* sm = reinterpret_cast<V*>(dyn);
+  constexpr int kSm = kTsvdSmem / sizeof(V);
+  __shared__ double s_w[8], s_norm[64], s_sig[256];
+  __shared__ int s_ord[256], s_flag, s_piv;
+  __shared__ V s_coef[256];
   int* rkp = Rk<NO>(d, X, n, b, p);
   const int r = *rkp;
   S* U = Up<NO, S>(d, X, n, b, p);
-  S* V = Vp<NO, S>(d, X, n, b, p);
+  S* Vf = Vp<NO, S>(d, X, n, b, p);
   double* Sv = Sp<NO>(d, X, n, b, p);
-  void* ring = ringX(d, X);
   // E <- new rows (and max |E| for the complex64 rounding floor below).  The
   // complex64 form reads them from its FP64 copies: rows free of storage
   // rounding, whose residuals against V hold real directions only.
-  double emax = 0.0;
-  for (long long e = tid; e < (long long)nb * ncol; e += blockDim.x) {
-    const int i = (int)(e / ncol), l = (int)(e % ncol);
-    const zd v = d.ring64[X] ? ld(el64<NO>(d, X, n, A + i, c0 + l) + p) : ld(el<NO, S>(ring, d, n, A + i, c0 + l) + p);
-    emax = fmax(emax, v.abs2());
-    st(Em + (long long)i * ncol + l, v);
+  {
+    void* ring = ringX(d, X);
+    double emax = 0.0;
+    for (int i = warp; i < nb; i += 8)
+      for (int l = lane; l < ncol; l += 32) {
+        V v;
+        if (d.ring64[X]) v = ld_split<S>(el64<NO>(d, X, n, A + i, c0 + l) + p);
+        else vset(v, ld(el<NO, S>(ring, d, n, A + i, c0 + l) + p));
+        emax = fmax(emax, (double)vnorm2(v));
+        Em[(long long)i * ncol + l] = v;
+      }
+    emax = warp_max(emax);
+    if (lane == 0) s_w[warp] = emax;
   }
-  emax = warp_max(emax);
-  if (lane == 0) s_wpart[warp] = emax;
-  __syncthreads();
-  for (int w2 = 0; w2 < nw; ++w2) emax = fmax(emax, s_wpart[w2]);
-  emax = sqrt(emax);
   __syncthreads();
   // Truncation threshold: eps_SVD, raised in the complex64 storage form to
   // the rounding floor of the appended rows.  Their rounding is a matrix of
@@ -556,226 +655,419 @@ __global__ void __launch_bounds__(256) k_tsvd(Dev d, int A, int nb, int n0) {
   // level are storage noise, and keeping them would let the rank grow by the
   // leaf size at every append.
   double tol = d.svd_tol;
-  if (sizeof(S) == sizeof(float2)) tol = fmax(tol, kF32Unit * emax * (sqrt((double)nb) + sqrt((double)ncol)));
-  // P = E V, E -= P V^dagger, twice (the second pass restores orthogonality
-  // to V lost to rounding).  The per-pass coefficients are staged in Q's
-  // storage (r <= ncol), which is free until the Gram-Schmidt below.
-  for (long long e = tid; e < (long long)nb * rmax; e += blockDim.x) Pm[e] = make_double2(0, 0);
-  __syncthreads();
-  for (int pass = 0; pass < 2 && r > 0; ++pass) {
-    for (int e = tid; e < nb * r; e += blockDim.x) {
-      const int i = e / r, q = e % r;
-      zd sacc = zd();
-      for (int l = 0; l < ncol; ++l) sacc = cfma(ld(Em + (long long)i * ncol + l), ld(V + (long long)l * rmax + q), sacc);
-      st(Pm + (long long)i * rmax + q, ld(Pm + (long long)i * rmax + q) + sacc);
-      st(Qm + (long long)i * ncol + q, sacc);
+  if (sizeof(S) == sizeof(float2)) {
+    double emax = 0.0;
+    for (int w2 = 0; w2 < 8; ++w2) emax = fmax(emax, s_w[w2]);
+    tol = fmax(tol, kF32Unit * sqrt(emax) * (sqrt((double)nb) + sqrt((double)ncol)));
+  }
+  constexpr int TC = 32;   // columns of a tile
+  // P = E V, E -= P V^dagger: once in the FP64 form, whose V is orthonormal to
+  // rounding; twice in the complex64 form, whose stored V is so to 2^-24 only (one
+  // pass leaves parts of that size along V in every row, about the threshold, and
+  // the ranks of the C2 run reached r_max).  The residual of a pass goes through
+  // its own coefficients, kept in Q's storage (r <= ncol), free until the
+  // Gram-Schmidt below.
+  constexpr int kPasses = sizeof(S) == sizeof(double2) ? 1 : 2;
+  for (int pass = 0; pass < (r > 0 ? kPasses : 1); ++pass) {
+  for (int qb = 0; qb < r; qb += 64) {   // the coefficients E V
+    const int rq = min(r - qb, 64), lg = rq <= 4 ? 2 : rq <= 8 ? 3 : rq <= 16 ? 4 : rq <= 32 ? 5 : 6;
+    const int q = tid & ((1 << lg) - 1), i0 = tid >> lg, di = blockDim.x >> lg;   // rows i0 + di o
+    V* Et = sm;                       // [64][TC + 1]
+    V* Vt = sm + 64 * (TC + 1);       // [TC][64]
+    DotC<S> acc[16];
+    for (int l0 = 0; l0 < ncol; l0 += TC) {
+      for (int e = tid; e < nb * TC; e += blockDim.x)
+        if (l0 + e % TC < ncol) Et[(e / TC) * (TC + 1) + e % TC] = Em[(long long)(e / TC) * ncol + l0 + e % TC];
+      for (int e = tid; e < TC * rq; e += blockDim.x)
+        if (l0 + e / rq < ncol) Vt[(e / rq) * 64 + e % rq] = vof(Vf[(long long)(l0 + e / rq) * rmax + qb + e % rq]);
+      __syncthreads();
+      const int lc = min(TC, ncol - l0);
+      if (q < rq)
+        for (int l = 0; l < lc; ++l) {
+          const V v = Vt[l * 64 + q];
+#pragma unroll
+          for (int o = 0; o < 16; ++o) {
+            const int i = i0 + di * o;
+            if (i >= nb) break;
+            acc[o].add(Et[i * (TC + 1) + l], v);
+          }
+        }
+      __syncthreads();
     }
-    __syncthreads();
-    for (long long e = tid; e < (long long)nb * ncol; e += blockDim.x) {
-      const int i = (int)(e / ncol), l = (int)(e % ncol);
-      zd sacc = ld(Em + e);
-      for (int q = 0; q < r; ++q) sacc -= ld(Qm + (long long)i * ncol + q) * ld(V + (long long)l * rmax + q).conj();
-      st(Em + e, sacc);
-    }
+    if (q < rq)
+#pragma unroll
+      for (int o = 0; o < 16; ++o) {
+        const int i = i0 + di * o;
+        if (i < nb) {
+          const V c = acc[o].get();
+          V* pp = Pm + (long long)i * rmax + qb + q;
+          *pp = pass == 0 ? c : vadd(*pp, c);
+          Qm[(long long)i * ncol + qb + q] = c;
+        }
+      }
     __syncthreads();
   }
-  for (long long e = tid; e < (long long)d.L * d.L; e += blockDim.x) Cm[e] = make_double2(0, 0);
+  // the residual, and the norms of its rows (rows w, w + 8, ... to warp w)
+  {
+    Nrm2<S> nr[8];
+    const int rows = (nb + 7) / 8;
+    for (int qb = 0; qb == 0 || qb < r; qb += 64) {
+      const int rq = max(0, min(r - qb, 64));
+      const bool lastq = qb + 64 >= r;
+      V* Pt = sm;                     // [64][64]
+      V* Vt = sm + 64 * 64;           // [TC][65]
+      for (int e = tid; e < nb * rq; e += blockDim.x) Pt[(e / rq) * 64 + e % rq] = vneg(Qm[(long long)(e / rq) * ncol + qb + e % rq]);
+      for (int l0 = 0; l0 < ncol; l0 += TC) {
+        for (int e = tid; e < TC * rq; e += blockDim.x)
+          if (l0 + e / rq < ncol) Vt[(e / rq) * 65 + e % rq] = vconj(vof(Vf[(long long)(l0 + e / rq) * rmax + qb + e % rq]));
+        __syncthreads();
+        if (l0 + lane < ncol) {
+#pragma unroll
+          for (int o = 0; o < 8; ++o) {
+            const int i = warp + 8 * o;
+            if (o >= rows || i >= nb) break;
+            V* ep = Em + (long long)i * ncol + l0 + lane;
+            V v = *ep;
+            if (rq) {
+              DotC<S> acc;
+              dot_from(acc, v);
+              for (int q = 0; q < rq; ++q) acc.add(Pt[i * 64 + q], Vt[lane * 65 + q]);
+              v = acc.get();
+              *ep = v;
+            }
+            if (lastq) nr[o].add(v);
+          }
+        }
+        __syncthreads();
+      }
+    }
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+      const R s = rsum(nr[o].get(), 32);
+      if (lane == 0 && warp + 8 * o < nb) s_norm[warp + 8 * o] = r64(s);
+    }
+  }
   __syncthreads();
-  // Two-pass Gram-Schmidt on the rows of E: E = C Q, rows of Q orthonormal.
-  // residual rows below a quarter of the threshold add no basis direction
+  }
+  for (int e = tid; e < L * L; e += blockDim.x) vset(Cm[e], zd());
+  __syncthreads();
+  // ---- Gram-Schmidt on the rows of E: E = C Q, rows of Q orthonormal.
+  // Residual rows below a quarter of the threshold add no basis direction
   // (a higher floor, the rounding level of one stored row, rejects rows that
   // are each at noise level but together carry a direction above the
-  // threshold: measured on the C4 batch, the ranks then grew about threefold)
-  const double delta = 0.25 * tol;
-  __shared__ zd s_coef[64];
-
-  // ke, the number of accepted basis rows, is kept in a register: every thread
-  // takes the same accept decision from the same (fixed-order) norm.
+  // threshold: measured on the C4 batch, the ranks then grew about threefold).
+  // Every thread takes the same decisions from the same sums.
+  const double delta = 0.25 * tol, delta2 = delta * delta;
   int ke = 0;
-  for (int i = 0; i < nb; ++i) {
-    double2* v = Em + (long long)i * ncol;
-    for (int pass = 0; pass < 2; ++pass) {
-      for (int e = warp; e < ke; e += nw) {  // coef_e = <Q_e, v>
-        const double2* qe = Qm + (long long)e * ncol;
-        zd s = zd();
-        for (int l = lane; l < ncol; l += 32) s = cfma(ld(qe + l).conj(), ld(v + l), s);
-        zd tmp[1] = {s};
-        warp_sum<1>(tmp);
-        if (lane == 0) s_coef[e] = tmp[0];
-      }
-      __syncthreads();
-      for (int l = tid; l < ncol; l += blockDim.x) {
-        zd s = ld(v + l);
-        for (int e = 0; e < ke; ++e) s -= s_coef[e] * ld(Qm + (long long)e * ncol + l);
-        st(v + l, s);
-      }
-      if (tid < ke) st(Cm + (long long)i * d.L + tid, ld(Cm + (long long)i * d.L + tid) + s_coef[tid]);
-      __syncthreads();
+  for (int j = 0; j < nb && r + ke < ncol; ++j) {
+    {   // the next row above the floor
+      const bool a = lane < nb && lane >= j && s_norm[lane] > delta2;
+      const bool c = lane + 32 < nb && lane + 32 >= j && s_norm[lane + 32] > delta2;
+      const unsigned lo = __ballot_sync(FULL, a), hi = __ballot_sync(FULL, c);
+      if (lo) j = __ffs(lo) - 1;
+      else if (hi) j = 31 + __ffs(hi);
+      else break;
     }
-    // norm of the residual
-    double part = 0.0;
-    for (int l = tid; l < ncol; l += blockDim.x) part += ld(v + l).abs2();
+    V* v = Em + (long long)j * ncol;
+    // second pass of the accepted row: against V, then against the rows of Q
+    for (int e = warp; e < r + ke; e += 8) {
+      DotC<S> s;
+      if (e < r)
+        for (int l = lane; l < ncol; l += 32) s.add(vof(Vf[(long long)l * rmax + e]), v[l]);
+      else
+        for (int l = lane; l < ncol; l += 32) s.add(vconj(Qm[(long long)(e - r) * ncol + l]), v[l]);
+      const V c = vsum(s.get(), 32);
+      if (lane == 0) s_coef[e] = c;
+    }
+    __syncthreads();
+    Nrm2<S> ns;
+    for (int l = tid; l < ncol; l += blockDim.x) {
+      DotC<S> s;
+      dot_from(s, v[l]);
+      for (int e = 0; e < r; ++e) s.add(vneg(s_coef[e]), vconj(vof(Vf[(long long)l * rmax + e])));
+      for (int e = 0; e < ke; ++e) s.add(vneg(s_coef[r + e]), Qm[(long long)e * ncol + l]);
+      const V x = s.get();
+      v[l] = x;
+      ns.add(x);
+    }
+    {
+      const R s = rsum(ns.get(), 32);
+      if (lane == 0) s_w[warp] = r64(s);
+    }
+    for (int e = tid; e < r + ke; e += blockDim.x) {
+      V* c = e < r ? Pm + (long long)j * rmax + e : Cm + (long long)j * L + e - r;
+      *c = vadd(*c, s_coef[e]);
+    }
+    __syncthreads();
+    double n2 = 0.0;
+    for (int w2 = 0; w2 < 8; ++w2) n2 += s_w[w2];
+    if (!(n2 > delta2)) continue;
+    const double nrm = sqrt(n2);
+    const R inv = rof(1.0 / nrm, (S*)nullptr);
+    V* q = Qm + (long long)ke * ncol;
+    for (int l = tid; l < ncol; l += blockDim.x) q[l] = vscl(v[l], inv);
+    if (tid == 0) vset(Cm[(long long)j * L + ke], zd(nrm));
+    __syncthreads();
+    // every later row loses its part along q; four rows at a time per warp
+    for (int ib = j + 1 + warp * 4; ib < nb; ib += 32) {
+      DotC<S> s[4];
+      for (int l = lane; l < ncol; l += 32) {
+        const V qc = vconj(q[l]);
 #pragma unroll
-    for (int off = 16; off; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
-    if (lane == 0) s_wpart[warp] = part;
-    __syncthreads();
-    double nsq = 0.0;  // fixed summation order: reproducible bit for bit
-    for (int w2 = 0; w2 < nw; ++w2) nsq += s_wpart[w2];
-    const double nrm = sqrt(nsq);
-    if (nrm > delta) {
-      for (int l = tid; l < ncol; l += blockDim.x) st(Qm + (long long)ke * ncol + l, ld(v + l) * (1.0 / nrm));
-      if (tid == 0) st(Cm + (long long)i * d.L + ke, zd(nrm));
-      ++ke;
+        for (int u = 0; u < 4; ++u)
+          if (ib + u < nb) s[u].add(qc, Em[(long long)(ib + u) * ncol + l]);
+      }
+      V c[4];
+      Nrm2<S> m2[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) c[u] = vsum(s[u].get(), 32);
+      for (int l = lane; l < ncol; l += 32) {
+        const V ql = q[l];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (ib + u < nb) {
+            V* ep = Em + (long long)(ib + u) * ncol + l;
+            const V x = vadd(*ep, vneg(vmul(c[u], ql)));
+            *ep = x;
+            m2[u].add(x);
+          }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const R t = rsum(m2[u].get(), 32);
+        if (lane == 0 && ib + u < nb) {
+          s_norm[ib + u] = r64(t);
+          Cm[(long long)(ib + u) * L + ke] = c[u];
+        }
+      }
     }
+    ++ke;
     __syncthreads();
-  }
-  const int m = r + nb, nk = r + ke;  // core rows, columns
-  // K = [[diag(S), 0], [P, C]] column-major; Vh = I
-  for (long long e = tid; e < (long long)ld_k * ld_k; e += blockDim.x) {
-    Km[e] = make_double2(0, 0);
-    Vh[e] = make_double2(0, 0);
   }
   __syncthreads();
+  const int m = r + nb, nk = r + ke;  // core rows, columns
+  // ---- the core K = [[diag(S), 0], [P, C]], column by column, and its column-pivoted QR ----
+  V* Xr = nk * nk <= kSm ? sm : g1;                                       // [col][nk] R^dagger
+  V* Kw = Xr == sm && nk * nk + m * nk <= kSm ? sm + nk * nk : g2;        // [col][m]
   for (int e = tid; e < nk * m; e += blockDim.x) {
     const int col = e / m, row = e % m;
-    zd v = zd();
-    if (row < r) v = (col == row) ? zd(Sv[row]) : zd();
-    else if (col < r) v = ld(Pm + (long long)(row - r) * rmax + col);
-    else v = ld(Cm + (long long)(row - r) * d.L + (col - r));
-    st(Km + (long long)col * ld_k + row, v);
+    V v;
+    if (row < r) vset(v, col == row ? zd(Sv[row]) : zd());
+    else if (col < r) v = Pm[(long long)(row - r) * rmax + col];
+    else v = Cm[(long long)(row - r) * L + (col - r)];
+    Kw[e] = v;
   }
-  for (int e = tid; e < nk; e += blockDim.x) st(Vh + (long long)e * ld_k + e, zd(1.0));
+  for (int e = tid; e < nk * nk; e += blockDim.x) vset(Xr[e], zd());
   __syncthreads();
-  // one-sided Jacobi (Hestenes) on the columns of K, round-robin pairing
-  const int npad = nk + (nk & 1);
-  __shared__ int s_rot;
+  for (int col = warp; col < nk; col += 8) {
+    Nrm2<S> s;
+    for (int i = lane; i < m; i += 32) s.add(Kw[col * m + i]);
+    const R t = rsum(s.get(), 32);
+    if (lane == 0) s_sig[col] = r64(t);
+  }
+  __syncthreads();
+  const double drop2 = 1e-14 * tol * tol;   // columns this far below the threshold add nothing
+  int nr = 0;                               // columns of R^dagger
+  for (; nr < nk; ++nr) {
+    if (warp == 0) {   // the largest remaining column (taken ones have norm -1)
+      double best = -1.0;
+      int arg = 0;
+      for (int col = lane; col < nk; col += 32)
+        if (s_sig[col] > best) { best = s_sig[col]; arg = col; }
+#pragma unroll
+      for (int off = 16; off; off >>= 1) {
+        const double b2 = __shfl_xor_sync(FULL, best, off);
+        const int a2 = __shfl_xor_sync(FULL, arg, off);
+        if (b2 > best || (b2 == best && a2 < arg)) { best = b2; arg = a2; }
+      }
+      if (lane == 0) { s_piv = best > drop2 ? arg : -1; s_w[0] = best; }
+    }
+    __syncthreads();
+    const int pv = s_piv;
+    if (pv < 0) break;
+    const double nrm = sqrt(s_w[0]);
+    const R inv = rof(1.0 / nrm, (S*)nullptr);
+    for (int i = tid; i < m; i += blockDim.x) Kw[pv * m + i] = vscl(Kw[pv * m + i], inv);
+    if (tid == 0) {
+      vset(Xr[nr * nk + pv], zd(nrm));
+      s_sig[pv] = -1.0;
+    }
+    __syncthreads();
+    for (int col = warp; col < nk; col += 8) {
+      if (s_sig[col] < 0.0) continue;
+      DotC<S> s;
+      for (int i = lane; i < m; i += 32) s.add(vconj(Kw[pv * m + i]), Kw[col * m + i]);
+      const V c = vsum(s.get(), 32);
+      Nrm2<S> t;
+      for (int i = lane; i < m; i += 32) {
+        const V x = vadd(Kw[col * m + i], vneg(vmul(c, Kw[pv * m + i])));
+        Kw[col * m + i] = x;
+        t.add(x);
+      }
+      const R t2 = rsum(t.get(), 32);
+      if (lane == 0) {
+        Xr[nr * nk + col] = vconj(c);
+        s_sig[col] = r64(t2);
+      }
+    }
+    __syncthreads();
+  }
+  __syncthreads();
+  // ---- one-sided Jacobi (Hestenes) on the columns of R^dagger, round-robin pairing, a half-warp per pair ----
+  const float small2 = (float)(1e-6 * tol * tol);   // two columns both this small are truncated: left as they are
+  const int npad = nr + (nr & 1);
   for (int sweep = 0; sweep < 40; ++sweep) {
-    if (tid == 0) s_rot = 0;
+    if (tid == 0) s_flag = 0;
     __syncthreads();
     for (int round = 0; round < npad - 1; ++round) {
-      for (int pr = warp; pr < npad / 2; pr += nw) {
-        // round-robin tournament: position 0 fixed, positions 1..npad-1 rotate
-        auto at = [&](int i) { return i == 0 ? 0 : ((i - 1 + round) % (npad - 1)) + 1; };
-        int a = at(pr), bq = at(npad - 1 - pr);
-        if (a > bq) { const int t2 = a; a = bq; bq = t2; }
-        if (bq >= nk) continue;
-        double2* ka = Km + (long long)a * ld_k;
-        double2* kb = Km + (long long)bq * ld_k;
-        double al = 0, be = 0;
-        zd ga = zd();
-        for (int i = lane; i < m; i += 32) {
-          const zd x = ld(ka + i), y = ld(kb + i);
-          al += x.abs2();
-          be += y.abs2();
-          ga = cfma(x.conj(), y, ga);
+      // round-robin tournament: position 0 fixed, positions 1..npad-1 rotate
+      auto at = [&](int i) { return i == 0 ? 0 : ((i - 1 + round) % (npad - 1)) + 1; };
+      for (int pr0 = warp * 2; pr0 < npad / 2; pr0 += 16) {
+        const int pr = pr0 + (lane >> 4), hl = lane & 15;
+        int ia = 0, ib = 0;
+        bool act = pr < npad / 2;
+        if (act) {
+          ia = at(pr);
+          ib = at(npad - 1 - pr);
+          act = ia < nr && ib < nr;
         }
-#pragma unroll
-        for (int off = 16; off; off >>= 1) {
-          al += __shfl_xor_sync(0xffffffffu, al, off);
-          be += __shfl_xor_sync(0xffffffffu, be, off);
-          ga.re += __shfl_xor_sync(0xffffffffu, ga.re, off);
-          ga.im += __shfl_xor_sync(0xffffffffu, ga.im, off);
-        }
-        const double g = sqrt(ga.abs2());
-        if (g <= 1e-14 * sqrt(al * be) || g == 0.0) continue;
-        if (lane == 0) s_rot = 1;
-        const zd ph(ga.re / g, -ga.im / g);  // e^{-i phi}
-        const double zeta = (be - al) / (2.0 * g);
-        const double tt = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-        const double cs = 1.0 / sqrt(1.0 + tt * tt), sn = cs * tt;
-        for (int i = lane; i < m; i += 32) {
-          const zd x = ld(ka + i), y = ld(kb + i) * ph;
-          st(ka + i, x * cs - y * sn);
-          st(kb + i, x * sn + y * cs);
-        }
-        double2* va = Vh + (long long)a * ld_k;
-        double2* vb = Vh + (long long)bq * ld_k;
-        for (int i = lane; i < nk; i += 32) {
-          const zd x = ld(va + i), y = ld(vb + i) * ph;
-          st(va + i, x * cs - y * sn);
-          st(vb + i, x * sn + y * cs);
+        V *xa = Xr + ia * nk, *xb = Xr + ib * nk;
+        Nrm2<S> na, nbm;
+        DotC<S> ng;
+        if (act)
+          for (int i = hl; i < nk; i += 16) {
+            const V x = xa[i], y = xb[i];
+            na.add(x);
+            nbm.add(y);
+            ng.add(vconj(x), y);
+          }
+        const R al = rsum(na.get(), 16), be = rsum(nbm.get(), 16);
+        const V ga = vsum(ng.get(), 16);
+        const float fa = r32(al), fb = r32(be);
+        // |<a, b>| in FP32, scaled by a power of two so that its square stays in range
+        const float gm = fmaxf(fabsf(r32(ga.re)), fabsf(r32(ga.im)));
+        const float sc = __uint_as_float((254u - min(max((__float_as_uint(gm) >> 23) & 0xffu, 1u), 253u)) << 23);
+        const V gs = vscl(ga, rof1(sc, (S*)nullptr));
+        const float fg = gm > 0.f ? sqrtf(vnorm32(gs)) / sc : 0.f;
+        const float eps = sizeof(S) == sizeof(double2) ? 1e-14f : 1e-13f;
+        act = act && gm > 0.f && !(fg * rsqrtf(fa) <= eps * sqrtf(fb)) && fmaxf(fa, fb) >= small2;
+        if (act) {
+          Nrm2<S> g2;
+          g2.add(gs);
+          V ph = vscl(vconj(gs), rsq(g2.get()));           // e^{-i phi}
+          const float zeta = (fb - fa) / (2.f * fg);
+          const float tf = fabsf(zeta) < 1e18f ? (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta)) : 0.5f / zeta;
+          R cs, sn;
+          if constexpr (sizeof(S) == sizeof(double2)) {
+            cs = rsq(fma((double)tf, (double)tf, 1.0));
+            sn = cs * (double)tf;
+          } else {
+            cs = rsq(ff_add(ff_mul({tf, 0.f}, {tf, 0.f}), {1.f, 0.f}));
+            sn = ff_mul(cs, {tf, 0.f});
+          }
+          if (hl == 0) s_flag = 1;
+          for (int i = hl; i < nk; i += 16) {
+            const V x = xa[i], y = vmul(xb[i], ph);
+            xa[i] = vadd(vscl(x, cs), vneg(vscl(y, sn)));
+            xb[i] = vadd(vscl(x, sn), vscl(y, cs));
+          }
         }
       }
       __syncthreads();
     }
-    if (!s_rot) break;
+    if (!s_flag) break;
     if (sweep == 39 && tid == 0) atomicAdd(d.status + 1, 1);
     __syncthreads();
   }
-  // singular values, sorted, truncated
-  for (int col = warp; col < nk; col += nw) {
-    double s2 = 0;
-    for (int i = lane; i < m; i += 32) s2 += ld(Km + (long long)col * ld_k + i).abs2();
+  // ---- singular values, sorted, truncated; W = the normalised columns ----
+  for (int col = warp; col < nr; col += 8) {
+    Nrm2<S> s;
+    for (int i = lane; i < nk; i += 32) s.add(Xr[col * nk + i]);
+    const R t = rsum(s.get(), 32);
+    if (lane == 0) s_sig[col] = sqrt(r64(t));
+  }
+  __syncthreads();
+  if (tid < nr) {   // position in descending order (ties by index)
+    const double s = s_sig[tid];
+    int pos = 0;
+    for (int i = 0; i < nr; ++i) pos += s_sig[i] > s || (s_sig[i] == s && i < tid);
+    s_ord[pos] = tid;
+  }
+  if (tid == 0) s_flag = 0;
+  __syncthreads();
+  if (tid < nr && s_sig[tid] > tol) atomicAdd(&s_flag, 1);
+  __syncthreads();
+  int rn = s_flag;
+  if (rn > rmax) {
+    if (tid == 0) atomicAdd(d.status, 1);
+    rn = rmax;
+  }
+  for (int e = tid; e < rn * nk; e += blockDim.x) {
+    V* x = Xr + s_ord[e / nk] * nk + e % nk;
+    *x = vscl(*x, rof(1.0 / s_sig[s_ord[e / nk]], (S*)nullptr));
+  }
+  __syncthreads();
+  // K W / sigma, [rn][m]: the first r rows S W / sigma, the others (P W + C W) / sigma
+  V* Kt = Xr == sm && nk * nk + rn * m <= kSm ? sm + nk * nk : g2;
+  for (int e = tid; e < rn * m; e += blockDim.x) {
+    const int jj = e / m, row = e % m;
+    const V* w = Xr + s_ord[jj] * nk;
+    const R inv = rof(1.0 / s_sig[s_ord[jj]], (S*)nullptr);
+    V v;
+    if (row < r) {
+      v = vscl(w[row], rof(Sv[row], (S*)nullptr));
+    } else {
+      DotC<S> s;
+      for (int q = 0; q < r; ++q) s.add(Pm[(long long)(row - r) * rmax + q], w[q]);
+      for (int q = 0; q < ke; ++q) s.add(Cm[(long long)(row - r) * L + q], w[r + q]);
+      v = s.get();
+    }
+    Kt[e] = vscl(v, inv);
+  }
+  __syncthreads();
+  // U' and V': lp lanes per row, up to four entries each; a row is read by its lanes before they write it
+  const int lp = rn <= 4 ? 4 : rn <= 8 ? 8 : rn <= 16 ? 16 : 32, sub = tid / lp, j0 = tid % lp, rstep = blockDim.x / lp;
+  auto rotate = [&](int rows, auto entry, S* out) {
+    for (int row0 = 0; row0 < rows; row0 += rstep) {
+      const int row = row0 + sub;
+      V res[4];
 #pragma unroll
-    for (int off = 16; off; off >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, off);
-    if (lane == 0) s_sig[col] = sqrt(s2);
-  }
-  __syncthreads();
-  if (tid == 0) {
-    for (int i = 0; i < nk; ++i) s_ord[i] = i;
-    for (int i = 0; i < nk; ++i) {  // selection sort, descending
-      int best = i;
-      for (int q = i + 1; q < nk; ++q)
-        if (s_sig[s_ord[q]] > s_sig[s_ord[best]]) best = q;
-      int t2 = s_ord[i]; s_ord[i] = s_ord[best]; s_ord[best] = t2;
-    }
-    int rn = 0;
-    while (rn < nk && s_sig[s_ord[rn]] > tol) ++rn;
-    if (rn > rmax) { atomicAdd(d.status, 1); rn = rmax; }
-    s_rnew = rn;
-  }
-  __syncthreads();
-  const int rn = s_rnew;
-  // U' = [[U, 0], [0, I]] Uhat : old rows r0..A-1, new rows A..A+nb-1
-  const int nold = A - r0;
-  for (int row = warp; row < nold + nb; row += nw) {
-    S* urow = U + (long long)row * rmax;
-    // compute U'[row][j] for j = lane, lane+32, ...
-    zd res[4];
-    for (int t2 = 0; t2 < 4; ++t2) res[t2] = zd();
-    for (int t2 = 0; t2 < 4; ++t2) {
-      const int jj = lane + 32 * t2;
-      if (jj >= rn) continue;
-      const int col = s_ord[jj];
-      const double inv = 1.0 / s_sig[col];
-      zd s = zd();
-      if (row < nold) {
-        for (int q = 0; q < r; ++q) s = cfma(ld(urow + q), ld(Km + (long long)col * ld_k + q), s);
-      } else {
-        s = ld(Km + (long long)col * ld_k + r + (row - nold));
+      for (int t2 = 0; t2 < 4; ++t2) {
+        const int jj = j0 + lp * t2;
+        vset(res[t2], zd());
+        if (jj < rn && row < rows) res[t2] = entry(row, jj);
       }
-      res[t2] = s * inv;
+      __syncwarp();
+      if (row < rows)
+        for (int t2 = 0; t2 * lp < rmax; ++t2) {
+          const int jj = j0 + lp * t2;
+          if (jj < rmax) {
+            V v = res[0];
+            if (t2 == 1) v = res[1];
+            if (t2 == 2) v = res[2];
+            if (t2 == 3) v = res[3];
+            if (jj >= rn) vset(v, zd());
+            if constexpr (sizeof(S) == sizeof(double2)) st(out + (long long)row * rmax + jj, v);
+            else out[(long long)row * rmax + jj] = make_float2(v.re.hi, v.im.hi);
+          }
+        }
+      __syncwarp();
     }
-    __syncwarp();
-    for (int t2 = 0; t2 < 4; ++t2) {
-      const int jj = lane + 32 * t2;
-      if (jj < rmax) st(urow + jj, jj < rn ? res[t2] : zd());
-    }
-    __syncwarp();
-  }
-  // V' = [V, Q^H] Vhat
-  for (int l = warp; l < ncol; l += nw) {
-    S* vrow = V + (long long)l * rmax;
-    zd res[4];
-    for (int t2 = 0; t2 < 4; ++t2) {
-      res[t2] = zd();
-      const int jj = lane + 32 * t2;
-      if (jj >= rn) continue;
-      const int col = s_ord[jj];
-      const double2* vh = Vh + (long long)col * ld_k;
-      zd s = zd();
-      for (int q = 0; q < r; ++q) s = cfma(ld(vrow + q), ld(vh + q), s);
-      for (int e = 0; e < ke; ++e) s = cfma(ld(Qm + (long long)e * ncol + l).conj(), ld(vh + r + e), s);
-      res[t2] = s;
-    }
-    __syncwarp();
-    for (int t2 = 0; t2 < 4; ++t2) {
-      const int jj = lane + 32 * t2;
-      if (jj < rmax) st(vrow + jj, jj < rn ? res[t2] : zd());
-    }
-    __syncwarp();
-  }
-  __syncthreads();
+  };
+  const int nold = A - r0;   // old rows r0..A-1, new rows A..A+nb-1
+  rotate(nold + nb, [&](int row, int jj) {
+    if (row >= nold) return Kt[jj * m + r + row - nold];
+    DotC<S> s;
+    for (int q = 0; q < r; ++q) s.add(vof(U[(long long)row * rmax + q]), Kt[jj * m + q]);
+    return s.get();
+  }, U);
+  rotate(ncol, [&](int l, int jj) {
+    const V* w = Xr + s_ord[jj] * nk;
+    DotC<S> s;
+    for (int q = 0; q < r; ++q) s.add(vof(Vf[(long long)l * rmax + q]), w[q]);
+    for (int e = 0; e < ke; ++e) s.add(vconj(Qm[(long long)e * ncol + l]), w[r + e]);
+    return s.get();
+  }, Vf);
   for (int q = tid; q < rmax; q += blockDim.x) Sv[q] = (q < rn) ? s_sig[s_ord[q]] : 0.0;
   if (tid == 0) *rkp = rn;
 }
@@ -966,16 +1258,16 @@ __global__ void __launch_bounds__(kLatMaxK) k_lattice_obs(Dev d, int t, double* 
   }
 }
 
-#define HK_DISPATCH(NOV, CALL)                                                  \
+#define HK_DISPATCH(NOV, ...)                                                   \
   switch ((NOV) * 2 + d.prec) {                                                 \
-    case 2: { constexpr int NO = 1; using S = double2; CALL; break; }           \
-    case 3: { constexpr int NO = 1; using S = float2; CALL; break; }            \
-    case 4: { constexpr int NO = 2; using S = double2; CALL; break; }           \
-    case 5: { constexpr int NO = 2; using S = float2; CALL; break; }            \
-    case 6: { constexpr int NO = 3; using S = double2; CALL; break; }           \
-    case 7: { constexpr int NO = 3; using S = float2; CALL; break; }            \
-    case 8: { constexpr int NO = 4; using S = double2; CALL; break; }           \
-    case 9: { constexpr int NO = 4; using S = float2; CALL; break; }            \
+    case 2: { constexpr int NO = 1; using S = double2; __VA_ARGS__; break; }           \
+    case 3: { constexpr int NO = 1; using S = float2; __VA_ARGS__; break; }            \
+    case 4: { constexpr int NO = 2; using S = double2; __VA_ARGS__; break; }           \
+    case 5: { constexpr int NO = 2; using S = float2; __VA_ARGS__; break; }            \
+    case 6: { constexpr int NO = 3; using S = double2; __VA_ARGS__; break; }           \
+    case 7: { constexpr int NO = 3; using S = float2; __VA_ARGS__; break; }            \
+    case 8: { constexpr int NO = 4; using S = double2; __VA_ARGS__; break; }           \
+    case 9: { constexpr int NO = 4; using S = float2; __VA_ARGS__; break; }            \
     default: return cudaErrorInvalidValue;                                      \
   }
 
@@ -1006,10 +1298,15 @@ cudaError_t launch_compress(const Dev& d, int A, int nb, cudaStream_t s) {
     dim3 g(64, d.n_inst);
     HK_DISPATCH(d.no, (k_comp_copy<NO, S><<<g, 256, 0, s>>>(d, A, nb)));
   }
-  for (int n0 = 0; n0 < d.n_inst; n0 += d.tsvd_group) {
-    dim3 g(4 * d.maxl * d.no * d.no, min(d.tsvd_group, d.n_inst - n0));
-    HK_DISPATCH(d.no, (k_tsvd<NO, S><<<g, 256, 0, s>>>(d, A, nb, n0)));
-  }
+  HK_DISPATCH(d.no, {
+    auto kern = k_tsvd<NO, S>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTsvdSmem);
+    if (e != cudaSuccess) return e;
+    for (int n0 = 0; n0 < d.n_inst; n0 += d.tsvd_group) {
+      dim3 g(4 * d.maxl * d.no * d.no, min(d.tsvd_group, d.n_inst - n0));
+      kern<<<g, 256, kTsvdSmem, s>>>(d, A, nb, n0);
+    }
+  })
   return cudaGetLastError();
 }
 cudaError_t launch_density_at(const Dev& d, int t, double2* out, cudaStream_t s) {
