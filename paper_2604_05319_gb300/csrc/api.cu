@@ -17,6 +17,8 @@
 using hk::Dev;
 using zc = std::complex<double>;
 
+constexpr int kAhead = 8;   // corrector iterations that are launched without waiting for one another
+
 struct hkbe_s {
   Dev d{};
   hkbe_params p{};
@@ -30,7 +32,7 @@ struct hkbe_s {
   int scheme = 0;              // HKBE_SCHEME_PAPER or HKBE_SCHEME_SWEEP_FREE
   std::vector<double> tau, om, gm_host, eps_host;
   hk::DLRMats dm;
-  int* any_dev = nullptr;
+  int* any_dev = nullptr;   // unused word (checkpoint files hold a copy of every buffer)
   size_t bytes = 0;
   std::vector<void*> allocs;
   std::vector<size_t> alloc_bytes;  // bytes of each entry of allocs (checkpoint files)
@@ -53,6 +55,8 @@ struct hkbe_s {
   double2* diagbuf = nullptr;  // [n_inst][no2] density matrices of one time
   std::vector<int> src_r0;   // first block row of each source-projection job (ascending)
   std::vector<void*> work;   // device buffers that are in neither snapshots nor files
+  int ahead = 1;             // corrector iterations of the last step
+  hk::IterResult *res = nullptr, *res_dev = nullptr;   // [kAhead][n_inst] outcomes, pinned host memory
   // points whose rows the chunk inverses hold (retarded [0, rowsR), lesser [1, rowsL))
   int rowsR = 0, rowsL = 1;
   // the rows of a growing chunk's inverse are rebuilt from the first step after a
@@ -497,6 +501,13 @@ int hkbe_create(const hkbe_params* p, const int32_t* nt_per_inst, void* stream, 
   h->scratch.insert(h->scratch.end(), {d.cinv_ws, h->diagbuf});
   {  // inverses of the retarded heads: rebuilt at every step, in neither snapshots nor files
     const size_t n2 = (size_t)d.no * d.no;
+    cudaError_t e = cudaHostAlloc((void**)&h->res, sizeof(hk::IterResult) * kAhead * d.n_inst, cudaHostAllocMapped);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&h->res_dev, h->res, 0);
+    if (e != cudaSuccess) {
+      g_create_error = std::string("cudaHostAlloc: ") + cudaGetErrorString(e);
+      hkbe_destroy(h);
+      return HKBE_ERR_NOMEM;
+    }
     if ((rc = walloc(h, &d.hinv, (size_t)d.n_inst * 4 * d.k * d.k * n2)) || (h->hodlr && (rc = src_jobs(h)))) {
       g_create_error = h->err;
       hkbe_destroy(h);
@@ -520,6 +531,7 @@ int hkbe_destroy(hkbe_t* h) {
   for (cudaEvent_t e : h->event_pool) cudaEventDestroy(e);
   for (void* p : h->allocs) cudaFree(p);
   for (void* p : h->work) cudaFree(p);
+  if (h->res) cudaFreeHost(h->res);
   for (void* p : h->snap_dev)
     if (p) cudaFree(p);
   delete h;
@@ -901,44 +913,51 @@ static int check_ready(hkbe_t* h) {
 // Run the iteration loop of one bootstrap or one time step; `pass` launches
 // one iteration.  Records per-instance iteration counts and final errors.
 // Instances with act0[n] == 0 (past their last step) take no part.
+//
+// After each iteration k_set_active writes every instance's error and flag
+// into pinned host memory and clears the flag of a converged instance, whose
+// kernels then do nothing.  So the host need not see the outcome of one
+// iteration before it launches the next: as many iterations as the step before
+// took (at most kAhead) go out at once, and the host waits for the last of them;
+// a step that needs more adds them one by one.  Waiting after every iteration
+// left the device idle for about 25 us each (two copies, two synchronisations
+// and the launches after them).
 template <typename F>
 static int iterate(hkbe_t* h, int max_iter, double tol, F pass, int32_t* iters, double* errs, bool* any_failed,
-                   const std::vector<int>* act0 = nullptr) {
+                   const std::vector<int>& act0, int* ahead) {
   Dev& d = h->d;
   const int N = d.n_inst;
-  std::vector<int> act(N, 1), it_of(N, 0);
-  if (act0) act = *act0;
-  std::vector<double> err(N, 0.0);
-  HK_CUDA(h, cudaMemcpyAsync(d.active, act.data(), N * sizeof(int), cudaMemcpyHostToDevice, h->s));
+  std::vector<int> act = act0, it_of(N, 0);
   const double tol_eff = h->self_consistent ? tol : INFINITY;
   const int min_iter = h->self_consistent ? 1 : 2;
-  int it = 0;
-  for (it = 1; it <= max_iter; ++it) {
-    HK_CUDA(h, cudaMemsetAsync(d.err, 0, N * sizeof(double), h->s));
-    HK_CUDA(h, cudaMemsetAsync(h->any_dev, 0, sizeof(int), h->s));
-    HK_CUDA(h, pass());
-    HK_CUDA(h, run_phase(h, HKBE_PHASE_CTRL, 1,
-                         [&]() { return hk::launch_set_active(d, tol_eff, it, min_iter, h->any_dev, h->s); }));
-    int any = 0;
-    HK_CUDA(h, cudaMemcpyAsync(err.data(), d.err, N * sizeof(double), cudaMemcpyDeviceToHost, h->s));
-    HK_CUDA(h, cudaMemcpyAsync(&any, h->any_dev, sizeof(int), cudaMemcpyDeviceToHost, h->s));
-    HK_CUDA(h, cudaStreamSynchronize(h->s));
-    for (int n = 0; n < N; ++n)
-      if (act[n]) {
-        it_of[n] = it;
-        if (errs) errs[n] = err[n];
-        if (!std::isfinite(err[n])) return fail(h, HKBE_ERR_NAN, "non-finite value during the self-consistency loop");
-      }
-    HK_CUDA(h, cudaMemcpyAsync(act.data(), d.active, N * sizeof(int), cudaMemcpyDeviceToHost, h->s));
+  const int coupled = d.model == HKBE_MODEL_LATTICE2B;   // k-points are coupled through Sigma: iterate all or none
+  int done = 0;
+  bool any = true;
+  while (any && done < max_iter) {
+    const int batch = done == 0 ? std::min({std::max(*ahead, 1), kAhead, max_iter}) : 1;
+    for (int i = 0; i < batch; ++i) {
+      HK_CUDA(h, pass());
+      HK_CUDA(h, run_phase(h, HKBE_PHASE_CTRL, 1, [&]() {
+        return hk::launch_set_active(d, tol_eff, done + i + 1, min_iter, coupled, h->res_dev + (size_t)i * N, h->s);
+      }));
+    }
     HK_CUDA(h, cudaStreamSynchronize(h->s));
     drain(h);
-    if (!any) break;
-    if (d.model == HKBE_MODEL_LATTICE2B) {  // k-points are coupled through Sigma: iterate all or none
-      if (act0) act = *act0;
-      else std::fill(act.begin(), act.end(), 1);
-      HK_CUDA(h, cudaMemcpyAsync(d.active, act.data(), N * sizeof(int), cudaMemcpyHostToDevice, h->s));
+    for (int i = 0; i < batch && any; ++i) {
+      const hk::IterResult* res = h->res + (size_t)i * N;
+      ++done;
+      any = false;
+      for (int n = 0; n < N; ++n) {
+        if (!act[n]) continue;
+        it_of[n] = done;
+        if (errs) errs[n] = res[n].err;
+        if (!std::isfinite(res[n].err)) return fail(h, HKBE_ERR_NAN, "non-finite value during the self-consistency loop");
+        act[n] = res[n].active;
+        any |= act[n] != 0;
+      }
     }
   }
+  *ahead = done;
   *any_failed = false;
   for (int n = 0; n < N; ++n) {
     if (iters) iters[n] = it_of[n];
@@ -1006,9 +1025,13 @@ int hkbe_bootstrap(hkbe_t* h, int max_iter, double tol, int32_t* iters, double* 
   if ((rc = hf_guess(h))) return rc;
   Dev& d = h->d;
   bool failed = false;
+  const std::vector<int> all(d.n_inst, 1);
+  HK_CUDA(h, cudaMemcpyAsync(d.active, all.data(), d.n_inst * sizeof(int), cudaMemcpyHostToDevice, h->s));
+  HK_CUDA(h, cudaMemsetAsync(d.err, 0, d.n_inst * sizeof(double), h->s));
+  int ahead = 1;
   rc = iterate(h, max_iter, tol,
                [&]() { return run_phase(h, HKBE_PHASE_BOOT, d.k + 4, [&]() { return hk::launch_boot(d, h->s); }); },
-               iters, err, &failed);
+               iters, err, &failed, all, &ahead);
   if (rc) return rc;
   if ((rc = finish_start(h))) return rc;
   if (failed) return fail(h, HKBE_ERR_NOCONV, "bootstrap did not converge");
@@ -1091,7 +1114,7 @@ int hkbe_step(hkbe_t* h, int n_steps, int32_t* iters, double* err) {
                      return e;
                    return cudaSuccess;
                  },
-                 iters ? iters + (size_t)st * N : nullptr, err ? err + (size_t)st * N : nullptr, &failed, &act0);
+                 iters ? iters + (size_t)st * N : nullptr, err ? err + (size_t)st * N : nullptr, &failed, act0, &h->ahead);
     if (rc) return rc;
     any_failed |= failed;
     h->cur = T;

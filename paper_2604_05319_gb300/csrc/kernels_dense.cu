@@ -229,6 +229,10 @@ __global__ void k_extrap(Dev d, int T) {
   const int n = blockIdx.y;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   const int k = d.k;
+  if (idx == 0) {   // the instances of this step, for its first iteration
+    d.active[n] = T <= d.last[n];
+    d.err[n] = 0.0;
+  }
   if (idx >= 2 * (T + 1) + d.r || T > d.last[n]) return;
   double e[6];
   {
@@ -985,14 +989,22 @@ __global__ void k_boot_les(Dev d) {
   if (lane == 0) atomic_max_nonneg(d.err + n, e);
 }
 
-// Per-instance convergence bookkeeping after an iteration.
-__global__ void k_set_active(Dev d, double tol, int iter, int min_iter, int* any) {
+// Per-instance convergence bookkeeping after an iteration: error and flag out
+// to the host, the error cleared for the next iteration.  Coupled instances (at
+// most one CTA of them) go on until all have converged.
+__global__ void k_set_active(Dev d, double tol, int iter, int min_iter, int coupled, IterResult* out) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= d.n_inst) return;
-  if (!d.active[n]) return;
-  const double e = d.err[n];
-  if ((e < tol && iter >= min_iter) || !(e == e)) d.active[n] = 0;
-  else atomicOr(any, 1);
+  const bool in = n < d.n_inst;
+  int a = in ? d.active[n] : 0;
+  const double e = in ? d.err[n] : 0.0;
+  const int on = a && !((e < tol && iter >= min_iter) || !(e == e));
+  const int any = coupled ? __syncthreads_or(on) : on;
+  if (!in) return;
+  a = a && any;
+  d.active[n] = a;
+  d.err[n] = 0.0;
+  out[n].err = e;
+  out[n].active = a;
 }
 
 // ---------------------------------------------------------------------------
@@ -1066,8 +1078,11 @@ cudaError_t launch_boot(const Dev& d, cudaStream_t s) {
   HK_DISPATCH(d.no, (k_boot_les<NO, S><<<d.n_inst, 32, 0, s>>>(d)));
   return cudaGetLastError();
 }
-cudaError_t launch_set_active(const Dev& d, double tol, int iter, int min_iter, int* any, cudaStream_t s) {
-  k_set_active<<<(d.n_inst + 127) / 128, 128, 0, s>>>(d, tol, iter, min_iter, any);
+cudaError_t launch_set_active(const Dev& d, double tol, int iter, int min_iter, int coupled, IterResult* out,
+                              cudaStream_t s) {
+  if (coupled && d.n_inst > 256) return cudaErrorInvalidValue;
+  const int nt = coupled ? 256 : 128;
+  k_set_active<<<(d.n_inst + nt - 1) / nt, nt, 0, s>>>(d, tol, iter, min_iter, coupled, out);
   return cudaGetLastError();
 }
 

@@ -1144,6 +1144,7 @@ template <typename S>
 __global__ void __launch_bounds__(128) k_sigma_lattice(Dev d, int T) {
   extern __shared__ __align__(16) zd grid[];   // [2][kLatT] grids of L rows of L + 1
   __shared__ zd tw[16];
+  if (!d.active[0]) return;   // (the k-points iterate together)
   const int L = (int)d.mpar[0], ys = (int)d.mpar[1], N = L * L, gsz = L * (L + 1);
   const int ntb = (T + kLatT) / kLatT, tid = threadIdx.x;
   lat_twiddles(tw, L);

@@ -111,7 +111,12 @@ cudaError_t launch_les(const Dev& d, int T, cudaStream_t s);
 cudaError_t launch_rho(const Dev& d, int T, cudaStream_t s);
 cudaError_t launch_boot(const Dev& d, cudaStream_t s);   // one bootstrap pass (Sigma + R/mixed/lesser)
 cudaError_t launch_diag_seed(const Dev& d, cudaStream_t s);  // diag64[t] = G^<(t,t), t <= k
-cudaError_t launch_set_active(const Dev& d, double tol, int iter, int min_iter, int* any_active_dev, cudaStream_t s);
+// outcome of an iteration for one instance: its error, and whether it goes on
+struct IterResult {
+  double err;
+  int active, pad;
+};
+cudaError_t launch_set_active(const Dev& d, double tol, int iter, int min_iter, int coupled, IterResult* out, cudaStream_t s);
 // compressed (HODLR) form
 cudaError_t launch_ret_h(const Dev& d, int T, cudaStream_t s);
 cudaError_t launch_les_h(const Dev& d, int T, cudaStream_t s);
