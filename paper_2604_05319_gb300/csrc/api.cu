@@ -508,7 +508,7 @@ int hkbe_create(const hkbe_params* p, const int32_t* nt_per_inst, void* stream, 
       hkbe_destroy(h);
       return HKBE_ERR_NOMEM;
     }
-    if ((rc = walloc(h, &d.hinv, (size_t)d.n_inst * 4 * d.k * d.k * n2)) || (h->hodlr && (rc = src_jobs(h)))) {
+    if ((rc = walloc(h, &d.nbose, d.n_inst)) || (rc = walloc(h, &d.hinv, (size_t)d.n_inst * 4 * d.k * d.k * n2)) || (h->hodlr && (rc = src_jobs(h)))) {
       g_create_error = h->err;
       hkbe_destroy(h);
       return rc;
@@ -804,6 +804,7 @@ int hkbe_set_model(hkbe_t* h, int model, const double* params, int nparams) {
   }
   d.model = model;
   HK_CUDA(h, cudaMemcpyAsync(d.mpar, mp.data(), mp.size() * sizeof(double), cudaMemcpyHostToDevice, h->s));
+  HK_CUDA(h, hk::launch_nbose(d, h->s));
   HK_CUDA(h, cudaStreamSynchronize(h->s));
   h->have_model = true;
   return HKBE_OK;
@@ -1633,6 +1634,11 @@ int hkbe_load(const char* path, void* stream, hkbe_t** out) {
   d.nfrozR = sc.nfrozR;
   d.nfrozL = sc.nfrozL;
   h->restart_rows();
+  if (hk::launch_nbose(d, h->s) != cudaSuccess || cudaStreamSynchronize(h->s) != cudaSuccess) {
+    hkbe_destroy(h);
+    g_create_error = "cannot start a kernel";
+    return HKBE_ERR_CUDA;
+  }
   *out = h;
   return HKBE_OK;
 }

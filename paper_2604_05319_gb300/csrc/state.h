@@ -78,6 +78,7 @@ struct Dev {
   double *tau, *e0, *ebeta, *rev, *q;  // [r], [r], [r], [r*r], [r*r]
   double *qrev;                // [r*r] Q Rev (null: the allocation-free entry point)
   double *mpar;                // [n][MP]
+  double *nbose;               // [n] phonon occupation n_B(w0) at beta (from mpar)
   double2 *qsrc;               // [n][nt][no2]   lesser source q(t) (complex64 form: float-float pairs)
   double2 *vvec;               // [n][r][no2]    v_a = sum_b Q_ab G^vt(tau_b, T)
   double2 *x0;                 // [n][no2]       -[G^tv(T,0)]^dagger
@@ -110,6 +111,7 @@ cudaError_t launch_src(const Dev& d, int T, cudaStream_t s);
 cudaError_t launch_les(const Dev& d, int T, cudaStream_t s);
 cudaError_t launch_rho(const Dev& d, int T, cudaStream_t s);
 cudaError_t launch_boot(const Dev& d, cudaStream_t s);   // one bootstrap pass (Sigma + R/mixed/lesser)
+cudaError_t launch_nbose(const Dev& d, cudaStream_t s);   // nbose from mpar
 cudaError_t launch_diag_seed(const Dev& d, cudaStream_t s);  // diag64[t] = G^<(t,t), t <= k
 // outcome of an iteration for one instance: its error, and whether it goes on
 struct IterResult {
