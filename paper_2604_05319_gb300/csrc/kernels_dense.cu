@@ -345,12 +345,12 @@ __global__ void __launch_bounds__(256) k_mixed(Dev d, int T) {
       for (int u = u0; u < u0 + 4; ++u) {
         const int l = l0 + NS * u;
         if (l < T) {
-          const R wl = (R)h * rule_wr<R>(W, T, l);
           cx<R> gv;
           if constexpr (MX) gv = zf(f32_of(g[u].x), f32_of(g[u].y));
           else gv = zd(g[u].x, g[u].y);
+          if (l <= k || T - l <= k || T < 2 * k + 1) gv = gv * rule_wr<R>(W, T, l);
 #pragma unroll
-          for (int x = 0; x < NO; ++x) pa[x] = cfma(ldr<R>(Sr + (long long)l * NO2 + x * NO) * wl, gv, pa[x]);
+          for (int x = 0; x < NO; ++x) pa[x] = cfma(ldr<R>(Sr + (long long)l * NO2 + x * NO), gv, pa[x]);
         }
       }
 #pragma unroll
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(256) k_mixed(Dev d, int T) {
   }
   zd acc[NO];
 #pragma unroll
-  for (int x = 0; x < NO; ++x) acc[x] = ka[x].get();
+  for (int x = 0; x < NO; ++x) acc[x] = ka[x].get() * h;
   const double2* C = d.wconv + ((long long)n * d.r * d.r + i0) * NO2 + (act ? el_ : 0);
   const double2* St = tv<NO>(d.STV, d, n, T, 0) + z;
 #pragma unroll 4
@@ -516,15 +516,26 @@ __global__ void k_src(Dev d, int T) {
 #pragma unroll
   for (int q = 0; q < NO2; ++q) acc[q] = zd();
   for (int l = lane; l <= T; l += 32) {
-    const double wl = h * rule_w(d.w, T, l);
-    M<NO> Sm;
+    const S* gp = el<NO, S>(d.GR, d, n, T, l);
+    const bool end = l <= d.k || T - l <= d.k || T < 2 * d.k + 1;   // (weight 1 elsewhere)
+    const double wl = end ? rule_w(d.w, T, l) : 1.0;
+    zd GA[NO2];   // G^A(l, T) times the weight
+#pragma unroll
+    for (int q = 0; q < NO2; ++q) {
+      GA[q] = ld(gp + (q % NO) * NO + q / NO).conj();
+      if (end) GA[q] = GA[q] * wl;
+    }
 #pragma unroll
     for (int x = 0; x < NO; ++x)
 #pragma unroll
-      for (int y = 0; y < NO; ++y) Sm.a[x][y] = sless<NO, S>(d, n, t, l, x, y);
-    M<NO> GA = dag<NO>(load<NO>(el<NO, S>(d.GR, d, n, T, l)));
-    mac<NO>(*reinterpret_cast<M<NO>*>(acc), Sm, GA, zd(wl));
+      for (int z = 0; z < NO; ++z) {
+        const zd sxz = sless<NO, S>(d, n, t, l, x, z);
+#pragma unroll
+        for (int y = 0; y < NO; ++y) acc[x * NO + y] = cfma(sxz, GA[z * NO + y], acc[x * NO + y]);
+      }
   }
+#pragma unroll
+  for (int q = 0; q < NO2; ++q) acc[q] = acc[q] * h;
   for (int a = lane; a < d.r; a += 32) {
     M<NO> Sm = load<NO>(tv<NO>(d.STV, d, n, t, a));
     M<NO> V = load<NO>(d.vvec + ((long long)n * d.r + a) * NO2);
@@ -708,11 +719,22 @@ __global__ void __launch_bounds__(256) k_rho(Dev d, int T) {
 #pragma unroll
   for (int q = 0; q < NO2; ++q) acc[q] = zd();
   for (int l = tid; l < T; l += blockDim.x) {
-    const double wl = h * rule_w(d.w, T, l);
     M<NO> Sm = load<NO>(el<NO, S>(d.SR, d, n, T, l));
     M<NO> X = load<NO>(el<NO, S>(d.GL, d, n, T, l));
-    mac<NO>(*reinterpret_cast<M<NO>*>(acc), Sm, X, zd(wl));
+    if (l <= d.k || T - l <= d.k || T < 2 * d.k + 1) {   // (weight 1 elsewhere)
+      const double wl = rule_w(d.w, T, l);
+#pragma unroll
+      for (int q = 0; q < NO2; ++q) X.a[q / NO][q % NO] = X.a[q / NO][q % NO] * wl;
+    }
+#pragma unroll
+    for (int x = 0; x < NO; ++x)
+#pragma unroll
+      for (int z = 0; z < NO; ++z)
+#pragma unroll
+        for (int y = 0; y < NO; ++y) acc[x * NO + y] = cfma(Sm.a[x][z], X.a[z][y], acc[x * NO + y]);
   }
+#pragma unroll
+  for (int q = 0; q < NO2; ++q) acc[q] = acc[q] * h;
   if (tid < NO2)
     A[tid] = ld(epsp<NO>(d, n, T) + tid) + ld(el<NO, S>(d.SR, d, n, T, T) + tid) * (h * rule_w(d.w, T, T));
   warp_sum<NO2>(acc);

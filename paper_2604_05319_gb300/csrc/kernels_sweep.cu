@@ -586,12 +586,14 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
             for (int jj = 0; jj < FOLD; ++jj) {
               const int s2 = s0 + 8 * jj;
               if (s2 <= T) {
-                const R ws = rule_wr<R>(W, T - tp, T - s2);
+                const bool end = T - s2 <= k || s2 - tp <= k;   // (weight 1 elsewhere: no product)
+                const R ws = end ? rule_wr<R>(W, T - tp, T - s2) : (R)1;
                 const S* yl = sp(s2);
                 const S* sr = el<NO, S>(d.SR, d, n, s2, tp);
 #pragma unroll
                 for (int m = 0; m < NO; ++m) {
-                  const cx<R> ym = ldr<R>(yl + m) * ws;
+                  cx<R> ym = ldr<R>(yl + m);
+                  if (end) ym = ym * ws;
 #pragma unroll
                   for (int j = 0; j < NO; ++j) pa[j] = cfma(ym, ldr<R>(sr + m * NO + j), pa[j]);
                 }
@@ -903,11 +905,13 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
             for (int jj = 0; jj < FOLD; ++jj) {
               const int l = lb + 8 * jj;
               if (l < a) {
-                const R wl = rule_wr<R>(W, t, l);
+                const bool end = l <= k || t - l <= k || t < 2 * k + 1;
+                const R wl = end ? rule_wr<R>(W, t, l) : (R)1;
                 const S* sr = srow + (long long)l * NO2;
 #pragma unroll
                 for (int y = 0; y < NO; ++y) {
-                  const cx<R> xy = ldr<R>(sp(l) + y * NO + jc) * wl;
+                  cx<R> xy = ldr<R>(sp(l) + y * NO + jc);
+                  if (end) xy = xy * wl;
 #pragma unroll
                   for (int m = 0; m < NO; ++m) pa[m] = cfma(ldr<R>(sr + m * NO + y), xy, pa[m]);
                 }
