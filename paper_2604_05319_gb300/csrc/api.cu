@@ -1099,7 +1099,8 @@ int hkbe_step(hkbe_t* h, int n_steps, int32_t* iters, double* err) {
                           return h->scheme ? hk::launch_ret_sf(d, T, h->s) : hk::launch_ret_h(d, T, h->s);
                         })))
                      return e;
-                   if ((e = run_phase(h, HKBE_PHASE_MIXED, 1, [&]() { return hk::launch_mixed(d, T, h->s); })))
+                   if ((h->scheme || !hk::ret_takes_mixed(d)) &&
+                       (e = run_phase(h, HKBE_PHASE_MIXED, 1, [&]() { return hk::launch_mixed(d, T, h->s); })))
                      return e;
                    if ((e = run_phase(h, HKBE_PHASE_VT, 1, [&]() { return hk::launch_vt(d, T, h->s); }))) return e;
                    if ((e = run_phase(h, HKBE_PHASE_SRC, (h->hodlr && d.cdir > 0) ? 2 : 1, [&]() {

@@ -20,6 +20,7 @@
 //   k_rho    diagonal density-matrix update (Sec. 3.3), when selected
 // Each kernel folds max |new - old| of what it writes into err[instance].
 #include "dev_util.cuh"
+#include "mixed_nodes.cuh"
 
 namespace hk {
 
@@ -180,6 +181,7 @@ __device__ void nambu_sigma(const Dev& d, int n, int T, int idx, double nb) {
 
 template <int NO, typename S>
 __global__ void k_sigma(Dev d, int T) {
+  pdl_start();
   constexpr int NO2 = NO * NO;
   const int n = blockIdx.y;
   if (!d.active[n]) return;
@@ -238,6 +240,7 @@ __global__ void k_sigma(Dev d, int T) {
 // ---------------------------------------------------------------------------
 template <int NO, typename S>
 __global__ void k_extrap(Dev d, int T) {
+  pdl_start();
   constexpr int NO2 = NO * NO;
   const int n = blockIdx.y;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -285,138 +288,10 @@ __global__ void k_extrap(Dev d, int T) {
 constexpr int CH = 32;     // chunk of the sequential sweeps
 constexpr int NWARP = 8;   // warps per sweep CTA
 
-// ---------------------------------------------------------------------------
-// Mixed component at step T, Eq. KBET.  One CTA per instance and group of NI
-// nodes: a lane owns element (i, z, y) of the group's rows of G^tv (adjacent
-// elements, 16-byte loads) and all N_o products with column z of Sigma^R; the
-// warps, and the lanes left over by a small group, split the history l and the
-// convolution sum a.  Groups fill a warp (32 elements) where that gives a CTA to
-// every SM (256 lattice points: 38 us an iteration, 76 us with small groups);
-// with fewer, groups of 64 bytes or one node spread the FP64 products over more
-// SMs (3 instances, FP64, N_o = 1, T = 256: 19 us with groups of 32, 16 with 4).  (One
-// warp per node over all l read 16 bytes of every row and node apart, and its
-// lane 0 solved an N_o x N_o system per node: 158 us for 128 instances at
-// N_o = 2, T = 600; 110 us for 16 at N_o = 4, T = 290.)
-// ---------------------------------------------------------------------------
-template <int NO> constexpr int kNodes = 32 / (NO * NO);                      // nodes per CTA
-template <int NO> constexpr int kNodesFew = NO == 1 ? 4 : NO == 2 ? 2 : 1;    // with few instances
 template <int NO, typename S, int NI>
 __global__ void __launch_bounds__(256) k_mixed(Dev d, int T) {
-  constexpr int NO2 = NO * NO, E = NI * NO2, LS = 32 / E, NS = 8 * LS;   // elements, slices per warp and CTA
-  constexpr bool kLanes = LS > 1 && E * LS == 32;   // a warp's slices are combined by shuffles
-  constexpr int NR = kLanes ? 8 : NS;               // partial sums per element
-  constexpr bool MX = sizeof(S) == sizeof(float2);
-  using R = typename Bulk<S>::R;
-  const int n = blockIdx.y, i0 = blockIdx.x * NI;
-  if (!d.active[n]) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int k = d.k, ni = min(NI, d.r - i0);
-  const double h = d.h;
-  const DevW& W = d.w;
-  __shared__ zd red[NR][NO][E];
-  __shared__ zd Mi[NO2];       // inverse of the point's matrix
-  __shared__ double serr[8];
-  if (tid < NO2) {
-    const int x = tid / NO, y = tid % NO;
-    Mi[tid] = (x == y ? zd(0, W.a[0] / h) : zd()) - ld(epsp<NO>(d, n, T) + tid) -
-              ld(el<NO, S>(d.SR, d, n, T, T) + tid) * (h * rule_w(W, T, T));
-  }
-  const int el_ = lane % E, slice = warp * LS + lane / E;
-  const bool act = lane < LS * E && el_ < ni * NO2;
-  const int z = (el_ % NO2) / NO;
-  const double2* G = tv<NO>(d.GTV, d, n, 0, i0) + (act ? el_ : 0);
-  const long long gs = (long long)d.r * NO2;   // from row l to row l + 1
-  const S* Sr = el<NO, S>(d.SR, d, n, T, 0) + z;
-  constexpr int UB = 8;        // rows in flight
-  KAcc<R> ka[NO];              // h sum_l w_l Sigma^R(T,l) G^tv(l, tau_i): FP32 products, compensated, in the complex64 form
-  for (int l0 = slice; l0 < T; l0 += NS * UB) {
-    double2 g[UB];
-#pragma unroll
-    for (int u = 0; u < UB; ++u) {
-      const int l = l0 + NS * u;
-      g[u] = l < T ? G[l * gs] : make_double2(0, 0);
-    }
-#pragma unroll
-    for (int u0 = 0; u0 < UB; u0 += 4) {
-      cx<R> pa[NO];
-#pragma unroll
-      for (int x = 0; x < NO; ++x) pa[x] = cx<R>(0);
-#pragma unroll
-      for (int u = u0; u < u0 + 4; ++u) {
-        const int l = l0 + NS * u;
-        if (l < T) {
-          cx<R> gv;
-          if constexpr (MX) gv = zf(f32_of(g[u].x), f32_of(g[u].y));
-          else gv = zd(g[u].x, g[u].y);
-          if (l <= k || T - l <= k || T < 2 * k + 1) gv = gv * rule_wr<R>(W, T, l);
-#pragma unroll
-          for (int x = 0; x < NO; ++x) pa[x] = cfma(ldr<R>(Sr + (long long)l * NO2 + x * NO), gv, pa[x]);
-        }
-      }
-#pragma unroll
-      for (int x = 0; x < NO; ++x) ka[x].add(pa[x]);
-    }
-  }
-  zd acc[NO];
-#pragma unroll
-  for (int x = 0; x < NO; ++x) acc[x] = ka[x].get() * h;
-  const double2* C = d.wconv + ((long long)n * d.r * d.r + i0) * NO2 + (act ? el_ : 0);
-  const double2* St = tv<NO>(d.STV, d, n, T, 0) + z;
-#pragma unroll 4
-  for (int a = slice; a < d.r; a += NS) {   // sum_a Sigma^tv(T, tau_a) W[a][i]
-    const zd c = ld(C + (long long)a * gs);
-#pragma unroll
-    for (int x = 0; x < NO; ++x) acc[x] = cfma(ld(St + (long long)a * NO2 + x * NO), c, acc[x]);
-  }
-#pragma unroll
-  for (int x = 0; x < NO; ++x) {
-    if constexpr (kLanes) {
-#pragma unroll
-      for (int off = 16; off >= E; off >>= 1) acc[x] += wshfl(acc[x], off);
-      if (lane < E) red[warp][x][el_] = acc[x];
-    } else {
-      if (lane < LS * E) red[slice][x][el_] = acc[x];
-    }
-  }
-  __syncthreads();
-  if constexpr (NO == 1) {
-    if (tid == 0) Mi[0] = cdiv(zd(1.0), Mi[0]);
-    __syncthreads();
-  } else {
-    gj_inverse(NO, Mi, NO);
-  }
-  zd rhs = zd();
-  double e = 0.0;
-  const int i = tid / NO2, x = (tid % NO2) / NO, y = tid % NO;
-  if (tid < ni * NO2) {
-    for (int w2 = 0; w2 < NR; ++w2)
-#pragma unroll
-      for (int zz = 0; zz < NO; ++zz) rhs += red[w2][x][i * NO2 + zz * NO + y];
-    const double2* gp = tv<NO>(d.GTV, d, n, T, i0) + tid;
-    for (int j = 1; j <= k; ++j) {
-      const zd g = ld(gp - j * gs);
-      rhs += zd(W.ah[j] * g.im, -W.ah[j] * g.re);
-    }
-  }
-  __syncthreads();
-  zd* rs = &red[0][0][0];
-  if (tid < ni * NO2) rs[tid] = rhs;
-  __syncthreads();
-  if (tid < ni * NO2) {
-    zd v = zd();
-#pragma unroll
-    for (int m = 0; m < NO; ++m) v = cfma(Mi[x * NO + m], rs[i * NO2 + m * NO + y], v);
-    double2* p = tv<NO>(d.GTV, d, n, T, i0) + tid;
-    e = sqrt((v - ld(p)).abs2());
-    st(p, v);
-  }
-  e = warp_max(e);
-  if (lane == 0) serr[warp] = e;
-  __syncthreads();
-  if (tid == 0) {
-    for (int w2 = 1; w2 < 8; ++w2) e = fmax(e, serr[w2]);
-    atomic_max_nonneg(d.err + n, e);
-  }
+  pdl_start();
+  mixed_nodes<NO, S, NI>(d, T, blockIdx.x, blockIdx.y);
 }
 
 // v_a = sum_b Q_ab G^vt(tau_b, T), G^vt(tau_b, T) = -xi [G^tv(T, beta - tau_b)]^dagger,
@@ -426,6 +301,7 @@ __global__ void __launch_bounds__(256) k_mixed(Dev d, int T) {
 // after the other, a row per thread, took 15 us (N_o = 1) to 126 us (N_o = 4).
 template <int NO, typename S>
 __global__ void __launch_bounds__(256) k_vt_qr(Dev d, int T) {
+  pdl_start();
   constexpr int NO2 = NO * NO;
   const int n = blockIdx.y;
   if (!d.active[n]) return;
@@ -506,6 +382,7 @@ __global__ void k_vt(Dev d, int T) {
 // Lesser source q(t) = h sum_l w^(T)_l Sigma^<(t,l) G^A(l,T) - i sum_a Sigma^tv(t,tau_a) v_a
 template <int NO, typename S>
 __global__ void k_src(Dev d, int T) {
+  pdl_start();
   constexpr int NO2 = NO * NO;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -708,6 +585,7 @@ __global__ void __launch_bounds__(256) k_les(Dev d, int T) {
 // ---------------------------------------------------------------------------
 template <int NO, typename S>
 __global__ void __launch_bounds__(256) k_rho(Dev d, int T) {
+  pdl_start();
   constexpr int NO2 = NO * NO;
   const int n = blockIdx.x;
   if (!d.active[n]) return;
@@ -1028,6 +906,7 @@ __global__ void k_boot_les(Dev d) {
 // to the host, the error cleared for the next iteration.  Coupled instances (at
 // most one CTA of them) go on until all have converged.
 __global__ void k_set_active(Dev d, double tol, int iter, int min_iter, int coupled, IterResult* out) {
+  pdl_start();
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   const bool in = n < d.n_inst;
   int a = in ? d.active[n] : 0;
@@ -1060,34 +939,33 @@ __global__ void k_set_active(Dev d, double tol, int iter, int min_iter, int coup
 
 cudaError_t launch_extrapolate(const Dev& d, int T, cudaStream_t s) {
   dim3 g((2 * (T + 1) + d.r + 127) / 128, d.n_inst);
-  HK_DISPATCH(d.no, (k_extrap<NO, S><<<g, 128, 0, s>>>(d, T)));
-  return cudaGetLastError();
+  HK_DISPATCH(d.no, return launch_k(k_extrap<NO, S>, g, 128, 0, s, d, T));
+  return cudaSuccess;
 }
 cudaError_t launch_sigma(const Dev& d, int T, cudaStream_t s) {
   if (d.model == 4) return launch_sigma_lattice(d, T, s);
   dim3 g(((d.model == 3 ? (T + 128) / 128 * 128 : 2 * (T + 1)) + d.r + 127) / 128, d.n_inst);
-  HK_DISPATCH(d.no, (k_sigma<NO, S><<<g, 128, 0, s>>>(d, T)));
-  return cudaGetLastError();
+  HK_DISPATCH(d.no, return launch_k(k_sigma<NO, S>, g, 128, 0, s, d, T));
+  return cudaSuccess;
 }
 cudaError_t launch_mixed(const Dev& d, int T, cudaStream_t s) {
   HK_DISPATCH(d.no, {
     constexpr int N1 = kNodes<NO>, N2 = kNodesFew<NO>;
     if ((d.r + N1 - 1) / N1 * d.n_inst >= 152)
-      k_mixed<NO, S, N1><<<dim3((d.r + N1 - 1) / N1, d.n_inst), 256, 0, s>>>(d, T);
-    else
-      k_mixed<NO, S, N2><<<dim3((d.r + N2 - 1) / N2, d.n_inst), 256, 0, s>>>(d, T);
+      return launch_k(k_mixed<NO, S, N1>, dim3((d.r + N1 - 1) / N1, d.n_inst), 256, 0, s, d, T);
+    return launch_k(k_mixed<NO, S, N2>, dim3((d.r + N2 - 1) / N2, d.n_inst), 256, 0, s, d, T);
   })
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 cudaError_t launch_vt(const Dev& d, int T, cudaStream_t s) {
-  if (d.qrev) HK_DISPATCH(d.no, (k_vt_qr<NO, S><<<dim3((d.r + 16) / 16, d.n_inst), 256, 0, s>>>(d, T)))
+  if (d.qrev) HK_DISPATCH(d.no, return launch_k(k_vt_qr<NO, S>, dim3((d.r + 16) / 16, d.n_inst), 256, 0, s, d, T))
   else HK_DISPATCH(d.no, (k_vt<NO, S><<<d.n_inst, 128, d.r * NO * NO * sizeof(zd), s>>>(d, T)))
   return cudaGetLastError();
 }
 cudaError_t launch_src(const Dev& d, int T, cudaStream_t s) {
   const long long warps = (long long)d.n_inst * (T + 1);
-  HK_DISPATCH(d.no, (k_src<NO, S><<<(unsigned)((warps * 32 + 127) / 128), 128, 0, s>>>(d, T)));
-  return cudaGetLastError();
+  HK_DISPATCH(d.no, return launch_k(k_src<NO, S>, dim3((unsigned)((warps * 32 + 127) / 128)), 128, 0, s, d, T));
+  return cudaSuccess;
 }
 cudaError_t launch_les(const Dev& d, int T, cudaStream_t s) {
   dim3 g(d.no, d.n_inst);
@@ -1095,8 +973,8 @@ cudaError_t launch_les(const Dev& d, int T, cudaStream_t s) {
   return cudaGetLastError();
 }
 cudaError_t launch_rho(const Dev& d, int T, cudaStream_t s) {
-  HK_DISPATCH(d.no, (k_rho<NO, S><<<d.n_inst, 256, 0, s>>>(d, T)));
-  return cudaGetLastError();
+  HK_DISPATCH(d.no, return launch_k(k_rho<NO, S>, dim3(d.n_inst), 256, 0, s, d, T));
+  return cudaSuccess;
 }
 // n_B(w0) of each instance's phonon (NAMBU with g != 0; else 0)
 __global__ void k_nbose(Dev d) {
@@ -1128,8 +1006,7 @@ cudaError_t launch_set_active(const Dev& d, double tol, int iter, int min_iter, 
                               cudaStream_t s) {
   if (coupled && d.n_inst > 256) return cudaErrorInvalidValue;
   const int nt = coupled ? 256 : 128;
-  k_set_active<<<(d.n_inst + nt - 1) / nt, nt, 0, s>>>(d, tol, iter, min_iter, coupled, out);
-  return cudaGetLastError();
+  return launch_k(k_set_active, dim3((d.n_inst + nt - 1) / nt), nt, 0, s, d, tol, iter, min_iter, coupled, out);
 }
 
 }  // namespace hk

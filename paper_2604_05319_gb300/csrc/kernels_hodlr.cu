@@ -56,6 +56,7 @@ __device__ __forceinline__ cx<R>* Psrc(const Dev& d, int n, int b, int p, int wh
 // s_tab: (block, side, first row / 256, first slot of the side's partial sums).
 template <int NO, typename S>
 __global__ void __launch_bounds__(256) k_src_proj(Dev d, int T) {
+  pdl_start();
   constexpr int NO2 = NO * NO;
   using R = typename Bulk<S>::R;
   using V = typename Val<S>::t;
@@ -234,6 +235,7 @@ __device__ __forceinline__ cff vmul_mi(const cff& a) { return {a.im, ff_neg(a.re
 constexpr int kEB = 4;
 template <int NO, typename S>
 __global__ void __launch_bounds__(256) k_src_q(Dev d, int T, int uselist) {
+  pdl_start();
   constexpr int NO2 = NO * NO;
   using R = typename Bulk<S>::R;
   using V = typename Val<S>::t;
@@ -1142,6 +1144,7 @@ __global__ void k_density_at(Dev d, int t, double2* out) {
 // ---------------------------------------------------------------------------
 template <typename S>
 __global__ void __launch_bounds__(128) k_sigma_lattice(Dev d, int T) {
+  pdl_start();
   extern __shared__ __align__(16) zd grid[];   // [2][kLatT] grids of L rows of L + 1
   __shared__ zd tw[16];
   if (!d.active[0]) return;   // (the k-points iterate together)
@@ -1285,12 +1288,15 @@ static cudaError_t src_q(const Dev& d, int T, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(k_src_q<NO, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
   const int nrow = T + 1 - d.cdir;
-  k_src_q<NO, S><<<dim3(d.cdir / 32 + (nrow + 7) / 8, d.n_inst), 256, bytes, s>>>(d, T, uselist);
-  return cudaGetLastError();
+  return launch_k(k_src_q<NO, S>, dim3(d.cdir / 32 + (nrow + 7) / 8, d.n_inst), 256, bytes, s, d, T, uselist);
 }
 cudaError_t launch_src_h(const Dev& d, int T, int njob, cudaStream_t s) {
   if (d.cdir > 0 && T + 1 - d.cdir > kSrcRing) return cudaErrorInvalidValue;
-  if (njob > 0) HK_DISPATCH(d.no, (k_src_proj<NO, S><<<dim3(njob, d.n_inst), 256, 0, s>>>(d, T)));
+  if (njob > 0) {
+    cudaError_t e = cudaErrorInvalidValue;
+    HK_DISPATCH(d.no, e = launch_k(k_src_proj<NO, S>, dim3(njob, d.n_inst), 256, 0, s, d, T));
+    if (e != cudaSuccess) return e;
+  }
   HK_DISPATCH(d.no, return (src_q<NO, S>(d, T, s)));
   return cudaSuccess;
 }
@@ -1318,9 +1324,8 @@ cudaError_t launch_sigma_lattice(const Dev& d, int T, cudaStream_t s) {
   if (d.no != 1 || d.n_inst > kLatMaxK) return cudaErrorInvalidValue;
   const int nb = (T + kLatT) / kLatT + (d.r + kLatT - 1) / kLatT;
   const size_t smem = lat_smem(16);   // 35 KB
-  if (d.prec) k_sigma_lattice<float2><<<nb, 128, smem, s>>>(d, T);
-  else k_sigma_lattice<double2><<<nb, 128, smem, s>>>(d, T);
-  return cudaGetLastError();
+  if (d.prec) return launch_k(k_sigma_lattice<float2>, dim3(nb), 128, smem, s, d, T);
+  return launch_k(k_sigma_lattice<double2>, dim3(nb), 128, smem, s, d, T);
 }
 cudaError_t launch_lattice_obs(const Dev& d, int t, double* out, cudaStream_t s) {
   if (d.no != 1 || d.n_inst > kLatMaxK) return cudaErrorInvalidValue;

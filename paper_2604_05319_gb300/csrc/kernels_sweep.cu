@@ -30,6 +30,7 @@
 
 #include "bulk_copy.cuh"
 #include "hodlr_util.cuh"
+#include "mixed_nodes.cuh"
 
 namespace hk {
 
@@ -309,13 +310,21 @@ __device__ __forceinline__ void leaf_pack(const Dev& d, int A, bool cols, const 
 // complex64, 128 instances, T = 600), 1.34 -> 0.69 ms (one instance, T = 1089),
 // 0.75 -> 0.43 ms (N_o = 2, FP64, 16 instances, T = 300).
 // ---------------------------------------------------------------------------
-template <int NO, typename S>
+// MIX: the CTAs after the first N_o of an instance compute its mixed component.
+template <int NO, typename S, bool MIX>
 __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, int staged) {
+  pdl_start();
   constexpr int NO2 = NO * NO;
   constexpr bool MX = Row64<NO, S>::separate;
   using R = typename Bulk<S>::R;
   using V = typename Val<S>::t;
   const int n = blockIdx.y, irow = blockIdx.x;
+  if constexpr (MIX) {
+    if (irow >= NO) {
+      mixed_nodes<NO, S, kNodesFew<NO>>(d, T, irow - NO, n);
+      return;
+    }
+  }
   if (!d.active[n]) return;
   const int tid = threadIdx.x, lane = tid & 31;
   const int k = d.k, c = d.cdir, L = d.L;
@@ -696,6 +705,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
 // ---------------------------------------------------------------------------
 template <int NO, typename S>
 __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, int staged) {
+  pdl_start();
   constexpr int NO2 = NO * NO;
   constexpr bool MX = Row64<NO, S>::separate;
   using R = typename Bulk<S>::R;
@@ -1132,6 +1142,7 @@ __device__ void append_row(int s, int sb, const zd* crow, const P* Mi, int ld_m,
 
 template <int NO, typename S>
 __global__ void __launch_bounds__(256) k_inv_rows(Dev d, int T, int r0, int r1, int l0, int l1) {
+  pdl_start();
   constexpr int NO2 = NO * NO, LD = CK * NO, NH = 10 * NO;
   const int n = blockIdx.y, sys = blockIdx.x, tid = threadIdx.x;
   if (T > d.last[n]) return;   // the instance has ended
@@ -1217,16 +1228,16 @@ __global__ void __launch_bounds__(256) k_inv_rows(Dev d, int T, int r0, int r1, 
   }
 }
 
-#define HK_DISPATCH(NOV, CALL)                                                  \
+#define HK_DISPATCH(NOV, ...)                                                   \
   switch ((NOV) * 2 + d.prec) {                                                 \
-    case 2: { constexpr int NO = 1; using S = double2; CALL; break; }           \
-    case 3: { constexpr int NO = 1; using S = float2; CALL; break; }            \
-    case 4: { constexpr int NO = 2; using S = double2; CALL; break; }           \
-    case 5: { constexpr int NO = 2; using S = float2; CALL; break; }            \
-    case 6: { constexpr int NO = 3; using S = double2; CALL; break; }           \
-    case 7: { constexpr int NO = 3; using S = float2; CALL; break; }            \
-    case 8: { constexpr int NO = 4; using S = double2; CALL; break; }           \
-    case 9: { constexpr int NO = 4; using S = float2; CALL; break; }            \
+    case 2: { constexpr int NO = 1; using S = double2; __VA_ARGS__; break; }           \
+    case 3: { constexpr int NO = 1; using S = float2; __VA_ARGS__; break; }            \
+    case 4: { constexpr int NO = 2; using S = double2; __VA_ARGS__; break; }           \
+    case 5: { constexpr int NO = 2; using S = float2; __VA_ARGS__; break; }            \
+    case 6: { constexpr int NO = 3; using S = double2; __VA_ARGS__; break; }           \
+    case 7: { constexpr int NO = 3; using S = float2; __VA_ARGS__; break; }            \
+    case 8: { constexpr int NO = 4; using S = double2; __VA_ARGS__; break; }           \
+    case 9: { constexpr int NO = 4; using S = float2; __VA_ARGS__; break; }            \
     default: return cudaErrorInvalidValue;                                      \
   }
 
@@ -1252,15 +1263,25 @@ static size_t sweep_smem(const Dev& d, int* staged) {
   *staged = (d.ring && b <= 200 * 1024 && off32) ? 1 : 0;
   return *staged ? b : kBufBytes<NO>;
 }
+// Where the CTAs of the retarded sweep and of the mixed component's small node
+// groups all fit on the SMs at once (two per SM, one for N_o > 2), they are one
+// launch: the sweep is a chain on a few SMs, and the nodes need the others (3
+// instances, N_o = 1, FP64, T = 256: 106.9 -> 97.7 ms a pass).
+bool ret_takes_mixed(const Dev& d) {
+  const int ni = d.no == 1 ? kNodesFew<1> : d.no == 2 ? kNodesFew<2> : kNodesFew<3>;
+  return (long long)(d.no + (d.r + ni - 1) / ni) * d.n_inst <= (d.no <= 2 ? 2 : 1) * 152;
+}
 template <int NO, typename S>
 static cudaError_t sweep_ret(const Dev& d, int T, cudaStream_t s) {
   int staged = 0;
   const size_t bytes = sweep_smem<NO, S>(d, &staged);
-  cudaError_t e = allow_smem(k_ret2<NO, S>, bytes);
+  const bool with = ret_takes_mixed(d);
+  auto kern = with ? k_ret2<NO, S, true> : k_ret2<NO, S, false>;
+  cudaError_t e = allow_smem(kern, bytes);
   if (e != cudaSuccess) return e;
   if (d.ring && T + 1 - d.cdir > kRingRows && d.cdir > 0) return cudaErrorInvalidValue;
-  k_ret2<NO, S><<<dim3(d.no, d.n_inst), 256, bytes, s>>>(d, T, staged);
-  return cudaGetLastError();
+  const int mix = with ? (d.r + kNodesFew<NO> - 1) / kNodesFew<NO> : 0;
+  return launch_on(false, kern, dim3(NO + mix, d.n_inst), 256, bytes, s, d, T, staged);
 }
 template <int NO, typename S>
 static cudaError_t sweep_les(const Dev& d, int T, cudaStream_t s) {
@@ -1268,8 +1289,7 @@ static cudaError_t sweep_les(const Dev& d, int T, cudaStream_t s) {
   const size_t bytes = sweep_smem<NO, S>(d, &staged);
   cudaError_t e = allow_smem(k_les2<NO, S>, bytes);
   if (e != cudaSuccess) return e;
-  k_les2<NO, S><<<dim3(d.no, d.n_inst), 256, bytes, s>>>(d, T, staged);
-  return cudaGetLastError();
+  return launch_on(false, k_les2<NO, S>, dim3(d.no, d.n_inst), 256, bytes, s, d, T, staged);
 }
 cudaError_t launch_ret_h(const Dev& d, int T, cudaStream_t s) {
   HK_DISPATCH(d.no, return (sweep_ret<NO, S>(d, T, s)));
@@ -1280,8 +1300,8 @@ cudaError_t launch_les_h(const Dev& d, int T, cudaStream_t s) {
   return cudaSuccess;
 }
 cudaError_t launch_inv_rows(const Dev& d, int T, int r0, int r1, int l0, int l1, cudaStream_t s) {
-  HK_DISPATCH(d.no, (k_inv_rows<NO, S><<<dim3(3, d.n_inst), 256, 0, s>>>(d, T, r0, r1, l0, l1)));
-  return cudaGetLastError();
+  HK_DISPATCH(d.no, return launch_k(k_inv_rows<NO, S>, dim3(3, d.n_inst), 256, 0, s, d, T, r0, r1, l0, l1));
+  return cudaSuccess;
 }
 
 }  // namespace hk

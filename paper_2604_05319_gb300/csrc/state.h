@@ -121,6 +121,7 @@ struct IterResult {
 cudaError_t launch_set_active(const Dev& d, double tol, int iter, int min_iter, int coupled, IterResult* out, cudaStream_t s);
 // compressed (HODLR) form
 cudaError_t launch_ret_h(const Dev& d, int T, cudaStream_t s);
+bool ret_takes_mixed(const Dev& d);   // launch_ret_h computes the mixed component as well
 cudaError_t launch_les_h(const Dev& d, int T, cudaStream_t s);
 cudaError_t launch_src_h(const Dev& d, int T, int njob, cudaStream_t s);   // njob: jobs with built rows
 cudaError_t launch_compress(const Dev& d, int A, int nb, cudaStream_t s);
