@@ -245,6 +245,67 @@ __device__ __forceinline__ void lu_apply(int n, const zd* A, const int* piv, zd*
   }
 }
 
+// 1 / a: the real reciprocal from an FP32 estimate by two Newton steps (an FP64
+// division is a sequence of some ten dependent FP64 instructions, each holding
+// the pipe for 64 cycles of the warp).
+__device__ __forceinline__ zd crecip(const zd& a) {
+  const double d = a.abs2();
+  if (!(d > 1e-36 && d < 1e36)) return cdiv(zd(1.0), a);
+  double y = (double)(1.0f / (float)d);
+  y = y * fma(-d, y, 2.0);
+  y = y * fma(-d, y, 2.0);
+  return zd(a.re * y, -a.im * y);
+}
+// |a|^2 in FP32: a key to choose pivots by
+__device__ __forceinline__ float pivot_key(const zd& a) {
+  const float x = (float)a.re, y = (float)a.im;
+  return fmaf(x, x, y * y);
+}
+// Inverse of the NO x NO matrix A (shared memory, row-major) into out by one
+// warp, Gauss-Jordan with partial pivoting; lane e < NO^2 owns element e of A
+// and of out.  Every lane of the warp calls it.
+template <int NO>
+__device__ __forceinline__ void warp_inv(const zd* A, zd* tmp, zd* out) {
+  constexpr int NO2 = NO * NO;
+  const int lane = threadIdx.x & 31, r = lane / NO, c = lane % NO;
+  if constexpr (NO == 1) {
+    if (lane == 0) out[0] = crecip(A[0]);
+    __syncwarp();
+    return;
+  }
+  if (lane < NO2) {
+    tmp[lane] = A[lane];
+    out[lane] = zd(r == c ? 1.0 : 0.0);
+  }
+  __syncwarp();
+  for (int p = 0; p < NO; ++p) {
+    int pr = p;
+    float best = pivot_key(tmp[p * NO + p]);
+    for (int q = p + 1; q < NO; ++q) {
+      const float v = pivot_key(tmp[q * NO + p]);
+      if (v > best) { best = v; pr = q; }
+    }
+    zd a = zd(), o = zd(), f = zd(), ap = zd(), op = zd(), piv = tmp[pr * NO + p];
+    if (lane < NO2) {   // rows p and pr change places
+      const int src = r == p ? pr : r == pr ? p : r;
+      a = tmp[src * NO + c];
+      o = out[src * NO + c];
+      f = tmp[src * NO + p];
+      ap = tmp[pr * NO + c];
+      op = out[pr * NO + c];
+    }
+    __syncwarp();
+    const zd ip = crecip(piv);
+    if (lane < NO2) {
+      ap = ap * ip;
+      op = op * ip;
+      tmp[lane] = r == p ? ap : a - f * ap;
+      out[lane] = r == p ? op : o - f * op;
+    }
+    __syncwarp();
+  }
+}
+
 // In-place Gauss-Jordan inverse with partial pivoting of the n x n matrix A
 // (leading dimension ld, shared memory, n <= 20); every thread calls it.
 static __device__ __noinline__ void gj_inverse(int n, zd* A, int ld) {
@@ -253,18 +314,18 @@ static __device__ __noinline__ void gj_inverse(int n, zd* A, int ld) {
   const int tid = threadIdx.x;
   for (int c = 0; c < n; ++c) {
     if (tid < 32) {
-      double v = (tid >= c && tid < n) ? A[tid * ld + c].abs2() : -1.0;
+      float v = (tid >= c && tid < n) ? pivot_key(A[tid * ld + c]) : -1.f;
       int p = tid;
 #pragma unroll
       for (int off = 16; off; off >>= 1) {
-        const double v2 = __shfl_xor_sync(FULL, v, off);
+        const float v2 = __shfl_xor_sync(FULL, v, off);
         const int p2 = __shfl_xor_sync(FULL, p, off);
         if (v2 > v || (v2 == v && p2 < p)) { v = v2; p = p2; }
       }
       if (p != c && tid < n) { const zd t = A[c * ld + tid]; A[c * ld + tid] = A[p * ld + tid]; A[p * ld + tid] = t; }
       if (tid == 0) prow[c] = p;
       __syncwarp();
-      if (tid < n) col[tid] = tid == c ? cdiv(zd(1.0), A[c * ld + c]) : A[tid * ld + c];
+      if (tid < n) col[tid] = tid == c ? crecip(A[c * ld + c]) : A[tid * ld + c];
       __syncwarp();
       if (tid < n) A[c * ld + tid] = tid == c ? col[c] : A[c * ld + tid] * col[c];   // the scaled pivot row
     }

@@ -1096,28 +1096,21 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
 // of the whole chunk every 32 steps took 0.2 ms (N_o = 1) to 7 ms (N_o = 4) and
 // left the growing chunks without an inverse.
 // ---------------------------------------------------------------------------
-// Row s of an inverse: Mi(s, .) from the coefficients crow[u][m][p] = A(s,u)_mp,
-// u = 0..s (diagonal block last), and the rows u < s of Mi (leading dimension
-// ld_m, columns u N_o + p; the first sb rows are a full start block).  out(m,
-// col, value) stores.  Every thread calls it.
+// Row s of an inverse: Mi(s, .) from the coefficients crow[m][u N_o + p] =
+// A(s,u)_mp, u < s (leading dimension ld_c), the inverse dinv of A(s,s), and the
+// rows u < s of Mi (leading dimension ld_m, columns u N_o + p; the first sb rows
+// are a full start block).  out(m, col, value) stores.  Every thread calls it.
 template <int NO, typename P, typename OUT>
-__device__ void append_row(int s, int sb, const zd* crow, const P* Mi, int ld_m, zd* part, zd* dinv, OUT out) {
-  constexpr int NO2 = NO * NO, SL = NO == 1 ? 8 : NO == 2 ? 2 : 1;   // slices of the sum over u
+__device__ __forceinline__ void append_row(int s, int sb, const zd* crow, int ld_c, const zd* dinv, const P* Mi, int ld_m,
+                                           zd* part, OUT out) {
+  constexpr int SL = NO == 1 ? 8 : NO == 2 ? 2 : 1;   // slices of the sum over u
   const int tid = threadIdx.x, nc = s * NO, tps = blockDim.x / SL, slice = tid / tps;
-  if (tid == 0) {
-    M<NO> D;
-#pragma unroll
-    for (int q = 0; q < NO2; ++q) D.a[q / NO][q % NO] = crow[s * NO2 + q];
-    const M<NO> I = solve_left<NO>(D, M<NO>::eye(zd(1.0)));
-#pragma unroll
-    for (int q = 0; q < NO2; ++q) dinv[q] = I.a[q / NO][q % NO];
-  }
   for (int e = tid % tps; e < NO * nc; e += tps) {
     const int m = e / nc, col = e % nc;
     zd acc = zd();
     for (int u = (col < sb * NO ? 0 : col / NO) + slice; u < s; u += SL)
 #pragma unroll
-      for (int p = 0; p < NO; ++p) acc = cfma(crow[u * NO2 + m * NO + p], ldr<double>(Mi + (long long)(u * NO + p) * ld_m + col), acc);
+      for (int p = 0; p < NO; ++p) acc = cfma(crow[m * ld_c + u * NO + p], ldr<double>(Mi + (long long)(u * NO + p) * ld_m + col), acc);
     part[slice * (NO * nc) + e] = acc;
   }
   __syncthreads();
@@ -1150,8 +1143,8 @@ __global__ void __launch_bounds__(256) k_inv_rows(Dev d, int T, int r0, int r1, 
   const double h = d.h;
   const DevW& W = d.w;
   __shared__ zd part[NO <= 2 ? 256 : CK * NO2];
-  __shared__ zd crow[CK * NO2];
-  __shared__ zd dinv[NO2];
+  __shared__ zd crow[NO * (CK * NO)];
+  __shared__ zd dinv[8][NO2], dtmp[8][NO2], diag[8][NO2];
   __shared__ zd Hm[NH * NH];       // the head, or the lesser start block
   if (sys == 2) {
     const int hs = min(2 * k, T), kb = min(k, hs), nh = hs * NO, nb = kb * NO;
@@ -1164,16 +1157,22 @@ __global__ void __launch_bounds__(256) k_inv_rows(Dev d, int T, int r0, int r1, 
     };
     for (int e = tid; e < nh * nh; e += blockDim.x) {
       const int row = e / nh, col = e % nh;
-      Hm[e] = (row < nb && col < nb) ? coef(row / NO + 1, col / NO + 1, row % NO, col % NO) : zd();
+      // the start block, and below it the rows s > k up to their diagonal
+      Hm[e] = (row < nb ? col < nb : col / NO <= row / NO) ? coef(row / NO + 1, col / NO + 1, row % NO, col % NO) : zd();
     }
     __syncthreads();
-    gj_inverse(nb, Hm, nh);
-    for (int s = kb; s < hs; ++s) {
-      for (int e = tid; e < (s + 1) * NO2; e += blockDim.x)
-        crow[e] = coef(s + 1, e / NO2 + 1, (e % NO2) / NO, e % NO);
-      __syncthreads();
-      append_row<NO>(s, kb, crow, Hm, nh, part, dinv, [&](int m, int col, const zd& v) { Hm[(s * NO + m) * nh + col] = v; });
+    {   // the diagonal blocks' inverses of the rows s > k, a warp each (k <= 5 rows)
+      const int w = tid >> 5, l = tid & 31, s = kb + w;
+      if (s < hs) {
+        if (l < NO2) diag[w][l] = Hm[(s * NO + l / NO) * nh + s * NO + l % NO];
+        __syncwarp();
+        warp_inv<NO>(diag[w], dtmp[w], dinv[w]);
+      }
     }
+    gj_inverse(nb, Hm, nh);
+    for (int s = kb; s < hs; ++s)
+      append_row<NO>(s, kb, Hm + s * NO * nh, nh, dinv[s - kb], Hm, nh, part,
+                     [&](int m, int col, const zd& v) { Hm[(s * NO + m) * nh + col] = v; });
     double2* Hi = d.hinv + (long long)n * (4 * k * k * NO2);
     for (int e = tid; e < nh * nh; e += blockDim.x) st(Hi + e, Hm[e]);
     return;
@@ -1219,12 +1218,17 @@ __global__ void __launch_bounds__(256) k_inv_rows(Dev d, int T, int r0, int r1, 
       const double wl = sys == 1 ? rule_w(W, s, u) : dd <= k ? W.omega[dd] : 1.0;
       zd v = sr_any<NO, S>(d, n, s, u, m, p) * (-h * wl);
       if (dd <= k && m == p) v += zd(0, W.ah[dd]);
-      if (dd == 0) v -= ld(epsp<NO>(d, n, s) + m * NO + p);
-      crow[e] = v;
+      if (dd == 0) {
+        v -= ld(epsp<NO>(d, n, s) + m * NO + p);
+        diag[0][m * NO + p] = v;
+      } else {
+        crow[m * LD + (u - a) * NO + p] = v;
+      }
     }
     __syncthreads();
+    if (tid < 32) warp_inv<NO>(diag[0], dtmp[0], dinv[0]);   // (read after append_row's barrier)
     const int sb = sys == 1 && cc == 0 ? k : 0;   // rows of the start block in this chunk: full columns
-    append_row<NO>(ri, sb, crow, Mi, LD, part, dinv, [&](int m, int col, const zd& v) { put(ri * NO + m, col, v); });
+    append_row<NO>(ri, sb, crow, LD, dinv[0], Mi, LD, part, [&](int m, int col, const zd& v) { put(ri * NO + m, col, v); });
   }
 }
 
