@@ -74,13 +74,16 @@ struct Solver {
   std::vector<double> nu;        // r chosen frequencies
   hk::DLRMats dm;
 
-  bool init(int r_, const double* tau_, const double* om_, double beta_, int no_) {
+  // with_dlr: the DLR matrices too (the reversal of the host iteration); their
+  // quadratures take some 0.1 s, which the device solve, having them in its
+  // handle, need not spend again
+  bool init(int r_, const double* tau_, const double* om_, double beta_, int no_, bool with_dlr = true) {
     r = r_; no = no_; n2 = no * no; beta = beta_; xi = -1;
     tau.assign(tau_, tau_ + r); om.assign(om_, om_ + r);
     Kt.resize((size_t)r * r);
     for (int i = 0; i < r; ++i)
       for (int l = 0; l < r; ++l) Kt[(size_t)i * r + l] = hk::dlr_kernel(tau[i], om[l], beta);
-    if (!hk::dlr_build(r, tau_, om_, beta, xi, &dm)) return false;
+    if (with_dlr && !hk::dlr_build(r, tau_, om_, beta, xi, &dm)) return false;
     // frequency nodes: greedy pivoted Gram-Schmidt on the rows 1/(i nu_n - w_l)
     double wmax = 0.0;
     for (double w : om) wmax = std::max(wmax, std::abs(w));
@@ -176,7 +179,7 @@ struct Solver {
 bool hk::mats_maps(int r, const double* tau, const double* om, double beta, std::vector<zc>* F,
                    std::vector<zc>* B, std::vector<double>* nu) {
   Solver sv;
-  if (!sv.init(r, tau, om, beta, 1)) return false;
+  if (!sv.init(r, tau, om, beta, 1, false)) return false;
   auto tr = [r](const std::vector<zc>& M) {
     std::vector<zc> T((size_t)r * r);
     for (int i = 0; i < r; ++i)
