@@ -508,7 +508,8 @@ int hkbe_create(const hkbe_params* p, const int32_t* nt_per_inst, void* stream, 
       hkbe_destroy(h);
       return HKBE_ERR_NOMEM;
     }
-    if ((rc = walloc(h, &d.nbose, d.n_inst)) || (rc = walloc(h, &d.hinv, (size_t)d.n_inst * 4 * d.k * d.k * n2)) || (h->hodlr && (rc = src_jobs(h)))) {
+    if ((rc = walloc(h, &d.nbose, d.n_inst)) || (rc = walloc(h, &d.hinv, (size_t)d.n_inst * 4 * d.k * d.k * n2)) || (h->hodlr && (rc = src_jobs(h))) ||
+        (h->hodlr && (rc = walloc(h, &d.fring, (size_t)d.n_inst * (d.nt + hk::kRingRows) * n2)))) {
       g_create_error = h->err;
       hkbe_destroy(h);
       return rc;

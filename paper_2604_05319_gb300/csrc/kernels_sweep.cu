@@ -53,7 +53,11 @@ constexpr size_t kBufBytes = std::max((size_t)kInvStage<NO>, (size_t)8 * kPG<NO>
 // Leaf rows (of four per thread) that a chunk's far field keeps in flight.
 template <int NO, typename S> constexpr int kLB = NO == 1 ? 4 : NO == 2 ? (sizeof(S) == 8 ? 4 : 2) : 1;
 constexpr int kCopyWaitPolls = 1 << 20;   // bound of the wait for a staged inverse
-constexpr int kRingRows = 80;             // >= leaf + k + 1 uncompressed rows
+constexpr int kSplitRows = 192;           // compressed rows from which a sweep is split (see split_les)
+
+// What a sweep's launch covers: everything, or (see split_les) only the
+// uncompressed rows (retarded: with the head) or only the compressed leaves.
+enum { kAll = 0, kTop = 1, kLeaves = 2 };
 
 // Sum over the 8 lanes of an aligned lane group of their history
 // accumulators (every lane receives it).  Complex64 form: the compensated
@@ -109,28 +113,33 @@ __device__ __forceinline__ double2* Cinv(const Dev& d, int n, int cc, int which)
 // projections Ps[slot][rmax] of the blocks that cover the current leaf (slot =
 // (target m or j, level, other index), target-major), the same packed without
 // the gaps between ranks (Pk, and the factor entry Off each belongs to), and
-// per slot its factor base, rank, first packed entry and block, for this leaf
-// and the next (ranks and blocks).
+// per slot its factor base and first packed entry; per slot and level the rank
+// and the block with its geometry, for this leaf and the next.
+struct LeafBlk {
+  long long uoff, voff;
+  int b, r0, r1, c0, c1, pad;
+};
 template <int NO, typename R>
 struct SweepMem {
   cx<R>*Ps, *Pk;
   long long* base;
+  LeafBlk* blk;   // [2][maxl]
   unsigned* off;
-  int *start, *rk, *blk;
+  int *start, *rk;
   int nslot;
   __host__ __device__ static size_t bytes(int maxl, int rmax) {
     const size_t ns = (size_t)maxl * NO * NO;
-    return ns * rmax * (2 * sizeof(cx<R>) + 4) + ns * 8 + (ns + 1) * 4 + 2 * (ns + maxl) * 4 + 16;
+    return ns * rmax * (2 * sizeof(cx<R>) + 4) + ns * 8 + 2 * maxl * sizeof(LeafBlk) + (3 * ns + 1) * 4 + 16;
   }
   __device__ SweepMem(char* p, int maxl, int rmax) {
     nslot = maxl * NO * NO;
     Ps = reinterpret_cast<cx<R>*>(p);
     Pk = Ps + (size_t)nslot * rmax;
     base = reinterpret_cast<long long*>(Pk + (size_t)nslot * rmax);
-    off = reinterpret_cast<unsigned*>(base + nslot);
+    blk = reinterpret_cast<LeafBlk*>(base + nslot);
+    off = reinterpret_cast<unsigned*>(blk + 2 * maxl);
     start = reinterpret_cast<int*>(off + (size_t)nslot * rmax);
     rk = start + nslot + 1;
-    blk = rk + 2 * nslot;
   }
 };
 
@@ -145,14 +154,16 @@ struct SweepMem {
 // combined across a warp's rows by shuffles and across warps in red
 // ([8][group][64], shared memory).  out(p, q, value).  Every thread calls it.
 template <int NO, typename S, bool ROWS, typename VF, typename RK, typename OUT>
-__device__ __forceinline__ void proj_block(const Dev& d, int n, int blk, int l0, int l1, VF vf, RK rank_of, void* buf,
-                                           OUT out) {
+__device__ __forceinline__ void proj_block(const Dev& d, int n, const LeafBlk& B, int l0, int l1, VF vf, RK rank_of,
+                                           void* buf, OUT out) {
   constexpr int NO2 = NO * NO, PG = kPG<NO>;
   using R = typename Bulk<S>::R;
   using V = typename Val<S>::t;
   V* red = static_cast<V*>(buf);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int base = ROWS ? d.b_r0[blk] : d.b_c0[blk];
+  const int base = ROWS ? B.r0 : B.c0, len = ROWS ? B.r1 - B.r0 : B.c1 - B.c0;
+  const S* Fb = static_cast<const S*>(ROWS ? d.hod[2].U : d.hod[2].V) +
+                ((long long)n * (ROWS ? d.utot : d.vtot) + (ROWS ? B.uoff : B.voff)) * d.rmax;
 #pragma unroll 1
   for (int p0 = 0; p0 < NO2; p0 += PG) {
     int rk[PG], rkmax = 0;
@@ -160,7 +171,7 @@ __device__ __forceinline__ void proj_block(const Dev& d, int n, int blk, int l0,
 #pragma unroll
     for (int g = 0; g < PG; ++g) {
       rk[g] = rank_of(p0 + g);
-      F[g] = ROWS ? Up<NO, S>(d, 2, n, blk, p0 + g) : Vp<NO, S>(d, 2, n, blk, p0 + g);
+      F[g] = Fb + (long long)(p0 + g) * len * d.rmax;
       rkmax = max(rkmax, rk[g]);
     }
     for (int qb = 0; qb < rkmax; qb += 64) {   // 64 entries of the rank at a time
@@ -170,7 +181,7 @@ __device__ __forceinline__ void proj_block(const Dev& d, int n, int blk, int l0,
       double sv = 0.0;              // the singular value this thread multiplies at the end
       if (tid < PG * 64) {
         const int g = tid >> 6, q = qb + (tid & 63);
-        if (q < d.rmax) sv = Sp<NO>(d, 2, n, blk, p0 + g)[q];
+        if (q < d.rmax) sv = Sp<NO>(d, 2, n, B.b, p0 + g)[q];
       }
       KAcc<R> part[PG][2];
       for (int sb = l0 + warp * rps + sub; sb < l1; sb += stride * FOLD) {
@@ -239,10 +250,18 @@ __device__ __forceinline__ zf scale_sv(const cff& a, double s) {
   return zf(ff_mul(a.re, f).hi, ff_mul(a.im, f).hi);
 }
 
-// The blocks and ranks of Sigma^R that cover leaf jl (of tab = colblk or
-// rowblk; retarded: only blocks with built rows), slot by slot, into rk, blk.
+// Geometry of block b (b < 0: none), where it is not kept in shared memory.
+__device__ __forceinline__ LeafBlk block_at(const Dev& d, int b) {
+  if (b < 0) return {0, 0, -1, 0, 0, 0, 0, 0};
+  return {d.b_uoff[b], d.b_voff[b], b, d.b_r0[b], d.b_r1[b], d.b_c0[b], d.b_c1[b], 0};
+}
+__device__ __forceinline__ cff ff_split(const zd& z) { return {ff_of_bits(z.re), ff_of_bits(z.im)}; }
+
+// The blocks of Sigma^R that cover leaf jl (retarded: over its columns, only
+// blocks with built rows; lesser: over its rows), their geometry and ranks, into
+// blk and rk.  The kernels read them a leaf ahead.
 template <int NO, typename R>
-__device__ __forceinline__ void leaf_table(const Dev& d, int n, int jl, bool cols, int* rk, int* blk, int t0) {
+__device__ __forceinline__ void leaf_table(const Dev& d, int n, int jl, bool cols, int* rk, LeafBlk* blk, int t0) {
   constexpr int NO2 = NO * NO;
   const int* tab = cols ? d.colblk : d.rowblk;
   for (int e = t0; e < d.maxl * NO2; e += blockDim.x) {
@@ -251,14 +270,17 @@ __device__ __forceinline__ void leaf_table(const Dev& d, int n, int jl, bool col
     int b = tab[jl * d.maxl + lv];
     if (b >= 0 && cols && d.b_r0[b] >= d.cdir) b = -1;
     rk[e] = b >= 0 ? *Rk<NO>(d, 2, n, b, p) : 0;
-    if (tg == 0 && oth == 0) blk[lv] = b;
+    if (tg == 0 && oth == 0) {
+      blk[lv].b = b;
+      if (b >= 0) blk[lv] = {d.b_uoff[b], d.b_voff[b], b, d.b_r0[b], d.b_r1[b], d.b_c0[b], d.b_c1[b], 0};
+    }
   }
 }
 // Pack the projections of the current leaf: entry e of target tg belongs to
 // e in [start[tg maxl NO], start[(tg + 1) maxl NO]).  Every thread calls it.
 template <int NO, typename R>
 __device__ __forceinline__ void leaf_pack(const Dev& d, int A, bool cols, const SweepMem<NO, R>& sm, const int* rk,
-                                          const int* blk) {
+                                          const LeafBlk* blk) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (warp == 0) {   // first packed entry of each slot
     int carry = 0;
@@ -280,9 +302,9 @@ __device__ __forceinline__ void leaf_pack(const Dev& d, int A, bool cols, const 
     const int r = rk[s];
     if (!r) continue;
     const int tg = s / (d.maxl * NO), lv = (s / NO) % d.maxl, oth = s % NO, p = cols ? oth * NO + tg : tg * NO + oth;
-    const int b = blk[lv], r0 = d.b_r0[b], c0 = d.b_c0[b];
-    const long long base = cols ? (d.b_voff[b] + (long long)p * (d.b_c1[b] - c0) + (A - c0)) * d.rmax
-                                : (d.b_uoff[b] + (long long)p * (d.b_r1[b] - r0) + (A - r0)) * d.rmax;
+    const LeafBlk& B = blk[lv];
+    const long long base = cols ? (B.voff + (long long)p * (B.c1 - B.c0) + (A - B.c0)) * d.rmax
+                                : (B.uoff + (long long)p * (B.r1 - B.r0) + (A - B.r0)) * d.rmax;
     for (int q = lane; q < r; q += 32) {
       sm.Pk[sm.start[s] + q] = sm.Ps[(size_t)s * d.rmax + q];
       sm.off[sm.start[s] + q] = (unsigned)(base + q);
@@ -312,7 +334,7 @@ __device__ __forceinline__ void leaf_pack(const Dev& d, int A, bool cols, const 
 // ---------------------------------------------------------------------------
 // MIX: the CTAs after the first N_o of an instance compute its mixed component.
 template <int NO, typename S, bool MIX>
-__global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, int staged) {
+__global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, int staged, int part) {
   pdl_start();
   constexpr int NO2 = NO * NO;
   constexpr bool MX = Row64<NO, S>::separate;
@@ -362,11 +384,13 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
   auto yp = [&](int tp) { return rowy + (long long)tp * NO2 + irow * NO; };
   auto sp = [&](int tp) { return rowp + (long long)tp * NO2 + irow * NO; };
   decltype(vdist(V(), cx<R>())) myerr = 0;
-  if (staged && top >= 0 && c > 0) leaf_table<NO, R>(d, n, (min(c, top + 1) - 1) / L, true, sm.rk, sm.blk, tid);
+  const bool below = part != kTop, above = part != kLeaves;   // the compressed columns; the head and the others
+  if (staged && below && top >= 0 && c > 0)
+    leaf_table<NO, R>(d, n, (min(c, top + 1) - 1) / L, true, sm.rk, sm.blk, tid);
   // ---- the head: points T-s, s = 1..hs, and y(T) = -i.  Its right-hand side
   // is row T of Sigma^R (and the derivative's y(T) term) alone; 8 threads per
   // element of the product with the head's inverse ----
-  const int hs = min(2 * k, T), nh = hs * NO;
+  const int hs = above ? min(2 * k, T) : 0, nh = hs * NO;
   for (int e = tid; e < nh; e += blockDim.x) {
     const int s = e / NO + 1, j = e % NO;
     zd cc = ld(el<NO, S>(d.SR, d, n, T, T - s) + irow * NO + j) * (-h * (s <= k ? W.I0[s][0] : rule_w(W, s, 0)));
@@ -395,7 +419,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
       }
     }
   }
-  if (tid < NO) {
+  if (above && tid < NO) {
     V v;
     vset(v, (tid == irow) ? zd(0, -1) : zd());
     myerr = fmax(myerr, vdist(v, ldr<R>(sp(T) + tid)));
@@ -409,17 +433,30 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
       for (int e = blockDim.x - 1 - tid; e < wn * NO; e += blockDim.x)
         st(yp(wa + e / NO) + e % NO, cff_val(Yl[(wa + e / NO) & 63][e % NO]));
   };
-  bool first_comp = true;
+  bool first_comp = part == kAll;
   int wa = 0, wn = 0;
-  for (int cc = top >= 0 ? top / CK : -1; cc >= 0; --cc) {
+  if (part == kLeaves) {   // the points solved last by the part before
+    const int b0 = min(c, top + 1);
+    for (int e = tid; e < 64 * NO; e += blockDim.x) {
+      const int tp = b0 + e / NO;
+      if (tp > T) continue;
+      if constexpr (MX) Yl[tp & 63][e % NO] = ff_split(ld(yp(tp) + e % NO));
+      else Yl[tp & 63][e % NO] = ld(yp(tp) + e % NO);
+    }
+    __syncthreads();
+  }
+  const V* fr = reinterpret_cast<const V*>(d.fring) + ((long long)n * NO + irow) * d.nt * NO;
+  const int cstart = part == kLeaves ? min(c, top + 1) - 1 : top;
+  for (int cc = cstart >= 0 ? cstart / CK : -1; cc >= 0; --cc) {
     const int a = cc * CK, b = min(a + CK, top + 1), cn = b - a;
     const bool comp = (c > 0 && b <= c);
+    if (comp && !below) break;
     const int jl = comp ? a / L : 0, A = jl * L, E = comp ? (jl + 1) * L : 0;
     if (comp && (b == E || b == top + 1)) {   // (the top chunk may end inside its leaf)
       // Entering leaf jl from above.
       const int* rk = sm.rk + buf * sm.nslot;
-      const int* blks = sm.blk + buf * d.maxl;
-      const int nr = T + 1 - c;
+      const LeafBlk* blks = sm.blk + buf * d.maxl;
+      const int nr = part == kAll ? T + 1 - c : 0;   // uncompressed rows to sum here
       if (first_comp) {   // the uncompressed rows with their weights at the end T
         first_comp = false;
         for (int e = tid; e < nr * NO; e += blockDim.x) {
@@ -430,13 +467,12 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
       }
       // (1) projections pi_B = sum_s y(s) U_B(s,:) S_B of the blocks whose columns end at E
       for (int lv = 0; lv < d.maxl; ++lv) {
-        const int blk = staged ? blks[lv] : d.colblk[jl * d.maxl + lv];
-        if (blk < 0 || d.b_c1[blk] != E || d.b_r0[blk] >= c) continue;
-        const int r0 = d.b_r0[blk], rl = min(d.b_r1[blk], c);
+        const LeafBlk B = staged ? blks[lv] : block_at(d, d.colblk[jl * d.maxl + lv]);
+        if (B.b < 0 || B.c1 != E || B.r0 >= c) continue;
         auto slot = [&](int p) { return ((p % NO) * d.maxl + lv) * NO + p / NO; };
         proj_block<NO, S, true>(
-            d, n, blk, r0, rl, [&](int s2, int m) { return ldr<R>(sp(s2) + m); },
-            [&](int p) { return staged ? rk[slot(p)] : *Rk<NO>(d, 2, n, blk, p); }, dyn,
+            d, n, B, B.r0, min(B.r1, c), [&](int s2, int m) { return ldr<R>(sp(s2) + m); },
+            [&](int p) { return staged ? rk[slot(p)] : *Rk<NO>(d, 2, n, B.b, p); }, dyn,
             [&](int p, int q, const V& v, double sv) {
               if (staged) sm.Ps[(size_t)slot(p) * d.rmax + q] = scale_sv(v, sv);
               else reinterpret_cast<cx<R>*>(Pj<NO>(d, n, irow, lv, p))[q] = scale_sv(v, sv);
@@ -452,6 +488,12 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
       {
         const int lpc = blockDim.x / L, col = tid / lpc, sl = tid % lpc, tp = A + col;
         KAcc<R> ka[NO];   // FP32 history sums, compensated (FP64 in the FP64 form)
+        V fr0[NO];        // the uncompressed rows' part, if a kernel before this one has it
+#pragma unroll
+        for (int j = 0; j < NO; ++j) {
+          vset(fr0[j], zd());
+          if (part == kLeaves && sl == 0) fr0[j] = fr[(long long)tp * NO + j];
+        }
         constexpr int RB = NO == 1 ? 8 : NO == 2 ? (MX ? 4 : 2) : 1;   // rows in flight
         const S* Sr = static_cast<const S*>(d.SR) + ((long long)n * d.ring * d.nt + tp) * NO2;
         const int s0 = c % d.ring;
@@ -538,7 +580,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
             for (int off = 1; off < lpc; off <<= 1) acc[j] = vadd(acc[j], vshfl_xor(acc[j], off));
             r = vadd(r, acc[j]);
           }
-          if (sl == 0) FB[col][j] = r;
+          if (sl == 0) FB[col][j] = vadd(r, fr0[j]);
         }
       }
       buf ^= 1;
@@ -704,7 +746,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
 // same phases as the retarded sweep, upwards.
 // ---------------------------------------------------------------------------
 template <int NO, typename S>
-__global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, int staged) {
+__global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, int staged, int part) {
   pdl_start();
   constexpr int NO2 = NO * NO;
   constexpr bool MX = Row64<NO, S>::separate;
@@ -743,8 +785,15 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
   const double2* qs = d.qsrc + (long long)n * d.nt * NO2;
   decltype(vdist(V(), cx<R>())) myerr = 0;
   const int last = (d.rho_mode == 1) ? T - 1 : T;
-  if (staged && c > 0) leaf_table<NO, R>(d, n, 0, false, sm.rk, sm.blk, tid);
-  if (tid < NO) {  // x(0) = -[G^tv(T, 0+)]^dagger
+  if (staged && c > 0 && part != kTop) leaf_table<NO, R>(d, n, 0, false, sm.rk, sm.blk, tid);
+  if (part == kTop) {   // the points solved last by the part before
+    for (int e = tid; e < 64 * NO; e += blockDim.x) {
+      const int t = c - 1 - e / NO, m = e % NO;
+      if (t < 0) continue;
+      if constexpr (MX) Xl[t & 63][m] = ff_split(ld(xp(t) + m * NO + jc));
+      else Xl[t & 63][m] = ld(xp(t) + m * NO + jc);
+    }
+  } else if (tid < NO) {  // x(0) = -[G^tv(T, 0+)]^dagger
     const int m = tid;
     const zd x = ld(d.x0 + (long long)n * NO2 + m * NO + jc);
     V v;
@@ -761,27 +810,29 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
         st(xp(wa + e / NO) + (e % NO) * NO + jc, cff_val(Xl[(wa + e / NO) & 63][e % NO]));
   };
   int wa = 0, wn = 0;
-  for (int cc = 0; cc * CK <= last; ++cc) {
+  const V* fl = reinterpret_cast<const V*>(d.fring) + ((long long)d.n_inst * d.nt + (long long)n * kRingRows) * NO2;
+  const int chi = part == kLeaves ? c : last + 1;   // points below this
+  for (int cc = part == kTop ? c / CK : 0; cc * CK < chi; ++cc) {
     const int a = (cc == 0) ? 1 : cc * CK, b = min((cc + 1) * CK, last + 1), cn = b - a;
     if (cn <= 0) break;
     const bool comp = (c > 0 && b <= c);
     const int jl = comp ? a / L : 0, A = jl * L;
     if (comp && cc * CK == A) {
       const int* rk = sm.rk + buf * sm.nslot;
-      const int* blks = sm.blk + buf * d.maxl;
+      const LeafBlk* blks = sm.blk + buf * d.maxl;
       // Entering leaf jl.  (1) rho_B = S_B sum_l w_l conj(V_B(l,:)) x(l) for the
       // blocks whose rows start at A (w_l = omega_l for l <= k, else 1).
       for (int lv = 0; lv < d.maxl && jl > 0; ++lv) {
-        const int blk = staged ? blks[lv] : d.rowblk[jl * d.maxl + lv];
-        if (blk < 0 || d.b_r0[blk] != A) continue;
+        const LeafBlk B = staged ? blks[lv] : block_at(d, d.rowblk[jl * d.maxl + lv]);
+        if (B.b < 0 || B.r0 != A) continue;
         auto slot = [&](int p) { return ((p / NO) * d.maxl + lv) * NO + p % NO; };
         proj_block<NO, S, false>(
-            d, n, blk, d.b_c0[blk], d.b_c1[blk],
+            d, n, B, B.c0, B.c1,
             [&](int l, int nn) {
               const cx<R> x = ldr<R>(sp(l) + nn * NO + jc);
               return l <= k ? x * (R)W.omega[l] : x;
             },
-            [&](int p) { return staged ? rk[slot(p)] : *Rk<NO>(d, 2, n, blk, p); }, dyn,
+            [&](int p) { return staged ? rk[slot(p)] : *Rk<NO>(d, 2, n, B.b, p); }, dyn,
             [&](int p, int q, const V& v, double sv) {
               if (staged) sm.Ps[(size_t)slot(p) * d.rmax + q] = scale_sv(v, sv);
               else reinterpret_cast<cx<R>*>(Pj<NO>(d, n, jc, lv, p))[q] = scale_sv(v, sv);
@@ -907,7 +958,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
           for (int m = 0; m < NO; ++m) ka[m].add(pa[m]);
         } else {
           const S* srow = el<NO, S>(d.SR, d, n, t, 0);
-          for (int lb = sl; lb < a; lb += 8 * FOLD) {
+          for (int lb = (part == kTop ? c : 0) + sl; lb < a; lb += 8 * FOLD) {
             cx<R> pa[NO];
 #pragma unroll
             for (int m = 0; m < NO; ++m) pa[m] = cx<R>(0);
@@ -938,6 +989,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
       if (sl < NO && row < cn) {   // lane sl of the group finishes component sl
         V F = pick(r, sl), fb;
         if (comp && t > k) F = vadd(F, FB[t - A][sl]);
+        if (part == kTop) F = vadd(F, fl[((t - c) * NO + sl) * NO + jc]);   // the compressed columns
         F = vadd(vreal(F, h, W.hf), q);
         vset(fb, zd());
         if (t <= k) {   // start rows: only l = 0 lies left of chunk 0 (a derivative term: kept in Fb)
@@ -1071,6 +1123,144 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
   // after a timed-out wait, a copy may still be in flight into this CTA's
   // shared memory: wait for it (bounded) before the CTA exits
   if (kInvStage<NO> && tid == 0 && !s_stage) mbar_wait(&cbar, cphase ^ 1u, kCopyWaitPolls);
+}
+
+// ---------------------------------------------------------------------------
+// Between the two launches of a split sweep: the products of the uncompressed
+// rows of Sigma^R with the points the first launch has solved, which no later
+// point changes.  In the sweep's own chain they were its longest phases: an
+// SM's share of rows read one chunk (lesser) or leaf (retarded) at a time.
+// ---------------------------------------------------------------------------
+// Retarded: F(t')_ij = sum_{s in [c, T]} w_s y_i(s) Sigma^R(s, t') for t' < c, all
+// orbital rows i; 32 columns per CTA (adjacent elements of every row along the
+// lanes), the rows s over the 8 warps.
+template <int NO, typename S>
+__global__ void __launch_bounds__(256) k_ret_ring(Dev d, int T) {
+  pdl_start();
+  constexpr int NO2 = NO * NO;
+  using R = typename Bulk<S>::R;
+  using V = typename Val<S>::t;
+  const int n = blockIdx.y;
+  if (!d.active[n]) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, c = d.cdir, k = d.k, nr = T + 1 - c;
+  const DevW& W = d.w;
+  extern __shared__ __align__(16) char dyn[];
+  V* red = reinterpret_cast<V*>(dyn);                           // [8][NO2][32]
+  cx<R>* ys = reinterpret_cast<cx<R>*>(red + 8 * NO2 * 32);     // [kRingRows][i][m] y with its weight at the end T
+  const S* yrow = el<NO, S>(d.GR, d, n, T, 0);
+  for (int e = tid; e < nr * NO2; e += blockDim.x) {
+    const int s2 = c + e / NO2;
+    const cx<R> v = ldr<R>(yrow + (long long)c * NO2 + e);
+    ys[e] = T - s2 <= k ? v * rule_wr<R>(W, T + 2 * k + 1, T - s2) : v;
+  }
+  __syncthreads();
+  const int tp = blockIdx.x * 32 + lane;
+  const S* Sr = static_cast<const S*>(d.SR) + ((long long)n * d.ring * d.nt + tp) * NO2;
+  const int s0 = c % d.ring;
+  KAcc<R> ka[NO2];
+  for (int i0 = warp; i0 < nr; i0 += 8 * FOLD) {
+    cx<R> pa[NO2];
+#pragma unroll
+    for (int q = 0; q < NO2; ++q) pa[q] = cx<R>(0);
+#pragma unroll
+    for (int jj = 0; jj < FOLD; ++jj) {
+      const int i = i0 + 8 * jj;
+      if (i < nr) {
+        int slot = s0 + i;
+        if (slot >= d.ring) slot -= d.ring;
+        const S* sr = Sr + (long long)slot * d.nt * NO2;
+        const int dd = c + i - tp;
+        const bool near = dd <= k;
+        const R wd = near ? rule_wr<R>(W, 2 * k + 1 + dd, dd) : (R)1;
+#pragma unroll
+        for (int m = 0; m < NO; ++m)
+#pragma unroll
+          for (int j = 0; j < NO; ++j) {
+            cx<R> sv = ldr<R>(sr + m * NO + j);
+            if (near) sv = sv * wd;
+#pragma unroll
+            for (int x = 0; x < NO; ++x) pa[x * NO + j] = cfma(ys[(i * NO + x) * NO + m], sv, pa[x * NO + j]);
+          }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NO2; ++q) ka[q].add(pa[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < NO2; ++q) red[(warp * NO2 + q) * 32 + lane] = kacc_lanes(ka[q], 32, 32);
+  __syncthreads();
+  V* fr = reinterpret_cast<V*>(d.fring) + (long long)n * NO * d.nt * NO;
+  for (int e = tid; e < 32 * NO2; e += blockDim.x) {   // e: orbital row, column, j
+    const int x = e / (32 * NO), tt = (e / NO) % 32, j = e % NO;
+    V a[8];
+#pragma unroll
+    for (int w2 = 0; w2 < 8; ++w2) a[w2] = red[(w2 * NO2 + x * NO + j) * 32 + tt];
+#pragma unroll
+    for (int s2 = 4; s2; s2 >>= 1)
+#pragma unroll
+      for (int w2 = 0; w2 < s2; ++w2) a[w2] = vadd(a[w2], a[w2 + s2]);
+    fr[((long long)x * d.nt + blockIdx.x * 32 + tt) * NO + j] = a[0];
+  }
+}
+
+// Lesser: F(t)_mj = sum_{l < c} w^(t)_l Sigma^R(t, l) x_j(l) for the uncompressed
+// rows t >= c, all orbital columns j; 4 warps per row.
+template <int NO, typename S>
+__global__ void __launch_bounds__(256) k_les_ring(Dev d, int T) {
+  pdl_start();
+  constexpr int NO2 = NO * NO;
+  using R = typename Bulk<S>::R;
+  using V = typename Val<S>::t;
+  const int n = blockIdx.y;
+  if (!d.active[n]) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, c = d.cdir, k = d.k;
+  const DevW& W = d.w;
+  __shared__ V red[8][NO2];
+  const int t = c + blockIdx.x * 2 + (warp >> 2), i = tid & 127;
+  const bool row = t <= T;
+  const S* sr = el<NO, S>(d.SR, d, n, row ? t : T, 0);
+  const S* xr = el<NO, S>(d.GL, d, n, T, 0);
+  KAcc<R> ka[NO2];
+  for (int l0 = i; row && l0 < c; l0 += 128 * FOLD) {
+    cx<R> pa[NO2];
+#pragma unroll
+    for (int q = 0; q < NO2; ++q) pa[q] = cx<R>(0);
+#pragma unroll
+    for (int jj = 0; jj < FOLD; ++jj) {
+      const int l = l0 + 128 * jj;
+      if (l < c) {
+        const bool end = l <= k || t - l <= k;
+        const R wl = end ? rule_wr<R>(W, t, l) : (R)1;
+        cx<R> x[NO2];
+#pragma unroll
+        for (int q = 0; q < NO2; ++q) {
+          x[q] = ldr<R>(xr + (long long)l * NO2 + q);
+          if (end) x[q] = x[q] * wl;
+        }
+#pragma unroll
+        for (int m = 0; m < NO; ++m)
+#pragma unroll
+          for (int y = 0; y < NO; ++y) {
+            const cx<R> sv = ldr<R>(sr + (long long)l * NO2 + m * NO + y);
+#pragma unroll
+            for (int j = 0; j < NO; ++j) pa[m * NO + j] = cfma(sv, x[y * NO + j], pa[m * NO + j]);
+          }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NO2; ++q) ka[q].add(pa[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < NO2; ++q) {
+    const V v = kacc_lanes(ka[q], 1, 32);
+    if (lane == 0) red[warp][q] = v;
+  }
+  __syncthreads();
+  if (row && i < NO2) {
+    const int w0 = warp & 4;
+    const V v = vadd(vadd(red[w0][i], red[w0 + 1][i]), vadd(red[w0 + 2][i], red[w0 + 3][i]));
+    reinterpret_cast<V*>(d.fring)[((long long)d.n_inst * d.nt + (long long)n * kRingRows + (t - c)) * NO2 + i] = v;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1275,6 +1465,15 @@ bool ret_takes_mixed(const Dev& d) {
   const int ni = d.no == 1 ? kNodesFew<1> : d.no == 2 ? kNodesFew<2> : kNodesFew<3>;
   return (long long)(d.no + (d.r + ni - 1) / ni) * d.n_inst <= (d.no <= 2 ? 2 : 1) * 152;
 }
+// A sweep runs as two launches with its ring kernel between them once kSplitRows
+// rows are compressed: before that, the ring's products in the chain cost less
+// than two more launches (complex64, T = 150, 64 to 128 rows: 4.4 -> 4.8 ms of
+// lesser sweeps in 49 steps).  From there on, the lesser sweep: 35 -> 31 ms (128
+// instances, N_o = 2, T = 600), 43.5 -> 38.4 (1, FP64, T = 384).  The retarded
+// sweep, whose ring phases are shorter, gains only while its CTAs leave SMs
+// idle: 43 -> 36 ms (1, FP64, T = 384), but 19.7 -> 21.6 (304, complex64).
+static bool split_les(const Dev& d) { return d.cdir >= kSplitRows; }
+static bool split_ret(const Dev& d) { return d.cdir >= kSplitRows && d.no * d.n_inst <= 152; }
 template <int NO, typename S>
 static cudaError_t sweep_ret(const Dev& d, int T, cudaStream_t s) {
   int staged = 0;
@@ -1285,7 +1484,17 @@ static cudaError_t sweep_ret(const Dev& d, int T, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   if (d.ring && T + 1 - d.cdir > kRingRows && d.cdir > 0) return cudaErrorInvalidValue;
   const int mix = with ? (d.r + kNodesFew<NO> - 1) / kNodesFew<NO> : 0;
-  return launch_on(false, kern, dim3(NO + mix, d.n_inst), 256, bytes, s, d, T, staged);
+  const bool split = split_ret(d);
+  if ((e = launch_on(false, kern, dim3(NO + mix, d.n_inst), 256, bytes, s, d, T, staged, split ? (int)kTop : (int)kAll)) !=
+          cudaSuccess ||
+      !split)
+    return e;
+  const size_t rb = NO * NO * (8 * 32 * 16 + kRingRows * sizeof(S));
+  auto leaves = k_ret2<NO, S, false>;
+  if ((e = allow_smem(k_ret_ring<NO, S>, rb)) != cudaSuccess || (e = allow_smem(leaves, bytes)) != cudaSuccess ||
+      (e = launch_k(k_ret_ring<NO, S>, dim3(d.cdir / 32, d.n_inst), 256, rb, s, d, T)) != cudaSuccess)
+    return e;
+  return launch_on(false, leaves, dim3(NO, d.n_inst), 256, bytes, s, d, T, staged, (int)kLeaves);
 }
 template <int NO, typename S>
 static cudaError_t sweep_les(const Dev& d, int T, cudaStream_t s) {
@@ -1293,7 +1502,15 @@ static cudaError_t sweep_les(const Dev& d, int T, cudaStream_t s) {
   const size_t bytes = sweep_smem<NO, S>(d, &staged);
   cudaError_t e = allow_smem(k_les2<NO, S>, bytes);
   if (e != cudaSuccess) return e;
-  return launch_on(false, k_les2<NO, S>, dim3(d.no, d.n_inst), 256, bytes, s, d, T, staged);
+  const bool split = split_les(d);
+  const int rows = T + 1 - d.cdir;
+  if (split && rows > kRingRows) return cudaErrorInvalidValue;
+  if ((e = launch_on(false, k_les2<NO, S>, dim3(NO, d.n_inst), 256, bytes, s, d, T, staged,
+                     split ? (int)kLeaves : (int)kAll)) != cudaSuccess ||
+      !split)
+    return e;
+  if ((e = launch_k(k_les_ring<NO, S>, dim3((rows + 1) / 2, d.n_inst), 256, 0, s, d, T)) != cudaSuccess) return e;
+  return launch_on(false, k_les2<NO, S>, dim3(NO, d.n_inst), 256, bytes, s, d, T, staged, (int)kTop);
 }
 cudaError_t launch_ret_h(const Dev& d, int T, cudaStream_t s) {
   HK_DISPATCH(d.no, return (sweep_ret<NO, S>(d, T, s)));

@@ -61,6 +61,7 @@ struct Dev {
   // the diagonal stay zero from the allocation
   double2* cinv;
   double2* cinv_ws;    // [n][2][(32 no)^2] complex64 form: FP64 rows of the growing chunks
+  double2* fring;      // products of the uncompressed rows, retarded [n][no][nt][no], then lesser [n][kRingRows][no2]
   double2* hinv;       // [n][(2k no)^2] inverse of the retarded head of the current step
   int nchunk;          // ceil(nt / 32)
   int nfrozR, nfrozL;  // chunks [0, nfroz) of each sweep have a complete inverse
@@ -100,6 +101,7 @@ struct Dev {
   const int *last;             // [n] last time step of each instance (N_t of the instance - 1)
 };
 
+constexpr int kRingRows = 80;    // >= leaf + k + 1 uncompressed rows
 constexpr int kSrcChunk = 256;   // rows of a block side that one CTA of the source projections takes
 
 // ---- launchers (all on `s`) ----
