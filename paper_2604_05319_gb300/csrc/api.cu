@@ -383,9 +383,17 @@ int hkbe_create(const hkbe_params* p, const int32_t* nt_per_inst, void* stream, 
     d.w.omegaf[i] = (float)w.omega[i];
     auto pair = [](double x) { const float hi = (float)x; return make_float2(hi, (float)(x - (double)hi)); };
     d.w.hf = pair(p->h);
+    d.w.ext[i] = 0.0;
     d.w.ahf[i] = pair(d.w.ah[i]);
     d.w.wm1f[i] = pair(w.omega[i] - 1.0);
     for (int j = 0; j < 6; ++j) d.w.I0f[i][j] = (float)w.I0[i][j];
+  }
+  {
+    double c = 1.0;   // C(k+1, l+1)
+    for (int l = 0; l <= p->k; ++l) {
+      c = c * (p->k + 1 - l) / (l + 1);
+      d.w.ext[l] = (l & 1) ? -c : c;
+    }
   }
   h->hodlr = p->svd_tol > 0;
   size_t tri = (size_t)d.n_inst * d.ntri * d.no * d.no;
@@ -938,7 +946,7 @@ static int iterate(hkbe_t* h, int max_iter, double tol, F pass, int32_t* iters, 
   while (any && done < max_iter) {
     const int batch = done == 0 ? std::min({std::max(*ahead, 1), kAhead, max_iter}) : 1;
     for (int i = 0; i < batch; ++i) {
-      HK_CUDA(h, pass());
+      HK_CUDA(h, pass(done + i));
       HK_CUDA(h, run_phase(h, HKBE_PHASE_CTRL, 1, [&]() {
         return hk::launch_set_active(d, tol_eff, done + i + 1, min_iter, coupled, h->res_dev + (size_t)i * N, h->s);
       }));
@@ -1032,7 +1040,7 @@ int hkbe_bootstrap(hkbe_t* h, int max_iter, double tol, int32_t* iters, double* 
   HK_CUDA(h, cudaMemsetAsync(d.err, 0, d.n_inst * sizeof(double), h->s));
   int ahead = 1;
   rc = iterate(h, max_iter, tol,
-               [&]() { return run_phase(h, HKBE_PHASE_BOOT, d.k + 4, [&]() { return hk::launch_boot(d, h->s); }); },
+               [&](int) { return run_phase(h, HKBE_PHASE_BOOT, d.k + 4, [&]() { return hk::launch_boot(d, h->s); }); },
                iters, err, &failed, all, &ahead);
   if (rc) return rc;
   if ((rc = finish_start(h))) return rc;
@@ -1092,9 +1100,11 @@ int hkbe_step(hkbe_t* h, int n_steps, int32_t* iters, double* err) {
     for (int n = 0; n < N; ++n) act0[n] = T <= h->last[n] ? 1 : 0;
     bool failed = false;
     rc = iterate(h, h->p.max_iter, h->p.tol,
-                 [&]() -> cudaError_t {
+                 [&](int it) -> cudaError_t {
                    cudaError_t e;
-                   if ((e = run_phase(h, HKBE_PHASE_SIGMA, 1, [&]() { return hk::launch_sigma(d, T, h->s); })))
+                   // a Sigma that does not depend on G stays as the step's first iteration left it
+                   if ((it == 0 || h->self_consistent) &&
+                       (e = run_phase(h, HKBE_PHASE_SIGMA, 1, [&]() { return hk::launch_sigma(d, T, h->s); })))
                      return e;
                    if ((e = run_phase(h, HKBE_PHASE_RET, 1, [&]() {
                           return h->scheme ? hk::launch_ret_sf(d, T, h->s) : hk::launch_ret_h(d, T, h->s);

@@ -250,14 +250,7 @@ __global__ void k_extrap(Dev d, int T) {
     d.err[n] = 0.0;
   }
   if (idx >= 2 * (T + 1) + d.r || T > d.last[n]) return;
-  double e[6];
-  {
-    double c = 1.0;  // C(k+1, l+1) built incrementally
-    for (int l = 0; l <= k; ++l) {
-      c = (l == 0) ? (double)(k + 1) : c * (double)(k + 1 - l) / (double)(l + 1);
-      e[l] = (l & 1) ? -c : c;
-    }
-  }
+  const double* e = d.w.ext;   // (-1)^l C(k+1, l+1); built per thread, its divisions were most of the kernel's FP64 work
   zd acc[NO2];
   for (int q = 0; q < NO2; ++q) acc[q] = zd();
   if (idx <= 2 * T + 1) {   // G^R row (X = 0) or G^< column (X = 1), from the FP64 copies where kept

@@ -11,6 +11,7 @@ struct DevW {
   int k;
   double a[6], omega[6], D[6][6], I0[6][6];
   float omegaf[6], I0f[6][6];   // float copies for the bulk sums of the complex64 form
+  double ext[6];                 // extrapolation weights of a step's first guess
   double ah[6];                  // a_j / h (the BDF coefficients of the time derivative)
   float2 hf, ahf[6], wm1f[6];    // h, a_j / h and omega_i - 1 as float-float pairs (complex64 form)
 };
