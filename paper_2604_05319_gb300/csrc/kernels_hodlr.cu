@@ -232,6 +232,9 @@ __device__ __forceinline__ cff vmul_mi(const cff& a) { return {a.im, ff_neg(a.re
 // and source together took 554 us at N_o = 2, complex64, 128 instances, T = 600
 // (now 360), 400 us in FP64 at 16 instances, T = 300 (123), 970 us at N_o = 4,
 // complex64, 16 instances, T = 290 (152).
+// With the rows' g staged in shared memory and each entry's pointers kept there:
+// 25.1 -> 18.8 ms of a pass at N_o = 1, complex64, 304 instances, T = 384, and
+// 46.3 -> 37.0 at N_o = 2, 128 instances, T = 600.
 constexpr int kEB = 4;
 template <int NO, typename S>
 __global__ void __launch_bounds__(256) k_src_q(Dev d, int T, int uselist) {
@@ -288,26 +291,31 @@ __global__ void __launch_bounds__(256) k_src_q(Dev d, int T, int uselist) {
         }
   };
   if ((int)blockIdx.x >= ntile) {   // uncompressed rows, one warp each, lanes along the row
-    __syncthreads();
     const int t = c + ((int)blockIdx.x - ntile) * 8 + warp;
-    if (t > T) return;
-    cx<R> g[NO2], s[NO2];
-    for (int l0 = lane; l0 <= T; l0 += 32 * FOLD) {
+    const bool row = t <= T;
+    const S* srow = el<NO, S>(d.SL, d, n, row ? t : T, 0);
+    cx<R>* gt = reinterpret_cast<cx<R>*>(red);   // [256][NO2] w_l g_l, shared by the CTA's rows
+    cx<R> s[NO2];
+    for (int lt = 0; lt <= T; lt += 256) {
+      const int ln = min(256, T + 1 - lt);
+      __syncthreads();
+      for (int e = tid; e < ln * NO2; e += blockDim.x) gt[e] = gw(lt + e / NO2, (e % NO2) / NO, e % NO);
+      __syncthreads();
+      if (row) {
 #pragma unroll
-      for (int jj = 0; jj < FOLD; ++jj) {
-        const int l = l0 + 32 * jj;
-        if (l <= T) {
-          const S* sp = l >= t ? el<NO, S>(d.SL, d, n, l, t) : el<NO, S>(d.SL, d, n, t, l);
+        for (int jj = 0; jj < FOLD; ++jj) {
+          const int li = lane + 32 * jj, l = lt + li;
+          if (li < ln) {
+            const S* sp = l >= t ? el<NO, S>(d.SL, d, n, l, t) : srow + (long long)l * NO2;
 #pragma unroll
-          for (int q = 0; q < NO2; ++q) {
-            s[q] = ldr<R>(sp + q);
-            g[q] = gw(l, q / NO, q % NO);
+            for (int q = 0; q < NO2; ++q) s[q] = ldr<R>(sp + q);
+            mac(s, l < t, gt + li * NO2);
           }
-          mac(s, l < t, g);
         }
+        fold();
       }
-      fold();
     }
+    if (!row) return;
     V hist[NO2];
 #pragma unroll
     for (int q = 0; q < NO2; ++q) hist[q] = vreal(kacc_lanes(ka[q], 1, 32), d.h, W.hf);
@@ -328,9 +336,9 @@ __global__ void __launch_bounds__(256) k_src_q(Dev d, int T, int uselist) {
   int* rk = reinterpret_cast<int*>(gl + 64 * NO2);            // per slot (target x, side, level, other index): rank,
   const int nslot = 2 * d.maxl * NO2;
   int* start = rk + nslot;                                    // first packed entry,
-  int* blk = start + nslot + 1;                               // block,
-  long long* base = reinterpret_cast<long long*>(((unsigned long long)(blk + nslot) + 7) & ~7ull);   // factor row of t0
-  unsigned short* list = reinterpret_cast<unsigned short*>(base + nslot);   // entries: slot * 128 + q
+  const S** fp = reinterpret_cast<const S**>(((unsigned long long)(start + nslot + 1) + 7) & ~7ull);   // factor row of the first t,
+  const cx<R>** pp = reinterpret_cast<const cx<R>**>(fp + nslot);           // and projections [q][y]
+  unsigned short* list = reinterpret_cast<unsigned short*>(pp + nslot);     // entries: slot * 128 + q
   const int nr = T + 1 - c;
   for (int e = tid; e < nr * NO2; e += blockDim.x) gr[e] = gw(c + e / NO2, (e % NO2) / NO, e % NO);
   for (int e = tid; e < L * NO2; e += blockDim.x) gl[e] = gw(A + e / NO2, (e % NO2) / NO, e % NO);
@@ -339,12 +347,11 @@ __global__ void __launch_bounds__(256) k_src_q(Dev d, int T, int uselist) {
     const int p = which == 0 ? x * NO + z : z * NO + x;
     int b = (which == 0 ? d.colblk : d.rowblk)[jt * d.maxl + lv];
     if (b >= 0 && d.b_r0[b] >= c) b = -1;
-    blk[s] = b;
     rk[s] = b >= 0 ? *Rk<NO>(d, 3, n, b, p) : 0;
     if (b >= 0) {
-      const int r0 = d.b_r0[b], c0 = d.b_c0[b];
-      base[s] = which == 0 ? ((long long)n * d.vtot + d.b_voff[b] + (long long)p * (d.b_c1[b] - c0) + (blockIdx.x * 32 - c0)) * d.rmax
-                           : ((long long)n * d.utot + d.b_uoff[b] + (long long)p * (d.b_r1[b] - r0) + (blockIdx.x * 32 - r0)) * d.rmax;
+      fp[s] = which == 0 ? Vp<NO, S>(d, 3, n, b, p) + (long long)(blockIdx.x * 32 - d.b_c0[b]) * d.rmax
+                         : Up<NO, S>(d, 3, n, b, p) + (long long)(blockIdx.x * 32 - d.b_r0[b]) * d.rmax;
+      pp[s] = Psrc<NO, R>(d, n, b, p, which);
     }
   }
   __syncthreads();
@@ -370,12 +377,16 @@ __global__ void __launch_bounds__(256) k_src_q(Dev d, int T, int uselist) {
     __syncthreads();
   }
   cx<R> s[NO2];
+  const int ring0 = c % d.ring;
+  const S* sring = static_cast<const S*>(d.SL) + ((long long)n * d.ring * d.nt + t) * NO2;
   for (int l0 = warp; l0 < nr; l0 += 8 * FOLD) {   // the uncompressed rows
 #pragma unroll
     for (int jj = 0; jj < FOLD; ++jj) {
       const int l = l0 + 8 * jj;
       if (l < nr) {
-        const S* sp = el<NO, S>(d.SL, d, n, c + l, t);
+        int slot = ring0 + l;
+        if (slot >= d.ring) slot -= d.ring;
+        const S* sp = sring + (long long)slot * d.nt * NO2;
 #pragma unroll
         for (int q = 0; q < NO2; ++q) s[q] = ldr<R>(sp + q);
         mac(s, false, gr + l * NO2);
@@ -383,12 +394,14 @@ __global__ void __launch_bounds__(256) k_src_q(Dev d, int T, int uselist) {
     }
     fold();
   }
+  const S* leaf = static_cast<const S*>(d.hod[3].leaf) + ((long long)n * d.leaftot + (long long)jt * (L * (L + 1) / 2)) * NO2;
   for (int l0 = warp; l0 < L; l0 += 8 * FOLD) {   // the leaf, both triangles
 #pragma unroll
     for (int jj = 0; jj < FOLD; ++jj) {
       const int l = A + l0 + 8 * jj;
       if (l < A + L) {
-        const S* sp = Lf<NO, S>(d, 3, n, jt, max(l, t), min(l, t));
+        const int hi = max(l, t) - A, lo = min(l, t) - A;
+        const S* sp = leaf + (hi * (hi + 1) / 2 + lo) * NO2;
 #pragma unroll
         for (int q = 0; q < NO2; ++q) s[q] = ldr<R>(sp + q);
         mac(s, l < t, gl + (l - A) * NO2);
@@ -404,12 +417,9 @@ __global__ void __launch_bounds__(256) k_src_q(Dev d, int T, int uselist) {
 #pragma unroll
       for (int u = 0; u < kEB; ++u) {
         const int e = e0 + stride * u, le = at(min(e, e1 - 1)), sl = le >> 7, q = le & 127;
-        const int which = (sl / (d.maxl * NO)) & 1, z = sl % NO, p = which == 0 ? x * NO + z : z * NO + x;
-        const S* F = static_cast<const S*>(which == 0 ? d.hod[3].V : d.hod[3].U) + base[sl] + tstr;
-        const cx<R>* pp = Psrc<NO, R>(d, n, blk[sl], p, which) + q * NO;
-        f[u] = e < e1 ? ldr<R>(F + q).conj() : cx<R>(0);
+        f[u] = e < e1 ? ldr<R>(fp[sl] + tstr + q).conj() : cx<R>(0);
 #pragma unroll
-        for (int y = 0; y < NO; ++y) P[u][y] = pp[y];
+        for (int y = 0; y < NO; ++y) P[u][y] = pp[sl][q * NO + y];
       }
 #pragma unroll
       for (int y = 0; y < NO; ++y) {
@@ -1280,7 +1290,7 @@ __global__ void __launch_bounds__(kLatMaxK) k_lattice_obs(Dev d, int t, double* 
 template <int NO, typename S>
 static cudaError_t src_q(const Dev& d, int T, cudaStream_t s) {
   const size_t n2 = NO * NO, es = sizeof(S), ns = 2 * (size_t)d.maxl * n2;
-  size_t bytes = ((size_t)d.r * n2 + 8 * n2 * 32) * 16 + (kSrcRing + 64) * n2 * es + (3 * ns + 1) * 4 + 8 + ns * 8;
+  size_t bytes = ((size_t)d.r * n2 + 8 * n2 * 32) * 16 + (kSrcRing + 64) * n2 * es + (2 * ns + 1) * 4 + 8 + ns * 16;
   const size_t list = ns * d.rmax * 2;
   const int uselist = ns * 128 <= 65536 && bytes + list <= 200 * 1024;
   if (uselist) bytes += list;
