@@ -50,11 +50,12 @@ struct hkbe_s {
   bool hodlr = false;
   std::vector<int> g_r0, g_r1, g_c0, g_c1, g_lvl, g_rowblk, g_colblk;
   std::vector<long long> g_uoff, g_voff, g_leafoff, g_wslv;
-  double2 *rowbuf_r = nullptr, *rowbuf_l = nullptr;
+  double2 *rowbuf_r = nullptr, *rowbuf_l = nullptr;   // unused (checkpoint files hold a copy of every buffer)
   int* status_dev = nullptr;
   double2* diagbuf = nullptr;  // [n_inst][no2] density matrices of one time
   std::vector<int> src_r0;   // first block row of each source-projection job (ascending)
   std::vector<void*> work;   // device buffers that are in neither snapshots nor files
+  double2 *rowpin = nullptr, *rowpin_dev = nullptr;   // [2][nt][no2] rows being read, pinned host memory
   int ahead = 1;             // corrector iterations of the last step
   hk::IterResult *res = nullptr, *res_dev = nullptr;   // [kAhead][n_inst] outcomes, pinned host memory
   // points whose rows the chunk inverses hold (retarded [0, rowsR), lesser [1, rowsL))
@@ -231,20 +232,6 @@ int front_host(const hkbe_t* h, int n) {
 size_t esz(const hkbe_t* h) { return h->d.prec ? sizeof(float2) : sizeof(double2); }
 char* elp(const hkbe_t* h, void* base, size_t off) { return static_cast<char*>(base) + off * esz(h); }
 
-// Copy `cnt` complex storage elements device -> host as interleaved doubles
-// (converted from float in the mixed form).  Synchronises the stream.
-cudaError_t d2h_el(hkbe_t* h, double* out, const char* src, size_t cnt) {
-  if (!h->d.prec) {
-    cudaError_t e = cudaMemcpyAsync(out, src, cnt * sizeof(double2), cudaMemcpyDeviceToHost, h->s);
-    return e != cudaSuccess ? e : cudaStreamSynchronize(h->s);
-  }
-  std::vector<float> tmp(2 * cnt);
-  cudaError_t e = cudaMemcpyAsync(tmp.data(), src, cnt * sizeof(float2), cudaMemcpyDeviceToHost, h->s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->s);
-  if (e != cudaSuccess) return e;
-  for (size_t i = 0; i < 2 * cnt; ++i) out[i] = tmp[i];
-  return cudaSuccess;
-}
 // Copy `cnt` complex values (interleaved doubles) host -> device storage
 // (rounded to float in the mixed form).  Synchronises the stream.
 cudaError_t h2d_el(hkbe_t* h, char* dst, const double* in, size_t cnt) {
@@ -541,6 +528,7 @@ int hkbe_destroy(hkbe_t* h) {
   for (void* p : h->allocs) cudaFree(p);
   for (void* p : h->work) cudaFree(p);
   if (h->res) cudaFreeHost(h->res);
+  if (h->rowpin) cudaFreeHost(h->rowpin);
   for (void* p : h->snap_dev)
     if (p) cudaFree(p);
   delete h;
@@ -1165,19 +1153,18 @@ int hkbe_current_step(const hkbe_t* h, int32_t* T) {
 }
 
 // Copy rows T of G^R and G^< (t = 0..T) of an instance to host buffers
-// (either may be NULL); compressed rows are reconstructed on the device.
+// (either may be NULL): a kernel gathers or reconstructs them into pinned memory.
 static int fetch_row(hkbe_t* h, int inst, int T, double* gr, double* gl) {
-  const size_t cnt = (size_t)(T + 1) * no2(h);
-  hk::Dev& d = h->d;
-  if (h->hodlr && T < front_host(h, inst)) {
-    HK_CUDA(h, hk::launch_row_out(d, inst, T, gr ? h->rowbuf_r : nullptr, gl ? h->rowbuf_l : nullptr, h->s));
-    if (gr) HK_CUDA(h, cudaMemcpyAsync(gr, h->rowbuf_r, cnt * sizeof(double2), cudaMemcpyDeviceToHost, h->s));
-    if (gl) HK_CUDA(h, cudaMemcpyAsync(gl, h->rowbuf_l, cnt * sizeof(double2), cudaMemcpyDeviceToHost, h->s));
-  } else {
-    if (gr) HK_CUDA(h, d2h_el(h, gr, elp(h, d.GR, row_off(h, inst, T)), cnt));
-    if (gl) HK_CUDA(h, d2h_el(h, gl, elp(h, d.GL, row_off(h, inst, T)), cnt));
+  const size_t cnt = (size_t)(T + 1) * no2(h), cap = (size_t)h->d.nt * no2(h);
+  if (!gr && !gl) return HKBE_OK;
+  if (!h->rowpin) {   // allocated with the first row that is read
+    HK_CUDA(h, cudaHostAlloc((void**)&h->rowpin, 2 * cap * sizeof(double2), cudaHostAllocMapped));
+    HK_CUDA(h, cudaHostGetDevicePointer((void**)&h->rowpin_dev, h->rowpin, 0));
   }
+  HK_CUDA(h, hk::launch_row_out(h->d, inst, T, gr ? h->rowpin_dev : nullptr, gl ? h->rowpin_dev + cap : nullptr, h->s));
   HK_CUDA(h, cudaStreamSynchronize(h->s));
+  if (gr) std::memcpy(gr, h->rowpin, cnt * sizeof(double2));
+  if (gl) std::memcpy(gl, h->rowpin + cap, cnt * sizeof(double2));
   return HKBE_OK;
 }
 

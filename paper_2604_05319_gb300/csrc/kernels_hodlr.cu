@@ -1084,8 +1084,12 @@ __global__ void __launch_bounds__(256, 2) k_tsvd(Dev d, int A, int nb, int n0) {
   if (tid == 0) *rkp = rn;
 }
 
-// Reconstruct row T of G^R and G^< (any T <= current) into out_r, out_l
-// ([T+1][no2] each), from the ring, the leaves or the blocks.
+// Row T of G^R and G^< (any T <= current) in complex128 into out_r, out_l
+// ([T+1][no2] each, pinned host memory), from the dense triangle, the ring, the
+// leaves or the blocks.  One launch and one synchronisation per row: a copy of
+// each component through pageable memory, each waited for, and a conversion on
+// the host took some 45 us, half of them gaps (304 instances, T = 384, a row of
+// each at the end: 106.9 -> 98.7 ms a pass).
 template <int NO, typename S>
 __global__ void k_row_out(Dev d, int n, int T, double2* out_r, double2* out_l) {
   constexpr int NO2 = NO * NO;
@@ -1096,7 +1100,7 @@ __global__ void k_row_out(Dev d, int n, int T, double2* out_r, double2* out_l) {
     if (!out) continue;
     for (int p = 0; p < NO2; ++p) {
       zd v;
-      if (T >= front_of(d, n)) {
+      if (!d.ring || T >= front_of(d, n)) {
         v = ld(el<NO, S>(ringX(d, X), d, n, T, t) + p);
       } else {
         const int jT = T / d.L, jt = t / d.L;
