@@ -113,25 +113,24 @@ HD zd cff_val(const cff& a) { return zd(ff_val(a.re), ff_val(a.im)); }
 // instruction per element would cost more than the products.
 __device__ __forceinline__ float f32_of(double x) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const int e = (int)((hi >> 20) & 0x7ffu) - 1023 + 127;
-  const unsigned sign = hi & 0x80000000u;
-  if (e <= 0) return __uint_as_float(sign);
-  if (e >= 255) return __uint_as_float(sign | 0x7f800000u);
-  const unsigned mag = ((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-  return __uint_as_float(sign | (mag + ((lo >> 28) & 1u)));
+  const int h = (int)(hi & 0x7fffffffu) - (896 << 20);   // exponent rebiased, in place
+  unsigned mag = __funnelshift_l(lo, (unsigned)h, 3) + ((lo >> 28) & 1u);
+  if (h < 1 << 20) mag = 0u;
+  if (h >= 255 << 20) mag = 0x7f800000u;
+  return __uint_as_float((hi & 0x80000000u) | mag);
 }
 // The same as an unevaluated pair: hi the top 24 bits of x (truncated), lo the
 // 29 bits after them (rounded to 24): x to about 2^-47 of it, without an FP64
 // instruction.  Magnitudes below 2^-74 keep hi only, below the FP32 range 0.
 __device__ __forceinline__ ffl ff_of_bits(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const int e = (int)((hi >> 20) & 0x7ffu) - 1023 + 127;
-  const unsigned sign = hi & 0x80000000u;
-  if (e <= 0) return {__uint_as_float(sign), 0.f};
-  if (e >= 255) return {__uint_as_float(sign | 0x7f800000u), 0.f};
-  const float h = __uint_as_float(sign | ((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
-  const float l = e > 52 ? (float)(lo & 0x1fffffffu) * __uint_as_float(sign | ((unsigned)(e - 52) << 23)) : 0.f;
-  return {h, l};
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), sign = hi & 0x80000000u;
+  const int h = (int)(hi & 0x7fffffffu) - (896 << 20);   // exponent rebiased, in place
+  unsigned mag = __funnelshift_l(lo, (unsigned)h, 3);
+  unsigned sc = (unsigned)((h >> 20) - 52) << 23;        // 2^(exponent - 52)
+  if (h < 53 << 20) sc = 0u;
+  if (h < 1 << 20) mag = 0u;
+  if (h >= 255 << 20) { mag = 0x7f800000u; sc = 0u; }
+  return {__uint_as_float(sign | mag), (float)(lo & 0x1fffffffu) * __uint_as_float(sign | sc)};
 }
 __device__ __forceinline__ zf ld_f32(const double2* p) {
   const double2 v = *p;

@@ -17,7 +17,9 @@ namespace hk {
 // SMs (3 instances, FP64, N_o = 1, T = 256: 19 us with groups of 32, 16 with 4).  (One
 // warp per node over all l read 16 bytes of every row and node apart, and its
 // lane 0 solved an N_o x N_o system per node: 158 us for 128 instances at
-// N_o = 2, T = 600; 110 us for 16 at N_o = 4, T = 290.)
+// N_o = 2, T = 600; 110 us for 16 at N_o = 4, T = 290.)  Bound by latency at two
+// CTAs per SM, so a thread's addresses advance by constants and the BDF rows are
+// loaded before their sum (128 x 600: 16.7 -> 14.7 ms of a pass).
 // ---------------------------------------------------------------------------
 template <int NO> constexpr int kNodes = 32 / (NO * NO);                      // nodes per CTA
 template <int NO> constexpr int kNodesFew = NO == 1 ? 4 : NO == 2 ? 2 : 1;    // with few instances
@@ -50,13 +52,14 @@ __device__ __forceinline__ void mixed_nodes(const Dev& d, int T, int group, int 
   const S* Sr = el<NO, S>(d.SR, d, n, T, 0) + z;
   constexpr int UB = 8;        // rows in flight
   KAcc<R> ka[NO];              // h sum_l w_l Sigma^R(T,l) G^tv(l, tau_i): FP32 products, compensated, in the complex64 form
-  for (int l0 = slice; l0 < T; l0 += NS * UB) {
+  const bool start = T < 2 * k + 1;   // the rule of the first steps has weights everywhere
+  const double2* Gl = G + slice * gs;
+  const S* Sl = Sr + (long long)slice * NO2;
+  const long long gst = NS * gs;      // between a slice's rows
+  for (int l0 = slice; l0 < T; l0 += NS * UB, Gl += UB * gst, Sl += UB * NS * NO2) {
     double2 g[UB];
 #pragma unroll
-    for (int u = 0; u < UB; ++u) {
-      const int l = l0 + NS * u;
-      g[u] = l < T ? G[l * gs] : make_double2(0, 0);
-    }
+    for (int u = 0; u < UB; ++u) g[u] = l0 + NS * u < T ? Gl[u * gst] : make_double2(0, 0);
 #pragma unroll
     for (int u0 = 0; u0 < UB; u0 += 4) {
       cx<R> pa[NO];
@@ -69,9 +72,9 @@ __device__ __forceinline__ void mixed_nodes(const Dev& d, int T, int group, int 
           cx<R> gv;
           if constexpr (MX) gv = zf(f32_of(g[u].x), f32_of(g[u].y));
           else gv = zd(g[u].x, g[u].y);
-          if (l <= k || T - l <= k || T < 2 * k + 1) gv = gv * rule_wr<R>(W, T, l);
+          if (start || l <= k || T - l <= k) gv = gv * rule_wr<R>(W, T, l);
 #pragma unroll
-          for (int x = 0; x < NO; ++x) pa[x] = cfma(ldr<R>(Sr + (long long)l * NO2 + x * NO), gv, pa[x]);
+          for (int x = 0; x < NO; ++x) pa[x] = cfma(ldr<R>(Sl + u * NS * NO2 + x * NO), gv, pa[x]);
         }
       }
 #pragma unroll
@@ -114,10 +117,11 @@ __device__ __forceinline__ void mixed_nodes(const Dev& d, int T, int group, int 
 #pragma unroll
       for (int zz = 0; zz < NO; ++zz) rhs += red[w2][x][i * NO2 + zz * NO + y];
     const double2* gp = tv<NO>(d.GTV, d, n, T, i0) + tid;
-    for (int j = 1; j <= k; ++j) {
-      const zd g = ld(gp - j * gs);
-      rhs += zd(W.ah[j] * g.im, -W.ah[j] * g.re);
-    }
+    zd g[5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) g[j] = j < k ? ld(gp - (j + 1) * gs) : zd();
+#pragma unroll
+    for (int j = 0; j < 5; ++j) rhs += zd(W.ah[j + 1] * g[j].im, -W.ah[j + 1] * g[j].re);
   }
   __syncthreads();
   zd* rs = &red[0][0][0];
