@@ -177,7 +177,7 @@ int walloc(hkbe_t* h, T** p, size_t count) {
   return e == cudaSuccess ? HKBE_OK : fail(h, HKBE_ERR_CUDA, cudaGetErrorString(e));
 }
 
-// Jobs of the source projections (block, side, chunk of kSrcChunk rows, first
+// Jobs of the source projections (block, side, chunk of src_chunk rows, first
 // partial-sum slot of a side longer than one chunk), sorted by the block's
 // first row so that the jobs of the built blocks come first.
 int src_jobs(hkbe_t* h) {
@@ -191,7 +191,7 @@ int src_jobs(hkbe_t* h) {
   for (int b : order)
     for (int side = 0; side < 2; ++side) {
       const int len = side == 0 ? h->g_r1[b] - h->g_r0[b] : h->g_c1[b] - h->g_c0[b];
-      const int nch = (len + hk::kSrcChunk - 1) / hk::kSrcChunk;
+      const int nch = (len + hk::src_chunk(len) - 1) / hk::src_chunk(len);
       for (int c = 0; c < nch; ++c) {
         tab.push_back(make_int4(b, side, c, parts));
         h->src_r0.push_back(h->g_r0[b]);

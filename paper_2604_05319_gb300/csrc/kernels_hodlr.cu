@@ -45,7 +45,7 @@ __device__ __forceinline__ cx<R>* Psrc(const Dev& d, int n, int b, int p, int wh
                                   ((((long long)n * d.nblk + b) * (NO * NO) + p) * 2 + which) * d.rmax * NO);
 }
 
-// The projections: one CTA per instance, block side and 256 of its rows (or
+// The projections: one CTA per instance, block side and 256 rows of it (or
 // columns), so that a block of a thousand rows is not one warp's loop over
 // all of them.  A warp takes one pair (N_o = 1, 2: 8 or 2 warps share a pair's
 // rows), all y, lanes packed by the pair's rank (8, 16 or 32 per factor row,
@@ -53,7 +53,12 @@ __device__ __forceinline__ cx<R>* Psrc(const Dev& d, int n, int b, int p, int wh
 // sum per CTA in spart; the CTA that finds itself the last of its side (a
 // counter that it sets back) adds them in their order, so the sum does not
 // depend on which one that is.
-// s_tab: (block, side, first row / 256, first slot of the side's partial sums).
+// In sides longer than that the chunks are of 128 rows: the chain per CTA halves,
+// and the sums over chunks are there anyway (1 instance, N_o = 2, T = 1089: 10.4 ->
+// 7.6 ms of a pass; 128 instances, T = 600: 36.4 -> 35.6).  128 rows everywhere
+// would split sides that need no partial sums (16 instances, N_o = 4, T = 290:
+// 17.6 -> 19.3).
+// s_tab: (block, side, chunk, first slot of the side's partial sums).
 template <int NO, typename S>
 __global__ void __launch_bounds__(256) k_src_proj(Dev d, int T) {
   pdl_start();
@@ -65,7 +70,8 @@ __global__ void __launch_bounds__(256) k_src_proj(Dev d, int T) {
   const int c = d.cdir;
   if (!d.active[n] || d.b_r0[b] >= c) return;
   const int lo = which == 0 ? d.b_r0[b] : d.b_c0[b], hi = which == 0 ? min(d.b_r1[b], c) : d.b_c1[b];
-  const int l0 = lo + ch * kSrcChunk, l1 = min(l0 + kSrcChunk, hi), nch = (hi - lo + kSrcChunk - 1) / kSrcChunk;
+  const int rows = src_chunk(which == 0 ? d.b_r1[b] - d.b_r0[b] : d.b_c1[b] - d.b_c0[b]);
+  const int l0 = lo + ch * rows, l1 = min(l0 + rows, hi), nch = (hi - lo + rows - 1) / rows;
   if (l0 >= hi) return;
   const DevW& W = d.w;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

@@ -103,7 +103,8 @@ struct Dev {
 };
 
 constexpr int kRingRows = 80;    // >= leaf + k + 1 uncompressed rows
-constexpr int kSrcChunk = 256;   // rows of a block side that one CTA of the source projections takes
+// rows of a block side of len rows that one CTA of the source projections takes
+__host__ __device__ constexpr int src_chunk(int len) { return len > 256 ? 128 : 256; }
 
 // ---- launchers (all on `s`) ----
 cudaError_t launch_extrapolate(const Dev& d, int T, cudaStream_t s);
