@@ -1457,13 +1457,16 @@ static size_t sweep_smem(const Dev& d, int* staged) {
   *staged = (d.ring && b <= 200 * 1024 && off32) ? 1 : 0;
   return *staged ? b : kBufBytes<NO>;
 }
-// Where the CTAs of the retarded sweep and of the mixed component's small node
-// groups all fit on the SMs at once (two per SM, one for N_o > 2), they are one
-// launch: the sweep is a chain on a few SMs, and the nodes need the others (3
-// instances, N_o = 1, FP64, T = 256: 106.9 -> 97.7 ms a pass).
+// In small batches the retarded sweep and the mixed component, in small node
+// groups, are one launch: the sweep is a chain on a few SMs, and the nodes need
+// the others.  In FP64 up to a CTA per SM (3 instances, T = 256: 97.0 -> 91.6 ms
+// a pass); beyond that the nodes hold FP64 pipes that the sweeps wait for (20 x
+// 150: 40.4 -> 41.9; N_o = 2, 10 x 150: 40.1 -> 44.5).  In complex64 up to four
+// (60 x 150: 22.4 -> 20.9; N_o = 4, 16 x 290: 111.3 -> 108.1); large batches fill
+// the SMs in large groups (N_o = 2, 128 x 600: 158 -> 179 in one launch).
 bool ret_takes_mixed(const Dev& d) {
   const int ni = d.no == 1 ? kNodesFew<1> : d.no == 2 ? kNodesFew<2> : kNodesFew<3>;
-  return (long long)(d.no + (d.r + ni - 1) / ni) * d.n_inst <= (d.no <= 2 ? 2 : 1) * 152;
+  return (long long)(d.no + (d.r + ni - 1) / ni) * d.n_inst <= (d.prec ? 4 : 1) * 152;
 }
 // A sweep runs as two launches with its ring kernel between them once kSplitRows
 // rows are compressed: before that, the ring's products in the chain cost less
