@@ -17,7 +17,7 @@ constexpr unsigned FULL = 0xffffffffu;
 // 15.8 -> 14.9; 8 x 300, N_o = 2, FP64: 73.5 -> 71.9).  Larger batches place
 // their CTAs worse when they come early, next to those still running (12 x 300,
 // N_o = 2, FP64: 76.6 -> 81.7; 40 x 150, FP64: 43.8 -> 44.8; lattice of 256,
-// T = 360: 90.7 -> 97.6), and the sweeps never come early for the same reason.
+// T = 360: 90.7 -> 97.6); for the sweeps themselves see early_sweep.
 constexpr int kEarlyCtas = 16;
 __device__ __forceinline__ void pdl_start() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -1477,6 +1477,11 @@ bool ret_takes_mixed(const Dev& d) {
 // idle: 43 -> 36 ms (1, FP64, T = 384), but 19.7 -> 21.6 (304, complex64).
 static bool split_les(const Dev& d) { return d.cdir >= kSplitRows; }
 static bool split_ret(const Dev& d) { return d.cdir >= kSplitRows && d.no * d.n_inst <= 152; }
+// A sweep comes early (see pdl_start) in the dense form with up to four CTAs: 1 x
+// 64, FP64, 10.7 -> 10.2 ms; 3 x 256 91.5 -> 90.8; 4 x 200 58.6 -> 57.6. Compressed
+// forms gain nothing there (4 x 300, FP64, 55.9 -> 56.6), and more CTAs end up two
+// to an SM next to the kernel before them (N_o = 2, 8 x 300, FP64, 79.8 -> 112.8).
+static bool early_sweep(const Dev& d) { return !d.ring && d.no * d.n_inst <= 4; }
 template <int NO, typename S>
 static cudaError_t sweep_ret(const Dev& d, int T, cudaStream_t s) {
   int staged = 0;
@@ -1488,7 +1493,7 @@ static cudaError_t sweep_ret(const Dev& d, int T, cudaStream_t s) {
   if (d.ring && T + 1 - d.cdir > kRingRows && d.cdir > 0) return cudaErrorInvalidValue;
   const int mix = with ? (d.r + kNodesFew<NO> - 1) / kNodesFew<NO> : 0;
   const bool split = split_ret(d);
-  if ((e = launch_on(false, kern, dim3(NO + mix, d.n_inst), 256, bytes, s, d, T, staged, split ? (int)kTop : (int)kAll)) !=
+  if ((e = launch_on(early_sweep(d), kern, dim3(NO + mix, d.n_inst), 256, bytes, s, d, T, staged, split ? (int)kTop : (int)kAll)) !=
           cudaSuccess ||
       !split)
     return e;
@@ -1497,7 +1502,7 @@ static cudaError_t sweep_ret(const Dev& d, int T, cudaStream_t s) {
   if ((e = allow_smem(k_ret_ring<NO, S>, rb)) != cudaSuccess || (e = allow_smem(leaves, bytes)) != cudaSuccess ||
       (e = launch_k(k_ret_ring<NO, S>, dim3(d.cdir / 32, d.n_inst), 256, rb, s, d, T)) != cudaSuccess)
     return e;
-  return launch_on(false, leaves, dim3(NO, d.n_inst), 256, bytes, s, d, T, staged, (int)kLeaves);
+  return launch_on(early_sweep(d), leaves, dim3(NO, d.n_inst), 256, bytes, s, d, T, staged, (int)kLeaves);
 }
 template <int NO, typename S>
 static cudaError_t sweep_les(const Dev& d, int T, cudaStream_t s) {
@@ -1508,12 +1513,12 @@ static cudaError_t sweep_les(const Dev& d, int T, cudaStream_t s) {
   const bool split = split_les(d);
   const int rows = T + 1 - d.cdir;
   if (split && rows > kRingRows) return cudaErrorInvalidValue;
-  if ((e = launch_on(false, k_les2<NO, S>, dim3(NO, d.n_inst), 256, bytes, s, d, T, staged,
+  if ((e = launch_on(early_sweep(d), k_les2<NO, S>, dim3(NO, d.n_inst), 256, bytes, s, d, T, staged,
                      split ? (int)kLeaves : (int)kAll)) != cudaSuccess ||
       !split)
     return e;
   if ((e = launch_k(k_les_ring<NO, S>, dim3((rows + 1) / 2, d.n_inst), 256, 0, s, d, T)) != cudaSuccess) return e;
-  return launch_on(false, k_les2<NO, S>, dim3(NO, d.n_inst), 256, bytes, s, d, T, staged, (int)kTop);
+  return launch_on(early_sweep(d), k_les2<NO, S>, dim3(NO, d.n_inst), 256, bytes, s, d, T, staged, (int)kTop);
 }
 cudaError_t launch_ret_h(const Dev& d, int T, cudaStream_t s) {
   HK_DISPATCH(d.no, return (sweep_ret<NO, S>(d, T, s)));
