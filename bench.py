@@ -172,7 +172,7 @@ def phase_flops(phase, T, k, no, L, blocks, ranks, hodlr):
 
 
 KERNEL_OF = {"ret": "k_ret2", "les": "k_les2", "src": "k_src_q"}
-_SWEEP_SRC = ["kernels_sweep.cu", "bulk_copy.cuh", "hodlr_util.cuh", "dev_util.cuh", "common.cuh", "state.h"]
+_SWEEP_SRC = ["kernels_sweep.cu", "mixed_nodes.cuh", "bulk_copy.cuh", "hodlr_util.cuh", "dev_util.cuh", "common.cuh", "state.h"]
 _SRC_SRC = ["kernels_hodlr.cu", "lattice.cuh", "hodlr_util.cuh", "dev_util.cuh", "common.cuh", "state.h"]
 SOURCE_OF = {"ret": _SWEEP_SRC, "les": _SWEEP_SRC, "src": _SRC_SRC}
 
