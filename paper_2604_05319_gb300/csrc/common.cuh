@@ -271,17 +271,31 @@ template <int N> HD M<N> dag(const M<N>& x) {
     for (int j = 0; j < N; ++j) m.a[i][j] = x.a[j][i].conj();
   return m;
 }
-template <int N> HD double maxabs_diff(const M<N>& x, const M<N>& y) {
+#ifdef __CUDACC__
+// The larger of two magnitudes by their bit patterns: values >= 0 order like
+// integers, infinity above every number and a NaN (sign aside) above infinity.
+// The measures of an iteration's change are folded with it, since fmax would
+// drop a NaN and a row of them would pass as converged; it takes no FP64
+// instruction.
+__device__ __forceinline__ double max_mag(double a, double b) {
+  const long long m = 0x7fffffffffffffffll, x = __double_as_longlong(a) & m, y = __double_as_longlong(b) & m;
+  return __longlong_as_double(x > y ? x : y);
+}
+__device__ __forceinline__ float max_mag(float a, float b) {
+  return __int_as_float(max(__float_as_int(a) & 0x7fffffff, __float_as_int(b) & 0x7fffffff));
+}
+template <int N> __device__ double maxabs_diff(const M<N>& x, const M<N>& y) {
   double e = 0;
 #pragma unroll
   for (int i = 0; i < N; ++i)
 #pragma unroll
     for (int j = 0; j < N; ++j) {
       zd d = x.a[i][j] - y.a[i][j];
-      e = fmax(e, sqrt(d.abs2()));
+      e = max_mag(e, sqrt(d.abs2()));
     }
   return e;
 }
+#endif
 // Solve A X = B (left) by Gauss-Jordan with partial pivoting; A is copied.
 template <int N> HD M<N> solve_left(M<N> A, M<N> B) {
 #pragma unroll
@@ -331,7 +345,7 @@ template <int N> HD M<N> solve_right(const M<N>& A, const M<N>& B) {
 
 // ---- atomics ----------------------------------------------------------------
 __device__ __forceinline__ void atomic_max_nonneg(double* addr, double v) {
-  // for non-negative doubles the IEEE bit pattern orders like unsigned ints
+  // for non-negative doubles the IEEE bit pattern orders like unsigned ints, a NaN above all others
   atomicMax(reinterpret_cast<unsigned long long*>(addr), (unsigned long long)__double_as_longlong(v));
 }
 

@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
       if (sl == 0) {
         V v;
         vset(v, y);
-        myerr = fmax(myerr, vdist(v, ldr<R>(sp(T - s) + j)));
+        myerr = max_mag(myerr, vdist(v, ldr<R>(sp(T - s) + j)));
         Yl[(T - s) & 63][j] = v;
         st(yp(T - s) + j, y);
         if constexpr (MX) vstore(sp(T - s) + j, v);
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
   if (above && tid < NO) {
     V v;
     vset(v, (tid == irow) ? zd(0, -1) : zd());
-    myerr = fmax(myerr, vdist(v, ldr<R>(sp(T) + tid)));
+    myerr = max_mag(myerr, vdist(v, ldr<R>(sp(T) + tid)));
     st(yp(T) + tid, v64(v));
     if constexpr (MX) vstore(sp(T) + tid, v);
   }
@@ -721,7 +721,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
 #pragma unroll
         for (int off = 1; off < 8; off <<= 1) out = vadd(out, vshfl_xor(out, off));
         if (sl == 0 && ti < cn) {
-          myerr = fmax(myerr, vdist(out, Old[ti][j]));
+          myerr = max_mag(myerr, vdist(out, Old[ti][j]));
           Yl[(a + ti) & 63][j] = out;
           vstore(sp(a + ti) + j, out);
         }
@@ -733,7 +733,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
   }
   write64(wa, wn);
   const double e1 = sqrt(warp_max((double)myerr));
-  if (lane == 0 && e1 > 0) atomic_max_nonneg(&serr, e1);
+  if (lane == 0) atomic_max_nonneg(&serr, e1);
   __syncthreads();
   if (tid == 0) atomic_max_nonneg(d.err + n, serr);
   // after a timed-out wait, a copy may still be in flight into this CTA's
@@ -798,7 +798,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
     const zd x = ld(d.x0 + (long long)n * NO2 + m * NO + jc);
     V v;
     vset(v, x);
-    myerr = fmax(myerr, vdist(v, ldr<R>(sp(0) + m * NO + jc)));
+    myerr = max_mag(myerr, vdist(v, ldr<R>(sp(0) + m * NO + jc)));
     Xl[0][m] = v;
     st(xp(0) + m * NO + jc, x);
     if constexpr (MX) vstore(sp(0) + m * NO + jc, v);
@@ -1059,7 +1059,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
 #pragma unroll
         for (int off = 1; off < 8; off <<= 1) out = vadd(out, vshfl_xor(out, off));
         if (sl == 0 && ti < fn) {
-          myerr = fmax(myerr, vdist(out, Old[ti][m]));
+          myerr = max_mag(myerr, vdist(out, Old[ti][m]));
           Xl[(a + ti) & 63][m] = out;
           vstore(sp(a + ti) + m * NO + jc, out);
         }
@@ -1106,7 +1106,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
           for (int m = 0; m < NO; ++m) {
             V v;
             vset(v, x[m]);
-            myerr = fmax(myerr, vdist(v, Old[fn][m]));
+            myerr = max_mag(myerr, vdist(v, Old[fn][m]));
             st(xp(T) + m * NO + jc, x[m]);
             if constexpr (MX) vstore(sp(T) + m * NO + jc, v);
           }
@@ -1117,7 +1117,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
   }
   write64(wa, wn);
   const double e1 = sqrt(warp_max((double)myerr));
-  if (lane == 0 && e1 > 0) atomic_max_nonneg(&serr, e1);
+  if (lane == 0) atomic_max_nonneg(&serr, e1);
   __syncthreads();
   if (tid == 0) atomic_max_nonneg(d.err + n, serr);
   // after a timed-out wait, a copy may still be in flight into this CTA's

@@ -56,17 +56,17 @@ __global__ void __launch_bounds__(32) k_ret_sf_start(Dev d, int T) {
   for (int row = lane; row < ns; row += 32) {
     const int s = row / NO + 1, j = row % NO;
     double2* p = el<NO, S>(d.GR, d, n, T, T - s) + irow * NO + j;
-    err = fmax(err, sqrt((sB[row] - ld(p)).abs2()));
+    err = max_mag(err, sqrt((sB[row] - ld(p)).abs2()));
     st(p, sB[row]);
   }
   if (lane < NO) {
     double2* p = el<NO, S>(d.GR, d, n, T, T) + irow * NO + lane;
     const zd v = lane == irow ? zd(0, -1) : zd();
-    err = fmax(err, sqrt((v - ld(p)).abs2()));
+    err = max_mag(err, sqrt((v - ld(p)).abs2()));
     st(p, v);
   }
   err = warp_max(err);
-  if (lane == 0 && err > 0) atomic_max_nonneg(d.err + n, err);
+  if (lane == 0) atomic_max_nonneg(d.err + n, err);
 }
 
 // t' = T - n, n > k: one thread per (t', instance).  The threads of a block

@@ -139,7 +139,7 @@ __device__ __forceinline__ void mixed_nodes(const Dev& d, int T, int group, int 
   if (lane == 0) serr[warp] = e;
   __syncthreads();
   if (tid == 0) {
-    for (int w2 = 1; w2 < 8; ++w2) e = fmax(e, serr[w2]);
+    for (int w2 = 1; w2 < 8; ++w2) e = max_mag(e, serr[w2]);
     atomic_max_nonneg(d.err + n, e);
   }
 }
