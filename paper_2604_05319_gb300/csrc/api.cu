@@ -510,9 +510,11 @@ int hkbe_create(const hkbe_params* p, const int32_t* nt_per_inst, void* stream, 
       return rc;
     }
   }
-  cudaError_t e = cudaStreamSynchronize(h->s);
+  cudaError_t e = hk::open_sweeps(d);
+  if (e == cudaSuccess) e = hk::open_history(d);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->s);
   if (e != cudaSuccess) {
-    g_create_error = std::string("cudaStreamSynchronize: ") + cudaGetErrorString(e);
+    g_create_error = std::string("hkbe_create: ") + cudaGetErrorString(e);
     hkbe_destroy(h);
     return HKBE_ERR_CUDA;
   }

@@ -42,6 +42,25 @@ inline cudaError_t launch_k(void (*kern)(P...), dim3 grid, int threads, size_t s
   return launch_on(d.no * d.n_inst <= kEarlyCtas, kern, grid, threads, smem, s, d, args...);
 }
 
+// Let a kernel ask for all the dynamic shared memory that its static arrays leave
+// of a CTA's opt-in limit; *room is lowered to that size.  The setting belongs to
+// the kernel and the device, not to a handle: it is made when a handle is created,
+// always to this same value, and a launch never touches it.  Set to a launch's own
+// size before each launch, one thread's handle could lower it between another
+// thread's setting and launch, which was then refused.
+template <typename K>
+inline cudaError_t open_smem(K kern, int* room) {
+  int dev = 0, cap = 0;
+  cudaFuncAttributes a;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kern);
+  if (e != cudaSuccess) return e;
+  const int left = cap - (int)a.sharedSizeBytes;
+  *room = left < *room ? left : *room;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, left);
+}
+
 __device__ __forceinline__ long long tri(int T) { return (long long)T * (T + 1) / 2; }
 
 // First uncompressed row of instance n.  An instance whose last step comes

@@ -1304,11 +1304,16 @@ static cudaError_t src_q(const Dev& d, int T, cudaStream_t s) {
   const size_t list = ns * d.rmax * 2;
   const int uselist = ns * 128 <= 65536 && bytes + list <= 200 * 1024;
   if (uselist) bytes += list;
-  if (bytes > 227 * 1024) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(k_src_q<NO, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
   const int nrow = T + 1 - d.cdir;
   return launch_k(k_src_q<NO, S>, dim3(d.cdir / 32 + (nrow + 7) / 8, d.n_inst), 256, bytes, s, d, T, uselist);
+}
+cudaError_t open_history(const Dev& d) {
+  cudaError_t e = cudaErrorInvalidValue;
+  int room = 1 << 30;
+  HK_DISPATCH(d.no, {
+    if ((e = open_smem(k_src_q<NO, S>, &room)) == cudaSuccess) e = open_smem(k_tsvd<NO, S>, &room);
+  })
+  return e;
 }
 cudaError_t launch_src_h(const Dev& d, int T, int njob, cudaStream_t s) {
   if (d.cdir > 0 && T + 1 - d.cdir > kSrcRing) return cudaErrorInvalidValue;
@@ -1326,12 +1331,9 @@ cudaError_t launch_compress(const Dev& d, int A, int nb, cudaStream_t s) {
     HK_DISPATCH(d.no, (k_comp_copy<NO, S><<<g, 256, 0, s>>>(d, A, nb)));
   }
   HK_DISPATCH(d.no, {
-    auto kern = k_tsvd<NO, S>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTsvdSmem);
-    if (e != cudaSuccess) return e;
     for (int n0 = 0; n0 < d.n_inst; n0 += d.tsvd_group) {
       dim3 g(4 * d.maxl * d.no * d.no, min(d.tsvd_group, d.n_inst - n0));
-      kern<<<g, 256, kTsvdSmem, s>>>(d, A, nb, n0);
+      k_tsvd<NO, S><<<g, 256, kTsvdSmem, s>>>(d, A, nb, n0);
     }
   })
   return cudaGetLastError();

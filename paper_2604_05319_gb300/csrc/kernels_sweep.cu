@@ -1435,26 +1435,15 @@ __global__ void __launch_bounds__(256) k_inv_rows(Dev d, int T, int r0, int r1, 
     default: return cudaErrorInvalidValue;                                      \
   }
 
-// Static plus dynamic shared memory above the 48 KB default needs an opt-in
-// per kernel (the static arrays of the sweeps take 24-31 KB).
-template <typename K>
-static cudaError_t allow_smem(K kern, size_t bytes) {
-  cudaFuncAttributes a;
-  cudaError_t e = cudaFuncGetAttributes(&a, kern);
-  if (e != cudaSuccess) return e;
-  if (a.sharedSizeBytes + bytes <= 48 * 1024) return cudaSuccess;
-  if (a.sharedSizeBytes + bytes > 227 * 1024) return cudaErrorInvalidValue;
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
 // Dynamic shared memory of a sweep: the buffer of the staged inverse and, in
 // the compressed form, the projections of the blocks over a leaf, unless ranks
-// and levels make them larger than 200 KB in all (then they stay in global
-// memory).
+// and levels make them larger than 200 KB in all, or than the kernels' static
+// arrays leave room for (4 to 27 KB of them; then they stay in global memory).
 template <int NO, typename S>
 static size_t sweep_smem(const Dev& d, int* staged) {
   const size_t b = kBufBytes<NO> + (d.ring ? SweepMem<NO, typename Bulk<S>::R>::bytes(d.maxl, d.rmax) : 0);
   const bool off32 = std::max(d.utot, d.vtot) * d.rmax < (1ll << 32);
-  *staged = (d.ring && b <= 200 * 1024 && off32) ? 1 : 0;
+  *staged = (d.ring && b <= std::min<size_t>(200 * 1024, d.sweep_room) && off32) ? 1 : 0;
   return *staged ? b : kBufBytes<NO>;
 }
 // In small batches the retarded sweep and the mixed component, in small node
@@ -1488,8 +1477,7 @@ static cudaError_t sweep_ret(const Dev& d, int T, cudaStream_t s) {
   const size_t bytes = sweep_smem<NO, S>(d, &staged);
   const bool with = ret_takes_mixed(d);
   auto kern = with ? k_ret2<NO, S, true> : k_ret2<NO, S, false>;
-  cudaError_t e = allow_smem(kern, bytes);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   if (d.ring && T + 1 - d.cdir > kRingRows && d.cdir > 0) return cudaErrorInvalidValue;
   const int mix = with ? (d.r + kNodesFew<NO> - 1) / kNodesFew<NO> : 0;
   const bool split = split_ret(d);
@@ -1498,18 +1486,14 @@ static cudaError_t sweep_ret(const Dev& d, int T, cudaStream_t s) {
       !split)
     return e;
   const size_t rb = NO * NO * (8 * 32 * 16 + kRingRows * sizeof(S));
-  auto leaves = k_ret2<NO, S, false>;
-  if ((e = allow_smem(k_ret_ring<NO, S>, rb)) != cudaSuccess || (e = allow_smem(leaves, bytes)) != cudaSuccess ||
-      (e = launch_k(k_ret_ring<NO, S>, dim3(d.cdir / 32, d.n_inst), 256, rb, s, d, T)) != cudaSuccess)
-    return e;
-  return launch_on(early_sweep(d), leaves, dim3(NO, d.n_inst), 256, bytes, s, d, T, staged, (int)kLeaves);
+  if ((e = launch_k(k_ret_ring<NO, S>, dim3(d.cdir / 32, d.n_inst), 256, rb, s, d, T)) != cudaSuccess) return e;
+  return launch_on(early_sweep(d), k_ret2<NO, S, false>, dim3(NO, d.n_inst), 256, bytes, s, d, T, staged, (int)kLeaves);
 }
 template <int NO, typename S>
 static cudaError_t sweep_les(const Dev& d, int T, cudaStream_t s) {
   int staged = 0;
   const size_t bytes = sweep_smem<NO, S>(d, &staged);
-  cudaError_t e = allow_smem(k_les2<NO, S>, bytes);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   const bool split = split_les(d);
   const int rows = T + 1 - d.cdir;
   if (split && rows > kRingRows) return cudaErrorInvalidValue;
@@ -1519,6 +1503,18 @@ static cudaError_t sweep_les(const Dev& d, int T, cudaStream_t s) {
     return e;
   if ((e = launch_k(k_les_ring<NO, S>, dim3((rows + 1) / 2, d.n_inst), 256, 0, s, d, T)) != cudaSuccess) return e;
   return launch_on(early_sweep(d), k_les2<NO, S>, dim3(NO, d.n_inst), 256, bytes, s, d, T, staged, (int)kTop);
+}
+cudaError_t open_sweeps(Dev& d) {
+  cudaError_t e = cudaErrorInvalidValue;
+  int ring = 1 << 30;
+  d.sweep_room = 1 << 30;
+  HK_DISPATCH(d.no, {
+    if ((e = open_smem(k_ret2<NO, S, true>, &d.sweep_room)) == cudaSuccess &&
+        (e = open_smem(k_ret2<NO, S, false>, &d.sweep_room)) == cudaSuccess &&
+        (e = open_smem(k_les2<NO, S>, &d.sweep_room)) == cudaSuccess)
+      e = open_smem(k_ret_ring<NO, S>, &ring);
+  })
+  return e;
 }
 cudaError_t launch_ret_h(const Dev& d, int T, cudaStream_t s) {
   HK_DISPATCH(d.no, return (sweep_ret<NO, S>(d, T, s)));

@@ -65,6 +65,7 @@ struct Dev {
   double2* fring;      // products of the uncompressed rows, retarded [n][no][nt][no], then lesser [n][kRingRows][no2]
   double2* hinv;       // [n][(2k no)^2] inverse of the retarded head of the current step
   int nchunk;          // ceil(nt / 32)
+  int sweep_room;      // largest dynamic shared memory that both sweeps may ask for
   int nfrozR, nfrozL;  // chunks [0, nfroz) of each sweep have a complete inverse
   long long ntri;  // nt*(nt+1)/2
   double h, beta;
@@ -105,6 +106,11 @@ struct Dev {
 constexpr int kRingRows = 80;    // >= leaf + k + 1 uncompressed rows
 // rows of a block side of len rows that one CTA of the source projections takes
 __host__ __device__ constexpr int src_chunk(int len) { return len > 256 ? 128 : 256; }
+
+// Shared-memory limits of the kernels that a handle of this form launches (and
+// d.sweep_room); once per handle, before its first step.
+cudaError_t open_sweeps(Dev& d);
+cudaError_t open_history(const Dev& d);
 
 // ---- launchers (all on `s`) ----
 cudaError_t launch_extrapolate(const Dev& d, int T, cudaStream_t s);
