@@ -367,8 +367,9 @@ int hkbe_rewind(hkbe_t* h);
  * memory instead).  hkbe_snapshot_save copies every device buffer of the
  * handle that holds state (all but its scratch workspaces) into a second
  * device allocation made on the first call and reused afterwards, together
- * with the step counter and the compression front.  hkbe_snapshot_restore copies it back: stepping the
- * restored handle repeats the run from the saved step bit for bit.
+ * with the step counter, the model and the compression front.
+ * hkbe_snapshot_restore copies it back: stepping the restored handle repeats
+ * the run from the saved step bit for bit, whatever model was set in between.
  * hkbe_snapshot_free releases the copy (hkbe_destroy does too).  Both run on
  * the handle's stream and return after it has finished.  Errors:
  * HKBE_ERR_ARG (null, before the bootstrap, restore without a saved copy),

@@ -75,6 +75,8 @@ struct hkbe_s {
   std::vector<const void*> scratch;  // buffers whose contents do not outlive a kernel phase
   size_t snap_bytes = 0;
   int snap_cur = -1, snap_cdir = 0, snap_nfrozR = 0, snap_nfrozL = 0;
+  int snap_model = 0, snap_lat_L = 0, snap_lat_ys = 0;
+  bool snap_self_consistent = false;
 };
 
 namespace {
@@ -1364,6 +1366,10 @@ int hkbe_snapshot_save(hkbe_t* h) {
   h->snap_cdir = h->d.cdir;
   h->snap_nfrozR = h->d.nfrozR;
   h->snap_nfrozL = h->d.nfrozL;
+  h->snap_model = h->d.model;
+  h->snap_lat_L = h->lat_L;
+  h->snap_lat_ys = h->lat_ys;
+  h->snap_self_consistent = h->self_consistent;
   return HKBE_OK;
 }
 
@@ -1374,6 +1380,12 @@ int hkbe_snapshot_restore(hkbe_t* h) {
   for (size_t i = 0; i < h->allocs.size(); ++i)
     if (h->snap_dev[i])
       HK_CUDA(h, cudaMemcpyAsync(h->allocs[i], h->snap_dev[i], h->alloc_bytes[i], cudaMemcpyDeviceToDevice, h->s));
+  // the model whose parameters came back, and what is derived from them
+  h->d.model = h->snap_model;
+  h->lat_L = h->snap_lat_L;
+  h->lat_ys = h->snap_lat_ys;
+  h->self_consistent = h->snap_self_consistent;
+  HK_CUDA(h, hk::launch_nbose(h->d, h->s));
   HK_CUDA(h, cudaStreamSynchronize(h->s));
   h->cur = h->snap_cur;
   h->d.cdir = h->snap_cdir;
