@@ -266,19 +266,24 @@ __device__ __forceinline__ void lu_apply(int n, const zd* A, const int* piv, zd*
 
 // 1 / a: the real reciprocal from an FP32 estimate by two Newton steps (an FP64
 // division is a sequence of some ten dependent FP64 instructions, each holding
-// the pipe for 64 cycles of the warp).
+// the pipe for 64 cycles of the warp).  The exponent of |a|^2 is set aside
+// meanwhile, so the estimate covers the range of FP64.
 __device__ __forceinline__ zd crecip(const zd& a) {
   const double d = a.abs2();
-  if (!(d > 1e-36 && d < 1e36)) return cdiv(zd(1.0), a);
-  double y = (double)(1.0f / (float)d);
-  y = y * fma(-d, y, 2.0);
-  y = y * fma(-d, y, 2.0);
+  const int hi = __double2hiint(d), e = (hi >> 20) - 1023;
+  if (e < -1021 || e > 1020) return cdiv(zd(1.0), a);   // zero, subnormal, about to overflow, not finite
+  const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(d));   // d = m 2^e
+  double y = (double)(1.0f / (float)m);
+  y = y * fma(-m, y, 2.0);
+  y = y * fma(-m, y, 2.0);
+  y = __hiloint2double(__double2hiint(y) - (e << 20), __double2loint(y));
   return zd(a.re * y, -a.im * y);
 }
-// |a|^2 in FP32: a key to choose pivots by
-__device__ __forceinline__ float pivot_key(const zd& a) {
-  const float x = (float)a.re, y = (float)a.im;
-  return fmaf(x, x, y * y);
+// A key to choose pivots by: the upper words of max(|re|, |im|), which order like
+// the values over the range of FP64 (squares in FP32 order nothing outside 1e-22
+// to 1.8e19) and take no FP64 instruction.
+__device__ __forceinline__ int pivot_key(const zd& a) {
+  return max(__double2hiint(a.re) & 0x7fffffff, __double2hiint(a.im) & 0x7fffffff);
 }
 // Inverse of the NO x NO matrix A (shared memory, row-major) into out by one
 // warp, Gauss-Jordan with partial pivoting; lane e < NO^2 owns element e of A
@@ -299,9 +304,9 @@ __device__ __forceinline__ void warp_inv(const zd* A, zd* tmp, zd* out) {
   __syncwarp();
   for (int p = 0; p < NO; ++p) {
     int pr = p;
-    float best = pivot_key(tmp[p * NO + p]);
+    int best = pivot_key(tmp[p * NO + p]);
     for (int q = p + 1; q < NO; ++q) {
-      const float v = pivot_key(tmp[q * NO + p]);
+      const int v = pivot_key(tmp[q * NO + p]);
       if (v > best) { best = v; pr = q; }
     }
     zd a = zd(), o = zd(), f = zd(), ap = zd(), op = zd(), piv = tmp[pr * NO + p];
@@ -333,11 +338,11 @@ static __device__ __noinline__ void gj_inverse(int n, zd* A, int ld) {
   const int tid = threadIdx.x;
   for (int c = 0; c < n; ++c) {
     if (tid < 32) {
-      float v = (tid >= c && tid < n) ? pivot_key(A[tid * ld + c]) : -1.f;
+      int v = (tid >= c && tid < n) ? pivot_key(A[tid * ld + c]) : -1;
       int p = tid;
 #pragma unroll
       for (int off = 16; off; off >>= 1) {
-        const float v2 = __shfl_xor_sync(FULL, v, off);
+        const int v2 = __shfl_xor_sync(FULL, v, off);
         const int p2 = __shfl_xor_sync(FULL, p, off);
         if (v2 > v || (v2 == v && p2 < p)) { v = v2; p = p2; }
       }
