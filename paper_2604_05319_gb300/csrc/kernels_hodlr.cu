@@ -550,6 +550,8 @@ __device__ __forceinline__ cff vconj(const cff& a) { return {a.re, ff_neg(a.im)}
 __device__ __forceinline__ zd vof(const double2& a) { return zd(a.x, a.y); }
 __device__ __forceinline__ cff vof(const float2& a) { return {{a.x, 0.f}, {a.y, 0.f}}; }
 __device__ __forceinline__ double vnorm2(const zd& a) { return a.abs2(); }
+__device__ __forceinline__ float vtop(const zd&) { return 0.f; }
+__device__ __forceinline__ float vtop(const cff& a) { return fmaxf(fabsf(a.re.hi), fabsf(a.im.hi)); }
 __device__ __forceinline__ float vnorm2(const cff& a) { return a.re.hi * a.re.hi + a.im.hi * a.im.hi; }
 // 1 / sqrt(x) from an FP32 estimate by two Newton steps
 __device__ __forceinline__ double rsq(double x) {
@@ -569,14 +571,35 @@ __device__ __forceinline__ ffl rsq(const ffl& x) {
   for (int i = 0; i < 2; ++i) y = ff_mul(y, ff_add(ff_mul(ff_mul(xh, y), y), {1.5f, 0.f}));
   return y;
 }
-__device__ __forceinline__ float r32(double x) { return (float)x; }
-__device__ __forceinline__ float r32(const ffl& x) { return x.hi; }
+// x >= 0 as m 4^e, m in [1, 4), of FP32 precision (zero: m = 0), on the integer
+// pipes: the decisions on a rotation are taken in FP32 without its range
+struct Quad {
+  float m;
+  int e;
+};
+__device__ __forceinline__ Quad quad_of(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), f = hi >> 20 & 0x7ffu, e = f - 1023u;
+  const unsigned m = (127u + (e & 1u)) << 23 | (hi & 0xfffffu) << 3 | (unsigned)__double2loint(x) >> 29;
+  return {f ? __uint_as_float(m) : 0.f, (int)e >> 1};
+}
+__device__ __forceinline__ Quad quad_of(const ffl& x) {
+  const unsigned b = __float_as_uint(x.hi), f = b >> 23 & 0xffu, e = f - 127u;
+  return {f ? __uint_as_float((127u + (e & 1u)) << 23 | (b & 0x7fffffu)) : 0.f, (int)e >> 1};
+}
+// a 2^e (e kept within the exponents of normal numbers)
+__device__ __forceinline__ zd vldexp(const zd& a, int e) {
+  return a * __hiloint2double((1023 + min(max(e, -1022), 1022)) << 20, 0);
+}
+__device__ __forceinline__ cff vldexp(const cff& a, int e) {
+  const float s = __int_as_float((127 + min(max(e, -126), 126)) << 23);
+  return {{a.re.hi * s, a.re.lo * s}, {a.im.hi * s, a.im.lo * s}};
+}
+__device__ __forceinline__ double rtop(double x) { return x; }
+__device__ __forceinline__ float rtop(const ffl& x) { return x.hi; }
 __device__ __forceinline__ double r64(double x) { return x; }
 __device__ __forceinline__ double r64(const ffl& x) { return ff_val(x); }
 template <typename S> struct Re { using t = double; };
 template <> struct Re<float2> { using t = ffl; };
-__device__ __forceinline__ double rof1(float x, double2*) { return (double)x; }
-__device__ __forceinline__ ffl rof1(float x, float2*) { return {x, 0.f}; }
 __device__ __forceinline__ float vnorm32(const zd& a) { return (float)a.abs2(); }
 __device__ __forceinline__ float vnorm32(const cff& a) { return vnorm2(a); }
 __device__ __forceinline__ double rof(double x, double2*) { return x; }
@@ -651,6 +674,7 @@ __global__ void __launch_bounds__(256, 2) k_tsvd(Dev d, int A, int nb, int n0) {
   // E <- new rows (and max |E| for the complex64 rounding floor below).  The
   // complex64 form reads them from its FP64 copies: rows free of storage
   // rounding, whose residuals against V hold real directions only.
+  float top = 0.f;
   {
     void* ring = ringX(d, X);
     double emax = 0.0;
@@ -660,19 +684,45 @@ __global__ void __launch_bounds__(256, 2) k_tsvd(Dev d, int A, int nb, int n0) {
         if (d.ring64[X]) v = ld_split<S>(el64<NO>(d, X, n, A + i, c0 + l) + p);
         else vset(v, ld(el<NO, S>(ring, d, n, A + i, c0 + l) + p));
         emax = fmax(emax, (double)vnorm2(v));
+        top = fmaxf(top, vtop(v));
         Em[(long long)i * ncol + l] = v;
       }
     emax = warp_max(emax);
-    if (lane == 0) s_w[warp] = emax;
+    top = (float)warp_max((double)top);
+    if (lane == 0) { s_w[warp] = emax; s_norm[warp] = top; }
   }
   __syncthreads();
+  // The complex64 form's squares have the range of FP32: rows and singular values
+  // far from 1 are brought there by a power of two, which changes no digit, and the
+  // new singular values taken back.
+  double up = 1.0, down = 1.0;
+  if constexpr (sizeof(S) == sizeof(float2)) {
+    double big = r > 0 ? Sv[0] : 0.0;
+    for (int w2 = 0; w2 < 8; ++w2) big = fmax(big, s_norm[w2]);
+    if (big > 0.0 && (big < 0x1p-20 || big > 0x1p50)) {   // (the same for every thread)
+      const int e = min(max((__double2hiint(big) >> 20) - 1023, -126), 126);
+      up = __hiloint2double((1023 - e) << 20, 0);
+      down = __hiloint2double((1023 + e) << 20, 0);
+      __syncthreads();
+      double emax = 0.0;
+      for (int i = warp; i < nb; i += 8)
+        for (int l = lane; l < ncol; l += 32) {
+          const V v = vldexp(Em[(long long)i * ncol + l], -e);
+          emax = fmax(emax, (double)vnorm2(v));
+          Em[(long long)i * ncol + l] = v;
+        }
+      emax = warp_max(emax);
+      if (lane == 0) s_w[warp] = emax;
+      __syncthreads();
+    }
+  }
   // Truncation threshold: eps_SVD, raised in the complex64 storage form to
   // the rounding floor of the appended rows.  Their rounding is a matrix of
   // independent entries below 2^-24 max|E|, whose largest singular value
   // stays below 2^-24 max|E| (sqrt(nb) + sqrt(ncol)); directions under that
   // level are storage noise, and keeping them would let the rank grow by the
   // leaf size at every append.
-  double tol = d.svd_tol;
+  double tol = d.svd_tol * up;
   if (sizeof(S) == sizeof(float2)) {
     double emax = 0.0;
     for (int w2 = 0; w2 < 8; ++w2) emax = fmax(emax, s_w[w2]);
@@ -870,7 +920,7 @@ __global__ void __launch_bounds__(256, 2) k_tsvd(Dev d, int A, int nb, int n0) {
   for (int e = tid; e < nk * m; e += blockDim.x) {
     const int col = e / m, row = e % m;
     V v;
-    if (row < r) vset(v, col == row ? zd(Sv[row]) : zd());
+    if (row < r) vset(v, col == row ? zd(Sv[row] * up) : zd());
     else if (col < r) v = Pm[(long long)(row - r) * rmax + col];
     else v = Cm[(long long)(row - r) * L + (col - r)];
     Kw[e] = v;
@@ -932,7 +982,7 @@ __global__ void __launch_bounds__(256, 2) k_tsvd(Dev d, int A, int nb, int n0) {
   }
   __syncthreads();
   // ---- one-sided Jacobi (Hestenes) on the columns of R^dagger, round-robin pairing, a half-warp per pair ----
-  const float small2 = (float)(1e-6 * tol * tol);   // two columns both this small are truncated: left as they are
+  const auto small2 = (decltype(rtop(R())))(1e-6 * tol * tol);   // two columns both this small are truncated: left as they are
   const int npad = nr + (nr & 1);
   for (int sweep = 0; sweep < 40; ++sweep) {
     if (tid == 0) s_flag = 0;
@@ -961,20 +1011,24 @@ __global__ void __launch_bounds__(256, 2) k_tsvd(Dev d, int A, int nb, int n0) {
           }
         const R al = rsum(na.get(), 16), be = rsum(nbm.get(), 16);
         const V ga = vsum(ng.get(), 16);
-        const float fa = r32(al), fb = r32(be);
-        // |<a, b>| in FP32, scaled by a power of two so that its square stays in range
-        const float gm = fmaxf(fabsf(r32(ga.re)), fabsf(r32(ga.im)));
-        const float sc = __uint_as_float((254u - min(max((__float_as_uint(gm) >> 23) & 0xffu, 1u), 253u)) << 23);
-        const V gs = vscl(ga, rof1(sc, (S*)nullptr));
-        const float fg = gm > 0.f ? sqrtf(vnorm32(gs)) / sc : 0.f;
+        const Quad qa = quad_of(al), qb = quad_of(be);   // |a|^2 = fa 4^ea, |b|^2 = fb 4^eb, <a, b> = gs 2^(ea + eb)
+        const V gs = vldexp(ga, -(qa.e + qb.e));
+        const float fa = qa.m, fb = qb.m, fg = sqrtf(vnorm32(gs));
+        const int de = qb.e - qa.e;
         const float eps = sizeof(S) == sizeof(double2) ? 1e-14f : 1e-13f;
-        act = act && gm > 0.f && !(fg * rsqrtf(fa) <= eps * sqrtf(fb)) && fmaxf(fa, fb) >= small2;
+        act = act && fa * fb > 0.f && fg > eps * sqrtf(fa * fb) && (rtop(al) >= small2 || rtop(be) >= small2) && abs(de) <= 100;
         if (act) {
           Nrm2<S> g2;
           g2.add(gs);
           V ph = vscl(vconj(gs), rsq(g2.get()));           // e^{-i phi}
-          const float zeta = (fb - fa) / (2.f * fg);
-          const float tf = fabsf(zeta) < 1e18f ? (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta)) : 0.5f / zeta;
+          float tf;   // tan of the angle: 1 / (zeta + sign sqrt(1 + zeta^2)), zeta = (|b|^2 - |a|^2) / (2 |<a, b>|)
+          if (abs(de) > 20) {   // 1 / (2 zeta)
+            tf = (de > 0 ? fg / fb : -fg / fa) * __int_as_float((127 - abs(de)) << 23);
+          } else {
+            const float u = __int_as_float((127 + de) << 23), v = __int_as_float((127 - de) << 23);
+            const float zeta = (fb * u - fa * v) / (2.f * fg);
+            tf = fabsf(zeta) < 1e18f ? (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta)) : 0.5f / zeta;
+          }
           R cs, sn;
           if constexpr (sizeof(S) == sizeof(double2)) {
             cs = rsq(fma((double)tf, (double)tf, 1.0));
@@ -1033,7 +1087,7 @@ __global__ void __launch_bounds__(256, 2) k_tsvd(Dev d, int A, int nb, int n0) {
     const R inv = rof(1.0 / s_sig[s_ord[jj]], (S*)nullptr);
     V v;
     if (row < r) {
-      v = vscl(w[row], rof(Sv[row], (S*)nullptr));
+      v = vscl(w[row], rof(Sv[row] * up, (S*)nullptr));
     } else {
       DotC<S> s;
       for (int q = 0; q < r; ++q) s.add(Pm[(long long)(row - r) * rmax + q], w[q]);
@@ -1086,7 +1140,7 @@ __global__ void __launch_bounds__(256, 2) k_tsvd(Dev d, int A, int nb, int n0) {
     for (int e = 0; e < ke; ++e) s.add(vconj(Qm[(long long)e * ncol + l]), w[r + e]);
     return s.get();
   }, Vf);
-  for (int q = tid; q < rmax; q += blockDim.x) Sv[q] = (q < rn) ? s_sig[s_ord[q]] : 0.0;
+  for (int q = tid; q < rmax; q += blockDim.x) Sv[q] = (q < rn) ? s_sig[s_ord[q]] * down : 0.0;
   if (tid == 0) *rkp = rn;
 }
 

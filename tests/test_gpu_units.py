@@ -1,7 +1,9 @@
 """Other units of energy and time.  Energies times 2^m, times by 2^-m: G^R, G^<
 and G^tv are the same numbers, Sigma is 2^2m times as large, and a power of two
 commutes with every rounding, so an FP64 run gives the same bits as long as
-nothing leaves the range of FP64 (pivots and reciprocals included)."""
+nothing leaves the range of FP64 (pivots and reciprocals included).  With
+compressed history (an absolute tolerance) the compressed run is compared with the
+dense run of the same units, at Sigma about 2^72: its squares are beyond FP32."""
 import numpy as np
 import pytest
 
@@ -29,3 +31,15 @@ def _run(no, nt, m, rho_mode=0, mixed=False, **form):
 def test_dense_bits(no, rho_mode, m):
     a, b = _run(no, 75, 0, rho_mode).dense(), _run(no, 75, m, rho_mode).dense()
     assert all(np.array_equal(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("no,nt,mixed", [(1, 160, False), (2, 150, False), (1, 160, True), (2, 150, True)])
+def test_compressed(no, nt, mixed):
+    # blocks of 64 columns at most, so no rank exceeds r_max; bounds: the compressed FP64 form's rounding
+    # floor; the complex64 form's bar plus ten times its SVD tolerance
+    a = _run(no, nt, 36, mixed=mixed, svd_tol=1e-8 if mixed else 1e-12, leaf=32, r_max=64)
+    b = _run(no, nt, 36)
+    bound = 1e-6 + 1e-7 if mixed else 1e-9
+    for T in (nt - 1, nt - 40, 90, 70):
+        for x, y in zip(a.row(0, T) + (a.tv(0, T),), b.row(0, T) + (b.tv(0, T),)):
+            assert np.abs(x - y).max() < bound, T
