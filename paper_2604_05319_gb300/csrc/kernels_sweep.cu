@@ -102,7 +102,11 @@ struct Row64<NO, double2> {
 // and the BDF terms reaching across the chunk edge (k rows), which carry the
 // implicit recursion and get hi + lo in float-float (about 48 bits); a plain
 // complex64 inverse would put 2^-24 times the BDF amplitude a_j / h into
-// every chunk and accumulate.
+// every chunk and accumulate.  In a chunk that is still growing the far field
+// goes through hi + lo too: the next steps' BDF terms come from its points (rms
+// error of the density matrix against FP64, N_o = 1, runs of 40 points: 5.7e-8
+// with the FP32 product, 4.5e-8 so; no time: 99.1 -> 99.3 ms at 304 x 384, 158.1 ->
+// 158.0 at N_o = 2, 128 x 600).
 template <int NO>
 __device__ __forceinline__ double2* Cinv(const Dev& d, int n, int cc, int which) {
   const long long nn = (long long)(CK * NO) * (CK * NO);
@@ -255,7 +259,6 @@ __device__ __forceinline__ LeafBlk block_at(const Dev& d, int b) {
   if (b < 0) return {0, 0, -1, 0, 0, 0, 0, 0};
   return {d.b_uoff[b], d.b_voff[b], b, d.b_r0[b], d.b_r1[b], d.b_c0[b], d.b_c1[b], 0};
 }
-__device__ __forceinline__ cff ff_split(const zd& z) { return {ff_of_bits(z.re), ff_of_bits(z.im)}; }
 
 // The blocks of Sigma^R that cover leaf jl (retarded: over its columns, only
 // blocks with built rows; lesser: over its rows), their geometry and ranks, into
@@ -440,7 +443,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
     for (int e = tid; e < 64 * NO; e += blockDim.x) {
       const int tp = b0 + e / NO;
       if (tp > T) continue;
-      if constexpr (MX) Yl[tp & 63][e % NO] = ff_split(ld(yp(tp) + e % NO));
+      if constexpr (MX) Yl[tp & 63][e % NO] = cff_of(ld(yp(tp) + e % NO));   // (hi rounded: it is used by itself too)
       else Yl[tp & 63][e % NO] = ld(yp(tp) + e % NO);
     }
     __syncthreads();
@@ -586,6 +589,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
       buf ^= 1;
       __syncthreads();
     }
+    const bool full = MX && cc >= d.nfrozR;   // still growing: all of its right-hand side in float-float
     // the inverse of this chunk into shared memory, overlapping the far field
     const bool stage_now = kInvStage<NO> && s_stage;
     if (stage_now && tid == 0) bulk_g2s(ctile, Cinv<NO>(d, n, cc, 0), kInvStage<NO>, &cbar);
@@ -667,7 +671,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
           for (int jj = b - tp; jj <= k; ++jj) fb = vbdf(fb, Yl[(tp + jj) & 63][sl], W, jj);
         if constexpr (MX) {
           Ff[col][sl] = vbulk(F);
-          Fb[col][sl] = fb;
+          Fb[col][sl] = full ? vadd(F, fb) : fb;
         } else {
           Ff[col][sl] = F + fb;
         }
@@ -700,12 +704,12 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
           const float2* Mh = reinterpret_cast<const float2*>(Mg);
           const float2* Ml = Mh + LD * LD;
           zf s32 = zf(0);
-          for (int si = (ti & ~7) + sl; si < cn; si += 8)
+          for (int si = (ti & ~7) + sl; si < cn && !full; si += 8)
 #pragma unroll
             for (int m = 0; m < NO; ++m)
               s32 = cfma(Ff[si][m], ldr<float>(Mh + (long long)(si * NO + m) * LD + ti * NO + j), s32);
           out = cff_of(s32);
-          for (int si = max(cn - k, 0) + sl; si < cn; si += 8)
+          for (int si = (full ? ti & ~7 : max(cn - k, 0)) + sl; si < cn; si += 8)
 #pragma unroll
             for (int m = 0; m < NO; ++m) {
               const long long e = (long long)(si * NO + m) * LD + ti * NO + j;
@@ -790,7 +794,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
     for (int e = tid; e < 64 * NO; e += blockDim.x) {
       const int t = c - 1 - e / NO, m = e % NO;
       if (t < 0) continue;
-      if constexpr (MX) Xl[t & 63][m] = ff_split(ld(xp(t) + m * NO + jc));
+      if constexpr (MX) Xl[t & 63][m] = cff_of(ld(xp(t) + m * NO + jc));
       else Xl[t & 63][m] = ld(xp(t) + m * NO + jc);
     }
   } else if (tid < NO) {  // x(0) = -[G^tv(T, 0+)]^dagger
@@ -910,6 +914,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
       __syncthreads();
     }
     const int fn = min(b, T) - a;   // rows solved with the chunk's inverse; row T, if it is here, follows them
+    const bool full = MX && cc >= d.nfrozL;   // still growing: all of its right-hand side in float-float
     // the inverse of this chunk into shared memory, overlapping the far field
     const bool stage_now = kInvStage<NO> && fn > 0 && s_stage;
     if (stage_now && tid == 0) bulk_g2s(ctile, Cinv<NO>(d, n, cc, 1), kInvStage<NO>, &cbar);
@@ -1006,7 +1011,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
         if (t == T) FT[sl] = vadd(F, fb);
         if constexpr (MX) {
           Ff[row][sl] = vbulk(F);
-          Fb[row][sl] = fb;
+          Fb[row][sl] = full ? vadd(F, fb) : fb;
         } else {
           Ff[row][sl] = F + fb;
         }
@@ -1038,12 +1043,12 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
           const float2* Mh = reinterpret_cast<const float2*>(Mg);
           const float2* Ml = Mh + LD * LD;
           zf s32 = zf(0);
-          for (int li = sl; li < le; li += 8)
+          for (int li = sl; li < le && !full; li += 8)
 #pragma unroll
             for (int y = 0; y < NO; ++y)
               s32 = cfma(ldr<float>(Mh + (long long)(ti * NO + m) * LD + li * NO + y), Ff[li][y], s32);
           out = cff_of(s32);
-          for (int li = sl; li < k && li < le; li += 8)
+          for (int li = sl; li < (full ? le : min(k, le)); li += 8)
 #pragma unroll
             for (int y = 0; y < NO; ++y) {
               const long long e = (long long)(ti * NO + m) * LD + li * NO + y;
