@@ -436,7 +436,10 @@ enum {
 int hkbe_set_profiling(hkbe_t* h, int on);
 
 /* Accumulated device milliseconds and launch count of `phase` since the last
- * hkbe_reset_counters (timing only while profiling is on; launches always). */
+ * hkbe_reset_counters (timing only while profiling is on; launches always,
+ * every kernel of a phase counted).  In small batches the retarded sweep's
+ * launch computes the mixed component as well: HKBE_PHASE_MIXED then has no
+ * launches, and its time is part of HKBE_PHASE_RET. */
 int hkbe_get_timing(const hkbe_t* h, int phase, double* ms, int64_t* launches);
 
 /* Zero the per-phase times and launch counts. */

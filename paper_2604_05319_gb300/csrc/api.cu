@@ -1098,7 +1098,7 @@ int hkbe_step(hkbe_t* h, int n_steps, int32_t* iters, double* err) {
                    if ((it == 0 || h->self_consistent) &&
                        (e = run_phase(h, HKBE_PHASE_SIGMA, 1, [&]() { return hk::launch_sigma(d, T, h->s); })))
                      return e;
-                   if ((e = run_phase(h, HKBE_PHASE_RET, 1, [&]() {
+                   if ((e = run_phase(h, HKBE_PHASE_RET, h->scheme ? 2 : hk::ret_launches(d), [&]() {
                           return h->scheme ? hk::launch_ret_sf(d, T, h->s) : hk::launch_ret_h(d, T, h->s);
                         })))
                      return e;
@@ -1110,7 +1110,7 @@ int hkbe_step(hkbe_t* h, int n_steps, int32_t* iters, double* err) {
                           return h->hodlr ? hk::launch_src_h(d, T, njob, h->s) : hk::launch_src(d, T, h->s);
                         })))
                      return e;
-                   if ((e = run_phase(h, HKBE_PHASE_LES, 1, [&]() {
+                   if ((e = run_phase(h, HKBE_PHASE_LES, h->scheme ? 1 : hk::les_launches(d), [&]() {
                           return h->scheme ? hk::launch_les_sf(d, T, h->s) : hk::launch_les_h(d, T, h->s);
                         })))
                      return e;
@@ -1126,7 +1126,7 @@ int hkbe_step(hkbe_t* h, int n_steps, int32_t* iters, double* err) {
     // update_blocks (Sec. 3.1): compress every whole leaf of rows older than k+1 steps
     while (h->hodlr && d.cdir + d.L <= T - d.k) {
       const int A = d.cdir;
-      HK_CUDA(h, run_phase(h, HKBE_PHASE_COMPRESS, 2, [&]() { return hk::launch_compress(d, A, d.L, h->s); }));
+      HK_CUDA(h, run_phase(h, HKBE_PHASE_COMPRESS, 1 + (N + d.tsvd_group - 1) / d.tsvd_group, [&]() { return hk::launch_compress(d, A, d.L, h->s); }));
       d.cdir += d.L;
     }
   }

@@ -1471,6 +1471,8 @@ bool ret_takes_mixed(const Dev& d) {
 // idle: 43 -> 36 ms (1, FP64, T = 384), but 19.7 -> 21.6 (304, complex64).
 static bool split_les(const Dev& d) { return d.cdir >= kSplitRows; }
 static bool split_ret(const Dev& d) { return d.cdir >= kSplitRows && d.no * d.n_inst <= 152; }
+int ret_launches(const Dev& d) { return split_ret(d) ? 3 : 1; }
+int les_launches(const Dev& d) { return split_les(d) ? 3 : 1; }
 // A sweep comes early (see pdl_start) in the dense form with up to four CTAs: 1 x
 // 64, FP64, 10.7 -> 10.2 ms; 3 x 256 91.5 -> 90.8; 4 x 200 58.6 -> 57.6. Compressed
 // forms gain nothing there (4 x 300, FP64, 55.9 -> 56.6), and more CTAs end up two

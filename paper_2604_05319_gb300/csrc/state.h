@@ -132,6 +132,8 @@ cudaError_t launch_set_active(const Dev& d, double tol, int iter, int min_iter, 
 // compressed (HODLR) form
 cudaError_t launch_ret_h(const Dev& d, int T, cudaStream_t s);
 bool ret_takes_mixed(const Dev& d);   // launch_ret_h computes the mixed component as well
+int ret_launches(const Dev& d);       // kernels of launch_ret_h and launch_les_h
+int les_launches(const Dev& d);
 cudaError_t launch_les_h(const Dev& d, int T, cudaStream_t s);
 cudaError_t launch_src_h(const Dev& d, int T, int njob, cudaStream_t s);   // njob: jobs with built rows
 cudaError_t launch_compress(const Dev& d, int A, int nb, cudaStream_t s);
