@@ -66,12 +66,17 @@ enum { kAll = 0, kTop = 1, kLeaves = 2 };
 template <typename R>
 __device__ __forceinline__ auto reduce8(const KAcc<R>& k) { return kacc_lanes(k, 1, 8); }
 
-// |new - old|^2, old a stored element
+// |new - old|^2, old a stored element; in the complex64 form |new - old|, the
+// squares taken with the exponent set aside (squares of FP32 overflow from 1.8e19)
 __device__ __forceinline__ double vdist(const zd& a, const zd& o) { return (a - o).abs2(); }
 __device__ __forceinline__ float vdist(const cff& a, const zf& o) {
   const float x = (a.re.hi - o.re) + a.re.lo, y = (a.im.hi - o.im) + a.im.lo;
-  return x * x + y * y;
+  const int e = min(max(__float_as_int(max_mag(x, y)) >> 23, 1), 253);
+  const float s = __int_as_float((254 - e) << 23), u = x * s, v = y * s;
+  return sqrtf(fmaf(u, u, v * v)) * __int_as_float(e << 23);
 }
+__device__ __forceinline__ double vdist_out(double d) { return sqrt(d); }
+__device__ __forceinline__ double vdist_out(float d) { return d; }
 __device__ __forceinline__ void vstore(double2* p, const zd& v) { st(p, v); }
 __device__ __forceinline__ void vstore(float2* p, const cff& v) { *p = make_float2(v.re.hi, v.im.hi); }
 // Where a sweep keeps the row it solves: in place (FP64 storage), or in FP64
@@ -736,7 +741,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
     __syncthreads();
   }
   write64(wa, wn);
-  const double e1 = sqrt(warp_max((double)myerr));
+  const double e1 = warp_max(vdist_out(myerr));
   if (lane == 0) atomic_max_nonneg(&serr, e1);
   __syncthreads();
   if (tid == 0) atomic_max_nonneg(d.err + n, serr);
@@ -1121,7 +1126,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
     __syncthreads();
   }
   write64(wa, wn);
-  const double e1 = sqrt(warp_max((double)myerr));
+  const double e1 = warp_max(vdist_out(myerr));
   if (lane == 0) atomic_max_nonneg(&serr, e1);
   __syncthreads();
   if (tid == 0) atomic_max_nonneg(d.err + n, serr);

@@ -43,3 +43,21 @@ def test_compressed(no, nt, mixed):
     for T in (nt - 1, nt - 40, 90, 70):
         for x, y in zip(a.row(0, T) + (a.tv(0, T),), b.row(0, T) + (b.tv(0, T),)):
             assert np.abs(x - y).max() < bound, T
+
+
+def test_large_occupations_complex64():
+    # G^M and with it G^<, G^tv times 2^100 (the equations are linear in them): the change from one iterate to
+    # the next has squares beyond FP32; bound: the complex64 form's bar, relative to the largest element
+    nt, no, V = 75, 2, np.array([[0.3, -0.4], [0.2, 0.5]]) + 0j
+    e0, eb = np.diag([0.2, -0.3]), wk.C5_BATH_LEVELS
+    tau, om = wk.dlr_grid(100.0, 1e-10, 5.0)
+    gm = wk.bath_gm(tau, 5.0, e0, V, eb)[None] * 2.0 ** 100
+    mp = np.concatenate([[2.0], eb, V.view(np.float64).ravel()])[None]
+    out = []
+    for prec in (pk.PREC_FP64, pk.PREC_MIXED):
+        st = pk.Stepper(nt, 0.05, 5, 5.0, nao=no, tol=1e-7, max_iter=80, precision=prec)
+        st.set_inputs(tau, om, gm, np.broadcast_to(e0, (1, nt + 1, no, no)).astype(complex), pk.MODEL_BATH, mp)
+        st.run()
+        out.append(st.dense())
+    for x, y in zip(*out):
+        assert np.abs(x - y).max() < 1e-6 * np.abs(x).max()
