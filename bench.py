@@ -171,6 +171,7 @@ def phase_flops(phase, T, k, no, L, blocks, ranks, hodlr):
     return int(8 * no * history_all_pairs(T, k, L, no, blocks, ranks, hodlr))
 
 
+DTYPE_MIXED = "c64 storage, f32 bulk sums, 2 x f32 chunk solves and TSVD, f64 inverses, head and density matrix"
 KERNEL_OF = {"ret": "k_ret2", "les": "k_les2", "src": "k_src_q"}
 _SWEEP_SRC = ["kernels_sweep.cu", "mixed_nodes.cuh", "bulk_copy.cuh", "hodlr_util.cuh", "dev_util.cuh", "common.cuh", "state.h"]
 _SRC_SRC = ["kernels_hodlr.cu", "lattice.cuh", "hodlr_util.cuh", "dev_util.cuh", "common.cuh", "state.h"]
@@ -527,7 +528,7 @@ def run_c5(args, pk, torch):
     total_steps = sum(int(np.sum(g["nt_per_inst"] - 1 - k)) for g in groups)
     line = {"metric": METRIC, "value": done / t_win, "unit": UNIT, "n_gpus": 1, "steps": K, "warmup": T_s - 1 - k,
             "ms_per_step": t_win / K * 1e3, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": "c64 storage, f32 bulk sums, f64 point solves and TSVD", "data": "synthetic",
+            "dtype": DTYPE_MIXED, "data": "synthetic",
             "config": {"workload": "C5", "desc": C5_DESC, "n_inst_per_gpu": 64,
                        "timed_window": f"time steps {T_s}..{T_s + K - 1} of every group (instances past their "
                                        f"N_t idle); host-timed between device synchronisations",
@@ -734,7 +735,7 @@ def main():
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world,
             "steps": K, "warmup": T_s - 1 - wl.k, "ms_per_step": t_win / K * 1e3,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": ("c64 storage, f32 bulk sums and TSVD, f64 point solves" if prec_name == "mixed" else "f64"),
+            "dtype": DTYPE_MIXED if prec_name == "mixed" else "f64",
             "data": "synthetic",
             "config": {"workload": wname, "desc": spec["desc"], "n_inst_per_gpu": n_inst,
                        "precision": prec_name, "nt": wl.nt, "h": wl.h, "k": wl.k,

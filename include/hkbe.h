@@ -64,12 +64,15 @@ enum {
                              arithmetic throughout                               */
   HKBE_PREC_MIXED = 1,    /* complex64 storage of the two-time components
                              (rows, HODLR factors, leaves, band); FP32 bulk
-                             history sums and FP32 TSVD; the row being solved,
-                             every point solve, the mixed components, weights
-                             and DLR matrices stay FP64.  Expected deviation
-                             from the FP64 form: about 1e-6 relative (single-
-                             precision rounding of the stored history; a GPU
-                             design choice, the paper computes in FP64)          */
+                             history sums, compensated; pairs of floats (about
+                             48 bits) in the solves, the lesser source and the
+                             TSVD; chunk inverses, the points next to the
+                             diagonal, density matrix, mixed components, copies
+                             of the rows being solved, weights and DLR matrices
+                             FP64.  Expected deviation from the FP64 form:
+                             about 1e-6 relative (single-precision rounding of
+                             the stored history; a GPU design choice, the paper
+                             computes in FP64)                                   */
   HKBE_PREC_TF32X3 = 2,   /* not provided: rejected by hkbe_create (see there) */
   HKBE_PREC_BF16X3 = 3    /* not provided: rejected by hkbe_create (see there) */
 };
@@ -279,8 +282,9 @@ int hkbe_set_initial_slices(hkbe_t* h, const double* gr, const double* gl, const
  * nt-1), HKBE_ERR_NOCONV (state kept; the step counter still advances: the
  * self-consistency loop reached max_iter, or, HODLR form, the Jacobi SVD of a
  * TSVD block core did not converge in 40 sweeps), HKBE_ERR_RANK (a block's
- * epsilon-rank was capped at r_max), HKBE_ERR_CUDA (a CUDA error, or a
- * sweep's bounded wait for the shared-memory copy of a frozen chunk inverse
+ * epsilon-rank was capped at r_max), HKBE_ERR_NAN (a value of the new row is
+ * not finite; the step counter stays), HKBE_ERR_CUDA (a CUDA error, or a
+ * sweep's bounded wait for the shared-memory copy of a chunk inverse
  * timed out; that chunk was then read from global memory).  The TSVD and
  * copy conditions are counted over the n_steps of this call and reset
  * afterwards. */

@@ -132,10 +132,6 @@ __device__ __forceinline__ ffl ff_of_bits(double x) {
   if (h >= 255 << 20) { mag = 0x7f800000u; sc = 0u; }
   return {__uint_as_float(sign | mag), (float)(lo & 0x1fffffffu) * __uint_as_float(sign | sc)};
 }
-__device__ __forceinline__ zf ld_f32(const double2* p) {
-  const double2 v = *p;
-  return zf(f32_of(v.x), f32_of(v.y));
-}
 
 // a float-float complex from lane (this lane ^ off) of the warp (all lanes call it)
 __device__ __forceinline__ cff cff_shfl_xor(const cff& a, int off) {
@@ -172,7 +168,7 @@ template <> struct KAcc<double> {
 // Sum of a history accumulator over the lanes reached by xor offsets from,
 // 2 from, ... below to (an aligned lane group); every lane of the group
 // receives it.  Compensated FP32: combined in float-float (FP32 pipes);
-// FP64: plain.  val_of gives the FP64 value (taken by the lane that uses it).
+// FP64: plain.
 __device__ __forceinline__ cff kacc_lanes(const KAcc<float>& k, int from, int to) {
   cff r = {ff_two_sum(k.s.re, -k.c.re), ff_two_sum(k.s.im, -k.c.im)};
   for (int off = from; off < to; off <<= 1) r = cff_add(r, cff_shfl_xor(r, off));
@@ -184,8 +180,6 @@ __device__ __forceinline__ zd kacc_lanes(const KAcc<double>& k, int from, int to
     v += zd(__shfl_xor_sync(0xffffffffu, v.re, off), __shfl_xor_sync(0xffffffffu, v.im, off));
   return v;
 }
-__device__ __forceinline__ zd val_of(const cff& a) { return cff_val(a); }
-__device__ __forceinline__ zd val_of(const zd& a) { return a; }
 #endif
 
 HD zd cdiv(const zd& a, const zd& b) {
@@ -199,7 +193,6 @@ struct M {
   zd a[N][N];
   HD M() {}
   HD static M zero() { M m; for (int i = 0; i < N; ++i) for (int j = 0; j < N; ++j) m.a[i][j] = zd(); return m; }
-  HD static M eye(zd d) { M m = zero(); for (int i = 0; i < N; ++i) m.a[i][i] = d; return m; }
   HD zd& operator()(int i, int j) { return a[i][j]; }
   HD const zd& operator()(int i, int j) const { return a[i][j]; }
 };
@@ -327,22 +320,6 @@ template <int N> HD M<N> solve_left(M<N> A, M<N> B) {
   }
   return B;
 }
-// Solve X A = B (right): X = B A^-1  <=>  A^T X^T = B^T
-template <int N> HD M<N> solve_right(const M<N>& A, const M<N>& B) {
-  M<N> At, Bt;
-#pragma unroll
-  for (int i = 0; i < N; ++i)
-#pragma unroll
-    for (int j = 0; j < N; ++j) { At.a[i][j] = A.a[j][i]; Bt.a[i][j] = B.a[j][i]; }
-  M<N> Xt = solve_left<N>(At, Bt);
-  M<N> X;
-#pragma unroll
-  for (int i = 0; i < N; ++i)
-#pragma unroll
-    for (int j = 0; j < N; ++j) X.a[i][j] = Xt.a[j][i];
-  return X;
-}
-
 // ---- atomics ----------------------------------------------------------------
 __device__ __forceinline__ void atomic_max_nonneg(double* addr, double v) {
   // for non-negative doubles the IEEE bit pattern orders like unsigned ints, a NaN above all others

@@ -7,6 +7,7 @@
 namespace hk {
 
 constexpr unsigned FULL = 0xffffffffu;
+constexpr int kSMs = 152;   // of a GB300: batches below a CTA for each of them leave SMs idle
 
 // The kernels of a time step run one after the other on one stream, and each
 // begins with pdl_start.  Where the sweeps have at most kEarlyCtas CTAs the
@@ -368,16 +369,7 @@ static __device__ __noinline__ void gj_inverse(int n, zd* A, int ld) {
   __syncthreads();
 }
 
-// small vector solves: y M = r (row vector) and M x = r (column vector)
-template <int NO>
-__device__ void solve_row(const M<NO>& Mm, const zd* r, zd* y) {
-  M<NO> B = M<NO>::zero();
-#pragma unroll
-  for (int j = 0; j < NO; ++j) B.a[0][j] = r[j];
-  M<NO> X = solve_right<NO>(Mm, B);
-#pragma unroll
-  for (int j = 0; j < NO; ++j) y[j] = X.a[0][j];
-}
+// small vector solve M x = r (column vector)
 template <int NO>
 __device__ void solve_col(const M<NO>& Mm, const zd* r, zd* x) {
   M<NO> B = M<NO>::zero();

@@ -944,7 +944,7 @@ cudaError_t launch_sigma(const Dev& d, int T, cudaStream_t s) {
 cudaError_t launch_mixed(const Dev& d, int T, cudaStream_t s) {
   HK_DISPATCH(d.no, {
     constexpr int N1 = kNodes<NO>, N2 = kNodesFew<NO>;
-    if ((d.r + N1 - 1) / N1 * d.n_inst >= 152)
+    if ((d.r + N1 - 1) / N1 * d.n_inst >= kSMs)
       return launch_k(k_mixed<NO, S, N1>, dim3((d.r + N1 - 1) / N1, d.n_inst), 256, 0, s, d, T);
     return launch_k(k_mixed<NO, S, N2>, dim3((d.r + N2 - 1) / N2, d.n_inst), 256, 0, s, d, T);
   })

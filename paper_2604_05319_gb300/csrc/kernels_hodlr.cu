@@ -16,17 +16,15 @@
 //
 // update_blocks (Sec. 3.1): whenever a whole leaf of rows is older than k+1
 // steps, its rows are appended to every block containing them by a batched
-// Brand update: P = R V, E = R - P V^dagger (projected twice), an orthonormal
-// basis Q of E's rows by two-pass Gram-Schmidt, the core
-// K = [[S, 0], [P, C]] (C = E Q^dagger), its SVD by one-sided Jacobi, truncation
-// of singular values below the SVD tolerance (Sec. 2.2), and rotation of U, V.
+// Brand update: P = R V, E = R - P V^dagger (projected twice in the complex64
+// form), an orthonormal basis Q of E's rows by Gram-Schmidt (a second pass for
+// the rows that add a direction), the core K = [[S, 0], [P, C]] (C = E Q^dagger),
+// its SVD by a column-pivoted QR and one-sided Jacobi on R^dagger, truncation of
+// singular values below the SVD tolerance (Sec. 2.2), and rotation of U, V.
 #include "hodlr_util.cuh"
 #include "lattice.cuh"
 
 namespace hk {
-
-
-constexpr int kSrcRing = 80;   // >= leaf + k + 1 uncompressed rows
 
 // ---------------------------------------------------------------------------
 // Lesser source with compressed Sigma^< (two-sided HODLR matvec).
@@ -337,8 +335,8 @@ __global__ void __launch_bounds__(256) k_src_q(Dev d, int T, int uselist) {
   }
   // 32 compressed columns
   const int t = blockIdx.x * 32 + lane, jt = blockIdx.x * 32 / L, A = jt * L;
-  cx<R>* gr = reinterpret_cast<cx<R>*>(red + 8 * NO2 * 32);   // [kSrcRing][NO2] w_l g_l of the uncompressed rows
-  cx<R>* gl = gr + kSrcRing * NO2;                            // [L][NO2] of the leaf
+  cx<R>* gr = reinterpret_cast<cx<R>*>(red + 8 * NO2 * 32);   // [kRingRows][NO2] w_l g_l of the uncompressed rows
+  cx<R>* gl = gr + kRingRows * NO2;                            // [L][NO2] of the leaf
   int* rk = reinterpret_cast<int*>(gl + 64 * NO2);            // per slot (target x, side, level, other index): rank,
   const int nslot = 2 * d.maxl * NO2;
   int* start = rk + nslot;                                    // first packed entry,
@@ -1354,7 +1352,7 @@ __global__ void __launch_bounds__(kLatMaxK) k_lattice_obs(Dev d, int t, double* 
 template <int NO, typename S>
 static cudaError_t src_q(const Dev& d, int T, cudaStream_t s) {
   const size_t n2 = NO * NO, es = sizeof(S), ns = 2 * (size_t)d.maxl * n2;
-  size_t bytes = ((size_t)d.r * n2 + 8 * n2 * 32) * 16 + (kSrcRing + 64) * n2 * es + (2 * ns + 1) * 4 + 8 + ns * 16;
+  size_t bytes = ((size_t)d.r * n2 + 8 * n2 * 32) * 16 + (kRingRows + 64) * n2 * es + (2 * ns + 1) * 4 + 8 + ns * 16;
   const size_t list = ns * d.rmax * 2;
   const int uselist = ns * 128 <= 65536 && bytes + list <= 200 * 1024;
   if (uselist) bytes += list;
@@ -1370,7 +1368,7 @@ cudaError_t open_history(const Dev& d) {
   return e;
 }
 cudaError_t launch_src_h(const Dev& d, int T, int njob, cudaStream_t s) {
-  if (d.cdir > 0 && T + 1 - d.cdir > kSrcRing) return cudaErrorInvalidValue;
+  if (d.cdir > 0 && T + 1 - d.cdir > kRingRows) return cudaErrorInvalidValue;
   if (njob > 0) {
     cudaError_t e = cudaErrorInvalidValue;
     HK_DISPATCH(d.no, e = launch_k(k_src_proj<NO, S>, dim3(njob, d.n_inst), 256, 0, s, d, T));

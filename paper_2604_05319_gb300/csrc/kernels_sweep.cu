@@ -330,12 +330,14 @@ __device__ __forceinline__ void leaf_pack(const Dev& d, int A, bool cols, const 
 // One CTA per (instance, orbital row) walks the chunks; its time is the
 // dependency chain of their phases, not bandwidth.  What keeps a phase short:
 // the last 64 solved points stay in shared memory (the far field of the lower
-// half of a leaf, the BDF terms and the band read them there), the complex64
-// form computes on the FP32 pipes throughout (FP64 copies of the row are
-// written a phase later, off the chain), the ranks of the next leaf are read
-// while this one is worked on, and the factors of all blocks over a leaf are
-// read as one packed list with eight loads in flight per thread (one block and
-// pair after the other, each waited for its rank and then for its row).
+// half of a leaf, the BDF terms and the band read them there), the chunks of the
+// complex64 form compute on the FP32 pipes but for the scaling of projections by
+// their singular values (FP64 copies of the row are written a phase later, off
+// the chain; the head and row T of the lesser column are FP64), the ranks of the
+// next leaf are read while this one is worked on, and the factors of all blocks
+// over a leaf are read as one packed list with eight loads in flight per thread
+// (one block and pair after the other, each waited for its rank and then for its
+// row).
 // Both sweeps of an iteration, before and after these: 1.05 -> 0.53 ms (N_o = 2,
 // complex64, 128 instances, T = 600), 1.34 -> 0.69 ms (one instance, T = 1089),
 // 0.75 -> 0.43 ms (N_o = 2, FP64, 16 instances, T = 300).
@@ -1465,7 +1467,7 @@ static size_t sweep_smem(const Dev& d, int* staged) {
 // the SMs in large groups (N_o = 2, 128 x 600: 158 -> 179 in one launch).
 bool ret_takes_mixed(const Dev& d) {
   const int ni = d.no == 1 ? kNodesFew<1> : d.no == 2 ? kNodesFew<2> : kNodesFew<3>;
-  return (long long)(d.no + (d.r + ni - 1) / ni) * d.n_inst <= (d.prec ? 4 : 1) * 152;
+  return (long long)(d.no + (d.r + ni - 1) / ni) * d.n_inst <= (d.prec ? 4 : 1) * kSMs;
 }
 // A sweep runs as two launches with its ring kernel between them once kSplitRows
 // rows are compressed: before that, the ring's products in the chain cost less
@@ -1475,7 +1477,7 @@ bool ret_takes_mixed(const Dev& d) {
 // sweep, whose ring phases are shorter, gains only while its CTAs leave SMs
 // idle: 43 -> 36 ms (1, FP64, T = 384), but 19.7 -> 21.6 (304, complex64).
 static bool split_les(const Dev& d) { return d.cdir >= kSplitRows; }
-static bool split_ret(const Dev& d) { return d.cdir >= kSplitRows && d.no * d.n_inst <= 152; }
+static bool split_ret(const Dev& d) { return d.cdir >= kSplitRows && d.no * d.n_inst <= kSMs; }
 int ret_launches(const Dev& d) { return split_ret(d) ? 3 : 1; }
 int les_launches(const Dev& d) { return split_les(d) ? 3 : 1; }
 // A sweep comes early (see pdl_start) in the dense form with up to four CTAs: 1 x

@@ -24,7 +24,8 @@ constexpr int MP = 64;  // doubles of model parameters per instance
 // leaf triangles plus U S V^dagger blocks, one scalar TSVD per orbital pair.
 // Element type of the two-time storage (U, V, leaves, band, ring or triangle
 // rows): double2 in the FP64 form, float2 in the mixed form.  Mixed
-// components, chunk inverses, singular values and projections are FP64 in both.
+// components and singular values are FP64 in both; chunk inverses are FP64 or
+// complex64 pairs hi + lo, projections are of the bulk type.
 struct Hod {
   void* U;       // [n][utot][rmax]   U of block b, pair p at (uoff[b] + p*rows_b) * rmax
   void* V;       // [n][vtot][rmax]   V of block b, pair p at (voff[b] + p*cols_b) * rmax
