@@ -265,18 +265,10 @@ template <int N> HD M<N> dag(const M<N>& x) {
   return m;
 }
 #ifdef __CUDACC__
-// The larger of two magnitudes by their bit patterns: values >= 0 order like
-// integers, infinity above every number and a NaN (sign aside) above infinity.
-// The measures of an iteration's change are folded with it, since fmax would
-// drop a NaN and a row of them would pass as converged; it takes no FP64
-// instruction.
-__device__ __forceinline__ double max_mag(double a, double b) {
-  const long long m = 0x7fffffffffffffffll, x = __double_as_longlong(a) & m, y = __double_as_longlong(b) & m;
-  return __longlong_as_double(x > y ? x : y);
-}
-__device__ __forceinline__ float max_mag(float a, float b) {
-  return __int_as_float(max(__float_as_int(a) & 0x7fffffff, __float_as_int(b) & 0x7fffffff));
-}
+// The larger of two changes from one iterate to the next; one that is not finite
+// counts as infinite (fmax by itself drops a NaN, and a row of them would pass as
+// converged).
+__device__ __forceinline__ double max_change(double a, double x) { return x < INFINITY ? fmax(a, x) : INFINITY; }
 template <int N> __device__ double maxabs_diff(const M<N>& x, const M<N>& y) {
   double e = 0;
 #pragma unroll
@@ -284,7 +276,7 @@ template <int N> __device__ double maxabs_diff(const M<N>& x, const M<N>& y) {
 #pragma unroll
     for (int j = 0; j < N; ++j) {
       zd d = x.a[i][j] - y.a[i][j];
-      e = max_mag(e, sqrt(d.abs2()));
+      e = max_change(e, sqrt(d.abs2()));
     }
   return e;
 }

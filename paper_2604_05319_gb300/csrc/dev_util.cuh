@@ -197,7 +197,7 @@ __device__ __forceinline__ void warp_sum(zd (&v)[L]) {
 }
 __device__ __forceinline__ double warp_max(double v) {
 #pragma unroll
-  for (int off = 16; off; off >>= 1) v = max_mag(v, __shfl_xor_sync(FULL, v, off));
+  for (int off = 16; off; off >>= 1) v = fmax(v, __shfl_xor_sync(FULL, v, off));
   return v;
 }
 

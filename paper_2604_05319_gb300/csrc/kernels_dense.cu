@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(256) k_les(Dev d, int T) {
       const int m = lane;
       zd v = ld(d.x0 + (long long)n * NO2 + m * NO + jc);
       S* p = xptr(0) + m * NO + jc;
-      myerr = max_mag(myerr, sqrt((v - ld(p)).abs2()));
+      myerr = max_change(myerr, sqrt((v - ld(p)).abs2()));
       st(p, v);
     }
     __syncwarp();
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(256) k_les(Dev d, int T) {
       const int t = row / NO + 1, m = row % NO;
       if (t > last) continue;
       S* p = xptr(t) + m * NO + jc;
-      myerr = max_mag(myerr, sqrt((sB[row] - ld(p)).abs2()));
+      myerr = max_change(myerr, sqrt((sB[row] - ld(p)).abs2()));
       st(p, sB[row]);
     }
   }
@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(256) k_les(Dev d, int T) {
 #pragma unroll
           for (int m = 0; m < NO; ++m) {
             S* p = xptr(t) + m * NO + jc;
-            myerr = max_mag(myerr, sqrt((x[m] - ld(p)).abs2()));
+            myerr = max_change(myerr, sqrt((x[m] - ld(p)).abs2()));
             st(p, x[m]);
             xch[tl][m] = x[m];
           }
@@ -650,7 +650,7 @@ __global__ void __launch_bounds__(256) k_rho(Dev d, int T) {
     for (int j = 0; j < NO2; ++j) x = cfma(Lm[tid * NO2 + j], b[j], x);
     x = x * zd(0, -xi);  // G^<(T,T) = -i xi rho
     S* p = el<NO, S>(d.GL, d, n, T, T);
-    e = sqrt((x - ld(p + tid)).abs2());
+    e = max_change(0.0, sqrt((x - ld(p + tid)).abs2()));
     st(p + tid, x);
     if (d.ring64[1]) st(el64<NO>(d, 1, n, T, T) + tid, x);
     if (!f64) st(d.diag64 + ((long long)n * d.nt + T) * NO2 + tid, x);
@@ -748,7 +748,7 @@ __global__ void __launch_bounds__(256) k_boot_mixed(Dev d) {
     for (int m = 1; m <= k; ++m)
       for (int x = 0; x < NO; ++x) {
         double2* p = tv<NO>(d.GTV, d, n, m, i) + x * NO + y;
-        e = max_mag(e, sqrt((b[(m - 1) * NO + x] - ld(p)).abs2()));
+        e = max_change(e, sqrt((b[(m - 1) * NO + x] - ld(p)).abs2()));
         st(p, b[(m - 1) * NO + x]);
       }
     atomic_max_nonneg(d.err + n, e);
@@ -800,7 +800,7 @@ __global__ void k_boot_ret(Dev d) {
       const int row = idx / NO, y = idx % NO;
       const int m = row / NO + c + 1, x = row % NO;
       S* p = el<NO, S>(d.GR, d, n, m, c) + x * NO + y;
-      e = max_mag(e, sqrt((sB[row * NO + y] - ld(p)).abs2()));
+      e = max_change(e, sqrt((sB[row * NO + y] - ld(p)).abs2()));
       st(p, sB[row * NO + y]);
     }
     __syncwarp();
@@ -830,7 +830,7 @@ __global__ void k_boot_les(Dev d) {
       for (int c = 0; c < r; ++c) s += ld(tv<NO>(d.GTV, d, n, m, c) + y * NO + x) * d.e0[c];
       x0s[lane] = -s.conj();
       S* p = el<NO, S>(d.GL, d, n, m, 0) + lane;
-      e = max_mag(e, sqrt((x0s[lane] - ld(p)).abs2()));
+      e = max_change(e, sqrt((x0s[lane] - ld(p)).abs2()));
       st(p, x0s[lane]);
     }
     for (int idx = lane; idx < r * NO2; idx += 32) {
@@ -886,7 +886,7 @@ __global__ void k_boot_les(Dev d) {
       const int t = row / NO + 1, x = row % NO;
       if (t > m) continue;
       S* p = el<NO, S>(d.GL, d, n, m, t) + x * NO + y;
-      e = max_mag(e, sqrt((sB[row * NO + y] - ld(p)).abs2()));
+      e = max_change(e, sqrt((sB[row * NO + y] - ld(p)).abs2()));
       st(p, sB[row * NO + y]);
     }
     __syncwarp();

@@ -27,6 +27,7 @@
 // T <= 64, and 820 of 1900 thousand at N_o = 4, T = 290; the two sweeps of
 // those runs went from 89 to 35 us and from 1650 to 1040 us.
 #include <algorithm>
+#include <type_traits>
 
 #include "bulk_copy.cuh"
 #include "hodlr_util.cuh"
@@ -66,17 +67,46 @@ enum { kAll = 0, kTop = 1, kLeaves = 2 };
 template <typename R>
 __device__ __forceinline__ auto reduce8(const KAcc<R>& k) { return kacc_lanes(k, 1, 8); }
 
-// |new - old|^2, old a stored element; in the complex64 form |new - old|, the
-// squares taken with the exponent set aside (squares of FP32 overflow from 1.8e19)
-__device__ __forceinline__ double vdist(const zd& a, const zd& o) { return (a - o).abs2(); }
-__device__ __forceinline__ float vdist(const cff& a, const zf& o) {
-  const float x = (a.re.hi - o.re) + a.re.lo, y = (a.im.hi - o.im) + a.im.lo;
-  const int e = min(max(__float_as_int(max_mag(x, y)) >> 23, 1), 253);
-  const float s = __int_as_float((254 - e) << 23), u = x * s, v = y * s;
-  return sqrtf(fmaf(u, u, v * v)) * __int_as_float(e << 23);
+// m: the largest |new - old|^2 of a thread, old a stored element; its root is the
+// measure of the iteration's change.  It sits at the end of every chunk of the
+// chain, so it stays one register: fmax would drop a NaN, and in FP64 a change that
+// is not finite goes to the CTA's measure serr at once; the complex64 form compares
+// the bits, in which a NaN is above infinity (change_out tells an overflow of the
+// square apart).  Bits in FP64 cost 1.5% (1 x 64: 10.15 -> 10.30 ms), a root per
+// element or a way of its own for large changes in the complex64 form 2%
+// (N_o = 2, 1 x 1089) and 1.0% (128 x 600).
+__device__ __forceinline__ void fold_change(double& m, const zd& a, const zd& o, double* serr) {
+  const double d = (a - o).abs2();
+  m = fmax(m, d);
+  if ((__double2hiint(d) & 0x7fffffff) >= 0x7ff00000) atomic_max_nonneg(serr, INFINITY);
 }
-__device__ __forceinline__ double vdist_out(double d) { return sqrt(d); }
-__device__ __forceinline__ double vdist_out(float d) { return d; }
+__device__ __forceinline__ void fold_change(float& m, const cff& a, const zf& o, double*) {
+  const float x = (a.re.hi - o.re) + a.re.lo, y = (a.im.hi - o.im) + a.im.lo;
+  m = __int_as_float(max(__float_as_int(m), __float_as_int(x * x + y * y) & 0x7fffffff));
+}
+// The warp's measure: bits in which a NaN is kept (complex64 form), or numbers.
+__device__ __forceinline__ double change_warp(double m) { return sqrt(warp_max(m)); }
+__device__ __forceinline__ double change_warp(float m) {
+  return sqrt((double)__int_as_float(__reduce_max_sync(FULL, __float_as_int(m))));
+}
+// The CTA's measure, by one thread: where a square left FP32 but every element of
+// the row (one component, elements `step` apart) is finite, the change was large,
+// at least the root of the largest square, and the step goes on.
+template <int NO, typename S>
+__device__ __forceinline__ double change_out(double e, const S* row, int T, int step) {
+  if constexpr (sizeof(S) == sizeof(float2)) {
+    if (!(e < INFINITY)) {
+      bool finite = true;
+      for (int t = 0; t <= T; ++t)
+        for (int j = 0; j < NO; ++j) {
+          const float2 v = row[(long long)t * NO * NO + j * step];
+          finite &= isfinite(v.x) && isfinite(v.y);
+        }
+      if (finite) e = 1.8446743e19;
+    }
+  }
+  return e;
+}
 __device__ __forceinline__ void vstore(double2* p, const zd& v) { st(p, v); }
 __device__ __forceinline__ void vstore(float2* p, const cff& v) { *p = make_float2(v.re.hi, v.im.hi); }
 // Where a sweep keeps the row it solves: in place (FP64 storage), or in FP64
@@ -393,7 +423,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
   Y* rowy = Row64<NO, S>::get(d, n, 0, T, rowp);
   auto yp = [&](int tp) { return rowy + (long long)tp * NO2 + irow * NO; };
   auto sp = [&](int tp) { return rowp + (long long)tp * NO2 + irow * NO; };
-  decltype(vdist(V(), cx<R>())) myerr = 0;
+  std::conditional_t<MX, float, double> myerr = 0;
   const bool below = part != kTop, above = part != kLeaves;   // the compressed columns; the head and the others
   if (staged && below && top >= 0 && c > 0)
     leaf_table<NO, R>(d, n, (min(c, top + 1) - 1) / L, true, sm.rk, sm.blk, tid);
@@ -422,7 +452,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
       if (sl == 0) {
         V v;
         vset(v, y);
-        myerr = max_mag(myerr, vdist(v, ldr<R>(sp(T - s) + j)));
+        fold_change(myerr, v, ldr<R>(sp(T - s) + j), &serr);
         Yl[(T - s) & 63][j] = v;
         st(yp(T - s) + j, y);
         if constexpr (MX) vstore(sp(T - s) + j, v);
@@ -432,7 +462,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
   if (above && tid < NO) {
     V v;
     vset(v, (tid == irow) ? zd(0, -1) : zd());
-    myerr = max_mag(myerr, vdist(v, ldr<R>(sp(T) + tid)));
+    fold_change(myerr, v, ldr<R>(sp(T) + tid), &serr);
     st(yp(T) + tid, v64(v));
     if constexpr (MX) vstore(sp(T) + tid, v);
   }
@@ -732,7 +762,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
 #pragma unroll
         for (int off = 1; off < 8; off <<= 1) out = vadd(out, vshfl_xor(out, off));
         if (sl == 0 && ti < cn) {
-          myerr = max_mag(myerr, vdist(out, Old[ti][j]));
+          fold_change(myerr, out, Old[ti][j], &serr);
           Yl[(a + ti) & 63][j] = out;
           vstore(sp(a + ti) + j, out);
         }
@@ -743,10 +773,10 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_ret2(Dev d, int T, i
     __syncthreads();
   }
   write64(wa, wn);
-  const double e1 = warp_max(vdist_out(myerr));
-  if (lane == 0) atomic_max_nonneg(&serr, e1);
+  const double e1 = change_warp(myerr);
+  if (lane == 0 && !(e1 <= 0)) atomic_max_nonneg(&serr, e1);
   __syncthreads();
-  if (tid == 0) atomic_max_nonneg(d.err + n, serr);
+  if (tid == 0) atomic_max_nonneg(d.err + n, change_out<NO, S>(serr, sp(0), T, 1));
   // after a timed-out wait, a copy may still be in flight into this CTA's
   // shared memory: wait for it (bounded) before the CTA exits
   if (kInvStage<NO> && tid == 0 && !s_stage) mbar_wait(&cbar, cphase ^ 1u, kCopyWaitPolls);
@@ -788,13 +818,14 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
     s_stage = 1;
     if (kInvStage<NO>) mbar_init(&cbar);
   }
+  __syncwarp();   // (serr, for the lanes that fold x(0))
   // FP64 column during the sweep (see k_ret2); xp: as solved, sp: storage
   S* colp = el<NO, S>(d.GL, d, n, T, 0);
   Y* coly = Row64<NO, S>::get(d, n, 1, T, colp);
   auto xp = [&](int t) { return coly + (long long)t * NO2; };  // element [m*NO + jc]
   auto sp = [&](int t) { return colp + (long long)t * NO2; };
   const double2* qs = d.qsrc + (long long)n * d.nt * NO2;
-  decltype(vdist(V(), cx<R>())) myerr = 0;
+  std::conditional_t<MX, float, double> myerr = 0;
   const int last = (d.rho_mode == 1) ? T - 1 : T;
   if (staged && c > 0 && part != kTop) leaf_table<NO, R>(d, n, 0, false, sm.rk, sm.blk, tid);
   if (part == kTop) {   // the points solved last by the part before
@@ -809,7 +840,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
     const zd x = ld(d.x0 + (long long)n * NO2 + m * NO + jc);
     V v;
     vset(v, x);
-    myerr = max_mag(myerr, vdist(v, ldr<R>(sp(0) + m * NO + jc)));
+    fold_change(myerr, v, ldr<R>(sp(0) + m * NO + jc), &serr);
     Xl[0][m] = v;
     st(xp(0) + m * NO + jc, x);
     if constexpr (MX) vstore(sp(0) + m * NO + jc, v);
@@ -1071,7 +1102,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
 #pragma unroll
         for (int off = 1; off < 8; off <<= 1) out = vadd(out, vshfl_xor(out, off));
         if (sl == 0 && ti < fn) {
-          myerr = max_mag(myerr, vdist(out, Old[ti][m]));
+          fold_change(myerr, out, Old[ti][m], &serr);
           Xl[(a + ti) & 63][m] = out;
           vstore(sp(a + ti) + m * NO + jc, out);
         }
@@ -1118,7 +1149,7 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
           for (int m = 0; m < NO; ++m) {
             V v;
             vset(v, x[m]);
-            myerr = max_mag(myerr, vdist(v, Old[fn][m]));
+            fold_change(myerr, v, Old[fn][m], &serr);
             st(xp(T) + m * NO + jc, x[m]);
             if constexpr (MX) vstore(sp(T) + m * NO + jc, v);
           }
@@ -1128,10 +1159,10 @@ __global__ void __launch_bounds__(256, (NO <= 2) ? 2 : 1) k_les2(Dev d, int T, i
     __syncthreads();
   }
   write64(wa, wn);
-  const double e1 = warp_max(vdist_out(myerr));
-  if (lane == 0) atomic_max_nonneg(&serr, e1);
+  const double e1 = change_warp(myerr);
+  if (lane == 0 && !(e1 <= 0)) atomic_max_nonneg(&serr, e1);
   __syncthreads();
-  if (tid == 0) atomic_max_nonneg(d.err + n, serr);
+  if (tid == 0) atomic_max_nonneg(d.err + n, change_out<NO, S>(serr, sp(0) + jc, T, NO));
   // after a timed-out wait, a copy may still be in flight into this CTA's
   // shared memory: wait for it (bounded) before the CTA exits
   if (kInvStage<NO> && tid == 0 && !s_stage) mbar_wait(&cbar, cphase ^ 1u, kCopyWaitPolls);

@@ -56,13 +56,13 @@ __global__ void __launch_bounds__(32) k_ret_sf_start(Dev d, int T) {
   for (int row = lane; row < ns; row += 32) {
     const int s = row / NO + 1, j = row % NO;
     double2* p = el<NO, S>(d.GR, d, n, T, T - s) + irow * NO + j;
-    err = max_mag(err, sqrt((sB[row] - ld(p)).abs2()));
+    err = max_change(err, sqrt((sB[row] - ld(p)).abs2()));
     st(p, sB[row]);
   }
   if (lane < NO) {
     double2* p = el<NO, S>(d.GR, d, n, T, T) + irow * NO + lane;
     const zd v = lane == irow ? zd(0, -1) : zd();
-    err = max_mag(err, sqrt((v - ld(p)).abs2()));
+    err = max_change(err, sqrt((v - ld(p)).abs2()));
     st(p, v);
   }
   err = warp_max(err);

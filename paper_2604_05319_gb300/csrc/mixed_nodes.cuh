@@ -132,14 +132,14 @@ __device__ __forceinline__ void mixed_nodes(const Dev& d, int T, int group, int 
 #pragma unroll
     for (int m = 0; m < NO; ++m) v = cfma(Mi[x * NO + m], rs[i * NO2 + m * NO + y], v);
     double2* p = tv<NO>(d.GTV, d, n, T, i0) + tid;
-    e = sqrt((v - ld(p)).abs2());
+    e = max_change(0.0, sqrt((v - ld(p)).abs2()));
     st(p, v);
   }
   e = warp_max(e);
   if (lane == 0) serr[warp] = e;
   __syncthreads();
   if (tid == 0) {
-    for (int w2 = 1; w2 < 8; ++w2) e = max_mag(e, serr[w2]);
+    for (int w2 = 1; w2 < 8; ++w2) e = fmax(e, serr[w2]);
     atomic_max_nonneg(d.err + n, e);
   }
 }
